@@ -49,6 +49,7 @@ struct Ctx {
     PhaseTimer *tm = nullptr;   // optional phase timing and launch counting
     int ph_hash = kPhNumHash, ph_dense = kPhNumDense;
     bool stage_items = false;   // heavy items take their counts from pcnt_in
+    bool sort = false;          // the pass writes C itself in row order (opts.sort_output)
     const int64_t *f = nullptr; // flops per column of the full product (hybrid accumulator)
     int tbegin(int phase, cudaStream_t st) const { return tm ? tm->begin(phase, st) : -1; }
     void tend(int idx, cudaStream_t st) const { if (tm) tm->end(idx, st); }
@@ -75,6 +76,7 @@ inline TierCommon common_of(const Ctx &c) {
     t.P = c.P; t.log2R = c.tun.log2R; t.Rs = c.Rs; t.Q = c.Q;
     t.flops = c.f;
     t.hybrid_sort = c.tun.hybrid_sort;
+    t.sort = c.sort ? 1 : 0;
     return t;
 }
 
@@ -1001,7 +1003,10 @@ template <class I, class V> struct Engine : EngineBase {
         Ctx cx = make_ctx(ps);
         const int64_t n = ps.n;
         const int64_t *hc = ps.h_colptr.as<int64_t>();
+        // the pass that writes C (not the stages of a k-split)
+        const bool sort = ps.opts.sort_output && !ps.defer_sort;
         if (ps.s == 1) {
+            cx.sort = sort;
             NumOut<I, V> o{ps.colptr.as<int64_t>(), hc[b.c0], (I *)C->rowidx, (V *)C->vals};
             GA ga = gemm_args(ps, 0, ps.k);
             SPG_ST((num_pass<SrcGemm<I, V>, SrcPanel<I, V>, SrcPanelRange<I, V>>(
@@ -1037,6 +1042,7 @@ template <class I, class V> struct Engine : EngineBase {
             // sort-free hash merge of the stage partials (Sec. IV-D)
             cx.ph_hash = kPhMerge;
             cx.ph_dense = kPhMerge;
+            cx.sort = sort;
             PA pa{ps.parts_tab.as<PartDev<I, V>>() + (size_t)t * ps.s, ps.s, ps.m};
             NumOut<I, V> o{ps.colptr.as<int64_t>(), hc[b.c0], (I *)C->rowidx, (V *)C->vals};
             SPG_ST((num_pass<SrcParts<I, V>, SrcPartsPanel<I, V>, SrcPartsRange<I, V>>(
@@ -1046,10 +1052,11 @@ template <class I, class V> struct Engine : EngineBase {
                 ps.list_num.as<int32_t>(), ps.off_num.as<int32_t>(), st, ps.items.as<HeavyItem>(),
                 bitems.n, bitems.order)));
         }
-        if (ps.opts.sort_output && !ps.defer_sort)
-            SPG_ST(sort_batch(cx, ps.colptr.as<int64_t>(), hc[b.c0], b.c0, b.c1, (I *)C->rowidx, (V *)C->vals,
-                              b.heavy > 0 ? ps.items.as<HeavyItem>() : nullptr,
-                              ps.item_off.as<int64_t>() + ps.nheavy, ps.n_items, st));
+        // the hash tiers wrote their columns in row order, dense items are in row
+        // order: what is left are the hash-range items of the heavy columns
+        if (sort && b.heavy > 0)
+            SPG_ST(sort_items(cx, ps.colptr.as<int64_t>(), hc[b.c0], b.c0, b.c1, (I *)C->rowidx, (V *)C->vals,
+                              ps.items.as<HeavyItem>(), ps.item_off.as<int64_t>() + ps.nheavy, ps.n_items, st));
         SPG_CK(rebase_colptr(ps.colptr.as<int64_t>() + b.c0, b.c1 - b.c0, C->colptr,
                              C->ptr_type == SPGEMM_I64, st));
         cx.launched();
@@ -1105,6 +1112,7 @@ template <class I, class V> struct Engine : EngineBase {
             } else {
                 NumOut<I, V> oc{ps.colptr.as<int64_t>(), hc[b.c0], (I *)C->rowidx, (V *)C->vals};
                 cx.stage_items = false;
+                cx.sort = ps.opts.sort_output && !ps.defer_sort;
                 SPG_ST((num_pass<SrcParts<I, V>, SrcPartsPanel<I, V>, SrcPartsRange<I, V>>(
                     cx, pa, pa, b.c0, b.c1, ps.cnt.as<int64_t>(), ps.cnt.as<int64_t>(), oc, b.tc[0].data(),
                     b.heavy > 0, ps.list_sym.as<int32_t>(), ps.off_sym.as<int32_t>(),
@@ -1118,25 +1126,12 @@ template <class I, class V> struct Engine : EngineBase {
     }
 
     // ---- sorted output and prune ---------------------------------------------
-    // Sort the rows of columns [c0, c1) of a batch in place: the light columns
-    // (warp bitonic up to 32 entries, shared-memory bitonic up to 8192) and the
-    // hash-range items of the heavy columns; dense items are in row order.
-    // colptr: the plan's global offsets, base = offset of column c0.
-    static spgemm_status sort_batch(const Ctx &cx, const int64_t *colptr, int64_t base, int64_t c0,
+    // Sort the hash-range items of the heavy columns in [c0, c1) of a batch in
+    // place. colptr: the plan's global offsets, base = offset of column c0.
+    static spgemm_status sort_items(const Ctx &cx, const int64_t *colptr, int64_t base, int64_t c0,
                                     int64_t c1, I *rows, V *vals, const HeavyItem *items,
                                     const int64_t *nitems_dev, int64_t n_items, cudaStream_t st) {
-        const int64_t nc = c1 - c0;
-        if (nc <= 0) return SPGEMM_OK;
-        const unsigned wb = (unsigned)std::max<int64_t>(1, std::min<int64_t>((nc + 7) / 8, 1 << 20));
-        k_sort_warp<I, V><<<wb, 256, 0, st>>>(colptr, base, c0, c1, rows, vals);
-        const int cap = cx.tun.hash_cap_max;
-        const unsigned bb = (unsigned)std::max<int64_t>(1, std::min<int64_t>(nc, (int64_t)cx.nsm * 8));
-        k_sort_block<I, V, 1024><<<bb, 256, (int)(1024 * (4 + sizeof(V))), st>>>(colptr, base, c0, c1, 32,
-                                                                                 cap, rows, vals);
-        if (cap > 1024)
-            k_sort_block<I, V, 8192><<<bb, 512, (int)(8192 * (4 + sizeof(V))), st>>>(colptr, base, c0, c1,
-                                                                                   1024, cap, rows, vals);
-        if (items && n_items > 0) {
+        if (n_items > 0) {
             // staging for the largest hash item (range_cap rows), a bitmap
             // over item row ranges of up to 16 panels and its 16-bit word
             // prefix (wider ranges fall back to the bitonic sort); two CTAs
@@ -1155,7 +1150,7 @@ template <class I, class V> struct Engine : EngineBase {
             if (range_cap(cx) <= 4096) launch(std::integral_constant<int, 4096>{});
             else launch(std::integral_constant<int, 8192>{});
         }
-        cx.launched(items ? 4 : 3);
+        cx.launched();
         SPG_CK(cudaGetLastError());
         return SPGEMM_OK;
     }

@@ -87,6 +87,7 @@ struct TierCommon {
     int range_cap;             // heavy hash items: at most this many output rows
     const int64_t *flops;      // flops per global column (hybrid accumulator), or null
     int hybrid_sort;           // CTA tiers: sort-accumulate columns with flops <= table size
+    int sort;                  // numeric tiers: write every column in row order
 };
 
 template <class I, class V> struct GemmArgs {
@@ -987,8 +988,15 @@ __global__ void __launch_bounds__(1024, 1) k_sym_bitmap(typename Src::Args sa, T
     }
 }
 
+}  // namespace spg
+
+#include "sort_smem.cuh"
+
+namespace spg {
+
 // ---------------------------------------------------------------------------
-// K3 / K4: numeric hash tiers (products or merge), unsorted output
+// K3 / K4: numeric hash tiers (products or merge); rows in table order, or
+// ascending with c.sort
 // ---------------------------------------------------------------------------
 template <class Src, int T>
 __global__ void __launch_bounds__(256) k_num_warp(typename Src::Args sa, TierCommon c,
@@ -1020,6 +1028,10 @@ __global__ void __launch_bounds__(256) k_num_warp(typename Src::Args sa, TierCom
         __syncwarp();
         const int64_t out0 = c.colptr[g] - c.out_base;
         const int64_t want = c.colptr[g + 1] - c.colptr[g];
+        if (c.sort) {
+            sorted_emit<false>(keys, vals, T, (int)want, nullptr, c.err, out_rows + out0, out_vals + out0);
+            continue;
+        }
         int pos = 0;
         for (int s0 = 0; s0 < T; s0 += 32) {
             const int s = s0 + lane;
@@ -1039,32 +1051,6 @@ __global__ void __launch_bounds__(256) k_num_warp(typename Src::Args sa, TierCom
         }
         if (lane == 0 && pos != want) atomicOr(c.err, kErrCount);
         __syncwarp();
-    }
-}
-
-// Bitonic sort of one segment of n <= CAP entries in shared memory (keys
-// padded with 0xffffffff to the next power of two). All threads call it.
-template <int CAP, class V>
-__device__ __forceinline__ void block_bitonic(uint32_t *sk, V *sv, int n) {
-    int np2 = 1;
-    while (np2 < n) np2 <<= 1;
-    for (int i = n + threadIdx.x; i < np2; i += blockDim.x) { sk[i] = 0xffffffffu; sv[i] = V(0); }
-    __syncthreads();
-    for (int k = 2; k <= np2; k <<= 1) {
-        for (int jj = k >> 1; jj > 0; jj >>= 1) {
-            for (int i = threadIdx.x; i < np2; i += blockDim.x) {
-                const int l = i ^ jj;
-                if (l > i) {
-                    const bool up = (i & k) == 0;
-                    const uint32_t a = sk[i], b = sk[l];
-                    if (up ? a > b : a < b) {
-                        sk[i] = b; sk[l] = a;
-                        const V t = sv[i]; sv[i] = sv[l]; sv[l] = t;
-                    }
-                }
-            }
-            __syncthreads();
-        }
     }
 }
 
@@ -1137,7 +1123,7 @@ __device__ __forceinline__ void num_block_sorted(const Src &src, const TierCommo
 }
 
 template <class Src, int T>
-__global__ void k_num_block(typename Src::Args sa, TierCommon c, typename Src::Idx *out_rows,
+__global__ void __launch_bounds__(1024) k_num_block(typename Src::Args sa, TierCommon c, typename Src::Idx *out_rows,
                             typename Src::Val *out_vals) {
     constexpr int LOG2T = Log2<T>::v;
     using V = typename Src::Val;
@@ -1146,6 +1132,7 @@ __global__ void k_num_block(typename Src::Args sa, TierCommon c, typename Src::I
     V *vals = reinterpret_cast<V *>(smem);
     uint32_t *keys = reinterpret_cast<uint32_t *>(smem + sizeof(V) * T);
     __shared__ BlockShared<V> sh;
+    __shared__ SortShared ss;
     __shared__ int s_it;
     if (threadIdx.x == 0) { sh.pos = 0; }
     const int lo = c.list_off[c.tier], hi = c.list_off[c.tier + 1];
@@ -1189,6 +1176,10 @@ __global__ void k_num_block(typename Src::Args sa, TierCommon c, typename Src::I
                 if (h >= 0) atomic_add_v(&vals[h], e.x);
             });
         block_walk<kWalkBatch>(src, emit, c.short_seg, c.huge_seg, sh);
+        if (c.sort) {
+            sorted_emit<true>(keys, vals, T, (int)want, &ss, c.err, out_rows + out0, out_vals + out0);
+            continue;
+        }
         for (int s0 = 0; s0 < T; s0 += blockDim.x) {
             const int s = s0 + threadIdx.x;
             const uint32_t key = s < T ? keys[s] : kEmpty;
