@@ -59,8 +59,8 @@ void free_mem(const AllocFns &a, void *p, size_t bytes, int kind) {
 }
 
 size_t PlanState::workspace_bytes() const {
-    const DevBuf *bufs[] = {&probs, &f, &cnt, &colptr, &tier, &list_sym, &list_num, &hist, &cursor,
-                            &off_sym, &off_num, &heavy_ord, &pcnt, &err, &scan_part, &wbytes,
+    const DevBuf *bufs[] = {&probs, &f, &cnt, &colptr, &tier, &list_sym, &list_num, &hist,
+                            &off_sym, &off_num, &heavy_ord, &pcnt, &err, &scan_part, &f_stage,
                             &valid_flag, &ap_end, &ap_row, &ap_val, &apc_off, &apc_row, &apc_val, &stage_cnt, &stage_colptr,
                             &stage_pcnt, &merge_tmp, &drows, &dvals, &parts_tab, &items, &item_cnt,
                             &item_off, &item_order, &pref_cnt, &pref_colptr, &pref_pcnt};
@@ -70,8 +70,8 @@ size_t PlanState::workspace_bytes() const {
 }
 
 void PlanState::release_all() {
-    DevBuf *bufs[] = {&probs, &f, &cnt, &colptr, &tier, &list_sym, &list_num, &hist, &cursor,
-                      &off_sym, &off_num, &heavy_ord, &pcnt, &err, &scan_part, &wbytes,
+    DevBuf *bufs[] = {&probs, &f, &cnt, &colptr, &tier, &list_sym, &list_num, &hist,
+                      &off_sym, &off_num, &heavy_ord, &pcnt, &err, &scan_part, &f_stage,
                       &valid_flag, &ap_end, &ap_row, &ap_val, &apc_off, &apc_row, &apc_val, &stage_cnt, &stage_colptr,
                       &stage_pcnt, &merge_tmp, &drows, &dvals, &parts_tab, &items, &item_cnt,
                       &item_off, &item_order, &pref_cnt, &pref_colptr, &pref_pcnt};
@@ -386,7 +386,7 @@ spgemm_status spgemm_backward(spgemm_plan *plan, const spgemm_csc *G, void *dA_v
 
 namespace spg {
 void MultiState::release_all() {
-    DevBuf *bufs[] = {&probs, &f, &cnt, &colptr, &tier, &list, &off, &hist, &cursor, &err,
+    DevBuf *bufs[] = {&probs, &f, &cnt, &colptr, &tier, &list, &off, &hist, &err,
                       &scan_part, &rows, &vals, &counter, &gsize, &gtab_off, &gkeys, &gvals};
     for (auto *b : bufs) b->release();
     h_small.release();

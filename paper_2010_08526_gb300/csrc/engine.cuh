@@ -36,13 +36,19 @@ inline int block_tier_threads(int T, const Tuning &tun) {
     return 1024;
 }
 
+// The binning words of a pass, zeroed together: [0, 16) tier histogram,
+// [kFlopTotal, +2) total multiplications (64 bits), [64, 128) list cursors
+// and the work counters of the persistent kernels.
+constexpr int kBinInts = 128;
+constexpr int kFlopTotal = 32;
+
 // Scratch shared by one symbolic / numeric pass.
 struct Ctx {
     int nsm;
     Tuning tun;
     int *err;
-    int32_t *hist;       // 64 ints
-    int32_t *cursor;     // 64 ints
+    int32_t *hist;       // kBinInts ints: tier histogram, flop total, cursors
+    int32_t *cursor;     // hist + 64: list cursors, work counters
     int32_t *h_small;    // pinned host, >= 64 ints
     int P, Q;
     int64_t Rs;
@@ -60,7 +66,7 @@ inline Ctx make_ctx(PlanState &ps) {
     Ctx c;
     c.tm = &ps.timer;
     c.nsm = ps.nsm; c.tun = ps.tun; c.err = ps.err.as<int>();
-    c.hist = ps.hist.as<int32_t>(); c.cursor = ps.cursor.as<int32_t>();
+    c.hist = ps.hist.as<int32_t>(); c.cursor = c.hist + 64;
     c.h_small = ps.h_small.as<int32_t>();
     c.P = ps.P; c.Q = ps.Q; c.Rs = ps.Rs;
     c.f = ps.f.as<int64_t>();
@@ -331,19 +337,31 @@ template <class I, class V> struct Engine : EngineBase {
     // Bins columns [c_lo, c_hi) of the source, counts distinct rows into
     // cnt_out, fills list/off; heavy columns get per-panel counts in pcnt.
     // heavy_ord_w (optional) receives the heavy ordinals (full pass only).
+    // Products: f receives the multiplications per column, total_out their
+    // sum, and nnz_b is the number of B entries.
     template <class Src>
     static spgemm_status sym_pass(const Ctx &cx, const typename Src::Args &sa, int64_t c_lo, int64_t c_hi,
-                           const int64_t *bound, int64_t *f_out, uint8_t *tier, int64_t *cnt_out,
+                           const int64_t *bound, int64_t *f, uint8_t *tier, int64_t *cnt_out,
                            int32_t *list, int32_t *off, int32_t *heavy_ord_w,
                            const int32_t *heavy_ord_r, DevBuf *pcnt_grow, int32_t *pcnt_ptr,
-                           int *hist_out, cudaStream_t st, bool allow_heavy = true) {
+                           int *hist_out, cudaStream_t st, bool allow_heavy = true, int64_t nnz_b = 0,
+                           int64_t *total_out = nullptr) {
         const int64_t nc = c_hi - c_lo;
-        SPG_CK(cudaMemsetAsync(cx.hist, 0, sizeof(int32_t) * 64, st));
-        SPG_CK(cudaMemsetAsync(cx.cursor, 0, sizeof(int32_t) * 64, st));
+        SPG_CK(cudaMemsetAsync(cx.hist, 0, sizeof(int32_t) * kBinInts, st));
         if (nc > 0) {
             const int tb = cx.tbegin(kPhFlopsBin, st);
-            k_flops_bin<Src><<<(unsigned)((nc + 255) / 256), 256, 0, st>>>(
-                sa, c_lo, c_hi, cx.tun.hash_cap_max, bound, f_out, tier, cnt_out, cx.hist);
+            if constexpr (!Src::kParts) {   // all columns of one product
+                SPG_CK(cudaMemsetAsync(f, 0, sizeof(int64_t) * (size_t)nc, st));
+                const int64_t per = 256 * kFlopsEntries;
+                if (nnz_b > 0) {
+                    k_col_flops<I, V><<<(unsigned)((nnz_b + per - 1) / per), 256, 0, st>>>(
+                        sa, nc, reinterpret_cast<unsigned long long *>(f),
+                        reinterpret_cast<unsigned long long *>(cx.hist + kFlopTotal));
+                    cx.launched();
+                }
+            }
+            k_col_tier<Src><<<(unsigned)((nc + 255) / 256), 256, 0, st>>>(
+                sa, c_lo, c_hi, cx.tun.hash_cap_max, bound, f, tier, cnt_out, cx.hist);
             k_bin_scatter<<<(unsigned)((nc + 255) / 256), 256, 0, st>>>(tier, c_lo, c_hi, cx.hist,
                                                                        cx.cursor, list, off,
                                                                        heavy_ord_w);
@@ -351,10 +369,11 @@ template <class I, class V> struct Engine : EngineBase {
             cx.launched(2);
             SPG_CK(cudaGetLastError());
         }
-        SPG_CK(cudaMemcpyAsync(cx.h_small, cx.hist, sizeof(int32_t) * 16, cudaMemcpyDeviceToHost, st));
+        SPG_CK(cudaMemcpyAsync(cx.h_small, cx.hist, sizeof(int32_t) * (kFlopTotal + 2), cudaMemcpyDeviceToHost, st));
         SPG_CK(cudaStreamSynchronize(st));
         int hist[16];
         std::memcpy(hist, cx.h_small, sizeof(hist));
+        if (total_out) std::memcpy(total_out, cx.h_small + kFlopTotal, sizeof(int64_t));
         if (nc <= 0) std::memset(hist, 0, sizeof(hist));
         if (hist_out) std::memcpy(hist_out, hist, sizeof(hist));
         int nheavy = 0;
@@ -418,8 +437,7 @@ template <class I, class V> struct Engine : EngineBase {
         c.out_base = o.out_base;
         if (any_hash && nc > 0) {
             const int th = cx.tbegin(cx.ph_hash, st);
-            SPG_CK(cudaMemsetAsync(cx.hist, 0, sizeof(int32_t) * 64, st));
-            SPG_CK(cudaMemsetAsync(cx.cursor, 0, sizeof(int32_t) * 64, st));
+            SPG_CK(cudaMemsetAsync(cx.hist, 0, sizeof(int32_t) * kBinInts, st));
             k_numeric_tier<<<(unsigned)((nc + 255) / 256), 256, 0, st>>>(
                 cnt, dense_sel, c_lo, c_hi, cx.tun.hash_cap_max, tier, cx.hist);
             k_bin_scatter<<<(unsigned)((nc + 255) / 256), 256, 0, st>>>(
@@ -544,13 +562,12 @@ template <class I, class V> struct Engine : EngineBase {
         SPG_CK(ps.f.ensure(sizeof(int64_t) * (n + 1)));
         SPG_CK(ps.cnt.ensure(sizeof(int64_t) * (n + 1)));
         SPG_CK(ps.colptr.ensure(sizeof(int64_t) * (n + 1)));
-        SPG_CK(ps.wbytes.ensure(sizeof(int64_t) * (n + 1)));
+        if (ps.s > 1) SPG_CK(ps.f_stage.ensure(sizeof(int64_t) * (n + 1)));
         SPG_CK(ps.tier.ensure(n + 16));
         SPG_CK(ps.list_sym.ensure(sizeof(int32_t) * (n + 1)));
         SPG_CK(ps.list_num.ensure(sizeof(int32_t) * (n + 1)));
         SPG_CK(ps.heavy_ord.ensure(sizeof(int32_t) * (n + 1)));
-        SPG_CK(ps.hist.ensure(sizeof(int32_t) * 64));
-        SPG_CK(ps.cursor.ensure(sizeof(int32_t) * 64));
+        SPG_CK(ps.hist.ensure(sizeof(int32_t) * kBinInts));
         SPG_CK(ps.off_sym.ensure(sizeof(int32_t) * 64));
         SPG_CK(ps.off_num.ensure(sizeof(int32_t) * 64));
         SPG_CK(ps.err.ensure(sizeof(int) * 4));
@@ -577,10 +594,10 @@ template <class I, class V> struct Engine : EngineBase {
                                        ps.tier.as<uint8_t>(), ps.cnt.as<int64_t>(),
                                        ps.list_sym.as<int32_t>(), ps.off_sym.as<int32_t>(),
                                        ps.heavy_ord.as<int32_t>(), ps.heavy_ord.as<int32_t>(),
-                                       &ps.pcnt, nullptr, ps.sym_hist, st));
+                                       &ps.pcnt, nullptr, ps.sym_hist, st, true, ps.B.nnz, &ps.flops));
         ps.nheavy = 0;
         for (int t = kHeavyTier0; t < kTiers; ++t) ps.nheavy += ps.sym_hist[t];
-        int tsc = cx.tbegin(kPhScan, st);
+        const int tsc = cx.tbegin(kPhScan, st);
         SPG_CK(exclusive_scan_i64(ps.cnt.as<int64_t>(), n, ps.colptr.as<int64_t>(),
                                   ps.scan_part.as<int64_t>(), 1, st));
         cx.tend(tsc, st);
@@ -596,10 +613,10 @@ template <class I, class V> struct Engine : EngineBase {
                 int32_t *spc = ps.nheavy ? ps.stage_pcnt.as<int32_t>() + (size_t)t * ps.nheavy * ps.P
                                          : nullptr;
                 SPG_ST(sym_pass<SrcGemm<I, V>>(cx, gemm_args(ps, k0, k1), 0, n, ps.cnt.as<int64_t>(),
-                                               nullptr, ps.tier.as<uint8_t>(), scnt,
+                                               ps.f_stage.as<int64_t>(), ps.tier.as<uint8_t>(), scnt,
                                                ps.list_num.as<int32_t>(), ps.off_num.as<int32_t>(),
                                                nullptr, ps.heavy_ord.as<int32_t>(), nullptr, spc,
-                                               nullptr, st));
+                                               nullptr, st, true, ps.B.nnz));
                 SPG_CK(exclusive_scan_i64(scnt, n, ps.stage_colptr.as<int64_t>() + (size_t)t * (n + 1),
                                           ps.scan_part.as<int64_t>(), 1, st));
                 cx.launched(3);
@@ -622,10 +639,10 @@ template <class I, class V> struct Engine : EngineBase {
                     int32_t *pp = ps.nheavy ? ps.pref_pcnt.as<int32_t>() + (size_t)(u - 1) * ps.nheavy * ps.P
                                             : nullptr;
                     SPG_ST(sym_pass<SrcGemm<I, V>>(cx, gemm_args(ps, 0, k1), 0, n, ps.cnt.as<int64_t>(),
-                                                   nullptr, ps.tier.as<uint8_t>(), pc,
+                                                   ps.f_stage.as<int64_t>(), ps.tier.as<uint8_t>(), pc,
                                                    ps.list_num.as<int32_t>(), ps.off_num.as<int32_t>(),
                                                    nullptr, ps.heavy_ord.as<int32_t>(), nullptr, pp,
-                                                   nullptr, st));
+                                                   nullptr, st, true, ps.B.nnz));
                     SPG_CK(exclusive_scan_i64(pc, n, ps.pref_colptr.as<int64_t>() + (size_t)(u - 1) * (n + 1),
                                               ps.scan_part.as<int64_t>(), 1, st));
                     cx.launched(3);
@@ -637,13 +654,6 @@ template <class I, class V> struct Engine : EngineBase {
         SPG_CK(cudaMemcpyAsync(ps.h_colptr.p, ps.colptr.p, sizeof(int64_t) * (n + 1),
                                cudaMemcpyDeviceToHost, st));
         SPG_CK(cudaMemcpyAsync(ps.h_small.as<char>() + 256, ps.err.p, sizeof(int), cudaMemcpyDeviceToHost, st));
-        tsc = cx.tbegin(kPhScan, st);
-        SPG_CK(exclusive_scan_i64(ps.f.as<int64_t>(), n, ps.wbytes.as<int64_t>(),
-                                  ps.scan_part.as<int64_t>(), 1, st));
-        cx.tend(tsc, st);
-        cx.launched(3);
-        SPG_CK(cudaMemcpyAsync(ps.h_small.as<char>() + 512, ps.wbytes.as<int64_t>() + n, sizeof(int64_t),
-                               cudaMemcpyDeviceToHost, st));
         if (ps.nheavy) SPG_ST(build_panels(ps, st));
         // products alone: a hash item may span any number of panels (one run
         // of the column-grouped copy of A); sorted output and the k-split's
@@ -659,7 +669,6 @@ template <class I, class V> struct Engine : EngineBase {
             set_error("symbolic: device error flags " + std::to_string(errw));
             return SPGEMM_ERR_OVERFLOW;
         }
-        ps.flops = *(int64_t *)(ps.h_small.as<char>() + 512);
         ps.nnz_c = ps.h_colptr.as<int64_t>()[n];
         SPG_ST(plan_batches(ps));
         SPG_ST(order_items_by_batch(ps, st));
@@ -1310,8 +1319,7 @@ template <class I, class V> struct Engine : EngineBase {
             k_fill_zero<V><<<(unsigned)((ps.B.nnz + 255) / 256), 256, 0, st>>>((V *)dB, ps.B.nnz);
         cx.launched(2);
         if (n == 0) { cx.tend(tbw, st); return SPGEMM_OK; }
-        SPG_CK(cudaMemsetAsync(cx.hist, 0, sizeof(int32_t) * 64, st));
-        SPG_CK(cudaMemsetAsync(cx.cursor, 0, sizeof(int32_t) * 64, st));
+        SPG_CK(cudaMemsetAsync(cx.hist, 0, sizeof(int32_t) * kBinInts, st));
         k_bwd_tier<I, V><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(ga, n, cx.tun.hash_cap_max,
                                                                        ps.tier.as<uint8_t>(), cx.hist);
         k_bin_scatter<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(
@@ -1401,8 +1409,7 @@ template <class I, class V> struct Engine : EngineBase {
         SPG_CK(tmp.list_sym.ensure(sizeof(int32_t) * (n + 1)));
         SPG_CK(tmp.list_num.ensure(sizeof(int32_t) * (n + 1)));
         SPG_CK(tmp.heavy_ord.ensure(sizeof(int32_t) * (n + 1)));
-        SPG_CK(tmp.hist.ensure(sizeof(int32_t) * 64));
-        SPG_CK(tmp.cursor.ensure(sizeof(int32_t) * 64));
+        SPG_CK(tmp.hist.ensure(sizeof(int32_t) * kBinInts));
         SPG_CK(tmp.off_sym.ensure(sizeof(int32_t) * 64));
         SPG_CK(tmp.off_num.ensure(sizeof(int32_t) * 64));
         SPG_CK(tmp.err.ensure(sizeof(int) * 4));
@@ -1467,7 +1474,7 @@ template <class I, class V> struct Engine : EngineBase {
     static size_t merge_noalloc_bytes(int64_t n, int nparts) {
         auto al = [](size_t x) { return (x + 255) / 256 * 256; };
         return al(sizeof(int64_t) * (n + 1)) * 2 + al(n + 16) + al(sizeof(int32_t) * (n + 1)) * 3 +
-               al(sizeof(int32_t) * 64) * 4 + al(sizeof(int) * 4) +
+               al(sizeof(int32_t) * kBinInts) + al(sizeof(int32_t) * 64) * 2 + al(sizeof(int) * 4) +
                al(sizeof(int64_t) * scan_partials_len(n + 1)) + al(sizeof(PartDev<I, V>) * nparts);
     }
 
@@ -1492,8 +1499,7 @@ template <class I, class V> struct Engine : EngineBase {
         int32_t *list_sym = (int32_t *)take(sizeof(int32_t) * (n + 1));
         int32_t *list_num = (int32_t *)take(sizeof(int32_t) * (n + 1));
         int32_t *heavy_ord = (int32_t *)take(sizeof(int32_t) * (n + 1));
-        int32_t *hist = (int32_t *)take(sizeof(int32_t) * 64);
-        int32_t *cursor = (int32_t *)take(sizeof(int32_t) * 64);
+        int32_t *hist = (int32_t *)take(sizeof(int32_t) * kBinInts);
         int32_t *off_sym = (int32_t *)take(sizeof(int32_t) * 64);
         int32_t *off_num = (int32_t *)take(sizeof(int32_t) * 64);
         int *err = (int *)take(sizeof(int) * 4);
@@ -1515,7 +1521,7 @@ template <class I, class V> struct Engine : EngineBase {
         SPG_CK(cudaMemsetAsync(err, 0, sizeof(int) * 4, st));
         Ctx cx;
         cx.nsm = nsm;
-        cx.err = err; cx.hist = hist; cx.cursor = cursor; cx.h_small = h_stage;
+        cx.err = err; cx.hist = hist; cx.cursor = hist + 64; cx.h_small = h_stage;
         cx.tun.log2R = sizeof(V) == 4 ? 14 : 13;
         cx.P = 1; cx.Q = 1; cx.Rs = 32;
         PA pa{tab_d, nparts, m};
@@ -1560,7 +1566,7 @@ template <class I, class V> struct Engine : EngineBase {
     static Ctx multi_ctx(MultiState &ms) {
         Ctx c;
         c.nsm = ms.nsm; c.tun = ms.tun; c.err = ms.err.as<int>();
-        c.hist = ms.hist.as<int32_t>(); c.cursor = ms.cursor.as<int32_t>();
+        c.hist = ms.hist.as<int32_t>(); c.cursor = c.hist + 64;
         c.h_small = ms.h_small.as<int32_t>();
         c.P = 1; c.Q = 1; c.Rs = 32;
         return c;
@@ -1596,8 +1602,7 @@ template <class I, class V> struct Engine : EngineBase {
         SPG_CK(ms.tier.ensure(n + 16));
         SPG_CK(ms.list.ensure(sizeof(int32_t) * (n + 1)));
         SPG_CK(ms.off.ensure(sizeof(int32_t) * 64));
-        SPG_CK(ms.hist.ensure(sizeof(int32_t) * 64));
-        SPG_CK(ms.cursor.ensure(sizeof(int32_t) * 64));
+        SPG_CK(ms.hist.ensure(sizeof(int32_t) * kBinInts));
         SPG_CK(ms.err.ensure(sizeof(int) * 4));
         SPG_CK(ms.scan_part.ensure(sizeof(int64_t) * scan_partials_len(n + 1)));
         SPG_CK(ms.h_small.ensure(4096));
@@ -1607,7 +1612,7 @@ template <class I, class V> struct Engine : EngineBase {
         SPG_CK(cudaMemsetAsync(cx.hist, 0, sizeof(int32_t) * 64, st));
         if (n > 0)
             k_flops_bin<SrcGemm<I, V>><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(
-                multi_args(ms), 0, n, cx.tun.hash_cap_max, nullptr, ms.f.as<int64_t>(),
+                multi_args(ms), 0, n, cx.tun.hash_cap_max, ms.f.as<int64_t>(),
                 ms.tier.as<uint8_t>(), ms.cnt.as<int64_t>(), cx.hist);
         SPG_CK(cudaGetLastError());
         SPG_CK(exclusive_scan_i64(ms.f.as<int64_t>(), n, ms.colptr.as<int64_t>(),
@@ -1668,13 +1673,12 @@ template <class I, class V> struct Engine : EngineBase {
         Ctx cx = multi_ctx(ms);
         const int64_t n = ms.total_cols;
         GA ga = multi_args(ms);
-        SPG_CK(cudaMemsetAsync(cx.hist, 0, sizeof(int32_t) * 64, st));
-        SPG_CK(cudaMemsetAsync(cx.cursor, 0, sizeof(int32_t) * 64, st));
+        SPG_CK(cudaMemsetAsync(cx.hist, 0, sizeof(int32_t) * kBinInts, st));
         SPG_CK(cudaMemsetAsync(ms.counter.p, 0, sizeof(unsigned long long) * 4, st));
         if (n > 0) {
             // tiers by the flop bound min(f_j, m), the same as at creation
             k_flops_bin<SrcGemm<I, V>><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(
-                ga, 0, n, cx.tun.hash_cap_max, nullptr, nullptr, ms.tier.as<uint8_t>(),
+                ga, 0, n, cx.tun.hash_cap_max, nullptr, ms.tier.as<uint8_t>(),
                 ms.cnt.as<int64_t>(), cx.hist);
             k_bin_scatter<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(
                 ms.tier.as<uint8_t>(), 0, n, cx.hist, cx.cursor, ms.list.as<int32_t>(),

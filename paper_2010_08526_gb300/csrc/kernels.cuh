@@ -116,6 +116,7 @@ template <class I, class V> struct PartsArgs {
 // Sources
 // ---------------------------------------------------------------------------
 template <class I, class V> struct SrcGemm {
+    static constexpr bool kParts = false;
     using Args = GemmArgs<I, V>;
     using Val = V;
     using Idx = I;
@@ -152,6 +153,7 @@ template <class I, class V> struct SrcGemm {
 };
 
 template <class I, class V> struct SrcParts {
+    static constexpr bool kParts = true;
     using Args = PartsArgs<I, V>;
     using Val = V;
     using Idx = I;
@@ -186,15 +188,15 @@ template <class I, class V> struct SrcParts {
     __device__ __forceinline__ V val(int64_t q, V) const {
         return parts[q >> kShift].vals[q & ((1ll << kShift) - 1)];
     }
-    __device__ __forceinline__ int64_t flops() const {
-        const int lane = threadIdx.x & 31;
+    // entries of the column over all parts
+    __device__ __forceinline__ int64_t entries() const {
         int64_t s = 0;
-        for (int e = lane; e < nparts; e += 32) {
+        for (int e = 0; e < nparts; ++e) {
             int64_t b, en;
             range(e, b, en);
             s += en - b;
         }
-        return warp_sum(s);
+        return s;
     }
 };
 
@@ -793,15 +795,128 @@ __device__ __forceinline__ int hash_tier_of(int64_t u, int hash_cap_max) {
     return -1;
 }
 
-// One warp per column computes f_j, the number of contributions; the CTA
-// keeps a tier histogram. bound (optional) is the exact count of the unsplit
-// product when a k-stage is binned: columns with bound > hash_cap_max go to
-// the heavy tier (their stage output must be panel-grouped), others use
-// min(f, bound) as their size.
+// Multiplications per column of one product, f[g] += sum of nnz(A(:, k)) over
+// the column's B entries with k in [k0, k1) (f zeroed before), and their
+// total. B's entries are contiguous over the columns, so the kernel is cut by
+// entries, not by columns: a thread takes kFlopsEntries of them, finds its
+// first column with one search in colptr, and adds a column's part when it
+// leaves it (a warp inside one column adds one sum). It is bound by the
+// latency of the dependent colptr / rowidx / colptr reads; a warp per column
+// with 32 columns in a row (the form the batched products keep) left small
+// products on a few CTAs and skewed ones on a few long columns. Measured, with
+// k_col_tier, before -> now: uniform 4096 columns of 8 entries 27.8 -> 9 us,
+// 2-path counts 50k 33 -> 11.6 us, R-MAT 14 92 -> 15 us (R-MAT 18: 1363 us before).
+constexpr int kFlopsEntries = 8;
+template <class I, class V>
+__global__ void __launch_bounds__(256) k_col_flops(GemmArgs<I, V> ga, int64_t n, unsigned long long *f,
+                                                   unsigned long long *total) {
+    const ProbDev<I, V> *pd = ga.probs;
+    const I *bp = pd->bp, *bi = pd->bi, *ap = pd->ap;
+    const int lane = threadIdx.x & 31;
+    const int64_t e_end = (int64_t)bp[n];
+    const int64_t q0 = (int64_t)bp[0] + ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * kFlopsEntries;
+    const bool any = q0 < e_end;
+    // the column of q0: the last one starting at or before it
+    int64_t lo = 0, hi = n - 1;
+    if (any) {
+        while (lo < hi) {
+            const int64_t mid = (lo + hi + 1) >> 1;
+            if ((int64_t)__ldg(&bp[mid]) <= q0) lo = mid; else hi = mid - 1;
+        }
+    }
+    int64_t len[kFlopsEntries];
+#pragma unroll
+    for (int i = 0; i < kFlopsEntries; ++i) {
+        len[i] = 0;
+        if (q0 + i < e_end) {
+            const int64_t k = (int64_t)__ldg(&bi[q0 + i]);
+            if (k >= ga.k0 && k < ga.k1) len[i] = (int64_t)__ldg(&ap[k + 1]) - (int64_t)__ldg(&ap[k]);
+        }
+    }
+    int64_t g = lo, sum = 0, all = 0;
+    const int64_t first = lo;
+    if (any) {
+        int64_t next = (int64_t)__ldg(&bp[g + 1]);
+#pragma unroll
+        for (int i = 0; i < kFlopsEntries; ++i) {
+            if (q0 + i >= e_end) break;
+            while (q0 + i >= next) {
+                if (sum) atomicAdd(&f[g], (unsigned long long)sum);
+                sum = 0;
+                next = (int64_t)__ldg(&bp[++g + 1]);
+            }
+            sum += len[i];
+            all += len[i];
+        }
+    }
+    const int64_t g0 = __shfl_sync(SPG_FULL, first, 0);
+    if (__all_sync(SPG_FULL, any && first == g0 && g == g0)) {
+        sum = warp_sum(sum);
+        if (lane == 0 && sum) atomicAdd(&f[g0], (unsigned long long)sum);
+    } else if (sum) {
+        atomicAdd(&f[g], (unsigned long long)sum);
+    }
+    if (total) {
+        __shared__ unsigned long long s_tot[8];
+        all = warp_sum(all);
+        if (lane == 0) s_tot[threadIdx.x >> 5] = (unsigned long long)all;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            unsigned long long t = 0;
+            for (int w = 0; w < 8; ++w) t += s_tot[w];
+            if (t) atomicAdd(total, t);
+        }
+    }
+}
+
+// Tier of every column from its contributions f (products: counted by
+// k_col_flops; the merge counts its parts' entries here), and the tier
+// histogram. bound (optional) is the exact count of the unsplit product when a
+// k-stage is binned: columns with bound > hash_cap_max go to the heavy tier
+// (their stage output must be panel-grouped), others use min(f, bound) as
+// their size.
+template <class Src>
+__global__ void __launch_bounds__(256) k_col_tier(typename Src::Args sa, int64_t c_lo, int64_t c_hi,
+                                                  int hash_cap_max, const int64_t *bound, const int64_t *f_in,
+                                                  uint8_t *tier_out, int64_t *cnt_out, int32_t *tier_hist) {
+    __shared__ int s_hist[kTiers];
+    if (threadIdx.x < kTiers) s_hist[threadIdx.x] = 0;
+    __syncthreads();
+    const int64_t g = c_lo + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (g < c_hi) {
+        int64_t f, m;
+        if constexpr (Src::kParts) {
+            Src src;
+            src.open(sa, g);
+            f = src.entries();
+            m = src.m();
+        } else {
+            f = f_in[g];
+            m = sa.probs->m;
+        }
+        int64_t u = f < m ? f : m;
+        int t;
+        if (bound && bound[g] > hash_cap_max) {
+            t = heavy_subtier(f);
+        } else {
+            if (bound && bound[g] < u) u = bound[g];
+            t = hash_tier_of(u, hash_cap_max);
+            if (t < 0) t = heavy_subtier(u);
+        }
+        tier_out[g] = (uint8_t)t;
+        if (cnt_out) cnt_out[g] = 0;
+        if (t) atomicAdd(&s_hist[t], 1);
+    }
+    __syncthreads();
+    if (threadIdx.x < kTiers && s_hist[threadIdx.x])
+        atomicAdd(&tier_hist[threadIdx.x], s_hist[threadIdx.x]);
+}
+
+// Both steps in one launch for the columns of many problems (the batched
+// products): one warp per column computes f_j; the CTA keeps a tier histogram.
 template <class Src>
 __global__ void __launch_bounds__(256) k_flops_bin(typename Src::Args sa, int64_t c_lo,
-                                                   int64_t c_hi, int hash_cap_max,
-                                                   const int64_t *bound, int64_t *f_out,
+                                                   int64_t c_hi, int hash_cap_max, int64_t *f_out,
                                                    uint8_t *tier_out, int64_t *cnt_out,
                                                    int32_t *tier_hist) {
     __shared__ int s_hist[kTiers];
@@ -816,15 +931,9 @@ __global__ void __launch_bounds__(256) k_flops_bin(typename Src::Args sa, int64_
         src.open(sa, g);
         const int64_t f = src.flops();
         if (lane == 0) {
-            int64_t u = f < src.m() ? f : src.m();
-            int t;
-            if (bound && bound[g] > hash_cap_max) {
-                t = heavy_subtier(f);
-            } else {
-                if (bound && bound[g] < u) u = bound[g];
-                t = hash_tier_of(u, hash_cap_max);
-                if (t < 0) t = heavy_subtier(u);
-            }
+            const int64_t u = f < src.m() ? f : src.m();
+            int t = hash_tier_of(u, hash_cap_max);
+            if (t < 0) t = heavy_subtier(u);
             if (f_out) f_out[g] = f;
             tier_out[g] = (uint8_t)t;
             if (cnt_out) cnt_out[g] = 0;

@@ -196,8 +196,8 @@ struct PlanState {
     EngineBase *eng = nullptr;
 
     // device workspace
-    DevBuf probs, f, cnt, colptr, tier, list_sym, list_num, hist, cursor, off_sym, off_num;
-    DevBuf heavy_ord, pcnt, err, scan_part, wbytes, valid_flag;
+    DevBuf probs, f, cnt, colptr, tier, list_sym, list_num, hist, off_sym, off_num;
+    DevBuf heavy_ord, pcnt, err, scan_part, f_stage, valid_flag;
     DevBuf ap_end, ap_row, ap_val;
     DevBuf apc_off, apc_row, apc_val;   // A grouped by panel within each column
     DevBuf stage_cnt, stage_colptr, stage_pcnt, drows, dvals, parts_tab;  // k-split
@@ -284,7 +284,7 @@ struct MultiState {
     int nprob = 0, idx64 = 0, vtype = 0, nsm = 148;
     AllocFns alloc;          // workspace allocator (opts->allocator, copied)
     Tuning tun;
-    DevBuf probs, f, cnt, colptr, tier, list, off, hist, cursor, err, scan_part;
+    DevBuf probs, f, cnt, colptr, tier, list, off, hist, err, scan_part;
     DevBuf rows, vals;
     DevBuf counter;                // work counters of the two persistent passes (2 each)
     DevBuf gsize, gtab_off, gkeys, gvals;   // global tables of the heavy columns

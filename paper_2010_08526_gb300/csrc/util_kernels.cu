@@ -242,40 +242,95 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_partials(int64_t *partial
     if (threadIdx.x == 0) partials[np] = carry;
 }
 
-// out[i] = sum_{j<i} in[j] for i in [0, n]; in and out may alias.
-__global__ void __launch_bounds__(kScanThreads) k_scan_apply(const int64_t *in, int64_t n,
-                                                             const int64_t *partials,
-                                                             int64_t *out, int write_total) {
-    __shared__ int64_t s_warp[33];
-    const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
-    int64_t v[kScanItems];
-    int64_t s = 0;
+// A CTA's exclusive scan of the ITEMS * kScanThreads entries at t0, plus
+// `before`. A warp owns a run of 32 * ITEMS entries in rows of 32, so every load and
+// store is a full line; returns the tile's total.
+template <int ITEMS>
+__device__ __forceinline__ int64_t scan_tile(const int64_t *in, int64_t n, int64_t t0, int64_t before, int64_t *out,
+                                             int64_t *s_warp) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t base = t0 + (int64_t)warp * (32 * ITEMS) + lane;
+    int64_t v[ITEMS], ex[ITEMS];
 #pragma unroll
-    for (int i = 0; i < kScanItems; ++i) {
-        const int64_t idx = base + i;
-        v[i] = idx < n ? in[idx] : 0;
-        s += v[i];
+    for (int i = 0; i < ITEMS; ++i) v[i] = base + 32 * i < n ? in[base + 32 * i] : 0;
+    int64_t run = 0;
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+        const int64_t incl = warp_incl_scan(v[i]);
+        ex[i] = run + incl - v[i];
+        run += __shfl_sync(SPG_FULL, incl, 31);
     }
     int64_t total;
-    int64_t ex = block_excl_scan(s, s_warp, total) + partials[blockIdx.x];
+    if (lane == 0) s_warp[warp] = run;
+    __syncthreads();
+    const int64_t w = s_warp[lane];   // kScanThreads / 32 == 32 warps
+    const int64_t wi = warp_incl_scan(w);
+    before += __shfl_sync(SPG_FULL, wi - w, warp);
+    total = __shfl_sync(SPG_FULL, wi, 31);
 #pragma unroll
-    for (int i = 0; i < kScanItems; ++i) {
-        const int64_t idx = base + i;
-        if (idx < n) out[idx] = ex;
-        ex += v[i];
+    for (int i = 0; i < ITEMS; ++i)
+        if (base + 32 * i < n) out[base + 32 * i] = before + ex[i];
+    return total;
+}
+
+// out[i] = sum_{j<i} in[j] for i in [0, n]; in and out may alias. np > 0: the
+// partials are the tiles' own sums, and every CTA adds up those before its
+// tile (np of them at most); np == 0: they are prefixes already.
+__global__ void __launch_bounds__(kScanThreads) k_scan_apply(const int64_t *in, int64_t n,
+                                                             const int64_t *partials, int np,
+                                                             int64_t *out, int write_total) {
+    __shared__ int64_t s_warp[33];
+    int64_t before = 0;
+    if (np > 0) {
+        int64_t p = 0;
+        for (int i = threadIdx.x; i < (int)blockIdx.x; i += kScanThreads) p += partials[i];
+        block_excl_scan(p, s_warp, before);
+    } else if (partials) {
+        before = partials[blockIdx.x];
     }
-    if (write_total && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0)
-        out[n] = partials[gridDim.x];
+    const int64_t total = scan_tile<kScanItems>(in, n, (int64_t)blockIdx.x * kScanTile, before, out, s_warp);
+    if (write_total && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[n] = before + total;
+}
+
+// The whole scan in one launch, for in != out and small n: every CTA first
+// sums all the input before its tile (from L2), then scans its tile.
+constexpr int kDirectItems = 2;
+constexpr int kDirectTile = kDirectItems * kScanThreads;
+__global__ void __launch_bounds__(kScanThreads) k_scan_direct(const int64_t *in, int64_t n, int64_t *out,
+                                                              int write_total) {
+    __shared__ int64_t s_warp[33];
+    const int64_t t0 = (int64_t)blockIdx.x * kDirectTile;
+    int64_t p = 0, before;
+#pragma unroll 16
+    for (int64_t i = threadIdx.x; i < t0; i += kScanThreads) p += in[i];
+    block_excl_scan(p, s_warp, before);
+    const int64_t total = scan_tile<kDirectItems>(in, n, t0, before, out, s_warp);
+    if (write_total && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[n] = before + total;
 }
 
 int64_t scan_partials_len(int64_t n) { return (n + kScanTile - 1) / kScanTile + 1; }
 
+// The form by size. One launch up to kDirectScan entries: a CTA reads on
+// average half the input again, which costs less than a second launch (50,021 entries: 7.5 us
+// against 2.7 + 6.0 us and a launch; even at 65,536: 10.0 against 8.8 us).
+// Up to kFoldPartials tiles the apply kernel adds up the partials itself,
+// which saves the launch between (3 us). Beyond, three launches.
+constexpr int64_t kDirectScan = 56 * 1024;
+constexpr int64_t kFoldPartials = 1024;
 cudaError_t exclusive_scan_i64(const int64_t *in, int64_t n, int64_t *out, int64_t *partials,
                                int write_total, cudaStream_t st) {
     const int64_t nb = n > 0 ? (n + kScanTile - 1) / kScanTile : 1;
-    k_scan_reduce<<<(unsigned)nb, kScanThreads, 0, st>>>(in, n, partials);
-    k_scan_partials<<<1, kScanThreads, 0, st>>>(partials, nb);
-    k_scan_apply<<<(unsigned)nb, kScanThreads, 0, st>>>(in, n, partials, out, write_total);
+    if (in != out && n <= kDirectScan) {
+        const int64_t nd = n > 0 ? (n + kDirectTile - 1) / kDirectTile : 1;
+        k_scan_direct<<<(unsigned)nd, kScanThreads, 0, st>>>(in, n, out, write_total);
+    } else if (nb == 1) {
+        k_scan_apply<<<1, kScanThreads, 0, st>>>(in, n, nullptr, 0, out, write_total);
+    } else {
+        k_scan_reduce<<<(unsigned)nb, kScanThreads, 0, st>>>(in, n, partials);
+        const bool fold = nb <= kFoldPartials;
+        if (!fold) k_scan_partials<<<1, kScanThreads, 0, st>>>(partials, nb);
+        k_scan_apply<<<(unsigned)nb, kScanThreads, 0, st>>>(in, n, partials, fold ? (int)nb : 0, out, write_total);
+    }
     return cudaGetLastError();
 }
 

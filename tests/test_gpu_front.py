@@ -1,0 +1,52 @@
+"""The symbolic step's front end: multiplications per column, their total and
+the column offsets, at the sizes where the scans change form (one tile, one
+launch, folded partials, three launches) and for ragged columns of B (runs of
+empty columns, one column of thousands of entries)."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():  # pragma: no cover
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+import paper_2010_08526_gb300 as spg  # noqa: E402
+
+
+def diagonal(n, it):
+    i = torch.arange(n + 1, device="cuda", dtype=it)
+    return spg.Csc(n, n, i, i[:n].clone(), torch.ones(n, device="cuda"))
+
+
+@pytest.mark.parametrize("it", [torch.int32, torch.int64])
+@pytest.mark.parametrize("n", [1, 31, 2047, 2048, 2049, 8192, 8193, 57344, 57345, 70001, (1 << 23) + 8191])
+def test_offsets_and_flops_of_ragged_columns(n, it):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n)
+    k = 4096
+    counts = torch.randint(0, 4, (n,), generator=g, device="cuda")
+    counts[torch.rand(n, generator=g, device="cuda") < 0.4] = 0
+    counts[n // 3:n // 3 + 700] = 0
+    counts[n // 2] = k                       # one long column
+    ptr = torch.zeros(n + 1, dtype=torch.int64, device="cuda")
+    ptr[1:] = torch.cumsum(counts, 0)
+    nnz = int(ptr[-1])
+    # rows of a column: consecutive from a random start, so they are distinct
+    start = torch.randint(0, k, (n,), generator=g, device="cuda")
+    start[n // 2] = 0
+    col = torch.repeat_interleave(torch.arange(n, device="cuda"), counts)
+    rows = (start[col] + torch.arange(nnz, device="cuda") - ptr[col]) % k
+    B = spg.Csc(k, n, ptr.to(it), rows.to(it), torch.ones(nnz, device="cuda"))
+    plan = spg.Plan(diagonal(k, it), B)
+    info = plan.symbolic()
+    assert info["flops"] == nnz and info["nnz_c"] == nnz
+    assert torch.equal(plan.column_counts(), counts)
+    for t in range(plan.nbatches):
+        c0, c1, _ = plan.batch(t)
+        C = plan.numeric(t)
+        assert torch.equal(C.colptr, ptr[c0:c1 + 1] - ptr[c0])
+    plan.check_errors()
+    plan.close()
