@@ -172,9 +172,12 @@ template <class I, class V> struct Engine : EngineBase {
         set_smem(k_multi_pass<SrcGemm<I, V>, 256, 1>, mx);
         set_smem(k_multi_pass<SrcGemm<I, V>, 128, 0>, mx);
         set_smem(k_multi_pass<SrcGemm<I, V>, 128, 1>, mx);
-        set_smem(k_num_heavy32<I, V, 1>, mx);
-        set_smem(k_num_heavy32<I, V, 2>, mx);
-        set_smem(k_num_heavy32<I, V, 3>, mx);
+        set_smem(k_num_heavy32<I, V, 1, false>, mx);
+        set_smem(k_num_heavy32<I, V, 1, true>, mx);
+        set_smem(k_num_heavy32<I, V, 2, false>, mx);
+        set_smem(k_num_heavy32<I, V, 2, true>, mx);
+        set_smem(k_num_heavy32<I, V, 3, false>, mx);
+        set_smem(k_num_heavy32<I, V, 3, true>, mx);
         set_smem(k_sort_block<I, V, 1024>, mx);
         set_smem(k_sort_block<I, V, 8192>, mx);
         set_smem(k_sort_items<I, V, 8192>, mx);
@@ -275,6 +278,13 @@ template <class I, class V> struct Engine : EngineBase {
         int cap = 64;
         while (cap * 2 <= fit && cap * 2 <= kRangeCap) cap *= 2;
         return cap;
+    }
+
+    // Whether the products of heavy columns run in k_num_heavy32: every entry
+    // index < nnz(A) < 2^31, and the largest hash table of an item lies inside
+    // the accumulator.
+    static bool heavy32(const Ctx &cx, const GA &ga) {
+        return ga.lean_dense && 2 * range_cap(cx) * (int)(sizeof(V) + 4) <= (1 << cx.tun.log2R) * (int)sizeof(V);
     }
 
     static int heavy_smem(const Ctx &cx) {
@@ -470,12 +480,8 @@ template <class I, class V> struct Engine : EngineBase {
                 const int per_sm = (3 * (smem + stat) <= 227 * 1024) ? 3 : 2;
                 const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(n_items, (int64_t)cx.nsm * per_sm));
                 if constexpr (std::is_same<RSrc, SrcPanelRange<I, V>>::value) {
-                    // products: all heavy items in the kernel with 32-bit
-                    // offsets (every entry index < nnz(A) < 2^31), whose
-                    // largest hash table lies inside the accumulator
-                    const bool table_fits =
-                        2 * range_cap(cx) * (int)(sizeof(V) + 4) <= (1 << cx.tun.log2R) * (int)sizeof(V);
-                    if (da.lean_dense && table_fits) {
+                    // products: all heavy items in the kernel with 32-bit offsets
+                    if (heavy32(cx, da)) {
                         // three CTAs per SM when their shared memory allows it
                         // (registers are then capped at 40 per thread), else two
                         const int dsm = heavy32_smem(cx);
@@ -486,15 +492,14 @@ template <class I, class V> struct Engine : EngineBase {
                         // the item counter (the last int of the binning cursors)
                         int *next_item = cx.cursor + 63;
                         SPG_CK(cudaMemsetAsync(next_item, 0, sizeof(int), st));
-                        if (dper >= 3)
-                            k_num_heavy32<I, V, 3><<<dblocks, kDenseChunk, dsm, st>>>(da, c, items, item_order,
-                                                                                     n_items, next_item, o.rows, o.vals);
-                        else if (dper == 2)
-                            k_num_heavy32<I, V, 2><<<dblocks, kDenseChunk, dsm, st>>>(da, c, items, item_order,
-                                                                                     n_items, next_item, o.rows, o.vals);
-                        else
-                            k_num_heavy32<I, V, 1><<<dblocks, kDenseChunk, dsm, st>>>(da, c, items, item_order,
-                                                                                     n_items, next_item, o.rows, o.vals);
+                        auto kern = cx.sort ? (dper >= 3   ? k_num_heavy32<I, V, 3, true>
+                                               : dper == 2 ? k_num_heavy32<I, V, 2, true>
+                                                           : k_num_heavy32<I, V, 1, true>)
+                                            : (dper >= 3   ? k_num_heavy32<I, V, 3, false>
+                                               : dper == 2 ? k_num_heavy32<I, V, 2, false>
+                                                           : k_num_heavy32<I, V, 1, false>);
+                        kern<<<dblocks, kDenseChunk, dsm, st>>>(da, c, items, item_order, n_items, next_item, o.rows,
+                                                                o.vals);
                         cx.tend(tdd, st);
                         cx.launched();
                         SPG_CK(cudaGetLastError());
@@ -656,9 +661,10 @@ template <class I, class V> struct Engine : EngineBase {
         SPG_CK(cudaMemcpyAsync(ps.h_small.as<char>() + 256, ps.err.p, sizeof(int), cudaMemcpyDeviceToHost, st));
         if (ps.nheavy) SPG_ST(build_panels(ps, st));
         // products alone: a hash item may span any number of panels (one run
-        // of the column-grouped copy of A); sorted output and the k-split's
-        // part-by-part merges keep the narrower items
-        const int max_panels = (ps.opts.sort_output || ps.s > 1 || !ps.A.nnz || ps.A.nnz >= (int64_t(1) << 31))
+        // of the column-grouped copy of A); the items that k_sort_items orders
+        // and the k-split's part-by-part merges keep the narrower form
+        const int max_panels = (ps.s > 1 || !ps.A.nnz || (ps.opts.sort_output && !heavy32(cx, gemm_args(ps, 0, ps.k))) ||
+                                ps.A.nnz >= (int64_t(1) << 31))
                                    ? kRangeMaxPanels : std::max(kRangeMaxPanels, ps.P);
         SPG_ST(build_items(cx, ps.nheavy, ps.list_sym.as<int32_t>(), ps.off_sym.as<int32_t>(),
                            ps.cnt.as<int64_t>(), ps.pcnt.as<int32_t>(), n, ps.items, ps.item_cnt,
@@ -1061,9 +1067,9 @@ template <class I, class V> struct Engine : EngineBase {
                 ps.list_num.as<int32_t>(), ps.off_num.as<int32_t>(), st, ps.items.as<HeavyItem>(),
                 bitems.n, bitems.order)));
         }
-        // the hash tiers wrote their columns in row order, dense items are in row
-        // order: what is left are the hash-range items of the heavy columns
-        if (sort && b.heavy > 0)
+        // the hash tiers and k_num_heavy32 write in row order, and so do dense
+        // items: what is left are the hash-range items of the other heavy kernel
+        if (sort && b.heavy > 0 && !(ps.s == 1 && heavy32(cx, gemm_args(ps, 0, ps.k))))
             SPG_ST(sort_items(cx, ps.colptr.as<int64_t>(), hc[b.c0], b.c0, b.c1, (I *)C->rowidx, (V *)C->vals,
                               ps.items.as<HeavyItem>(), ps.item_off.as<int64_t>() + ps.nheavy, ps.n_items, st));
         SPG_CK(rebase_colptr(ps.colptr.as<int64_t>() + b.c0, b.c1 - b.c0, C->colptr,

@@ -151,19 +151,24 @@ __device__ __forceinline__ void sort_front(uint32_t *keys, V *vals, int T, int n
         if (lane == 0) { atomicMin(&ss->lo, lo); atomicMax(&ss->hi, hi); }
     }
     sort_sync<BLOCK>();   // the front is complete: the upper half is free
-    for (int i = t; i < NB; i += nt) hist[i] = 0u;
+    for (int i = t; i < NB / 4; i += nt) reinterpret_cast<uint4 *>(hist)[i] = make_uint4(0u, 0u, 0u, 0u);
     if constexpr (BLOCK) { lo = ss->lo; hi = ss->hi; }
     const int bits = 32 - __clz((int)(hi - lo));      // of the span (0: a single row)
     const int shift = max(0, bits - (31 - __clz(NB)));
     sort_sync<BLOCK>();
     for (int i = t; i < n; i += nt) atomicAdd(&hist[(keys[i] - lo) >> shift], 1u);
     sort_sync<BLOCK>();
-    // exclusive prefix of the bucket counts, a run of buckets per thread
-    const int per = (NB + nt - 1) / nt;
-    const int b0 = min(NB, t * per), b1 = min(NB, b0 + per);
+    // exclusive prefix of the bucket counts, a run of buckets (in fours) per thread
+    uint4 *hist4 = reinterpret_cast<uint4 *>(hist);
+    const int per = (NB / 4 + nt - 1) / nt;
+    const int b0 = min(NB / 4, t * per), b1 = min(NB / 4, b0 + per);
     int sum = 0;
     uint32_t most = 0;
-    for (int b = b0; b < b1; ++b) { const uint32_t c = hist[b]; sum += (int)c; most = max(most, c); }
+    for (int b = b0; b < b1; ++b) {
+        const uint4 c = hist4[b];
+        sum += (int)(c.x + c.y + c.z + c.w);
+        most = max(most, max(max(c.x, c.y), max(c.z, c.w)));
+    }
     const int incl = warp_incl_scan(sum);
     int run = incl - sum;
     if constexpr (BLOCK) {
@@ -181,7 +186,12 @@ __device__ __forceinline__ void sort_front(uint32_t *keys, V *vals, int T, int n
             return;
         }
     }
-    for (int b = b0; b < b1; ++b) { const uint32_t c = hist[b]; hist[b] = (uint32_t)run; run += (int)c; }
+    for (int b = b0; b < b1; ++b) {
+        const uint4 c = hist4[b];
+        const uint32_t x = (uint32_t)run, y = x + c.x, z = y + c.y, w = z + c.z;
+        hist4[b] = make_uint4(x, y, z, w);
+        run = (int)(w + c.w);
+    }
     sort_sync<BLOCK>();
     for (int i = t; i < n; i += nt) {
         const uint32_t key = keys[i];
@@ -219,7 +229,15 @@ __device__ __forceinline__ void sorted_emit(uint32_t *keys, V *vals, int T, int 
     if (n != want && t == 0) atomicOr(err, kErrCount);
     if (n <= (T >> 1)) sort_front<BLOCK>(keys, vals, T, n, lo, hi, want, ss, out_rows, out_vals);
     sort_sync<BLOCK>();
-    for (int s = t; s < T; s += nt) { keys[s] = kEmpty; vals[s] = V(0); }
+    // empty slots again, 16 bytes at a time (tables start on 16-byte boundaries)
+    uint4 *k4 = reinterpret_cast<uint4 *>(keys);
+    struct alignas(16) Vals { V v[16 / sizeof(V)]; };
+    Vals *v4 = reinterpret_cast<Vals *>(vals);
+    Vals none;
+#pragma unroll
+    for (int i = 0; i < 16 / (int)sizeof(V); ++i) none.v[i] = V(0);
+    for (int s = t; s < T / 4; s += nt) k4[s] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
+    for (int s = t; s < T * (int)sizeof(V) / 16; s += nt) v4[s] = none;
     sort_sync<BLOCK>();
 }
 

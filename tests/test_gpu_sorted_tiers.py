@@ -64,3 +64,30 @@ def test_hash_tiers_write_ascending_rows(layout, m, vt, it, semiring, stages):
         order = np.sort(cols[j])
         assert np.array_equal(rows[colptr[j]:colptr[j + 1]], order), f"column of {SIZES[j]}"
         assert np.array_equal(got[colptr[j]:colptr[j + 1]], np.array([want[r] for r in order.tolist()], dtype=vt))
+
+
+@pytest.mark.parametrize("vt,it", [(np.float32, np.int32), (np.float64, np.int32), (np.int64, np.int64)])
+@pytest.mark.parametrize("cap", [256, 8192])
+def test_heavy_columns_write_ascending_rows(vt, it, cap):
+    """Hash-range items over many sparse panels, some with clusters far from
+    the rest (the bitonic fallback), between dense panels."""
+    rng = np.random.default_rng(cap)
+    m = 1 << 20
+    cols = []
+    for count in (257, 600, 3000, 8193, 20000):
+        far = rng.integers(m // 2, m, count // 3)
+        cluster = 300000 + np.arange(min(1500, count // 3))          # one bucket of a wide item
+        near = rng.integers(0, 40000, count)                          # denser panels
+        rows = np.unique(np.concatenate([far, cluster, near]))
+        cols.append(rng.permutation(rows)[:count])
+    ptr = np.concatenate([[0], np.cumsum([c.size for c in cols])])
+    vals = [rng.integers(1, 9, c.size) for c in cols]
+    n = len(cols)
+    A = CSC(m, n, ptr.astype(it), np.concatenate(cols).astype(it), np.concatenate(vals).astype(vt))
+    I = CSC(n, n, np.arange(n + 1).astype(it), np.arange(n).astype(it), np.ones(n, vt))
+    C = spg.spgemm(to_dev(A), to_dev(I), sort_output=True, tuning=spg.Tuning(hash_max_cap=cap))
+    colptr, rows, got = (x.cpu().numpy() for x in (C.colptr, C.rowidx, C.vals))
+    for j in range(n):
+        order = np.argsort(cols[j])
+        assert np.array_equal(rows[colptr[j]:colptr[j + 1]], cols[j][order])
+        assert np.array_equal(got[colptr[j]:colptr[j + 1]], vals[j][order].astype(vt))
