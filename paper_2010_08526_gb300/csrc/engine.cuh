@@ -750,27 +750,26 @@ template <class I, class V> struct Engine : EngineBase {
         SPG_CK(ps.ap_val.ensure(sizeof(V) * (nnzA + 8)));
         SPG_CK(ps.merge_tmp.ensure(sizeof(int64_t) * scan_partials_len(N + 1)));
         const int tp = ps.timer.begin(kPhPanels, st);
-        SPG_CK(cudaMemsetAsync(ps.ap_end.p, 0, sizeof(int64_t) * (N + 1), st));
-        const int blocks = ps.nsm * 8;
-        k_panel_count<I><<<blocks, 256, 0, st>>>((const I *)ps.A.colptr, (const I *)ps.A.rowidx, ka,
-                                                 ps.tun.log2R, ps.ap_end.as<unsigned long long>());
-        SPG_CK(exclusive_scan_i64(ps.ap_end.as<int64_t>(), N, ps.ap_end.as<int64_t>(),
-                                  ps.merge_tmp.as<int64_t>(), 0, st));
-        k_panel_scatter<I, V><<<blocks, 256, 0, st>>>((const I *)ps.A.colptr, (const I *)ps.A.rowidx,
-                                                      (const V *)ps.A.vals, ka, ps.tun.log2R,
-                                                      ps.ap_end.as<unsigned long long>(),
-                                                      ps.ap_row.as<uint16_t>(), ps.ap_val.as<V>());
-        // the column-grouped copy read by hash-range items
         SPG_CK(ps.apc_off.ensure(sizeof(int32_t) * (size_t)(ka * ((int64_t)ps.P + 1))));
         SPG_CK(ps.apc_row.ensure(sizeof(uint32_t) * (nnzA + 8)));
         SPG_CK(ps.apc_val.ensure(sizeof(V) * (nnzA + 8)));
+        const I *ap = (const I *)ps.A.colptr, *ai = (const I *)ps.A.rowidx;
+        int32_t *apo = ps.apc_off.as<int32_t>();
+        SPG_CK(cudaMemsetAsync(apo, 0, sizeof(int32_t) * (size_t)(ka * ((int64_t)ps.P + 1)), st));
+        const unsigned eb = (unsigned)((nnzA + 8 * kPanelWindow - 1) / (8 * kPanelWindow));   // 8 warps per CTA
+        if (nnzA > 0)
+            k_panel_count<I><<<eb, 256, 0, st>>>(ap, ai, ka, nnzA, ps.tun.log2R, ps.P, apo);
         const unsigned kb = (unsigned)std::max<int64_t>(1, std::min<int64_t>((ka + 255) / 256, 1 << 20));
-        k_colpanel_offsets<<<kb, 256, 0, st>>>(ps.ap_end.as<int64_t>(), ka, ps.P, ps.apc_off.as<int32_t>());
-        k_colpanel_copy<I, V><<<dim3(kb, (unsigned)std::min(ps.P, 65535)), 256, 0, st>>>(
-            (const I *)ps.A.colptr, ps.ap_end.as<int64_t>(), ps.ap_row.as<uint16_t>(), ps.ap_val.as<V>(), ka,
-            ps.P, ps.tun.log2R, ps.apc_off.as<int32_t>(), ps.apc_row.as<uint32_t>(), ps.apc_val.as<V>());
+        k_panel_starts<<<kb, 256, 0, st>>>(ka, ps.P, apo, ps.ap_end.as<int64_t>());
+        SPG_CK(exclusive_scan_i64(ps.ap_end.as<int64_t>(), N, ps.ap_end.as<int64_t>(),
+                                  ps.merge_tmp.as<int64_t>(), 0, st));
+        if (nnzA > 0)
+            k_panel_scatter<I, V><<<eb, 256, 0, st>>>(ap, ai, (const V *)ps.A.vals, ka, nnzA, ps.tun.log2R, ps.P,
+                                                      ps.ap_end.as<unsigned long long>(), apo,
+                                                      ps.ap_row.as<uint16_t>(), ps.ap_val.as<V>(),
+                                                      ps.apc_row.as<uint32_t>(), ps.apc_val.as<V>());
         ps.timer.end(tp, st);
-        ps.timer.launches += 7;
+        ps.timer.launches += 6;
         SPG_CK(cudaGetLastError());
         ps.panels_built = true;
         return SPGEMM_OK;

@@ -50,3 +50,32 @@ def test_offsets_and_flops_of_ragged_columns(n, it):
         assert torch.equal(C.colptr, ptr[c0:c1 + 1] - ptr[c0])
     plan.check_errors()
     plan.close()
+
+
+@pytest.mark.parametrize("ordered", [True, False])
+@pytest.mark.parametrize("entries", [257, 383, 384, 385, 511, 512, 513, 5000])
+def test_panel_copies_at_window_edges(entries, ordered):
+    """Heavy columns read the panelised copies of A, built in windows of 128
+    entries: totals around a window, runs cut by it, empty columns between."""
+    rng = np.random.default_rng(entries)
+    m = 6000
+    counts = [0, 257, 0, 0, min(entries - 257, m - 1), 0]
+    rows = [rng.permutation(m)[:c] for c in counts]
+    if ordered:
+        rows = [np.sort(r) for r in rows]
+    ptr = np.concatenate([[0], np.cumsum(counts)])
+    vals = rng.integers(1, 9, int(ptr[-1])).astype(np.float32)
+    n = len(counts)
+
+    def csc(nrows, ncols, p, r, v):
+        t = [torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in (p.astype(np.int32), r.astype(np.int32), v)]
+        return spg.Csc(nrows, ncols, *t)
+
+    A = csc(m, n, ptr, np.concatenate(rows), vals)
+    B = csc(n, 1, np.array([0, n]), np.arange(n), np.ones(n, np.float32))     # the sum of all columns
+    C = spg.spgemm(A, B, sort_output=True, tuning=spg.Tuning(hash_max_cap=256, panel_rows=1024))
+    dense = np.zeros(m)
+    np.add.at(dense, np.concatenate(rows), vals)
+    where = np.flatnonzero(dense)
+    assert np.array_equal(C.rowidx.cpu().numpy(), where)
+    assert np.array_equal(C.vals.cpu().numpy(), dense[where].astype(np.float32))
