@@ -60,7 +60,7 @@ void free_mem(const AllocFns &a, void *p, size_t bytes, int kind) {
 
 size_t PlanState::workspace_bytes() const {
     const DevBuf *bufs[] = {&probs, &f, &cnt, &colptr, &tier, &list_sym, &list_num, &hist,
-                            &off_sym, &off_num, &heavy_ord, &pcnt, &err, &scan_part, &f_stage,
+                            &off_sym, &off_num, &heavy_ord, &pcnt, &err, &scan_part, &col_ws,
                             &valid_flag, &ap_end, &ap_row, &ap_val, &apc_off, &apc_row, &apc_val, &stage_cnt, &stage_colptr,
                             &stage_pcnt, &merge_tmp, &drows, &dvals, &parts_tab, &items, &item_cnt,
                             &item_off, &item_order, &pref_cnt, &pref_colptr, &pref_pcnt};
@@ -71,7 +71,7 @@ size_t PlanState::workspace_bytes() const {
 
 void PlanState::release_all() {
     DevBuf *bufs[] = {&probs, &f, &cnt, &colptr, &tier, &list_sym, &list_num, &hist,
-                      &off_sym, &off_num, &heavy_ord, &pcnt, &err, &scan_part, &f_stage,
+                      &off_sym, &off_num, &heavy_ord, &pcnt, &err, &scan_part, &col_ws,
                       &valid_flag, &ap_end, &ap_row, &ap_val, &apc_off, &apc_row, &apc_val, &stage_cnt, &stage_colptr,
                       &stage_pcnt, &merge_tmp, &drows, &dvals, &parts_tab, &items, &item_cnt,
                       &item_off, &item_order, &pref_cnt, &pref_colptr, &pref_pcnt};
@@ -81,6 +81,7 @@ void PlanState::release_all() {
     h_small.release();
     h_stage_colptr.release();
     h_parts.release();
+    h_tier_blk.release();
     for (auto &b : ring_pcol) b.release();
     for (auto &b : ring_prow) b.release();
     for (auto &b : ring_pval) b.release();

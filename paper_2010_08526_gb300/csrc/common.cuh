@@ -34,6 +34,20 @@ __host__ __device__ constexpr int tier_cap(int t) {
     return t == 1 ? 32 : t == 2 ? 128 : (128 << (t - 2));
 }
 
+// Numeric tier of a column with n distinct rows: 0 empty, 1..8 hash tiers,
+// kHeavyTier0 above the largest table. sel (0: none) is the column's exact
+// count in C when n counts a stage of it: C's heavy columns are heavy in
+// every stage.
+__host__ __device__ inline int num_tier(int64_t n, int64_t sel, int hash_cap_max) {
+    if (sel > hash_cap_max || n > hash_cap_max) return kHeavyTier0;
+    if (n == 0) return 0;
+    for (int t = 1; t <= 8; ++t)
+        if (n <= tier_cap(t)) return t;
+    return kHeavyTier0;
+}
+// columns per entry of k_tier_blocks
+constexpr int kTierBlock = 256;
+
 // Multiplicative (Fibonacci) hashing: the top log2(T) bits of key * 2^32/phi.
 __device__ __forceinline__ uint32_t hash_slot(uint32_t key, int log2T) {
     return (key * 0x9E3779B1u) >> (32 - log2T);

@@ -567,7 +567,7 @@ template <class I, class V> struct Engine : EngineBase {
         SPG_CK(ps.f.ensure(sizeof(int64_t) * (n + 1)));
         SPG_CK(ps.cnt.ensure(sizeof(int64_t) * (n + 1)));
         SPG_CK(ps.colptr.ensure(sizeof(int64_t) * (n + 1)));
-        if (ps.s > 1) SPG_CK(ps.f_stage.ensure(sizeof(int64_t) * (n + 1)));
+        SPG_CK(ps.col_ws.ensure(std::max(sizeof(int64_t) * (size_t)(n + 1), sizeof(int32_t) * tier_words(ps))));
         SPG_CK(ps.tier.ensure(n + 16));
         SPG_CK(ps.list_sym.ensure(sizeof(int32_t) * (n + 1)));
         SPG_CK(ps.list_num.ensure(sizeof(int32_t) * (n + 1)));
@@ -618,7 +618,7 @@ template <class I, class V> struct Engine : EngineBase {
                 int32_t *spc = ps.nheavy ? ps.stage_pcnt.as<int32_t>() + (size_t)t * ps.nheavy * ps.P
                                          : nullptr;
                 SPG_ST(sym_pass<SrcGemm<I, V>>(cx, gemm_args(ps, k0, k1), 0, n, ps.cnt.as<int64_t>(),
-                                               ps.f_stage.as<int64_t>(), ps.tier.as<uint8_t>(), scnt,
+                                               ps.col_ws.as<int64_t>(), ps.tier.as<uint8_t>(), scnt,
                                                ps.list_num.as<int32_t>(), ps.off_num.as<int32_t>(),
                                                nullptr, ps.heavy_ord.as<int32_t>(), nullptr, spc,
                                                nullptr, st, true, ps.B.nnz));
@@ -644,7 +644,7 @@ template <class I, class V> struct Engine : EngineBase {
                     int32_t *pp = ps.nheavy ? ps.pref_pcnt.as<int32_t>() + (size_t)(u - 1) * ps.nheavy * ps.P
                                             : nullptr;
                     SPG_ST(sym_pass<SrcGemm<I, V>>(cx, gemm_args(ps, 0, k1), 0, n, ps.cnt.as<int64_t>(),
-                                                   ps.f_stage.as<int64_t>(), ps.tier.as<uint8_t>(), pc,
+                                                   ps.col_ws.as<int64_t>(), ps.tier.as<uint8_t>(), pc,
                                                    ps.list_num.as<int32_t>(), ps.off_num.as<int32_t>(),
                                                    nullptr, ps.heavy_ord.as<int32_t>(), nullptr, pp,
                                                    nullptr, st, true, ps.B.nnz));
@@ -658,7 +658,7 @@ template <class I, class V> struct Engine : EngineBase {
         }
         SPG_CK(cudaMemcpyAsync(ps.h_colptr.p, ps.colptr.p, sizeof(int64_t) * (n + 1),
                                cudaMemcpyDeviceToHost, st));
-        SPG_CK(cudaMemcpyAsync(ps.h_small.as<char>() + 256, ps.err.p, sizeof(int), cudaMemcpyDeviceToHost, st));
+        SPG_ST(count_tiers(ps, cx, st));
         if (ps.nheavy) SPG_ST(build_panels(ps, st));
         // products alone: a hash item may span any number of panels (one run
         // of the column-grouped copy of A); the items that k_sort_items orders
@@ -670,7 +670,7 @@ template <class I, class V> struct Engine : EngineBase {
                            ps.cnt.as<int64_t>(), ps.pcnt.as<int32_t>(), n, ps.items, ps.item_cnt,
                            ps.item_off, ps.scan_part, ps.item_order, &ps.n_items, st, max_panels));
         SPG_CK(cudaStreamSynchronize(st));
-        const int errw = *(int *)(ps.h_small.as<char>() + 256);
+        const int errw = ps.h_tier_blk.as<int32_t>()[tier_words(ps) - 1];
         if (errw) {
             set_error("symbolic: device error flags " + std::to_string(errw));
             return SPGEMM_ERR_OVERFLOW;
@@ -775,21 +775,63 @@ template <class I, class V> struct Engine : EngineBase {
         return SPGEMM_OK;
     }
 
-    static void tier_counts(const int64_t *cp, const int64_t *sel, int64_t c0, int64_t c1, int capmax,
-                            std::array<int, 16> &tc, int64_t *heavy) {
-        tc.fill(0);
-        int64_t hv = 0;
-        for (int64_t j = c0; j < c1; ++j) {
-            const int64_t x = cp[j + 1] - cp[j];
-            const int64_t s = sel ? sel[j + 1] - sel[j] : x;
-            if (s > capmax) { ++hv; continue; }
-            if (x == 0) continue;
-            for (int t = 1; t <= 8; ++t) {
-                if (tier_cap(t) > capmax) break;
-                if (x <= tier_cap(t)) { tc[t]++; break; }
-            }
+    // The launches of a batch's hash tiers need the tier populations of its
+    // columns on the host. k_tier_blocks counts them per block of
+    // kTierBlock columns; a batch adds up its whole blocks and looks at
+    // single columns only at its two ends. (Counting column by column on the
+    // host took 0.25 ms per 50,000 columns, a third of a 2-path count of that
+    // size, with the device idle.) Tables: [0] C, then (s > 1) the stages and
+    // the running sums M_1..M_{s-2} of the incremental merge.
+    static int tier_tables(const PlanState &ps) {
+        return ps.s == 1 ? 1 : 1 + ps.s + (incremental(ps) ? ps.s - 2 : 0);
+    }
+    static int64_t tier_block_count(int64_t n) { return (n + kTierBlock - 1) / kTierBlock; }
+
+    static size_t tier_words(const PlanState &ps) {   // the tables, then the error word
+        return (size_t)tier_tables(ps) * (size_t)tier_block_count(ps.n) * 16 + 1;
+    }
+
+    // Enqueues the counts and their copy to the host (with the error word last).
+    static spgemm_status count_tiers(PlanState &ps, const Ctx &cx, cudaStream_t st) {
+        const int64_t n = ps.n, nblk = tier_block_count(n);
+        const int nt = tier_tables(ps);
+        const size_t words = tier_words(ps);
+        SPG_CK(ps.h_tier_blk.ensure(sizeof(int32_t) * words));
+        int32_t *blk = ps.col_ws.as<int32_t>();   // the stages' flops are no longer needed
+        for (int i = 0; i < nt; ++i) {
+            const int64_t *cp = i == 0 ? ps.colptr.as<int64_t>()
+                                : i <= ps.s ? ps.stage_colptr.as<int64_t>() + (size_t)(i - 1) * (n + 1)
+                                            : ps.pref_colptr.as<int64_t>() + (size_t)(i - 1 - ps.s) * (n + 1);
+            k_tier_blocks<<<(unsigned)std::max<int64_t>(1, nblk), kTierBlock, 0, st>>>(
+                cp, i == 0 ? nullptr : ps.colptr.as<int64_t>(), n, cx.tun.hash_cap_max, blk + (size_t)i * nblk * 16,
+                ps.err.as<int>(), blk + words - 1);
         }
-        if (heavy) *heavy = hv;
+        cx.launched(nt);
+        SPG_CK(cudaGetLastError());
+        SPG_CK(cudaMemcpyAsync(ps.h_tier_blk.p, blk, sizeof(int32_t) * words, cudaMemcpyDeviceToHost, st));
+        return SPGEMM_OK;
+    }
+
+    // Tier populations of columns [c0, c1) from table i of the block counts;
+    // cp / sel: the host offsets that the table was counted from.
+    static void tier_counts(const PlanState &ps, int i, const int64_t *cp, const int64_t *sel, int64_t c0,
+                            int64_t c1, int capmax, std::array<int, 16> &tc, int64_t *heavy) {
+        tc.fill(0);
+        const int32_t *blk = ps.h_tier_blk.as<int32_t>() + (size_t)i * tier_block_count(ps.n) * 16;
+        auto single = [&](int64_t a, int64_t z) {
+            for (int64_t j = a; j < z; ++j)
+                tc[num_tier(cp[j + 1] - cp[j], sel ? sel[j + 1] - sel[j] : 0, capmax)]++;
+        };
+        const int64_t b0 = std::min(c1, (c0 + kTierBlock - 1) / kTierBlock * kTierBlock);
+        // the last block of the matrix is whole even when it is short
+        const int64_t b1 = c1 == ps.n ? c1 : std::max(b0, c1 / kTierBlock * kTierBlock);
+        single(c0, b0);
+        for (int64_t b = (b0 + kTierBlock - 1) / kTierBlock; b * kTierBlock < b1; ++b)
+            for (int t = 0; t < 16; ++t) tc[t] += blk[(size_t)b * 16 + t];
+        single(b1, c1);
+        if (heavy) *heavy = tc[kHeavyTier0];
+        for (int t = kHeavyTier0; t < 16; ++t) tc[t] = 0;
+        tc[0] = 0;
     }
 
     // Greedy contiguous column ranges under the per-batch cap, from the exact
@@ -897,24 +939,24 @@ template <class I, class V> struct Engine : EngineBase {
         for (auto &b : ps.batches) {
             if (ps.s == 1) {
                 b.tc.resize(1);
-                tier_counts(hc, nullptr, b.c0, b.c1, capmax, b.tc[0], &b.heavy);
+                tier_counts(ps, 0, hc, nullptr, b.c0, b.c1, capmax, b.tc[0], &b.heavy);
             } else {
                 // [0] the final merge, [1 + t] stage t, [s + u] the merge into
                 // the running sum M_u (incremental, u = 1..s-2)
                 b.tc.resize(ps.s + 1 + (inc ? ps.s - 2 : 0));
-                tier_counts(hc, nullptr, b.c0, b.c1, capmax, b.tc[0], &b.heavy);
+                tier_counts(ps, 0, hc, nullptr, b.c0, b.c1, capmax, b.tc[0], &b.heavy);
                 b.doff.resize(ps.s);
                 int64_t off = 0;
                 for (int t = 0; t < ps.s; ++t) {
                     const int64_t *sc = hs + (size_t)t * (n + 1);
-                    tier_counts(sc, hc, b.c0, b.c1, capmax, b.tc[1 + t], nullptr);
+                    tier_counts(ps, 1 + t, sc, hc, b.c0, b.c1, capmax, b.tc[1 + t], nullptr);
                     b.doff[t] = off;
                     off += sc[b.c1] - sc[b.c0];
                 }
                 if (inc)
                     for (int u = 1; u <= ps.s - 2; ++u)
-                        tier_counts(hp + (size_t)(u - 1) * (n + 1), hc, b.c0, b.c1, capmax, b.tc[ps.s + u],
-                                    nullptr);
+                        tier_counts(ps, ps.s + u, hp + (size_t)(u - 1) * (n + 1), hc, b.c0, b.c1, capmax,
+                                    b.tc[ps.s + u], nullptr);
             }
             total_unm += b.unmerged;
         }

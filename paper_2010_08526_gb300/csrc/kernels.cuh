@@ -1431,6 +1431,12 @@ __global__ void k_heavy_items(const int32_t *list, const int32_t *list_off, cons
                               int P, int dense_min, int range_cap, int max_panels, int mode,
                               int64_t *ncount, const int64_t *item_off, HeavyItem *items);
 
+// Tier populations per block of kTierBlock columns (blk[b * 16 + t]) from the
+// offsets cp (sel: the offsets of C when cp are a stage's), and the error word
+// (defined in util_kernels.cu).
+__global__ void k_tier_blocks(const int64_t *cp, const int64_t *sel, int64_t n, int hash_cap_max, int32_t *blk,
+                              const int *err, int32_t *err_out);
+
 // Panel-major item order (defined in util_kernels.cu).
 __global__ void k_items_by_panel(const HeavyItem *items, const int64_t *n_items_p, int mode,
                                  int32_t *panel_cnt, int32_t *order);

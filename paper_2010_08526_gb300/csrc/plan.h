@@ -197,7 +197,8 @@ struct PlanState {
 
     // device workspace
     DevBuf probs, f, cnt, colptr, tier, list_sym, list_num, hist, off_sym, off_num;
-    DevBuf heavy_ord, pcnt, err, scan_part, f_stage, valid_flag;
+    DevBuf heavy_ord, pcnt, err, scan_part, valid_flag;
+    DevBuf col_ws;   // flops of a k-stage while it is counted, then the tier counts by block
     DevBuf ap_end, ap_row, ap_val;
     DevBuf apc_off, apc_row, apc_val;   // A grouped by panel within each column
     DevBuf stage_cnt, stage_colptr, stage_pcnt, drows, dvals, parts_tab;  // k-split
@@ -206,7 +207,7 @@ struct PlanState {
     DevBuf items, item_cnt, item_off, item_order;  // heavy work items (dense panels / hash ranges)
     int64_t n_items = 0;
     std::vector<int64_t> batch_item_off;   // batch t's items: item_order[off[t], off[t+1])
-    HostBuf h_colptr, h_small, h_stage_colptr, h_parts, h_pref_colptr;
+    HostBuf h_colptr, h_small, h_stage_colptr, h_parts, h_pref_colptr, h_tier_blk;
     std::vector<DevBuf> ring_col, ring_row, ring_val;   // spgemm_run_batched device ring
     std::vector<DevBuf> ring_pcol, ring_prow, ring_pval;  // pruned copies (opts.prune)
     std::vector<HostBuf> ring_hpc;                        // their colptrs on the host

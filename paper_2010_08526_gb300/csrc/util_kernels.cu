@@ -5,16 +5,6 @@
 
 namespace spg {
 
-__device__ __forceinline__ int num_tier_of(int64_t n, int hash_cap_max) {
-    if (n == 0) return 0;
-    for (int t = 1; t <= 8; ++t) {
-        const int cap = tier_cap(t);
-        if (cap > hash_cap_max) break;
-        if (n <= cap) return t;
-    }
-    return kHeavyTier0;
-}
-
 __global__ void k_numeric_tier(const int64_t *cnt, const int64_t *dense_sel, int64_t c_lo,
                                int64_t c_hi, int hash_cap_max, uint8_t *tier_out,
                                int32_t *tier_hist) {
@@ -23,13 +13,26 @@ __global__ void k_numeric_tier(const int64_t *cnt, const int64_t *dense_sel, int
     __syncthreads();
     const int64_t g = c_lo + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (g < c_hi) {
-        int t = num_tier_of(cnt[g], hash_cap_max);
-        if (dense_sel && dense_sel[g] > hash_cap_max) t = kHeavyTier0;
+        const int t = num_tier(cnt[g], dense_sel ? dense_sel[g] : 0, hash_cap_max);
         tier_out[g] = (uint8_t)t;
         if (t) atomicAdd(&s_hist[t], 1);
     }
     __syncthreads();
     if (threadIdx.x < kTiers && s_hist[threadIdx.x]) atomicAdd(&tier_hist[threadIdx.x], s_hist[threadIdx.x]);
+}
+
+__global__ void __launch_bounds__(kTierBlock) k_tier_blocks(const int64_t *cp, const int64_t *sel, int64_t n,
+                                                             int hash_cap_max, int32_t *blk, const int *err,
+                                                             int32_t *err_out) {
+    __shared__ int s_hist[kTiers];
+    if (threadIdx.x < kTiers) s_hist[threadIdx.x] = 0;
+    __syncthreads();
+    const int64_t g = (int64_t)blockIdx.x * kTierBlock + threadIdx.x;
+    if (g < n)
+        atomicAdd(&s_hist[num_tier(cp[g + 1] - cp[g], sel ? sel[g + 1] - sel[g] : 0, hash_cap_max)], 1);
+    __syncthreads();
+    if (threadIdx.x < kTiers && n > 0) blk[(int64_t)blockIdx.x * 16 + threadIdx.x] = s_hist[threadIdx.x];
+    if (blockIdx.x == 0 && threadIdx.x == 0) *err_out = *err;
 }
 
 __global__ void k_bin_scatter(const uint8_t *tier, int64_t c_lo, int64_t c_hi,

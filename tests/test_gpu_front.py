@@ -79,3 +79,36 @@ def test_panel_copies_at_window_edges(entries, ordered):
     where = np.flatnonzero(dense)
     assert np.array_equal(C.rowidx.cpu().numpy(), where)
     assert np.array_equal(C.vals.cpu().numpy(), dense[where].astype(np.float32))
+
+
+@pytest.mark.parametrize("merge", ["end", "incremental"])
+@pytest.mark.parametrize("stages", [1, 3])
+def test_tier_counts_over_batches(stages, merge):
+    """The tier populations of a batch are added up from blocks of 256 columns
+    and single columns at its ends: batches cut anywhere, every hash tier."""
+    n, m = 1500, 9000
+    g = torch.Generator(device="cuda")
+    g.manual_seed(stages)
+    sizes = torch.tensor([0, 1, 33, 130, 300, 700, 1500, 3000, 5000], device="cuda")
+    counts = sizes[torch.randint(0, 9, (n,), generator=g, device="cuda")]
+    ptr = torch.zeros(n + 1, dtype=torch.int64, device="cuda")
+    ptr[1:] = torch.cumsum(counts, 0)
+    col = torch.repeat_interleave(torch.arange(n, device="cuda"), counts)
+    start = torch.randint(0, m, (n,), generator=g, device="cuda")
+    rows = (start[col] + torch.arange(col.numel(), device="cuda") - ptr[col]) % m
+    vals = torch.randint(1, 9, (col.numel(),), generator=g, device="cuda").to(torch.float64)
+    A = spg.Csc(m, n, ptr.int(), rows.int(), vals)
+    i = torch.arange(n + 1, device="cuda").int()
+    I = spg.Csc(n, n, i, i[:n].clone(), torch.ones(n, dtype=torch.float64, device="cuda"))
+    whole = spg.spgemm(A, I, sort_output=True)
+    probe = spg.Plan(A, I, budget=1 << 33, kstages=stages, merge=merge, sort_output=True)
+    spent = (1 << 33) - 2 * probe.symbolic()["batch_cap_bytes"]
+    probe.close()
+    for cut in (3, 17):
+        C = spg.spgemm(A, I, sort_output=True, kstages=stages, merge=merge,
+                       budget=spent + 2 * max(12 * 5000 * 4, 24 * whole.nnz // cut))
+        assert C.plan_info["nbatches"] > 1
+        assert torch.equal(C.colptr, whole.colptr)
+        assert torch.equal(C.rowidx, whole.rowidx) and torch.equal(C.vals, whole.vals)
+    order = torch.sort(col * m + rows)
+    assert torch.equal(whole.rowidx.long(), order.values % m) and torch.equal(whole.vals, vals[order.indices])
