@@ -351,15 +351,18 @@ def spgemm(A: Csc, B: Csc, *, budget: Optional[int] = None, kstages: int = 1,
         rows = torch.empty(nnz, dtype=A.rowidx.dtype, device=dev)
         vals = torch.empty(nnz, dtype=A.vals.dtype, device=dev)
         colptr = torch.empty(B.ncols + 1, dtype=ptr_dtype, device=dev)
-        scratch = torch.empty(int(info["max_batch_cols"]) + 1, dtype=torch.int64, device=dev)
-        off = 0
-        for t in range(plan.nbatches):
-            c0, c1, bn = plan.batch(t)
-            plan.numeric_into(t, scratch[: c1 - c0 + 1], rows[off:off + bn], vals[off:off + bn],
-                              stream)
-            off += bn
-        check(plan._lib.spgemm_plan_colptr(plan._h, ctypes.c_void_p(colptr.data_ptr()),
-                                           _IDX[ptr_dtype], _stream_handle(stream)))
+        if plan.nbatches == 1:   # the batch's offsets are C's
+            plan.numeric_into(0, colptr, rows, vals, stream)
+        else:
+            scratch = torch.empty(int(info["max_batch_cols"]) + 1, dtype=torch.int64, device=dev)
+            off = 0
+            for t in range(plan.nbatches):
+                c0, c1, bn = plan.batch(t)
+                plan.numeric_into(t, scratch[: c1 - c0 + 1], rows[off:off + bn], vals[off:off + bn],
+                                  stream)
+                off += bn
+            check(plan._lib.spgemm_plan_colptr(plan._h, ctypes.c_void_p(colptr.data_ptr()),
+                                               _IDX[ptr_dtype], _stream_handle(stream)))
         out = Csc(A.nrows, B.ncols, colptr, rows, vals)
         out.plan_info = info
         return out

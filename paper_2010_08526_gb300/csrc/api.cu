@@ -3,6 +3,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <string>
 
 #include "../../include/spgemm.h"
@@ -26,6 +27,48 @@ spgemm_status cuda_fail(cudaError_t e, const char *where) {
 
 thread_local AllocFns tl_alloc;
 
+namespace {
+constexpr int kMaxDevices = 64;
+struct CallBlock { void *p = nullptr; bool taken = false; };
+CallBlock g_call_block[kMaxDevices];
+std::mutex g_call_mu;
+
+// Frees the current device's idle block; whether there was one.
+bool drop_call_block() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return false;
+    std::lock_guard<std::mutex> lk(g_call_mu);
+    CallBlock &b = g_call_block[dev];
+    if (!b.p || b.taken) return false;
+    cudaFree(b.p);
+    b.p = nullptr;
+    return true;
+}
+}  // namespace
+
+CallScratch::CallScratch(DevBuf &arena, cudaStream_t st) : arena_(arena), st_(st) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return;
+    std::lock_guard<std::mutex> lk(g_call_mu);
+    CallBlock &b = g_call_block[dev];
+    if (b.taken) return;
+    if (!b.p && cudaMalloc(&b.p, kCallScratch) != cudaSuccess) {
+        cudaGetLastError();   // the call allocates what it needs itself
+        b.p = nullptr;
+        return;
+    }
+    b.taken = true;
+    dev_ = dev;
+    arena.borrow(b.p, kCallScratch);
+}
+
+CallScratch::~CallScratch() {
+    if (dev_ < 0) return;
+    cudaStreamSynchronize(st_);   // on every way out of the call
+    std::lock_guard<std::mutex> lk(g_call_mu);
+    g_call_block[dev_].taken = false;
+}
+
 void *alloc_mem(const AllocFns &a, size_t bytes, int kind, cudaError_t &e) {
     void *p = nullptr;
     if (a.alloc) {
@@ -40,6 +83,10 @@ void *alloc_mem(const AllocFns &a, size_t bytes, int kind, cudaError_t &e) {
         return p;
     }
     e = kind == SPGEMM_MEM_DEVICE ? cudaMalloc(&p, bytes) : cudaHostAlloc(&p, bytes, cudaHostAllocDefault);
+    if (e == cudaErrorMemoryAllocation && kind == SPGEMM_MEM_DEVICE && drop_call_block()) {
+        cudaGetLastError();
+        e = cudaMalloc(&p, bytes);
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();   // a failed allocation must not look like a failed launch later
         p = nullptr;
@@ -47,11 +94,11 @@ void *alloc_mem(const AllocFns &a, size_t bytes, int kind, cudaError_t &e) {
     return p;
 }
 
-void free_mem(const AllocFns &a, void *p, size_t bytes, int kind) {
+void free_mem(const AllocFns &a, void *p, size_t bytes, int kind, bool synced) {
     if (a.alloc) {
         // the caller's allocator may hand the block out again at once: every
         // use of it on the device must have finished (as cudaFree ensures)
-        cudaDeviceSynchronize();
+        if (!synced) cudaDeviceSynchronize();
         a.free(a.ctx, p, bytes, kind);
         return;
     }
@@ -70,28 +117,31 @@ size_t PlanState::workspace_bytes() const {
 }
 
 void PlanState::release_all() {
+    cudaDeviceSynchronize();   // once, for all blocks
     DevBuf *bufs[] = {&probs, &f, &cnt, &colptr, &tier, &list_sym, &list_num, &hist,
                       &off_sym, &off_num, &heavy_ord, &pcnt, &err, &scan_part, &col_ws,
                       &valid_flag, &ap_end, &ap_row, &ap_val, &apc_off, &apc_row, &apc_val, &stage_cnt, &stage_colptr,
                       &stage_pcnt, &merge_tmp, &drows, &dvals, &parts_tab, &items, &item_cnt,
                       &item_off, &item_order, &pref_cnt, &pref_colptr, &pref_pcnt};
-    for (auto *b : bufs) b->release();
-    h_colptr.release();
-    h_pref_colptr.release();
-    h_small.release();
-    h_stage_colptr.release();
-    h_parts.release();
-    h_tier_blk.release();
-    for (auto &b : ring_pcol) b.release();
-    for (auto &b : ring_prow) b.release();
-    for (auto &b : ring_pval) b.release();
-    for (auto &b : ring_hpc) b.release();
-    for (auto &w : ring_pws) w.release();
-    for (auto &b : ring_col) b.release();
-    for (auto &b : ring_row) b.release();
-    for (auto &b : ring_val) b.release();
-    for (auto &h : host_slots) h.release();
+    for (auto *b : bufs) b->release(true);
+    h_colptr.release(true);
+    h_pref_colptr.release(true);
+    h_small.release(true);
+    h_stage_colptr.release(true);
+    h_parts.release(true);
+    h_tier_blk.release(true);
+    for (auto &b : ring_pcol) b.release(true);
+    for (auto &b : ring_prow) b.release(true);
+    for (auto &b : ring_pval) b.release(true);
+    for (auto &b : ring_hpc) b.release(true);
+    for (auto &w : ring_pws) w.release(true);
+    for (auto &b : ring_col) b.release(true);
+    for (auto &b : ring_row) b.release(true);
+    for (auto &b : ring_val) b.release(true);
+    for (auto &h : host_slots) h.release(true);
     ring_col.clear(); ring_row.clear(); ring_val.clear(); host_slots.clear();
+    arena.release(true);
+    h_arena.release(true);
     timer.release();
 }
 
@@ -170,10 +220,11 @@ spgemm_status spgemm_plan_create(const spgemm_csc *A, const spgemm_csc *B, const
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
-    cudaDeviceProp prop;
-    e = cudaGetDeviceProperties(&prop, dev);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaGetDeviceProperties");
-    if (prop.major < 10) {
+    int major = 0, nsm = 0;
+    if ((e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev)) != cudaSuccess ||
+        (e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+        return cuda_fail(e, "cudaDeviceGetAttribute");
+    if (major < 10) {
         set_error("this library is built for sm_103a (Blackwell) devices");
         return SPGEMM_ERR_CUDA;
     }
@@ -193,7 +244,7 @@ spgemm_status spgemm_plan_create(const spgemm_csc *A, const spgemm_csc *B, const
     ps.idx64 = A->idx_type == SPGEMM_I64;
     ps.vtype = A->val_type;
     ps.m = A->nrows; ps.k = A->ncols; ps.n = B->ncols;
-    ps.dev = dev; ps.nsm = prop.multiProcessorCount;
+    ps.dev = dev; ps.nsm = nsm;
     // tuning
     const spgemm_tuning *tu = opts ? opts->tuning : nullptr;
     ps.tun.log2R = value_bytes((spgemm_value_t)ps.vtype) == 4 ? 14 : 13;
@@ -239,26 +290,31 @@ spgemm_status spgemm_plan_create(const spgemm_csc *A, const spgemm_csc *B, const
     ps.budget = (opts && opts->budget_bytes) ? opts->budget_bytes : (size_t)(0.8 * (double)freeb);
     ps.eng = make_engine(ps.idx64, ps.vtype, opts ? opts->semiring : SPGEMM_PLUS_TIMES);
     if (!ps.eng) { set_error("unsupported type combination"); delete plan; return SPGEMM_ERR_INVALID; }
-    // structural checks
-    auto read_last = [&](const spgemm_csc *M, int64_t *v) -> cudaError_t {
-        if (M->ptr_type == SPGEMM_I64)
-            return cudaMemcpy(v, (const int64_t *)M->colptr + M->ncols, 8, cudaMemcpyDeviceToHost);
-        int32_t x = 0;
-        cudaError_t ee = cudaMemcpy(&x, (const int32_t *)M->colptr + M->ncols, 4, cudaMemcpyDeviceToHost);
-        *v = x;
-        return ee;
-    };
-    int64_t la = 0, lb = 0;
-    if ((e = read_last(A, &la)) != cudaSuccess || (e = read_last(B, &lb)) != cudaSuccess) {
-        delete ps.eng; delete plan; return cuda_fail(e, "reading colptr");
-    }
-    if (la != A->nnz || lb != B->nnz) {
-        set_error("nnz does not match colptr[ncols]");
-        delete ps.eng; delete plan;
-        return SPGEMM_ERR_INVALID;
-    }
     s = ps.eng->setup(ps, stream);
     if (s != SPGEMM_OK) { ps.release_all(); delete ps.eng; delete plan; return s; }
+    // structural check: both last offsets, through pinned memory with one wait
+    {
+        char *h = ps.h_small.as<char>();
+        std::memset(h, 0, 16);
+        auto last = [&](const spgemm_csc *M, char *to) {
+            const size_t w = M->ptr_type == SPGEMM_I64 ? 8 : 4;
+            return cudaMemcpyAsync(to, (const char *)M->colptr + w * (size_t)M->ncols, w, cudaMemcpyDeviceToHost, 0);
+        };
+        auto value = [&](const spgemm_csc *M, const char *at) -> int64_t {
+            if (M->ptr_type == SPGEMM_I64) return *(const int64_t *)at;
+            return *(const int32_t *)at;
+        };
+        if ((e = last(A, h)) != cudaSuccess || (e = last(B, h + 8)) != cudaSuccess ||
+            (e = cudaStreamSynchronize(0)) != cudaSuccess) {
+            ps.release_all(); delete ps.eng; delete plan;
+            return cuda_fail(e, "reading colptr");
+        }
+        if (value(A, h) != A->nnz || value(B, h + 8) != B->nnz) {
+            set_error("nnz does not match colptr[ncols]");
+            ps.release_all(); delete ps.eng; delete plan;
+            return SPGEMM_ERR_INVALID;
+        }
+    }
     if (validate) {
         if ((e = ps.valid_flag.ensure(16)) != cudaSuccess ||
             (e = cudaMemsetAsync(ps.valid_flag.p, 0, 4, stream)) != cudaSuccess ||
@@ -517,9 +573,9 @@ spgemm_status spgemm_multi_create(int nprob, const spgemm_csc *As, const spgemm_
         set_error("an allocator needs both its alloc and free callbacks"); return SPGEMM_ERR_INVALID;
     }
     int dev = 0;
-    cudaDeviceProp prop;
+    int nsm = 0;
     cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaGetDeviceProperties(&prop, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return cuda_fail(e, "device query");
     auto *mh = new (std::nothrow) spgemm_multi_s();
     if (!mh) { set_error("host allocation failed"); return SPGEMM_ERR_OOM; }
@@ -533,7 +589,7 @@ spgemm_status spgemm_multi_create(int nprob, const spgemm_csc *As, const spgemm_
     ms.nprob = nprob;
     ms.idx64 = As[0].idx_type == SPGEMM_I64;
     ms.vtype = As[0].val_type;
-    ms.nsm = prop.multiProcessorCount;
+    ms.nsm = nsm;
     // defaults of the persistent passes: small shared tables and 128-thread
     // CTAs keep many CTAs resident per SM (batched problems are mostly small)
     ms.tun.hash_cap_max = 1024;

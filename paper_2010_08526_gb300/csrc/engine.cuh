@@ -561,30 +561,21 @@ template <class I, class V> struct Engine : EngineBase {
         pd.ap = (const I *)ps.A.colptr; pd.ai = (const I *)ps.A.rowidx; pd.av = (const V *)ps.A.vals;
         pd.bp = (const I *)ps.B.colptr; pd.bi = (const I *)ps.B.rowidx; pd.bv = (const V *)ps.B.vals;
         pd.m = ps.m; pd.gcol0 = 0; pd.ncols = ps.n; pd.ka = ps.k;
-        SPG_CK(ps.probs.ensure(sizeof(PD)));
-        SPG_CK(cudaMemcpyAsync(ps.probs.p, &pd, sizeof(PD), cudaMemcpyHostToDevice, st));
         const int64_t n = ps.n;
-        SPG_CK(ps.f.ensure(sizeof(int64_t) * (n + 1)));
-        SPG_CK(ps.cnt.ensure(sizeof(int64_t) * (n + 1)));
-        SPG_CK(ps.colptr.ensure(sizeof(int64_t) * (n + 1)));
-        SPG_CK(ps.col_ws.ensure(std::max(sizeof(int64_t) * (size_t)(n + 1), sizeof(int32_t) * tier_words(ps))));
-        SPG_CK(ps.tier.ensure(n + 16));
-        SPG_CK(ps.list_sym.ensure(sizeof(int32_t) * (n + 1)));
-        SPG_CK(ps.list_num.ensure(sizeof(int32_t) * (n + 1)));
-        SPG_CK(ps.heavy_ord.ensure(sizeof(int32_t) * (n + 1)));
-        SPG_CK(ps.hist.ensure(sizeof(int32_t) * kBinInts));
-        SPG_CK(ps.off_sym.ensure(sizeof(int32_t) * 64));
-        SPG_CK(ps.off_num.ensure(sizeof(int32_t) * 64));
-        SPG_CK(ps.err.ensure(sizeof(int) * 4));
-        SPG_CK(ps.scan_part.ensure(sizeof(int64_t) * scan_partials_len(n + 1)));
-        SPG_CK(ps.h_colptr.ensure(sizeof(int64_t) * (n + 1)));
-        SPG_CK(ps.h_small.ensure(4096));
+        const size_t c = (size_t)(n + 1), i64 = sizeof(int64_t), i32 = sizeof(int32_t);
+        const size_t stages = ps.s > 1 ? (size_t)ps.s * c : 0;
+        SPG_CK(carve<SPGEMM_MEM_DEVICE>(
+            ps.arena,
+            {{&ps.probs, sizeof(PD)}, {&ps.f, i64 * c}, {&ps.cnt, i64 * c}, {&ps.colptr, i64 * c},
+             {&ps.col_ws, std::max(i64 * c, i32 * tier_words(ps))}, {&ps.tier, c + 15}, {&ps.list_sym, i32 * c},
+             {&ps.list_num, i32 * c}, {&ps.heavy_ord, i32 * c}, {&ps.hist, i32 * kBinInts}, {&ps.off_sym, i32 * 64},
+             {&ps.off_num, i32 * 64}, {&ps.err, sizeof(int) * 4}, {&ps.scan_part, i64 * (size_t)scan_partials_len(n + 1)},
+             {&ps.stage_cnt, i64 * stages}, {&ps.stage_colptr, i64 * stages}}));
+        SPG_CK(carve<SPGEMM_MEM_PINNED_HOST>(
+            ps.h_arena, {{&ps.h_colptr, i64 * c}, {&ps.h_small, 4096}, {&ps.h_tier_blk, i32 * tier_words(ps)},
+                         {&ps.h_stage_colptr, i64 * stages}}));
+        SPG_CK(cudaMemcpyAsync(ps.probs.p, &pd, sizeof(PD), cudaMemcpyHostToDevice, st));
         SPG_CK(cudaMemsetAsync(ps.err.p, 0, sizeof(int) * 4, st));
-        if (ps.s > 1) {
-            SPG_CK(ps.stage_cnt.ensure(sizeof(int64_t) * (size_t)ps.s * (n + 1)));
-            SPG_CK(ps.stage_colptr.ensure(sizeof(int64_t) * (size_t)ps.s * (n + 1)));
-            SPG_CK(ps.h_stage_colptr.ensure(sizeof(int64_t) * (size_t)ps.s * (n + 1)));
-        }
         return SPGEMM_OK;
     }
 
@@ -796,7 +787,6 @@ template <class I, class V> struct Engine : EngineBase {
         const int64_t n = ps.n, nblk = tier_block_count(n);
         const int nt = tier_tables(ps);
         const size_t words = tier_words(ps);
-        SPG_CK(ps.h_tier_blk.ensure(sizeof(int32_t) * words));
         int32_t *blk = ps.col_ws.as<int32_t>();   // the stages' flops are no longer needed
         for (int i = 0; i < nt; ++i) {
             const int64_t *cp = i == 0 ? ps.colptr.as<int64_t>()
@@ -1286,6 +1276,7 @@ template <class I, class V> struct Engine : EngineBase {
             cp = cp64.as<int64_t>();
         }
         PruneWs ws;
+        CallScratch scratch(ws.arena, st);
         DevBuf tmp;
         const bool count_only = out->rowidx == nullptr;
         int64_t *ocp = (int64_t *)out->colptr;
@@ -1426,12 +1417,11 @@ template <class I, class V> struct Engine : EngineBase {
     static spgemm_status merge(const spgemm_csc *parts, int nparts, spgemm_csc *out, cudaStream_t st) {
         attrs();
         const int64_t n = parts[0].ncols, m = parts[0].nrows;
-        int dev = 0;
-        cudaDeviceProp prop;
+        int dev = 0, nsm = 0;
         SPG_CK(cudaGetDevice(&dev));
-        SPG_CK(cudaGetDeviceProperties(&prop, dev));
+        SPG_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
         PlanState tmp;   // scratch only
-        tmp.nsm = prop.multiProcessorCount;
+        tmp.nsm = nsm;
         tmp.tun.log2R = sizeof(V) == 4 ? 14 : 13;
         const int64_t R = 1ll << tmp.tun.log2R;
         tmp.P = (int)std::max<int64_t>(1, (m + R - 1) / R);
@@ -1440,6 +1430,7 @@ template <class I, class V> struct Engine : EngineBase {
         tmp.Rs = mpad <= maxbm ? (mpad > 0 ? mpad : R) : (maxbm / R) * R;
         tmp.Q = (int)std::max<int64_t>(1, (m + tmp.Rs - 1) / tmp.Rs);
         struct Guard { PlanState &p; ~Guard() { p.release_all(); } } guard{tmp};
+        CallScratch scratch(tmp.arena, st);
         std::vector<PartDev<I, V>> tab(nparts);
         for (int i = 0; i < nparts; ++i) {
             tab[i].colptr = parts[i].colptr;
@@ -1449,18 +1440,13 @@ template <class I, class V> struct Engine : EngineBase {
             tab[i].vals = (const V *)parts[i].vals;
             tab[i].pcnt = nullptr;
         }
-        SPG_CK(tmp.parts_tab.ensure(sizeof(PartDev<I, V>) * nparts));
-        SPG_CK(tmp.cnt.ensure(sizeof(int64_t) * (n + 1)));
-        SPG_CK(tmp.colptr.ensure(sizeof(int64_t) * (n + 1)));
-        SPG_CK(tmp.tier.ensure(n + 16));
-        SPG_CK(tmp.list_sym.ensure(sizeof(int32_t) * (n + 1)));
-        SPG_CK(tmp.list_num.ensure(sizeof(int32_t) * (n + 1)));
-        SPG_CK(tmp.heavy_ord.ensure(sizeof(int32_t) * (n + 1)));
-        SPG_CK(tmp.hist.ensure(sizeof(int32_t) * kBinInts));
-        SPG_CK(tmp.off_sym.ensure(sizeof(int32_t) * 64));
-        SPG_CK(tmp.off_num.ensure(sizeof(int32_t) * 64));
-        SPG_CK(tmp.err.ensure(sizeof(int) * 4));
-        SPG_CK(tmp.scan_part.ensure(sizeof(int64_t) * scan_partials_len(n + 1)));
+        const size_t c = (size_t)(n + 1), i64 = sizeof(int64_t), i32 = sizeof(int32_t);
+        SPG_CK(carve<SPGEMM_MEM_DEVICE>(
+            tmp.arena,
+            {{&tmp.parts_tab, sizeof(PartDev<I, V>) * (size_t)nparts}, {&tmp.cnt, i64 * c}, {&tmp.colptr, i64 * c},
+             {&tmp.tier, c + 15}, {&tmp.list_sym, i32 * c}, {&tmp.list_num, i32 * c}, {&tmp.heavy_ord, i32 * c},
+             {&tmp.hist, i32 * kBinInts}, {&tmp.off_sym, i32 * 64}, {&tmp.off_num, i32 * 64},
+             {&tmp.err, sizeof(int) * 4}, {&tmp.scan_part, i64 * (size_t)scan_partials_len(n + 1)}}));
         SPG_CK(tmp.h_small.ensure(4096));
         SPG_CK(cudaMemcpyAsync(tmp.parts_tab.p, tab.data(), sizeof(PartDev<I, V>) * nparts,
                                cudaMemcpyHostToDevice, st));

@@ -3,6 +3,7 @@
 
 #include <cstdint>
 #include <array>
+#include <initializer_list>
 #include <string>
 #include <vector>
 #include <cuda_runtime.h>
@@ -33,27 +34,34 @@ struct AllocScope {
 // Memory of `kind` from the current allocator; cudaErrorMemoryAllocation when
 // it fails (no CUDA error state is left behind).
 void *alloc_mem(const AllocFns &a, size_t bytes, int kind, cudaError_t &e);
-void free_mem(const AllocFns &a, void *p, size_t bytes, int kind);
+// synced: the device is known to be past every use of the block.
+void free_mem(const AllocFns &a, void *p, size_t bytes, int kind, bool synced = false);
 
 // A grow-only buffer of device (KIND = SPGEMM_MEM_DEVICE) or pinned host
-// memory; it owns its block (moved, never copied) and frees it when destroyed.
+// memory; it owns its block (moved, never copied) and frees it when
+// destroyed, or borrows a part of another buffer's block (carve()).
 template <int KIND> struct Buf {
     void *p = nullptr;
     size_t bytes = 0;
     AllocFns how;
+    bool borrowed = false;
     Buf() = default;
     Buf(const Buf &) = delete;
     Buf &operator=(const Buf &) = delete;
-    Buf(Buf &&o) noexcept : p(o.p), bytes(o.bytes), how(o.how) { o.p = nullptr; o.bytes = 0; }
+    Buf(Buf &&o) noexcept : p(o.p), bytes(o.bytes), how(o.how), borrowed(o.borrowed) { o.p = nullptr; o.bytes = 0; }
     Buf &operator=(Buf &&o) noexcept {
         if (this != &o) {
             release();
-            p = o.p; bytes = o.bytes; how = o.how;
+            p = o.p; bytes = o.bytes; how = o.how; borrowed = o.borrowed;
             o.p = nullptr; o.bytes = 0;
         }
         return *this;
     }
     ~Buf() { release(); }
+    void borrow(void *part, size_t n) {
+        release();
+        p = part; bytes = n; borrowed = true;
+    }
     cudaError_t ensure(size_t want) {
         if (want <= bytes && p) return cudaSuccess;
         release();
@@ -64,39 +72,85 @@ template <int KIND> struct Buf {
         if (e == cudaSuccess) bytes = want; else p = nullptr;
         return e;
     }
-    void release() {
-        if (p) free_mem(how, p, bytes, KIND);
+    void release(bool synced = false) {
+        if (p && !borrowed) free_mem(how, p, bytes, KIND, synced);
         p = nullptr;
         bytes = 0;
+        borrowed = false;
     }
     template <class T> T *as() const { return static_cast<T *>(p); }
 };
 using DevBuf = Buf<SPGEMM_MEM_DEVICE>;
 using HostBuf = Buf<SPGEMM_MEM_PINNED_HOST>;
 
+// Points every buffer of `want` into one block of `arena` (256-byte aligned
+// parts). A plan has some twenty buffers of a size known at its creation, and
+// an allocation and its release cost more than a small product's kernels:
+// one block for all took a 64 x 64 product from scratch from 335 to 235 us.
+template <int KIND> struct Want {
+    Buf<KIND> *buf;
+    size_t bytes;
+};
+template <int KIND> cudaError_t carve(Buf<KIND> &arena, std::initializer_list<Want<KIND>> want) {
+    auto up = [](size_t x) { return (x + 255) / 256 * 256; };
+    size_t total = 0;
+    for (const auto &w : want) total += up(w.bytes);
+    const cudaError_t e = arena.ensure(total);
+    if (e != cudaSuccess) return e;
+    char *p = static_cast<char *>(arena.p);
+    for (const auto &w : want) {
+        w.buf->borrow(p, w.bytes);
+        p += up(w.bytes);
+    }
+    return cudaSuccess;
+}
+
+// Scratch of the calls without a plan (transpose, prune, merge): a cudaMalloc
+// and its cudaFree cost them 60 to 150 us each. One block of kCallScratch bytes
+// per device is kept between calls; a call borrows it for its own length, and a
+// call that needs more, or finds it taken by another thread, allocates as
+// before. A call waits for its stream before it gives the block back, so the
+// next one may use it on any stream. A failing cudaMalloc of the library gives
+// the block back to the device and tries again.
+constexpr size_t kCallScratch = size_t(32) << 20;
+class CallScratch {
+  public:
+    CallScratch(DevBuf &arena, cudaStream_t st);   // lends the block to arena if it is free
+    ~CallScratch();
+    CallScratch(const CallScratch &) = delete;
+    CallScratch &operator=(const CallScratch &) = delete;
+
+  private:
+    DevBuf &arena_;
+    cudaStream_t st_;
+    int dev_ = -1;                                 // >= 0: this call has the block
+};
+
 int64_t scan_partials_len(int64_t n);
 
 // Workspace of the column prune (per column: kept count, mode, selection
 // list, selected key and tie quota; scan partials).
 struct PruneWs {
-    DevBuf keep, mode, sel, nsel, key, quota, part, row;
+    DevBuf arena, keep, mode, sel, nsel, key, quota, part, row;
+    int64_t cols = -1;   // columns that the parts hold
     cudaError_t ensure(int64_t ncols) {
-        cudaError_t e;
-        if ((e = keep.ensure(sizeof(int64_t) * (size_t)(ncols + 1))) != cudaSuccess) return e;
-        if ((e = mode.ensure((size_t)ncols + 16)) != cudaSuccess) return e;
-        if ((e = sel.ensure(sizeof(int64_t) * (size_t)(ncols + 1))) != cudaSuccess) return e;
-        if ((e = nsel.ensure(sizeof(unsigned long long) * 2)) != cudaSuccess) return e;
-        if ((e = key.ensure(sizeof(uint64_t) * (size_t)(ncols + 1))) != cudaSuccess) return e;
-        if ((e = quota.ensure(sizeof(int64_t) * (size_t)(ncols + 1))) != cudaSuccess) return e;
-        if ((e = row.ensure(sizeof(uint32_t) * (size_t)(ncols + 1))) != cudaSuccess) return e;
-        return part.ensure(sizeof(int64_t) * (size_t)scan_partials_len(ncols + 1));
+        if (ncols <= cols) return cudaSuccess;
+        const size_t c = (size_t)(ncols + 1);
+        cols = -1;
+        const cudaError_t e = carve<SPGEMM_MEM_DEVICE>(
+            arena, {{&keep, sizeof(int64_t) * c}, {&mode, c + 15}, {&sel, sizeof(int64_t) * c},
+                    {&nsel, sizeof(unsigned long long) * 2}, {&key, sizeof(uint64_t) * c},
+                    {&quota, sizeof(int64_t) * c}, {&row, sizeof(uint32_t) * c},
+                    {&part, sizeof(int64_t) * (size_t)scan_partials_len(ncols + 1)}});
+        if (e == cudaSuccess) cols = ncols;
+        return e;
     }
     size_t bytes() const {
         return keep.bytes + mode.bytes + sel.bytes + nsel.bytes + key.bytes + quota.bytes + part.bytes + row.bytes;
     }
-    void release() {
-        keep.release(); mode.release(); sel.release(); nsel.release(); key.release(); quota.release();
-        part.release(); row.release();
+    void release(bool synced = false) {
+        arena.release(synced);
+        cols = -1;
     }
 };
 
@@ -195,7 +249,9 @@ struct PlanState {
     int dev = 0, nsm = 148;
     EngineBase *eng = nullptr;
 
-    // device workspace
+    // device workspace; the buffers of fixed size share the arena's block
+    DevBuf arena;
+    HostBuf h_arena;
     DevBuf probs, f, cnt, colptr, tier, list_sym, list_num, hist, off_sym, off_num;
     DevBuf heavy_ord, pcnt, err, scan_part, valid_flag;
     DevBuf col_ws;   // flops of a k-stage while it is counted, then the tier counts by block

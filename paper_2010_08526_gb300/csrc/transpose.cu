@@ -56,12 +56,12 @@ __global__ void k_t_colptr(const int64_t *src, int64_t n, T *dst) {
 template <class P, class I, class W>
 static spgemm_status transpose_typed(const spgemm_csc *in, spgemm_csc *out, cudaStream_t st) {
     const int64_t m = in->nrows, n = in->ncols, nnz = in->nnz;
-    DevBuf count, scan, part, err;
-    cudaError_t e;
-    if ((e = count.ensure(sizeof(int64_t) * (size_t)(m + 1))) != cudaSuccess ||
-        (e = scan.ensure(sizeof(int64_t) * (size_t)(m + 1))) != cudaSuccess ||
-        (e = part.ensure(sizeof(int64_t) * (size_t)scan_partials_len(m + 1))) != cudaSuccess ||
-        (e = err.ensure(sizeof(int) * 4)) != cudaSuccess) {
+    DevBuf arena, count, scan, part, err;   // parts of one block
+    CallScratch scratch(arena, st);
+    cudaError_t e = carve<SPGEMM_MEM_DEVICE>(
+        arena, {{&count, sizeof(int64_t) * (size_t)(m + 1)}, {&scan, sizeof(int64_t) * (size_t)(m + 1)},
+                {&part, sizeof(int64_t) * (size_t)scan_partials_len(m + 1)}, {&err, sizeof(int) * 4}});
+    if (e != cudaSuccess) {
         if (e == cudaErrorMemoryAllocation) {
             set_error("transpose: workspace allocation failed");
             return SPGEMM_ERR_OOM;

@@ -112,3 +112,57 @@ def test_tier_counts_over_batches(stages, merge):
         assert torch.equal(C.rowidx, whole.rowidx) and torch.equal(C.vals, whole.vals)
     order = torch.sort(col * m + rows)
     assert torch.equal(whole.rowidx.long(), order.values % m) and torch.equal(whole.vals, vals[order.indices])
+
+
+def ragged(m, n, seed, dtype=torch.int32):
+    """Columns of 0, 1, 2 and a few hundred distinct rows."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    counts = torch.tensor([0, 0, 1, 2, 2, 300], device="cuda")[torch.randint(0, 6, (n,), generator=g, device="cuda")]
+    ptr = torch.zeros(n + 1, dtype=torch.int64, device="cuda")
+    ptr[1:] = torch.cumsum(counts, 0)
+    col = torch.repeat_interleave(torch.arange(n, device="cuda"), counts)
+    start = torch.randint(0, m, (n,), generator=g, device="cuda")
+    rows = (start[col] + 7 * (torch.arange(col.numel(), device="cuda") - ptr[col])) % m
+    vals = torch.randint(-9, 9, (col.numel(),), generator=g, device="cuda")
+    return spg.Csc(m, n, ptr.to(dtype), rows.to(dtype), vals), col
+
+
+def check_transpose(A, col, T):
+    key, order = torch.sort(A.rowidx.long() * A.ncols + col)
+    got = torch.repeat_interleave(torch.arange(A.nrows, device="cuda"), T.colptr.long().diff()) * A.ncols
+    k2, o2 = torch.sort(got + T.rowidx.long())
+    assert torch.equal(key, k2) and torch.equal(A.vals[order], T.vals[o2])
+
+
+@pytest.mark.parametrize("m,n", [(1, 40), (31, 33), (5003, 4001), ((1 << 21) + 3, 900)])
+def test_transpose_of_ragged_columns(m, n):
+    """The last shape needs more scratch than the block kept between calls."""
+    if m < 2200:
+        col = torch.arange(n, device="cuda")
+        A = spg.Csc(m, n, torch.arange(n + 1, device="cuda").int(), (col % m).int(), col.clone())
+    else:
+        A, col = ragged(m, n, m)
+    check_transpose(A, col, spg.transpose(A))
+
+
+def test_transposes_on_threads_and_streams():
+    import threading
+    work = [ragged(5003 + 100 * i, 3001, i) for i in range(4)]
+    torch.cuda.synchronize()
+    done = [None] * 4
+
+    def go(i):
+        s = torch.cuda.Stream()
+        with torch.cuda.stream(s):
+            for _ in range(8):
+                done[i] = spg.transpose(work[i][0])
+            s.synchronize()
+
+    threads = [threading.Thread(target=go, args=(i,)) for i in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for (A, col), T in zip(work, done):
+        check_transpose(A, col, T)
