@@ -149,7 +149,8 @@ template <class I, class V> struct Engine : EngineBase {
         set_smem(k_bwd_block<I, V, 8192>, mx);
         set_smem(k_bwd_block<I, V, 16384>, mx);
         set_smem(k_sym_bitmap<SrcGemm<I, V>>, mx);
-        set_smem(k_sym_heavy32<I, V>, mx);
+        set_smem(k_sym_heavy32<I, V, 1024, 1>, mx);
+        set_smem(k_sym_heavy32<I, V, 512, 3>, mx);
         set_smem(k_sym_bitmap<SrcParts<I, V>>, mx);
         set_smem(k_num_dense<SrcPanel<I, V>>, mx);
         set_smem(k_num_dense<SrcPartsPanel<I, V>>, mx);
@@ -415,7 +416,13 @@ template <class I, class V> struct Engine : EngineBase {
             bool lean = false;
             if constexpr (std::is_same<Src, SrcGemm<I, V>>::value) {
                 if (sa.lean_sym) {
-                    k_sym_heavy32<I, V><<<blocks, kSymChunk, smem, st>>>(sa, c);
+                    // CTAs of 512 threads, three or more per SM, where that many
+                    // bitmaps fit; one of 1024 threads per SM for wider ones
+                    const int per_sm = std::min(4, (227 * 1024) / (smem + (int)sizeof(SymShared<512>) + 1024));
+                    if (per_sm >= 3)
+                        k_sym_heavy32<I, V, 512, 3><<<(int)std::min<int64_t>(items, (int64_t)cx.nsm * per_sm), 512, smem, st>>>(sa, c);
+                    else
+                        k_sym_heavy32<I, V, 1024, 1><<<blocks, 1024, smem, st>>>(sa, c);
                     lean = true;
                 }
             }

@@ -13,23 +13,31 @@
 
 namespace spg {
 
-constexpr int kSymChunk = 1024;   // B entries per chunk (= threads per CTA)
+constexpr int kSymChunk = 1024;   // most B entries per chunk (= threads per CTA)
 constexpr int kSymBatch = 4;      // windows whose row loads a warp keeps in flight
 
-struct SymShared {
-    int start[kSymChunk + 1];     // stream start of compacted segment s; start[nz] = T
-    int qb[kSymChunk];            // segment begin (entry offset from colptr[0]) minus stream start
+template <int NT> struct SymShared {
+    int start[NT + 1];            // stream start of compacted segment s; start[nz] = T
+    int qb[NT];                   // segment begin (entry offset from colptr[0]) minus stream start
     int red_len[32];
     int red_cnt[32];
     int tot_len, tot_cnt;
     unsigned long long tot;
 };
 
-template <class I, class V>
-__global__ void __launch_bounds__(kSymChunk, 1) k_sym_heavy32(GemmArgs<I, V> ga, TierCommon c) {
+// NT threads, one B entry each per chunk. An item is a chain of dependent
+// loads and barriers (list, B column, colptr of A, rows), so several CTAs per SM
+// work on different items where their bitmaps fit. Three CTAs of 512 threads
+// against one of 1024: R-MAT 18 12.9 -> 10.5 ms, protein stand-in (100,000
+// columns) 1.27 -> 0.79 ms, the five passes of a 4-stage R-MAT 15 1.70 -> 1.24 ms.
+// 256 threads gain on the stand-in (0.69 ms) and lose on the hub columns of a
+// small R-MAT (R-MAT 14 0.37 against 0.28 ms). Looking at a bit before its
+// atomicOr costs more than the atomics it saves (R-MAT 18 13.8 ms).
+template <class I, class V, int NT, int MINB>
+__global__ void __launch_bounds__(NT, MINB) k_sym_heavy32(GemmArgs<I, V> ga, TierCommon c) {
     extern __shared__ __align__(16) unsigned char smem[];
     uint32_t *bm = reinterpret_cast<uint32_t *>(smem);
-    __shared__ SymShared sh;
+    __shared__ SymShared<NT> sh;
     const int nwords_max = (int)((c.Rs + 31) >> 5);
     for (int w = threadIdx.x; w < nwords_max; w += blockDim.x) bm[w] = 0u;
     if (threadIdx.x == 0) sh.tot = 0;
@@ -69,7 +77,7 @@ __global__ void __launch_bounds__(kSymChunk, 1) k_sym_heavy32(GemmArgs<I, V> ga,
         const int64_t r0 = (int64_t)q * c.Rs;
         const int64_t rows = (pd->m - r0) < c.Rs ? (pd->m - r0) : c.Rs;
         const bool filt = c.Q > 1;
-        for (int base = 0; base < nb; base += kSymChunk) {
+        for (int base = 0; base < nb; base += NT) {
             // 1. segments of this chunk's B entries
             const int e = base + (int)threadIdx.x;
             int len = 0, qrel = 0;
