@@ -294,53 +294,74 @@ template <class I, class V> struct Engine : EngineBase {
     }
 
     // Cut the heavy columns of the symbolic list into work items (dense
-    // panels and hash ranges) from their per-panel output counts; reads the
-    // item total back (one small synchronisation).
+    // panels and hash ranges) from their per-panel output counts, dense items
+    // before hash items, each by first panel. The total is left on the device
+    // (ioff[0]) and copied to item_total(cx), read by the caller after its next
+    // wait: with one panel a column has at most one item, so there is room for
+    // all before the total is known. Otherwise it is read here, between the
+    // count and the items. Few columns and panels take one launch (a product
+    // of 3,000 rows spent 55 us on eight launches and two waits).
     // max_panels: panels one hash item may span (any number for the products;
     // kRangeMaxPanels when the items are later sorted, or merged part by part)
+    static int64_t item_total(const Ctx &cx) {
+        int64_t t;
+        std::memcpy(&t, cx.h_small + 256, sizeof(t));
+        return t;
+    }
     static spgemm_status build_items(const Ctx &cx, int nheavy, const int32_t *sym_list,
                                      const int32_t *sym_off, const int64_t *sel,
-                                     const int32_t *pcnt, int64_t n, DevBuf &items, DevBuf &icnt,
-                                     DevBuf &ioff, DevBuf &scan_part, DevBuf &order,
-                                     int64_t *n_items, cudaStream_t st, int max_panels = kRangeMaxPanels) {
-        *n_items = 0;
+                                     const int32_t *pcnt, DevBuf &items, DevBuf &icnt,
+                                     DevBuf &ioff, DevBuf &order, cudaStream_t st,
+                                     int max_panels = kRangeMaxPanels) {
+        std::memset(cx.h_small + 256, 0, sizeof(int64_t));
         if (!nheavy) return SPGEMM_OK;
-        SPG_CK(icnt.ensure(sizeof(int64_t) * (nheavy + 1)));
+        SPG_CK(icnt.ensure(sizeof(int64_t) * (size_t)(std::max(nheavy, cx.P) + 1)));
         SPG_CK(ioff.ensure(sizeof(int64_t) * (nheavy + 1)));
-        SPG_CK(scan_part.ensure(sizeof(int64_t) * scan_partials_len(std::max<int64_t>(n, nheavy) + 1)));
         const int R = 1 << cx.tun.log2R;
         // a panel with at least R/8 output rows is a dense item; the rest are
         // grouped into hash items of at most range_cap rows, so a lone panel
         // below the dense threshold must fit one (dense_min - 1 <= range_cap)
         const int rcap = range_cap(cx);
         const int dmin = std::max(1, std::min(R / 8, rcap));
+        int64_t *total_d = ioff.as<int64_t>();
+        int32_t *bins = reinterpret_cast<int32_t *>(icnt.p);
+        const bool one = (int64_t)nheavy * cx.P <= kItemsOne && 2 * cx.P <= kItemBins;
         const unsigned nb = (unsigned)((nheavy + 255) / 256);
-        k_heavy_items<<<nb, 256, 0, st>>>(sym_list, sym_off, sel, cx.tun.hash_cap_max, 0, n, pcnt, cx.P,
-                                          dmin, rcap, max_panels, 0, icnt.as<int64_t>(), nullptr, nullptr);
-        SPG_CK(exclusive_scan_i64(icnt.as<int64_t>(), nheavy, ioff.as<int64_t>(),
-                                  scan_part.as<int64_t>(), 1, st));
-        int64_t total = 0;
-        SPG_CK(cudaMemcpyAsync(cx.h_small + 256, ioff.as<int64_t>() + nheavy, sizeof(int64_t),
-                               cudaMemcpyDeviceToHost, st));
-        SPG_CK(cudaStreamSynchronize(st));
-        std::memcpy(&total, cx.h_small + 256, sizeof(int64_t));
-        SPG_CK(items.ensure(sizeof(HeavyItem) * (size_t)(total + 1)));
-        k_heavy_items<<<nb, 256, 0, st>>>(sym_list, sym_off, sel, cx.tun.hash_cap_max, 0, n, pcnt, cx.P,
-                                          dmin, rcap, max_panels, 1, nullptr, ioff.as<int64_t>(), items.as<HeavyItem>());
-        // panel-major processing order: item indices sorted by first panel,
-        // stored after the items (icnt is reused for the panel histogram)
-        SPG_CK(order.ensure(sizeof(int32_t) * (size_t)(total + 1)));
-        SPG_CK(icnt.ensure(sizeof(int64_t) * (size_t)(std::max(nheavy, cx.P) + 1)));
-        int32_t *pc = reinterpret_cast<int32_t *>(icnt.p);
-        SPG_CK(cudaMemsetAsync(pc, 0, sizeof(int32_t) * (cx.P + 1), st));
-        const int64_t *tot_d = ioff.as<int64_t>() + nheavy;
-        const unsigned ob = (unsigned)std::max<int64_t>(1, std::min<int64_t>((total + 255) / 256, 4096));
-        k_items_by_panel<<<ob, 256, 0, st>>>(items.as<HeavyItem>(), tot_d, 0, pc, nullptr);
-        k_small_excl_scan<<<1, 1024, 0, st>>>(pc, cx.P);
-        k_items_by_panel<<<ob, 256, 0, st>>>(items.as<HeavyItem>(), tot_d, 1, pc, order.as<int32_t>());
-        cx.launched(8);
+        auto read_total = [&]() {
+            return cudaMemcpyAsync(cx.h_small + 256, total_d, sizeof(int64_t), cudaMemcpyDeviceToHost, st);
+        };
+        auto run_one = [&](int64_t room) {
+            k_heavy_items_one<<<1, 1024, 0, st>>>(sym_list, sym_off, sel, cx.tun.hash_cap_max, pcnt, cx.P, dmin, rcap,
+                                                  max_panels, room, items.as<HeavyItem>(), order.as<int32_t>(),
+                                                  total_d);
+            cx.launched();
+        };
+        auto run_bins = [&](int mode) {
+            k_heavy_items<<<nb, 256, 0, st>>>(sym_list, sym_off, sel, cx.tun.hash_cap_max, pcnt, cx.P, dmin, rcap,
+                                              max_panels, mode, bins, items.as<HeavyItem>(), order.as<int32_t>());
+            cx.launched();
+        };
+        auto size_items = [&](int64_t cnt) -> cudaError_t {
+            const cudaError_t e = items.ensure(sizeof(HeavyItem) * (size_t)(cnt + 1));
+            return e != cudaSuccess ? e : order.ensure(sizeof(int32_t) * (size_t)(cnt + 1));
+        };
+        if (cx.P == 1) SPG_CK(size_items(nheavy));
+        if (one) {
+            run_one(cx.P == 1 ? nheavy : 0);
+        } else {
+            SPG_CK(cudaMemsetAsync(bins, 0, sizeof(int32_t) * 2 * (size_t)cx.P, st));
+            run_bins(0);
+            k_small_excl_scan<<<1, 1024, 0, st>>>(bins, 2 * cx.P, total_d);
+            cx.launched();
+        }
+        SPG_CK(read_total());
+        if (cx.P > 1) {
+            SPG_CK(cudaStreamSynchronize(st));
+            SPG_CK(size_items(item_total(cx)));
+        }
+        if (!one) run_bins(1);
+        else if (cx.P > 1) run_one(item_total(cx));
         SPG_CK(cudaGetLastError());
-        *n_items = total;
         return SPGEMM_OK;
     }
 
@@ -550,7 +571,7 @@ template <class I, class V> struct Engine : EngineBase {
         a.ap_val = ps.ap_val.as<V>();
         a.apc_off = ps.apc_off.as<int32_t>();
         a.apc_row = ps.apc_row.as<uint32_t>();
-        a.apc_val = ps.apc_val.as<V>();
+        a.apc_val = ps.P == 1 ? ps.ap_val.as<V>() : ps.apc_val.as<V>();   // one panel: the same order
         a.lean_dense = ps.A.nnz < (int64_t(1) << 31) ? 1 : 0;
         // a chunk's stream is at most kSymChunk columns of A, each of at most
         // min(m, nnz(A)) entries
@@ -665,9 +686,10 @@ template <class I, class V> struct Engine : EngineBase {
                                 ps.A.nnz >= (int64_t(1) << 31))
                                    ? kRangeMaxPanels : std::max(kRangeMaxPanels, ps.P);
         SPG_ST(build_items(cx, ps.nheavy, ps.list_sym.as<int32_t>(), ps.off_sym.as<int32_t>(),
-                           ps.cnt.as<int64_t>(), ps.pcnt.as<int32_t>(), n, ps.items, ps.item_cnt,
-                           ps.item_off, ps.scan_part, ps.item_order, &ps.n_items, st, max_panels));
+                           ps.cnt.as<int64_t>(), ps.pcnt.as<int32_t>(), ps.items, ps.item_cnt,
+                           ps.item_off, ps.item_order, st, max_panels));
         SPG_CK(cudaStreamSynchronize(st));
+        ps.n_items = item_total(cx);
         const int errw = ps.h_tier_blk.as<int32_t>()[tier_words(ps) - 1];
         if (errw) {
             set_error("symbolic: device error flags " + std::to_string(errw));
@@ -692,6 +714,10 @@ template <class I, class V> struct Engine : EngineBase {
         ps.batch_item_off.clear();
         const int64_t nb = (int64_t)ps.batches.size();
         if (!ps.nheavy || ps.n_items <= 0 || nb < 1) return SPGEMM_OK;
+        if (nb == 1) {   // built in that order
+            ps.batch_item_off = {0, ps.n_items};
+            return SPGEMM_OK;
+        }
         const int64_t capw = (int64_t)(ps.item_cnt.bytes / sizeof(int64_t));
         const int64_t caps = (int64_t)(ps.scan_part.bytes / sizeof(int64_t));
         auto fits = [&](int64_t pe) {
@@ -750,19 +776,30 @@ template <class I, class V> struct Engine : EngineBase {
         const int tp = ps.timer.begin(kPhPanels, st);
         SPG_CK(ps.apc_off.ensure(sizeof(int32_t) * (size_t)(ka * ((int64_t)ps.P + 1))));
         SPG_CK(ps.apc_row.ensure(sizeof(uint32_t) * (nnzA + 8)));
-        SPG_CK(ps.apc_val.ensure(sizeof(V) * (nnzA + 8)));
         const I *ap = (const I *)ps.A.colptr, *ai = (const I *)ps.A.rowidx;
         int32_t *apo = ps.apc_off.as<int32_t>();
+        if (ps.P == 1) {
+            const int64_t w = std::max(ka, nnzA);
+            k_panel_single<I, V><<<(unsigned)std::max<int64_t>(1, std::min<int64_t>((w + 255) / 256, ps.nsm * 8)), 256, 0, st>>>(
+                ap, ai, (const V *)ps.A.vals, ka, ps.ap_end.as<int64_t>(), apo, ps.ap_row.as<uint16_t>(),
+                ps.apc_row.as<uint32_t>(), ps.ap_val.as<V>());
+            ps.timer.end(tp, st);
+            ps.timer.launches += 1;
+            SPG_CK(cudaGetLastError());
+            ps.panels_built = true;
+            return SPGEMM_OK;
+        }
+        SPG_CK(ps.apc_val.ensure(sizeof(V) * (nnzA + 8)));
         SPG_CK(cudaMemsetAsync(apo, 0, sizeof(int32_t) * (size_t)(ka * ((int64_t)ps.P + 1)), st));
         const unsigned eb = (unsigned)((nnzA + 8 * kPanelWindow - 1) / (8 * kPanelWindow));   // 8 warps per CTA
         if (nnzA > 0)
-            k_panel_count<I><<<eb, 256, 0, st>>>(ap, ai, ka, nnzA, ps.tun.log2R, ps.P, apo);
+            k_panel_count<I><<<eb, 256, 0, st>>>(ap, ai, ka, ps.tun.log2R, ps.P, apo);
         const unsigned kb = (unsigned)std::max<int64_t>(1, std::min<int64_t>((ka + 255) / 256, 1 << 20));
         k_panel_starts<<<kb, 256, 0, st>>>(ka, ps.P, apo, ps.ap_end.as<int64_t>());
         SPG_CK(exclusive_scan_i64(ps.ap_end.as<int64_t>(), N, ps.ap_end.as<int64_t>(),
                                   ps.merge_tmp.as<int64_t>(), 0, st));
         if (nnzA > 0)
-            k_panel_scatter<I, V><<<eb, 256, 0, st>>>(ap, ai, (const V *)ps.A.vals, ka, nnzA, ps.tun.log2R, ps.P,
+            k_panel_scatter<I, V><<<eb, 256, 0, st>>>(ap, ai, (const V *)ps.A.vals, ka, ps.tun.log2R, ps.P,
                                                       ps.ap_end.as<unsigned long long>(), apo,
                                                       ps.ap_row.as<uint16_t>(), ps.ap_val.as<V>(),
                                                       ps.apc_row.as<uint32_t>(), ps.apc_val.as<V>());
@@ -1109,7 +1146,7 @@ template <class I, class V> struct Engine : EngineBase {
         // items: what is left are the hash-range items of the other heavy kernel
         if (sort && b.heavy > 0 && !(ps.s == 1 && heavy32(cx, gemm_args(ps, 0, ps.k))))
             SPG_ST(sort_items(cx, ps.colptr.as<int64_t>(), hc[b.c0], b.c0, b.c1, (I *)C->rowidx, (V *)C->vals,
-                              ps.items.as<HeavyItem>(), ps.item_off.as<int64_t>() + ps.nheavy, ps.n_items, st));
+                              ps.items.as<HeavyItem>(), ps.item_off.as<int64_t>(), ps.n_items, st));
         SPG_CK(rebase_colptr(ps.colptr.as<int64_t>() + b.c0, b.c1 - b.c0, C->colptr,
                              C->ptr_type == SPGEMM_I64, st));
         cx.launched();
@@ -1486,10 +1523,11 @@ template <class I, class V> struct Engine : EngineBase {
         }
         int nheavy = 0;
         for (int t = kHeavyTier0; t < kTiers; ++t) nheavy += hist[t];
-        int64_t n_items = 0;
         SPG_ST(build_items(cx, nheavy, tmp.list_sym.as<int32_t>(), tmp.off_sym.as<int32_t>(),
-                           tmp.cnt.as<int64_t>(), tmp.pcnt.as<int32_t>(), n, tmp.items, tmp.item_cnt,
-                           tmp.item_off, tmp.scan_part, tmp.item_order, &n_items, st));
+                           tmp.cnt.as<int64_t>(), tmp.pcnt.as<int32_t>(), tmp.items, tmp.item_cnt,
+                           tmp.item_off, tmp.item_order, st));
+        SPG_CK(cudaStreamSynchronize(st));
+        const int64_t n_items = item_total(cx);
         NumOut<I, V> o{tmp.colptr.as<int64_t>(), 0, (I *)out->rowidx, (V *)out->vals};
         SPG_ST((num_pass<SrcParts<I, V>, SrcPartsPanel<I, V>, SrcPartsRange<I, V>>(
             cx, pa, pa, 0, n, tmp.cnt.as<int64_t>(), tmp.cnt.as<int64_t>(), o, nullptr, nheavy > 0,

@@ -1424,12 +1424,15 @@ struct HeavyItem {
 };
 
 // Cut heavy columns into work items (defined in util_kernels.cu).
-// mode 0: per-column item counts into ncount[h]; mode 1: write the items at
-// item_off[h] (exclusive scan of the counts).
-__global__ void k_heavy_items(const int32_t *list, const int32_t *list_off, const int64_t *sel,
-                              int hash_cap_max, int64_t c_lo, int64_t c_hi, const int32_t *pcnt,
-                              int P, int dense_min, int range_cap, int max_panels, int mode,
-                              int64_t *ncount, const int64_t *item_off, HeavyItem *items);
+constexpr int kItemBins = 2048;   // (kind, first panel) bins that a CTA counts in shared memory
+constexpr int kItemsOne = 16384;  // columns x panels that one CTA cuts by itself
+__global__ void k_heavy_items(const int32_t *list, const int32_t *list_off, const int64_t *sel, int hash_cap_max,
+                              const int32_t *pcnt, int P, int dense_min, int range_cap, int max_panels, int mode,
+                              int32_t *bins, HeavyItem *items, int32_t *order);
+__global__ void k_heavy_items_one(const int32_t *list, const int32_t *list_off, const int64_t *sel, int hash_cap_max,
+                                  const int32_t *pcnt, int P, int dense_min, int range_cap, int max_panels,
+                                  int64_t room, HeavyItem *items, int32_t *order, int64_t *total);
+__global__ void k_small_excl_scan(int32_t *a, int n, int64_t *total);
 
 // Tier populations per block of kTierBlock columns (blk[b * 16 + t]) from the
 // offsets cp (sel: the offsets of C when cp are a stage's), and the error word
@@ -1437,10 +1440,6 @@ __global__ void k_heavy_items(const int32_t *list, const int32_t *list_off, cons
 __global__ void k_tier_blocks(const int64_t *cp, const int64_t *sel, int64_t n, int hash_cap_max, int32_t *blk,
                               const int *err, int32_t *err_out);
 
-// Panel-major item order (defined in util_kernels.cu).
-__global__ void k_items_by_panel(const HeavyItem *items, const int64_t *n_items_p, int mode,
-                                 int32_t *panel_cnt, int32_t *order);
-__global__ void k_small_excl_scan(int32_t *a, int P);
 // Batch-major item order: by batch (the contiguous column ranges
 // bounds[0..nb]), then dense items before hash items, then by first panel
 // when pe > 1 (mode 0: histogram of the keys; mode 1: scatter at the scanned
@@ -1753,13 +1752,13 @@ constexpr int kPanelWindow = 128;
 // f(active, col, col_beg, panel, row, entry, leader lane, place in run, run length) for
 // every entry, by all lanes of a warp together. col_beg is colptr[col].
 template <class I, class F>
-__device__ __forceinline__ void panel_runs(const I *ap, const I *ai, int64_t ka, int64_t nnz, int log2R, F &f) {
+__device__ __forceinline__ void panel_runs(const I *ap, const I *ai, int64_t ka, int log2R, F &f) {
     const int lane = threadIdx.x & 31;
     const unsigned upto = 0xffffffffu >> (31 - lane);
-    const int64_t a0 = (int64_t)ap[0];
-    const int64_t w0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kPanelWindow;
-    if (w0 >= nnz) return;
-    const int64_t q0 = min(w0 + lane, nnz - 1) + a0;
+    const int64_t a0 = (int64_t)ap[0], a1 = (int64_t)ap[ka];
+    const int64_t w0 = a0 + (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kPanelWindow;
+    if (w0 >= a1) return;
+    const int64_t q0 = min(w0 + lane, a1 - 1);
     int64_t lo = 0, hi = ka - 1;
     while (lo < hi) {
         const int64_t mid = (lo + hi + 1) >> 1;
@@ -1768,8 +1767,8 @@ __device__ __forceinline__ void panel_runs(const I *ap, const I *ai, int64_t ka,
     int64_t col = lo, beg = (int64_t)__ldg(&ap[col]), end = (int64_t)__ldg(&ap[col + 1]);
 #pragma unroll
     for (int w = 0; w < kPanelWindow; w += 32) {
-        const int64_t q = a0 + w0 + w + lane;
-        const bool active = q < a0 + nnz;
+        const int64_t q = w0 + w + lane;
+        const bool active = q < a1;
         while (active && q >= end) { ++col; beg = end; end = (int64_t)__ldg(&ap[col + 1]); }
         const int64_t r = active ? (int64_t)__ldg(&ai[q]) : 0;
         const int64_t p = r >> log2R;
@@ -1784,14 +1783,36 @@ __device__ __forceinline__ void panel_runs(const I *ap, const I *ai, int64_t ka,
     }
 }
 
+// One panel holds all rows: its copies are A's own entries in order (both
+// copies share the values), so one launch takes the place of the count, the
+// scan and the scatter.
+template <class I, class V>
+__global__ void __launch_bounds__(256) k_panel_single(const I *ap, const I *ai, const V *av, int64_t ka, int64_t *ape,
+                                                      int32_t *apo, uint16_t *out_row, uint32_t *cr, V *out_val) {
+    const int64_t a0 = (int64_t)ap[0], n = (int64_t)ap[ka] - a0;
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    for (int64_t k = i0; k < ka; k += step) {
+        ape[k] = (int64_t)ap[k + 1] - a0;
+        apo[2 * k] = 0;
+        apo[2 * k + 1] = (int32_t)((int64_t)ap[k + 1] - (int64_t)ap[k]);
+    }
+    for (int64_t q = i0; q < n; q += step) {
+        const uint32_t r = (uint32_t)ai[a0 + q];
+        out_row[q] = (uint16_t)r;
+        cr[q] = r;
+        out_val[q] = av[a0 + q];
+    }
+}
+
 // apo[k*(P+1) + 1 + p] += entries of A(:, k) in row panel p (apo zeroed before).
 template <class I>
-__global__ void __launch_bounds__(256) k_panel_count(const I *ap, const I *ai, int64_t ka, int64_t nnz, int log2R,
-                                                     int P, int32_t *apo) {
+__global__ void __launch_bounds__(256) k_panel_count(const I *ap, const I *ai, int64_t ka, int log2R, int P,
+                                                     int32_t *apo) {
     auto f = [&](bool active, int64_t col, int64_t, int64_t p, int64_t, int64_t, int, int at, int len) {
         if (active && at == 0) atomicAdd(&apo[col * ((int64_t)P + 1) + 1 + p], len);
     };
-    panel_runs(ap, ai, ka, nnz, log2R, f);
+    panel_runs(ap, ai, ka, log2R, f);
 }
 
 // The counts, transposed into ape[p*ka + k], and their prefix over the panels
@@ -1803,7 +1824,7 @@ __global__ void k_panel_starts(int64_t ka, int P, int32_t *apo, int64_t *ape);
 // segment's end, apo[k*(P+1) + 1 + p] (its start within the column) at the
 // start of panel p + 1.
 template <class I, class V>
-__global__ void __launch_bounds__(256) k_panel_scatter(const I *ap, const I *ai, const V *av, int64_t ka, int64_t nnz,
+__global__ void __launch_bounds__(256) k_panel_scatter(const I *ap, const I *ai, const V *av, int64_t ka,
                                                        int log2R, int P, unsigned long long *ape, int32_t *apo,
                                                        uint16_t *out_row, V *out_val, uint32_t *cr, V *cv) {
     const int64_t mask = (1ll << log2R) - 1, a0 = (int64_t)ap[0];
@@ -1824,7 +1845,7 @@ __global__ void __launch_bounds__(256) k_panel_scatter(const I *ap, const I *ai,
         cr[d] = (uint32_t)r;
         cv[d] = v;
     };
-    panel_runs(ap, ai, ka, nnz, log2R, f);
+    panel_runs(ap, ai, ka, log2R, f);
 }
 
 // ---------------------------------------------------------------------------

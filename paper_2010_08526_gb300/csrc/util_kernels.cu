@@ -67,48 +67,114 @@ __global__ void k_bin_scatter(const uint8_t *tier, int64_t c_lo, int64_t c_hi,
     }
 }
 
-// mode 0: per-column item counts into ncount[h]; mode 1: write the items at
-// item_off[h] (exclusive scan of the counts). One thread per heavy column runs
-// the greedy cut over its P panel counts.
-__global__ void k_heavy_items(const int32_t *list, const int32_t *list_off, const int64_t *sel,
-                              int hash_cap_max, int64_t c_lo, int64_t c_hi, const int32_t *pcnt,
-                              int P, int dense_min, int range_cap, int max_panels, int mode,
-                              int64_t *ncount, const int64_t *item_off, HeavyItem *items) {
-    const int lo = list_off[kHeavyTier0], hi = list_off[kTiers];
-    const int nh = hi - lo;
-    const int64_t h = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (h >= nh) return;
-    const int64_t g = list[lo + h];
-    int64_t n_items = 0;
-    if (g >= c_lo && g < c_hi && sel[g] > hash_cap_max) {
-        const int32_t *pc = pcnt + h * P;
-        int64_t w = mode ? item_off[h] : 0;
-        int gp0 = -1, gcnt = 0, off = 0, goff = 0;
-        auto flush = [&](int p_end) {
-            if (gp0 >= 0 && gcnt > 0) {
-                if (mode) items[w++] = HeavyItem{(int32_t)g, gp0, p_end, gcnt, goff, 0};
-                ++n_items;
-            }
-            gp0 = -1; gcnt = 0;
-        };
-        for (int p = 0; p < P; ++p) {
-            const int x = pc[p];
-            if (x >= dense_min) {
-                flush(p);
-                if (mode) items[w++] = HeavyItem{(int32_t)g, p, p + 1, -x, off, 0};
-                ++n_items;
-                off += x;
-                continue;
-            }
-            if (gp0 >= 0 && (gcnt + x > range_cap || p - gp0 >= max_panels)) flush(p);
-            if (x == 0 && gp0 < 0) continue;      // no open group: skip empty panels
-            if (gp0 < 0) { gp0 = p; goff = off; }
-            gcnt += x;
+// Cuts heavy column h (global column g) into its items, in panel order:
+// emit(kind, HeavyItem) with kind 0 for dense and 1 for hash items.
+template <class F>
+__device__ __forceinline__ void cut_items(int64_t g, const int32_t *pc, int P, int dense_min, int range_cap,
+                                          int max_panels, F &&emit) {
+    int gp0 = -1, gcnt = 0, off = 0, goff = 0;
+    auto flush = [&](int p_end) {
+        if (gp0 >= 0 && gcnt > 0) emit(1, HeavyItem{(int32_t)g, gp0, p_end, gcnt, goff, 0});
+        gp0 = -1; gcnt = 0;
+    };
+    for (int p = 0; p < P; ++p) {
+        const int x = pc[p];
+        if (x >= dense_min) {
+            flush(p);
+            emit(0, HeavyItem{(int32_t)g, p, p + 1, -x, off, 0});
             off += x;
+            continue;
         }
-        flush(P);
+        if (gp0 >= 0 && (gcnt + x > range_cap || p - gp0 >= max_panels)) flush(p);
+        if (x == 0 && gp0 < 0) continue;      // no open group: skip empty panels
+        if (gp0 < 0) { gp0 = p; goff = off; }
+        gcnt += x;
+        off += x;
     }
-    if (!mode) ncount[h] = n_items;
+    flush(P);
+}
+
+// mode 0: bins[kind * P + first panel] += items; mode 1: bins hold the bins'
+// first positions, every item is written at the next position of its bin
+// (dense items before hash items, each by first panel). One thread per heavy
+// column runs the greedy cut over its P panel counts. For up to kItemBins bins
+// a CTA counts its items in shared memory and takes each bin's run with one
+// global atomic.
+__global__ void __launch_bounds__(256) k_heavy_items(const int32_t *list, const int32_t *list_off, const int64_t *sel,
+                                                     int hash_cap_max, const int32_t *pcnt, int P, int dense_min,
+                                                     int range_cap, int max_panels, int mode, int32_t *bins,
+                                                     HeavyItem *items, int32_t *order) {
+    __shared__ int s_cnt[kItemBins], s_base[kItemBins];
+    const int lo = list_off[kHeavyTier0], hi = list_off[kTiers];
+    const int64_t h = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int nbins = 2 * P;
+    const bool local = nbins <= kItemBins;
+    const int64_t g = h < hi - lo ? list[lo + h] : 0;
+    const bool mine = h < hi - lo && sel[g] > hash_cap_max;
+    const int32_t *pc = pcnt + h * P;
+    if (local) {
+        for (int b = threadIdx.x; b < nbins; b += blockDim.x) s_cnt[b] = 0;
+        __syncthreads();
+        if (mine)
+            cut_items(g, pc, P, dense_min, range_cap, max_panels,
+                      [&](int kind, const HeavyItem &it) { atomicAdd(&s_cnt[kind * P + it.p0], 1); });
+        __syncthreads();
+        for (int b = threadIdx.x; b < nbins; b += blockDim.x) {
+            s_base[b] = s_cnt[b] ? atomicAdd(&bins[b], s_cnt[b]) : 0;
+            s_cnt[b] = 0;
+        }
+        if (mode == 0) return;
+        __syncthreads();
+    }
+    if (mine)
+        cut_items(g, pc, P, dense_min, range_cap, max_panels, [&](int kind, const HeavyItem &it) {
+            const int b = kind * P + it.p0;
+            const int at = local ? s_base[b] + atomicAdd(&s_cnt[b], 1) : atomicAdd(&bins[b], 1);
+            if (mode) { items[at] = it; order[at] = at; }
+        });
+}
+
+// The same in one launch of one CTA, for few columns and panels (nheavy * P
+// <= kItemsOne): counts, bin prefix, items if there is room for them, and the
+// total.
+__global__ void __launch_bounds__(1024) k_heavy_items_one(const int32_t *list, const int32_t *list_off,
+                                                          const int64_t *sel, int hash_cap_max, const int32_t *pcnt,
+                                                          int P, int dense_min, int range_cap, int max_panels,
+                                                          int64_t room, HeavyItem *items, int32_t *order,
+                                                          int64_t *total) {
+    __shared__ int s_bin[kItemBins];
+    const int lo = list_off[kHeavyTier0], nh = list_off[kTiers] - lo;
+    const int nbins = 2 * P;
+    for (int b = threadIdx.x; b < nbins; b += blockDim.x) s_bin[b] = 0;
+    __syncthreads();
+    for (int h = threadIdx.x; h < nh; h += blockDim.x) {
+        const int64_t g = list[lo + h];
+        if (sel[g] > hash_cap_max)
+            cut_items(g, pcnt + (int64_t)h * P, P, dense_min, range_cap, max_panels,
+                      [&](int kind, const HeavyItem &it) { atomicAdd(&s_bin[kind * P + it.p0], 1); });
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        int carry = 0;
+        for (int b0 = 0; b0 < nbins; b0 += 32) {
+            const int b = b0 + threadIdx.x;
+            const int v = b < nbins ? s_bin[b] : 0;
+            const int incl = warp_incl_scan(v);
+            if (b < nbins) s_bin[b] = carry + incl - v;
+            carry += __shfl_sync(SPG_FULL, incl, 31);
+        }
+        if (threadIdx.x == 0) *total = carry;
+    }
+    __syncthreads();
+    for (int h = threadIdx.x; h < nh; h += blockDim.x) {
+        const int64_t g = list[lo + h];
+        if (sel[g] > hash_cap_max)
+            cut_items(g, pcnt + (int64_t)h * P, P, dense_min, range_cap, max_panels,
+                      [&](int kind, const HeavyItem &it) {
+                          const int at = atomicAdd(&s_bin[kind * P + it.p0], 1);
+                          if (at < room) { items[at] = it; order[at] = at; }
+                      });
+    }
 }
 
 __global__ void k_panel_starts(int64_t ka, int P, int32_t *apo, int64_t *ape) {
@@ -123,20 +189,6 @@ __global__ void k_panel_starts(int64_t ka, int P, int32_t *apo, int64_t *ape) {
             o[p] = run;
             run += c;
         }
-    }
-}
-
-// Panel-major order of the heavy items (counting sort by first panel), so
-// that the CTAs running at the same time read the same panel of A and of the
-// panel offsets from L2. mode 0: histogram; mode 1: scatter.
-__global__ void k_items_by_panel(const HeavyItem *items, const int64_t *n_items_p, int mode,
-                                 int32_t *panel_cnt, int32_t *order) {
-    const int64_t n = *n_items_p;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int p = items[i].p0;
-        if (mode == 0) atomicAdd(&panel_cnt[p], 1);
-        else order[atomicAdd(&panel_cnt[p], 1)] = (int32_t)i;
     }
 }
 
@@ -169,26 +221,26 @@ __global__ void k_batch_item_starts(const unsigned long long *cnt, int64_t nb, i
     start[t] = t == 0 ? 0 : t == nb ? n : (int64_t)cnt[t * 2 * pe - 1];
 }
 
-// exclusive scan of P ints in place (one CTA)
-__global__ void k_small_excl_scan(int32_t *a, int P) {
-    __shared__ int32_t s[1024];
-    int carry = 0;
-    for (int base = 0; base < P; base += blockDim.x) {
+// exclusive scan of n ints in place (one CTA); the sum goes to total
+__global__ void __launch_bounds__(1024) k_small_excl_scan(int32_t *a, int n, int64_t *total) {
+    __shared__ int32_t s_warp[33];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int32_t carry = 0;
+    for (int base = 0; base < n; base += 1024) {
         const int i = base + threadIdx.x;
-        const int v = i < P ? a[i] : 0;
-        s[threadIdx.x] = v;
+        const int32_t v = i < n ? a[i] : 0;
+        const int32_t incl = warp_incl_scan(v);
+        if (lane == 31) s_warp[warp] = incl;
         __syncthreads();
-        for (int o = 1; o < (int)blockDim.x; o <<= 1) {
-            const int t = threadIdx.x >= o ? s[threadIdx.x - o] : 0;
-            __syncthreads();
-            s[threadIdx.x] += t;
-            __syncthreads();
-        }
-        if (i < P) a[i] = carry + s[threadIdx.x] - v;
-        const int tot = s[blockDim.x - 1];
+        const int32_t w = s_warp[lane];
+        const int32_t wi = warp_incl_scan(w);
+        const int32_t before = __shfl_sync(SPG_FULL, wi - w, warp);
+        const int32_t all = __shfl_sync(SPG_FULL, wi, 31);
+        if (i < n) a[i] = carry + before + incl - v;
+        carry += all;
         __syncthreads();
-        carry += tot;
     }
+    if (threadIdx.x == 0) *total = carry;
 }
 
 // ---- exclusive scan of int64 (three phases, all on the device) ------------

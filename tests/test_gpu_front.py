@@ -166,3 +166,23 @@ def test_transposes_on_threads_and_streams():
         t.join()
     for (A, col), T in zip(work, done):
         check_transpose(A, col, T)
+
+
+@pytest.mark.parametrize("m,cols", [(1000, 5), (1000, 16500), (200000, 40), (200000, 1300), ((1 << 24) + 5000, 3)])
+def test_item_lists_of_every_form(m, cols):
+    """Heavy items cut by one CTA (one and several panels), by many CTAs with
+    bins in shared memory, and with more bins than fit there."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(m + cols)
+    count = 400
+    start = torch.randint(0, m, (cols,), generator=g, device="cuda")
+    step = torch.where(torch.arange(cols, device="cuda") % 2 == 0, 1, max(1, (m - 1) // count))
+    rows = (start[:, None] + step[:, None] * torch.arange(count, device="cuda")[None, :]) % m
+    vals = torch.randint(1, 9, (cols, count), generator=g, device="cuda").float()
+    ptr = (torch.arange(cols + 1, device="cuda") * count).int()
+    A = spg.Csc(m, cols, ptr, rows.reshape(-1).int(), vals.reshape(-1).contiguous())
+    C = spg.spgemm(A, diagonal(cols, torch.int32), sort_output=True,
+                   tuning=spg.Tuning(hash_max_cap=256, panel_rows=0 if m == 200000 else 1024))
+    order = torch.sort(rows, dim=1)
+    assert torch.equal(C.rowidx.long(), order.values.reshape(-1))
+    assert torch.equal(C.vals, torch.gather(vals, 1, order.indices).reshape(-1))
