@@ -248,8 +248,9 @@ spgemm_status spgemm_plan_create(const spgemm_csc *A, const spgemm_csc *B, const
     // tuning
     const spgemm_tuning *tu = opts ? opts->tuning : nullptr;
     ps.tun.log2R = value_bytes((spgemm_value_t)ps.vtype) == 4 ? 14 : 13;
+    while (ps.tun.log2R > 10 && (int64_t(1) << (ps.tun.log2R - 1)) >= ps.m) --ps.tun.log2R;   // one panel: no wider than m
     if (tu) {
-        if (tu->hash_max_cap) ps.tun.hash_cap_max = tu->hash_max_cap;
+        if (tu->hash_max_cap) { ps.tun.hash_cap_max = tu->hash_max_cap; ps.cap_rule = false; }
         if (tu->panel_rows) {
             int l = 0;
             while ((1 << l) < tu->panel_rows) ++l;
@@ -259,6 +260,7 @@ spgemm_status spgemm_plan_create(const spgemm_csc *A, const spgemm_csc *B, const
         if (tu->huge_seg) ps.tun.huge_seg = tu->huge_seg;
         if (tu->block_tier_threads) ps.tun.block_threads = tu->block_tier_threads;
         ps.tun.hybrid_sort = tu->hybrid_sort ? 1 : 0;
+        if (tu->panel_rows || tu->hybrid_sort) ps.cap_rule = false;
     }
     {
         bool ok = false;
@@ -274,6 +276,7 @@ spgemm_status spgemm_plan_create(const spgemm_csc *A, const spgemm_csc *B, const
             return SPGEMM_ERR_INVALID;
         }
     }
+    ps.cap_full = ps.tun.hash_cap_max;
     // panels
     const int64_t R = 1LL << ps.tun.log2R;
     ps.P = (int)((ps.m + R - 1) / R);

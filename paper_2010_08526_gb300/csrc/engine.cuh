@@ -6,6 +6,7 @@
 #include <array>
 #include <cmath>
 #include <cstring>
+#include <functional>
 #include <type_traits>
 #include <vector>
 
@@ -37,10 +38,12 @@ inline int block_tier_threads(int T, const Tuning &tun) {
 }
 
 // The binning words of a pass, zeroed together: [0, 16) tier histogram,
-// [kFlopTotal, +2) total multiplications (64 bits), [64, 128) list cursors
-// and the work counters of the persistent kernels.
+// [kFlopTotal, +2) total multiplications (64 bits), [kOverFull] columns above
+// the plan's largest hash table, [64, 128) list cursors and the work counters of
+// the persistent kernels.
 constexpr int kBinInts = 128;
 constexpr int kFlopTotal = 32;
+constexpr int kOverFull = 34;
 
 // Scratch shared by one symbolic / numeric pass.
 struct Ctx {
@@ -55,6 +58,8 @@ struct Ctx {
     PhaseTimer *tm = nullptr;   // optional phase timing and launch counting
     int ph_hash = kPhNumHash, ph_dense = kPhNumDense;
     bool stage_items = false;   // heavy items take their counts from pcnt_in
+    int cap_full = 8192;        // the plan's largest hash table
+    int over_full = 0;          // sym_pass: columns that may exceed it
     bool sort = false;          // the pass writes C itself in row order (opts.sort_output)
     const int64_t *f = nullptr; // flops per column of the full product (hybrid accumulator)
     int tbegin(int phase, cudaStream_t st) const { return tm ? tm->begin(phase, st) : -1; }
@@ -70,6 +75,7 @@ inline Ctx make_ctx(PlanState &ps) {
     c.h_small = ps.h_small.as<int32_t>();
     c.P = ps.P; c.Q = ps.Q; c.Rs = ps.Rs;
     c.f = ps.f.as<int64_t>();
+    c.cap_full = ps.cap_full;
     return c;
 }
 
@@ -370,42 +376,54 @@ template <class I, class V> struct Engine : EngineBase {
     // cnt_out, fills list/off; heavy columns get per-panel counts in pcnt.
     // heavy_ord_w (optional) receives the heavy ordinals (full pass only).
     // Products: f receives the multiplications per column, total_out their
-    // sum, and nnz_b is the number of B entries.
+    // sum, and nnz_b is the number of B entries. recap (optional) may lower or
+    // raise the hash cap once the total is known; the columns are then binned
+    // again.
     template <class Src>
-    static spgemm_status sym_pass(const Ctx &cx, const typename Src::Args &sa, int64_t c_lo, int64_t c_hi,
+    static spgemm_status sym_pass(Ctx &cx, const typename Src::Args &sa, int64_t c_lo, int64_t c_hi,
                            const int64_t *bound, int64_t *f, uint8_t *tier, int64_t *cnt_out,
                            int32_t *list, int32_t *off, int32_t *heavy_ord_w,
                            const int32_t *heavy_ord_r, DevBuf *pcnt_grow, int32_t *pcnt_ptr,
                            int *hist_out, cudaStream_t st, bool allow_heavy = true, int64_t nnz_b = 0,
-                           int64_t *total_out = nullptr) {
+                           int64_t *total_out = nullptr, const std::function<int(int64_t)> &recap = nullptr) {
         const int64_t nc = c_hi - c_lo;
-        SPG_CK(cudaMemsetAsync(cx.hist, 0, sizeof(int32_t) * kBinInts, st));
-        if (nc > 0) {
+        int hist[16];
+        int64_t total = 0;
+        for (bool again = false;; again = true) {
+          SPG_CK(cudaMemsetAsync(cx.hist, 0, sizeof(int32_t) * kBinInts, st));
+          if (nc > 0) {
             const int tb = cx.tbegin(kPhFlopsBin, st);
-            if constexpr (!Src::kParts) {   // all columns of one product
+            if (!Src::kParts && !again) {   // all columns of one product
                 SPG_CK(cudaMemsetAsync(f, 0, sizeof(int64_t) * (size_t)nc, st));
                 const int64_t per = 256 * kFlopsEntries;
-                if (nnz_b > 0) {
-                    k_col_flops<I, V><<<(unsigned)((nnz_b + per - 1) / per), 256, 0, st>>>(
-                        sa, nc, reinterpret_cast<unsigned long long *>(f),
-                        reinterpret_cast<unsigned long long *>(cx.hist + kFlopTotal));
-                    cx.launched();
+                if constexpr (!Src::kParts) {
+                    if (nnz_b > 0) {
+                        k_col_flops<I, V><<<(unsigned)((nnz_b + per - 1) / per), 256, 0, st>>>(
+                            sa, nc, reinterpret_cast<unsigned long long *>(f),
+                            reinterpret_cast<unsigned long long *>(cx.hist + kFlopTotal));
+                        cx.launched();
+                    }
                 }
             }
             k_col_tier<Src><<<(unsigned)((nc + 255) / 256), 256, 0, st>>>(
-                sa, c_lo, c_hi, cx.tun.hash_cap_max, bound, f, tier, cnt_out, cx.hist);
+                sa, c_lo, c_hi, cx.tun.hash_cap_max, cx.cap_full, bound, f, tier, cnt_out, cx.hist, cx.hist + kOverFull);
             k_bin_scatter<<<(unsigned)((nc + 255) / 256), 256, 0, st>>>(tier, c_lo, c_hi, cx.hist,
                                                                        cx.cursor, list, off,
                                                                        heavy_ord_w);
             cx.tend(tb, st);
             cx.launched(2);
             SPG_CK(cudaGetLastError());
+          }
+          SPG_CK(cudaMemcpyAsync(cx.h_small, cx.hist, sizeof(int32_t) * (kOverFull + 1), cudaMemcpyDeviceToHost, st));
+          SPG_CK(cudaStreamSynchronize(st));
+          cx.over_full = cx.h_small[kOverFull];
+          std::memcpy(hist, cx.h_small, sizeof(hist));
+          if (!again) std::memcpy(&total, cx.h_small + kFlopTotal, sizeof(int64_t));
+          const int cap = recap && !again ? recap(total) : cx.tun.hash_cap_max;
+          if (cap == cx.tun.hash_cap_max) break;
+          cx.tun.hash_cap_max = cap;
         }
-        SPG_CK(cudaMemcpyAsync(cx.h_small, cx.hist, sizeof(int32_t) * (kFlopTotal + 2), cudaMemcpyDeviceToHost, st));
-        SPG_CK(cudaStreamSynchronize(st));
-        int hist[16];
-        std::memcpy(hist, cx.h_small, sizeof(hist));
-        if (total_out) std::memcpy(total_out, cx.h_small + kFlopTotal, sizeof(int64_t));
+        if (total_out) *total_out = total;
         if (nc <= 0) std::memset(hist, 0, sizeof(hist));
         if (hist_out) std::memcpy(hist_out, hist, sizeof(hist));
         int nheavy = 0;
@@ -579,6 +597,43 @@ template <class I, class V> struct Engine : EngineBase {
         return a;
     }
 
+    // Columns above this many rows are heavy (k_sym_heavy32, k_num_heavy32),
+    // unless the caller gave hash_max_cap. The largest table that fits a CTA
+    // (8192 rows) is not the best line: a dense item accumulates without
+    // probing, leaves its rows in order, and three run per SM against one
+    // 1024-thread CTA with the 8192-row table. Measured steps (sorted, cap 8192 ->
+    // this rule's):
+    //   m in one panel, m / 16: R-MAT 14 1.88 -> 1.34 ms, R-MAT of 3,000 rows
+    //     0.48 -> 0.35 ms, fp64 min-plus of 7,919 rows 1.08 -> 0.79 ms, uniform 16384
+    //     with 3,600 rows a column 1.64 -> 1.15 ms (m / 32 loses where columns stay
+    //     sparse: uniform 10,000 with 1,000 rows a column 0.56 -> 0.73 ms);
+    //   more panels, 4096: protein stand-in 20,011 / 100,000 columns 2.11 -> 1.83 /
+    //     12.9 -> 12.5 ms, R-MAT of 60,000 rows 6.20 -> 5.89 ms; from about 500,000 rows
+    //     on, the symbolic bitmaps leave one CTA per SM (1,000,000 columns 133 -> 135 ms).
+    // A k-split keeps 8192 (its stages read every heavy column again: 4-stage R-MAT 15
+    // 8.07 -> 8.24 ms), and so does a product that the budget may cut into batches.
+    static int heavy_rule(const PlanState &ps) {
+        if (!ps.cap_rule || ps.s > 1 || ps.opts.prune || ps.A.nnz >= (int64_t(1) << 31)) return ps.cap_full;
+        if (ps.P == 1) {
+            int cap = 256;
+            while (cap < ps.cap_full && (int64_t)cap * 16 < ps.m) cap *= 2;
+            return cap;
+        }
+        return ps.m <= (int64_t(1) << 19) ? std::min(ps.cap_full, 4096) : ps.cap_full;
+    }
+
+    // Whether C fits one batch whatever its columns' overlap is: with as many
+    // entries as multiplications, and the heavy columns' workspace at its largest.
+    static bool one_batch(const PlanState &ps, int64_t flops) {
+        const int64_t si = ps.idx64 ? 8 : 4, sv = sizeof(V), r = si + sv;
+        const int64_t inputs = (int64_t)(ps.A.nnz + ps.B.nnz) * r + (ps.A.ncols + ps.B.ncols + 2) * si;
+        const int64_t heavy = ps.A.nnz * (2 + 4 + 2 * sv) + ps.k * ((int64_t)ps.P + 1) * 16 +
+                              ps.n * ((int64_t)ps.P * 4 + 64) + (1 << 20);
+        const int64_t items = ps.P == 1 ? 0 : std::min(ps.n * (int64_t)ps.P, flops) * 28;
+        const int ring = ps.opts.ring_depth > 0 ? ps.opts.ring_depth : 2;
+        return inputs + (int64_t)ps.workspace_bytes() + heavy + items + ring * (flops * r + 8 * ps.n) <= (int64_t)ps.budget;
+    }
+
     static bool incremental(const PlanState &ps) {
         return ps.s > 1 && ps.opts.merge_mode == SPGEMM_MERGE_INCREMENTAL;
     }
@@ -611,14 +666,22 @@ template <class I, class V> struct Engine : EngineBase {
         const int64_t n = ps.n;
         ps.have_symbolic = false;
         ps.panels_built = false;
+        ps.tun.hash_cap_max = heavy_rule(ps);
         Ctx cx = make_ctx(ps);
         SPG_CK(cudaMemsetAsync(ps.err.p, 0, sizeof(int) * 4, st));
+        // the rule's cap stays where the flops bound C to a single batch
+        const auto recap = [&](int64_t flops) {
+            return cx.tun.hash_cap_max == ps.cap_full || one_batch(ps, flops) ? cx.tun.hash_cap_max : ps.cap_full;
+        };
         // full product: flops, counts, heavy list
         SPG_ST(sym_pass<SrcGemm<I, V>>(cx, gemm_args(ps, 0, ps.k), 0, n, nullptr, ps.f.as<int64_t>(),
                                        ps.tier.as<uint8_t>(), ps.cnt.as<int64_t>(),
                                        ps.list_sym.as<int32_t>(), ps.off_sym.as<int32_t>(),
                                        ps.heavy_ord.as<int32_t>(), ps.heavy_ord.as<int32_t>(),
-                                       &ps.pcnt, nullptr, ps.sym_hist, st, true, ps.B.nnz, &ps.flops));
+                                       &ps.pcnt, nullptr, ps.sym_hist, st, true, ps.B.nnz, &ps.flops, recap));
+        ps.tun.hash_cap_max = cx.tun.hash_cap_max;
+        // heavy columns by the rule alone: their workspace is not the budget's
+        ps.rule_only = ps.tun.hash_cap_max < ps.cap_full && cx.over_full == 0;
         ps.nheavy = 0;
         for (int t = kHeavyTier0; t < kTiers; ++t) ps.nheavy += ps.sym_hist[t];
         const int tsc = cx.tbegin(kPhScan, st);
@@ -879,11 +942,15 @@ template <class I, class V> struct Engine : EngineBase {
         const int64_t ptr_bytes = 8;
         const int64_t inputs = (int64_t)(ps.A.nnz + ps.B.nnz) * r +
                                (ps.A.ncols + 1 + ps.B.ncols + 1) * (ps.idx64 ? 8 : 4);
+        // heavy columns that only heavy_rule made heavy: the product was shown to
+        // fit one batch with their workspace, which is left out here so that
+        // the reported cap per batch does not depend on the rule
         // the stage partial buffers are part of each batch's bytes (w_j counts
         // the unmerged entries), so they are not workspace here; this keeps the
         // plan identical across repeated symbolic calls on one plan
         const int64_t ws = (int64_t)ps.workspace_bytes() - (int64_t)ps.drows.bytes -
-                           (int64_t)ps.dvals.bytes - (int64_t)ps.parts_tab.bytes;
+                           (int64_t)ps.dvals.bytes - (int64_t)ps.parts_tab.bytes -
+                           (ps.rule_only ? (int64_t)ps.heavy_bytes() : 0);
         const int64_t avail = (int64_t)ps.budget - inputs - ws;
         const int ring = ps.opts.ring_depth > 0 ? ps.opts.ring_depth : 2;
         if (avail <= 0) {
@@ -1385,6 +1452,7 @@ template <class I, class V> struct Engine : EngineBase {
             return SPGEMM_ERR_INVALID;
         }
         Ctx cx = make_ctx(ps);
+        cx.tun.hash_cap_max = ps.cap_full;   // tiers by G's columns, not the product's heavy rule
         const int64_t n = ps.n;
         GradArgs<I, V> ga{};
         ga.gemm = gemm_args(ps, 0, ps.k);

@@ -874,13 +874,14 @@ __global__ void __launch_bounds__(256) k_col_flops(GemmArgs<I, V> ga, int64_t n,
 // histogram. bound (optional) is the exact count of the unsplit product when a
 // k-stage is binned: columns with bound > hash_cap_max go to the heavy tier
 // (their stage output must be panel-grouped), others use min(f, bound) as
-// their size.
+// their size. over counts the columns above cap_full, the largest line.
 template <class Src>
 __global__ void __launch_bounds__(256) k_col_tier(typename Src::Args sa, int64_t c_lo, int64_t c_hi,
-                                                  int hash_cap_max, const int64_t *bound, const int64_t *f_in,
-                                                  uint8_t *tier_out, int64_t *cnt_out, int32_t *tier_hist) {
-    __shared__ int s_hist[kTiers];
-    if (threadIdx.x < kTiers) s_hist[threadIdx.x] = 0;
+                                                  int hash_cap_max, int cap_full, const int64_t *bound, const int64_t *f_in,
+                                                  uint8_t *tier_out, int64_t *cnt_out, int32_t *tier_hist,
+                                                  int32_t *over) {
+    __shared__ int s_hist[kTiers + 1];
+    if (threadIdx.x <= kTiers) s_hist[threadIdx.x] = 0;
     __syncthreads();
     const int64_t g = c_lo + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (g < c_hi) {
@@ -895,6 +896,7 @@ __global__ void __launch_bounds__(256) k_col_tier(typename Src::Args sa, int64_t
             m = sa.probs->m;
         }
         int64_t u = f < m ? f : m;
+        if (u > cap_full) atomicAdd(&s_hist[kTiers], 1);
         int t;
         if (bound && bound[g] > hash_cap_max) {
             t = heavy_subtier(f);
@@ -910,6 +912,7 @@ __global__ void __launch_bounds__(256) k_col_tier(typename Src::Args sa, int64_t
     __syncthreads();
     if (threadIdx.x < kTiers && s_hist[threadIdx.x])
         atomicAdd(&tier_hist[threadIdx.x], s_hist[threadIdx.x]);
+    if (threadIdx.x == kTiers && s_hist[kTiers]) atomicAdd(over, s_hist[kTiers]);
 }
 
 // Both steps in one launch for the columns of many problems (the batched

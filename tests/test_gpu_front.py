@@ -186,3 +186,40 @@ def test_item_lists_of_every_form(m, cols):
     order = torch.sort(rows, dim=1)
     assert torch.equal(C.rowidx.long(), order.values.reshape(-1))
     assert torch.equal(C.vals, torch.gather(vals, 1, order.indices).reshape(-1))
+
+
+@pytest.mark.parametrize("m", [900, 5000, 20000])
+def test_heavy_rule_keeps_the_batch_plan(m):
+    """Which columns are heavy depends on the row count by default; whatever the
+    budget, the plan has the batches (or the refusal) of the fixed 8192-row line,
+    and the product is the same."""
+    n = 600
+    g = torch.Generator(device="cuda")
+    g.manual_seed(m)
+    counts = torch.randint(1, m // 2, (n,), generator=g, device="cuda")
+    ptr = torch.zeros(n + 1, dtype=torch.int64, device="cuda")
+    ptr[1:] = torch.cumsum(counts, 0)
+    col = torch.repeat_interleave(torch.arange(n, device="cuda"), counts)
+    start = torch.randint(0, m, (n,), generator=g, device="cuda")
+    rows = (start[col] + torch.arange(col.numel(), device="cuda") - ptr[col]) % m
+    vals = torch.randint(1, 5, (col.numel(),), generator=g, device="cuda").double()
+    A = spg.Csc(m, n, ptr.int(), rows.int(), vals)
+    B, _ = ragged(n, 700, m)
+    B = spg.Csc(n, 700, B.colptr, B.rowidx, B.vals.double())
+    whole = spg.spgemm(A, B, sort_output=True, tuning=spg.Tuning(hash_max_cap=8192))
+    need = 12 * whole.nnz
+    batches = set()
+    for budget in [1 << 20] + [int(need * f) + (60 << 20) for f in (0.2, 0.5, 1, 2, 4, 10, 40)]:
+        seen = []
+        for tun in (None, spg.Tuning(hash_max_cap=8192)):
+            try:
+                C = spg.spgemm(A, B, sort_output=True, budget=budget, tuning=tun)
+            except spg.SpgemmError as e:
+                seen.append(str(e.status))
+                continue
+            seen.append(C.plan_info["nbatches"])
+            assert torch.equal(C.colptr, whole.colptr) and torch.equal(C.rowidx, whole.rowidx)
+            assert torch.equal(C.vals, whole.vals)
+        assert seen[0] == seen[1]
+        batches.add(seen[0])
+    assert len(batches) > 1
