@@ -161,6 +161,9 @@ template <class I, class V> struct Engine : EngineBase {
         set_smem(k_num_dense<SrcPanel<I, V>>, mx);
         set_smem(k_num_dense<SrcPartsPanel<I, V>>, mx);
         set_smem(k_bwd_dense<I, V>, mx);
+        set_smem(k_light<I, V, 1024, 0>, mx);
+        set_smem(k_light<I, V, 512, 1>, mx);
+        set_smem(k_light<I, V, 1024, 1>, mx);
         set_smem(k_sym_warp<SrcGemm<I, V>, 1024>, mx);
         set_smem(k_sym_warp<SrcParts<I, V>, 1024>, mx);
         set_smem(k_num_warp<SrcGemm<I, V>, 512>, mx);
@@ -202,10 +205,21 @@ template <class I, class V> struct Engine : EngineBase {
         const int T = 2 * tier_cap(t);
         if (t <= kWarpTiers) {
             // one warp per column, 8 warps per CTA, warp-private tables
-            const int smem = 8 * T * 4;
+            const int smem = light_smem<V>(T, 0);
             const int per_sm = std::max(1, std::min(8, (228 * 1024) / (smem + 1024)));
             const int want = count < 0 ? cx.nsm * per_sm : (count + 7) / 8;
             const int blocks = std::max(1, std::min(want, cx.nsm * per_sm));
+            if constexpr (!Src::kParts) {
+                if (sa.lean_dense) {
+                    switch (T) {
+                        case 64: k_light<I, V, 64, 0><<<blocks, 256, smem, st>>>(sa, c, nullptr, nullptr); break;
+                        case 256: k_light<I, V, 256, 0><<<blocks, 256, smem, st>>>(sa, c, nullptr, nullptr); break;
+                        case 512: k_light<I, V, 512, 0><<<blocks, 256, smem, st>>>(sa, c, nullptr, nullptr); break;
+                        default: k_light<I, V, 1024, 0><<<blocks, 256, smem, st>>>(sa, c, nullptr, nullptr); break;
+                    }
+                    return;
+                }
+            }
             switch (T) {
                 case 64: k_sym_warp<Src, 64><<<blocks, 256, smem, st>>>(sa, c); break;
                 case 256: k_sym_warp<Src, 256><<<blocks, 256, smem, st>>>(sa, c); break;
@@ -236,10 +250,21 @@ template <class I, class V> struct Engine : EngineBase {
         c.tier = t;
         const int T = 2 * tier_cap(t);
         if (t <= kWarpTiers) {
-            const int smem = 8 * T * (int)(4 + sizeof(V));
+            const int smem = light_smem<V>(T, 1);
             const int per_sm = std::max(1, std::min(8, (228 * 1024) / (smem + 1024)));
             const int want = count < 0 ? cx.nsm * per_sm : (count + 7) / 8;
             const int blocks = std::max(1, std::min(want, cx.nsm * per_sm));
+            if constexpr (!Src::kParts) {
+                if (sa.lean_dense) {
+                    switch (T) {
+                        case 64: k_light<I, V, 64, 1><<<blocks, 256, smem, st>>>(sa, c, rows, vals); break;
+                        case 256: k_light<I, V, 256, 1><<<blocks, 256, smem, st>>>(sa, c, rows, vals); break;
+                        case 512: k_light<I, V, 512, 1><<<blocks, 256, smem, st>>>(sa, c, rows, vals); break;
+                        default: k_light<I, V, 1024, 1><<<blocks, 256, smem, st>>>(sa, c, rows, vals); break;
+                    }
+                    return;
+                }
+            }
             switch (T) {
                 case 64: k_num_warp<Src, 64><<<blocks, 256, smem, st>>>(sa, c, rows, vals); break;
                 case 256: k_num_warp<Src, 256><<<blocks, 256, smem, st>>>(sa, c, rows, vals); break;

@@ -2031,5 +2031,6 @@ template <class V> __global__ void k_fill_zero(V *p, int64_t n) {
 }  // namespace spg
 
 #include "dense_items.cuh"
+#include "light_cols.cuh"
 #include "sym_heavy32.cuh"
 #include "multi_persistent.cuh"

@@ -1,0 +1,201 @@
+// Light columns of a product, one warp each, with a warp-private hash table in
+// shared memory (C(:, j) = A * B(:, j), Sec. II-C's column formula): the
+// symbolic count and the numeric accumulation, with 32-bit entry offsets (the
+// caller guarantees nnz(A) < 2^31).
+//
+// A column of some hundred products is a chain of dependent loads (column
+// list, colptr of B, its rows, colptr of A, A's entries) around little work, so
+// the kernels are bound by that latency and by the warps the tables leave
+// room for. The chain is spread over the column before: its list entry is read
+// two columns ahead, the colptr of B when the previous column starts, B's rows
+// after that column's walk and the colptr of A after its output. Measured against
+// one chain per column (symbolic / numeric, us): 2-path counts of 200,000 vertices
+// with 4 entries a column 103 / 155 -> 75 / 132, uniform 100,000 columns of 11 84 / 174
+// -> 67 / 158, 2-path counts 50,021 x 16 97 / 316 -> 81 / 289. What is left is issue:
+// some 240 warp instructions per 32 products, the compare-and-swap loops of
+// the inserts and of the value adds first (issue slots 40 to 53% busy, a quarter to
+// half of the warps resident beside the tables).
+#pragma once
+
+namespace spg {
+
+// Dynamic shared memory of k_light: 8 tables and 8 segment lists.
+template <class V> constexpr int light_smem(int T, int mode) {
+    return 8 * (T + 32) * (4 + (mode == 1 ? (int)sizeof(V) : 0));
+}
+
+// MODE 0: symbolic (c.cnt[g]); MODE 1: numeric, rows in table order or
+// ascending (c.sort).
+template <class I, class V, int T, int MODE>
+__global__ void __launch_bounds__(256) k_light(GemmArgs<I, V> ga, TierCommon c, I *out_rows, V *out_vals) {
+    constexpr int LOG2T = Log2<T>::v;
+    constexpr int U = 4;   // windows whose loads are in flight
+    // how a lane finds its segment: a shuffle search over the lanes, or one
+    // OR-reduce of the segment starts and a table in shared memory (fewer
+    // instructions; the large numeric tables gain from the registers instead)
+    constexpr bool kSearch = MODE == 1 && T >= 512;
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    V *vals = MODE == 1 ? reinterpret_cast<V *>(smem) + warp * T : nullptr;
+    uint32_t *keys = reinterpret_cast<uint32_t *>(smem + (MODE == 1 ? sizeof(V) * 8 * T : 0)) + warp * T;
+    // per warp: the non-empty segments of a round, in stream order
+    unsigned char *segs = smem + (size_t)8 * T * (4 + (MODE == 1 ? sizeof(V) : 0));
+    V *s_bv = reinterpret_cast<V *>(segs) + warp * 32;
+    int *s_off = reinterpret_cast<int *>(segs + (MODE == 1 ? 8 * 32 * sizeof(V) : 0)) + warp * 32;
+    const ProbDev<I, V> *pd = ga.probs;
+    const I *bp = pd->bp, *bi = pd->bi, *ap = pd->ap, *ai = pd->ai;
+    const V *bv = pd->bv, *av = pd->av;
+    const int64_t k0 = ga.k0, k1 = ga.k1;
+    const unsigned below = (1u << lane) - 1u, upto = 0xffffffffu >> (31 - lane);
+    const int hi = c.list_off[c.tier + 1];
+    const int stride = gridDim.x * 8;
+    int it = c.list_off[c.tier] + blockIdx.x * 8 + warp;
+    if (it >= hi) return;
+    // the segment of A that B entry e holds
+    auto segment = [&](int64_t k, bool any, int &beg, int &len) {
+        beg = 0;
+        len = 0;
+        if (any && k >= k0 && k < k1) {
+            const int64_t a = (int64_t)__ldg(&ap[k]);
+            beg = (int)a;
+            len = (int)((int64_t)__ldg(&ap[k + 1]) - a);
+        }
+    };
+    int g = c.list[it];
+    int gn = it + stride < hi ? c.list[it + stride] : -1;
+    int64_t b0 = (int64_t)__ldg(&bp[g]);
+    int nb = (int)((int64_t)__ldg(&bp[g + 1]) - b0);
+    int64_t k = lane < nb ? (int64_t)__ldg(&bi[b0 + lane]) : 0;
+    V bval = V(0);
+    if (MODE == 1 && lane < nb) bval = __ldg(&bv[b0 + lane]);
+    int beg, len;
+    segment(k, lane < nb, beg, len);
+    // the table is cleared once; a column's output leaves it clean
+    for (int s = lane; s < T; s += 32) {
+        keys[s] = kEmpty;
+        if (MODE == 1) vals[s] = V(0);
+    }
+    __syncwarp();
+    for (;;) {
+        const int64_t b0n = gn >= 0 ? (int64_t)__ldg(&bp[gn]) : 0;
+        const int64_t b1n = gn >= 0 ? (int64_t)__ldg(&bp[gn + 1]) : 0;
+        const int gnn = it + 2 * (int64_t)stride < hi ? c.list[it + 2 * stride] : -1;
+        int64_t o0 = 0, o1 = 0;
+        if (MODE == 1) { o0 = c.colptr[g]; o1 = c.colptr[g + 1]; }
+        int mine = 0;
+        for (int base = 0;;) {
+            // this round's segments, one per lane, as a stream [0, tot)
+            const int incl = warp_incl_scan(len);
+            const int excl = incl - len;
+            const int tot = __shfl_sync(SPG_FULL, incl, 31);
+            const int off = beg - excl;   // stream position + off = entry index
+            if (!kSearch) {
+                // the non-empty segments in stream order
+                const unsigned nzm = __ballot_sync(SPG_FULL, len > 0);
+                if (len > 0) {
+                    const int rank = __popc(nzm & below);
+                    s_off[rank] = off;
+                    if (MODE == 1) s_bv[rank] = bval;
+                }
+                __syncwarp();
+            }
+            int before = -1;   // segments started before the window, minus one
+            for (int w = 0; w < tot; w += 32 * U) {
+                uint32_t r[U];
+                V x[U];
+                bool ok[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int p = w + 32 * u + lane;
+                    ok[u] = p < tot;
+                    int q;
+                    V vs;
+                    if (kSearch) {
+                        // the last lane whose segment starts at or before p
+                        int sl = 0;
+#pragma unroll
+                        for (int b = 16; b > 0; b >>= 1) {
+                            const int e = __shfl_sync(SPG_FULL, excl, sl + b);
+                            if (e <= p) sl += b;
+                        }
+                        q = __shfl_sync(SPG_FULL, off, sl) + p;
+                        if (MODE == 1) vs = shfl_bits(bval, sl);
+                    } else {
+                        // the segments started before the window plus the starts
+                        // at or below the lane
+                        const unsigned d = (unsigned)(excl - (w + 32 * u));
+                        const unsigned M = __reduce_or_sync(SPG_FULL, len > 0 && d < 32u ? 1u << d : 0u);
+                        const int sl = before + __popc(M & upto);
+                        before += __popc(M);
+                        q = ok[u] ? s_off[sl] + p : 0;
+                        if (MODE == 1 && ok[u]) vs = s_bv[sl];
+                    }
+                    if (ok[u]) {
+                        r[u] = (uint32_t)__ldg(&ai[q]);
+                        if (MODE == 1) x[u] = mul_v(__ldg(&av[q]), vs);
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    if (!ok[u]) continue;
+                    bool nw;
+                    const int h = hash_insert_dbl1(keys, LOG2T, r[u], c.err, nw);
+                    if (MODE == 0) mine += nw;
+                    else if (h >= 0) atomic_add_v(&vals[h], x[u]);
+                }
+            }
+            base += 32;
+            if (base >= nb) break;
+            if (!kSearch) __syncwarp();   // the segments are read: the next round may replace them
+            const bool any = base + lane < nb;
+            k = any ? (int64_t)__ldg(&bi[b0 + base + lane]) : 0;
+            if (MODE == 1 && any) bval = __ldg(&bv[b0 + base + lane]);
+            segment(k, any, beg, len);
+        }
+        // the next column's rows of B, on their way during this one's output
+        b0 = b0n;
+        nb = (int)(b1n - b0n);
+        k = lane < nb ? (int64_t)__ldg(&bi[b0 + lane]) : 0;
+        if (MODE == 1 && lane < nb) bval = __ldg(&bv[b0 + lane]);
+        __syncwarp();
+        if (MODE == 0) {
+            mine = warp_sum(mine);
+            if (lane == 0) c.cnt[g] = mine;
+            uint4 *k4 = reinterpret_cast<uint4 *>(keys);
+            for (int s = lane; s < T / 4; s += 32) k4[s] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
+        } else {
+            const int64_t out0 = o0 - c.out_base;
+            const int want = (int)(o1 - o0);
+            if (c.sort) {
+                sorted_emit<false>(keys, vals, T, want, nullptr, c.err, out_rows + out0, out_vals + out0);
+            } else {
+                int pos = 0;
+                for (int s0 = 0; s0 < T; s0 += 32) {
+                    const int s = s0 + lane;
+                    const uint32_t key = keys[s];
+                    const bool occ = key != kEmpty;
+                    const unsigned bal = __ballot_sync(SPG_FULL, occ);
+                    if (occ) {
+                        const int r = pos + __popc(bal & below);
+                        if (r < want) {
+                            out_rows[out0 + r] = (I)key;
+                            out_vals[out0 + r] = vals[s];
+                        }
+                        keys[s] = kEmpty;
+                        vals[s] = V(0);
+                    }
+                    pos += __popc(bal);
+                }
+                if (lane == 0 && pos != want) atomicOr(c.err, kErrCount);
+            }
+        }
+        if (gn < 0) return;
+        segment(k, lane < nb, beg, len);
+        g = gn;
+        gn = gnn;
+        it += stride;
+        __syncwarp();
+    }
+}
+
+}  // namespace spg

@@ -223,3 +223,38 @@ def test_heavy_rule_keeps_the_batch_plan(m):
         assert seen[0] == seen[1]
         batches.add(seen[0])
     assert len(batches) > 1
+
+
+@pytest.mark.parametrize("vt", [torch.float32, torch.int64])
+@pytest.mark.parametrize("stages,sort", [(1, True), (1, False), (3, True)])
+def test_light_columns_with_many_short_segments(vt, stages, sort):
+    """Columns of B around a warp's 32 entries and several rounds of them, over
+    columns of A with 0 to 3 entries (empty segments between), every warp tier."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(5)
+    m, k = 700, 2000
+    ca = torch.randint(0, 4, (k,), generator=g, device="cuda")
+    ap = torch.zeros(k + 1, dtype=torch.int64, device="cuda")
+    ap[1:] = torch.cumsum(ca, 0)
+    cola = torch.repeat_interleave(torch.arange(k, device="cuda"), ca)
+    ra = (torch.randint(0, m, (k,), generator=g, device="cuda")[cola] + 11 * (torch.arange(cola.numel(), device="cuda") - ap[cola])) % m
+    A = spg.Csc(m, k, ap.int(), ra.int(), torch.randint(1, 5, (cola.numel(),), generator=g, device="cuda").to(vt))
+    cb = torch.tensor([0, 1, 5, 31, 32, 33, 63, 64, 65, 128, 200, 300], device="cuda").repeat(9)
+    n = cb.numel()
+    bp = torch.zeros(n + 1, dtype=torch.int64, device="cuda")
+    bp[1:] = torch.cumsum(cb, 0)
+    colb = torch.repeat_interleave(torch.arange(n, device="cuda"), cb)
+    rb = (torch.randint(0, k, (n,), generator=g, device="cuda")[colb] + 3 * (torch.arange(colb.numel(), device="cuda") - bp[colb])) % k
+    B = spg.Csc(k, n, bp.int(), rb.int(), torch.randint(1, 5, (colb.numel(),), generator=g, device="cuda").to(vt))
+    C = spg.spgemm(A, B, sort_output=sort, kstages=stages, tuning=spg.Tuning(hash_max_cap=8192))
+    da = torch.zeros(m, k, dtype=torch.float64, device="cuda")
+    da[ra, cola] = A.vals.double()
+    db = torch.zeros(k, n, dtype=torch.float64, device="cuda")
+    db[rb, colb] = B.vals.double()
+    want, reached = (da @ db).T, ((da != 0).double() @ (db != 0).double()).T > 0
+    colc = torch.repeat_interleave(torch.arange(n, device="cuda"), C.colptr.diff())
+    got = torch.zeros(n, m, dtype=torch.float64, device="cuda")
+    got[colc, C.rowidx.long()] = C.vals.double()
+    assert torch.equal(C.colptr.diff(), reached.sum(1)) and torch.equal(got, want)
+    if sort:
+        assert torch.equal(colc * m + C.rowidx, torch.nonzero(reached.reshape(-1)).reshape(-1))
