@@ -188,8 +188,10 @@ template <class I, class V> struct Engine : EngineBase {
         set_smem(k_num_heavy32<I, V, 2, true>, mx);
         set_smem(k_num_heavy32<I, V, 3, false>, mx);
         set_smem(k_num_heavy32<I, V, 3, true>, mx);
-        set_smem(k_sort_block<I, V, 1024>, mx);
-        set_smem(k_sort_block<I, V, 8192>, mx);
+        set_smem(k_sort_cols<I, V, 512, false>, mx);
+        set_smem(k_sort_cols<I, V, 2048, true>, mx);
+        set_smem(k_sort_cols<I, V, 16384, true>, mx);
+        set_smem(k_prune_select<I, V, I>, mx);
         set_smem(k_sort_items<I, V, 8192>, mx);
         set_smem(k_sort_items<I, V, 4096>, mx);
         (void)sv;
@@ -1356,25 +1358,21 @@ template <class I, class V> struct Engine : EngineBase {
         else return V::raw(t);
     }
 
-    // prune workspace bytes per column (PruneWs: keep, sel, key, quota 8 B, row
-    // 4 B, mode 1 B, and the scan partials)
+    // bytes per column that the batch plan sets aside for the prune workspace
+    // (PruneWs: keep and sel 8 B, mode 1 B, and the scan partials; an upper bound)
     static constexpr int64_t kPruneWsPerCol = 40;
 
     // Prune step 1: kept count per column, the selections, and out_colptr =
     // exclusive scan of the counts (ncols + 1 entries, total last).
-    static spgemm_status prune_plan(const int64_t *colptr, const I *rows, const V *vals, int64_t ncols, V thr,
-                                    int64_t topk, int tie_by_row, PruneWs &ws, int64_t *out_colptr, int nsm,
-                                    cudaStream_t st) {
+    static spgemm_status prune_plan(const int64_t *colptr, const V *vals, int64_t ncols, V thr, int64_t topk,
+                                    PruneWs &ws, int64_t *out_colptr, cudaStream_t st) {
         SPG_CK(ws.ensure(ncols));
-        SPG_CK(cudaMemsetAsync(ws.nsel.p, 0, sizeof(unsigned long long), st));
+        SPG_CK(cudaMemsetAsync(ws.nsel.p, 0, 2 * sizeof(unsigned long long), st));
         if (ncols > 0) {
             const unsigned wb = (unsigned)std::max<int64_t>(1, std::min<int64_t>((ncols + 7) / 8, 1 << 20));
             k_prune_count<V><<<wb, 256, 0, st>>>(colptr, vals, ncols, thr, topk, ws.keep.as<int64_t>(),
                                                  ws.mode.as<int8_t>(), ws.sel.as<int64_t>(),
                                                  ws.nsel.as<unsigned long long>());
-            k_prune_select<I, V><<<(unsigned)nsm * 4, 512, 0, st>>>(
-                colptr, rows, vals, thr, topk, ws.sel.as<int64_t>(), ws.nsel.as<unsigned long long>(),
-                ws.key.as<uint64_t>(), ws.quota.as<int64_t>(), tie_by_row, ws.row.as<uint32_t>());
         }
         SPG_CK(exclusive_scan_i64(ws.keep.as<int64_t>(), ncols, out_colptr, ws.part.as<int64_t>(), 1, st));
         SPG_CK(cudaGetLastError());
@@ -1384,13 +1382,19 @@ template <class I, class V> struct Engine : EngineBase {
     // Prune step 2: the kept entries, in input order, at out_colptr.
     template <class IO>
     static spgemm_status prune_fill(const int64_t *colptr, const I *rows, const V *vals, int64_t ncols, V thr,
-                                    int tie_by_row, PruneWs &ws, const int64_t *out_colptr, IO *orows, V *ovals,
-                                    cudaStream_t st) {
+                                    int64_t topk, int tie_by_row, PruneWs &ws, const int64_t *out_colptr, IO *orows,
+                                    V *ovals, int nsm, cudaStream_t st) {
         if (ncols <= 0) return SPGEMM_OK;
         const unsigned wb = (unsigned)std::max<int64_t>(1, std::min<int64_t>((ncols + 7) / 8, 1 << 20));
-        k_prune_compact<I, V, IO><<<wb, 256, 0, st>>>(colptr, rows, vals, ncols, thr, ws.mode.as<int8_t>(),
-                                                      ws.key.as<uint64_t>(), ws.quota.as<int64_t>(), tie_by_row,
-                                                      ws.row.as<uint32_t>(), out_colptr, orows, ovals);
+        k_prune_compact<I, V, IO><<<wb, 256, 0, st>>>(colptr, rows, vals, ncols, thr, ws.mode.as<int8_t>(), out_colptr,
+                                                      orows, ovals);
+        if (topk > 0) {
+            // 100 KB of staged keys: two CTAs of 512 threads per SM
+            const int bytes = 100 * 1024, cap = bytes / (KeyBits<V>::v / 8);
+            k_prune_select<I, V, IO><<<(unsigned)nsm * 2, kPruneThreads, bytes, st>>>(
+                colptr, rows, vals, thr, topk, ws.sel.as<int64_t>(), ws.nsel.as<unsigned long long>(), tie_by_row, cap,
+                out_colptr, orows, ovals);
+        }
         SPG_CK(cudaGetLastError());
         return SPGEMM_OK;
     }
@@ -1398,6 +1402,7 @@ template <class I, class V> struct Engine : EngineBase {
     // spgemm_prune on a caller's CSC (two-call protocol).
     static spgemm_status prune(const spgemm_csc *in, double thr_d, int64_t topk, spgemm_csc *out,
                                cudaStream_t st) {
+        attrs();
         int dev = 0, nsm = 148;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -1420,7 +1425,7 @@ template <class I, class V> struct Engine : EngineBase {
             SPG_CK(tmp.ensure(sizeof(int64_t) * (size_t)(n + 1)));
             ocp = tmp.as<int64_t>();
         }
-        SPG_ST(prune_plan(cp, (const I *)in->rowidx, (const V *)in->vals, n, thr, topk, 0, ws, ocp, nsm, st));
+        SPG_ST(prune_plan(cp, (const V *)in->vals, n, thr, topk, ws, ocp, st));
         if (count_only) {
             int64_t total = 0;
             SPG_CK(cudaMemcpyAsync(&total, ocp + n, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
@@ -1429,8 +1434,8 @@ template <class I, class V> struct Engine : EngineBase {
             return SPGEMM_OK;
         }
         const int64_t *fin = (const int64_t *)out->colptr;
-        SPG_ST(prune_fill<I>(cp, (const I *)in->rowidx, (const V *)in->vals, n, thr, 0, ws, fin, (I *)out->rowidx,
-                             (V *)out->vals, st));
+        SPG_ST(prune_fill<I>(cp, (const I *)in->rowidx, (const V *)in->vals, n, thr, topk, 0, ws, fin,
+                             (I *)out->rowidx, (V *)out->vals, nsm, st));
         SPG_CK(cudaStreamSynchronize(st));   // the scratch buffers go out of scope
         return SPGEMM_OK;
     }
@@ -1443,22 +1448,22 @@ template <class I, class V> struct Engine : EngineBase {
         // the smaller rows, the order sorting would give), then sort only
         // the kept entries
         const int tie_by_row = ps.defer_sort ? 1 : 0;
-        SPG_ST(prune_plan(colptr, (const I *)rows, (const V *)vals, ncols, thr, ps.opts.prune_topk, tie_by_row, ws,
-                          ocolptr, ps.nsm, st));
-        SPG_ST(prune_fill<I>(colptr, (const I *)rows, (const V *)vals, ncols, thr, tie_by_row, ws, ocolptr,
-                             (I *)orows, (V *)ovals, st));
+        const int64_t topk = ps.opts.prune_topk;
+        SPG_ST(prune_plan(colptr, (const V *)vals, ncols, thr, topk, ws, ocolptr, st));
+        SPG_ST(prune_fill<I>(colptr, (const I *)rows, (const V *)vals, ncols, thr, topk, tie_by_row, ws, ocolptr,
+                             (I *)orows, (V *)ovals, ps.nsm, st));
         ps.timer.launches += 6;
-        if (ps.defer_sort) {
-            const int cap = (int)std::min<int64_t>(ps.opts.prune_topk, 8192);
-            const unsigned wbk = (unsigned)std::max<int64_t>(1, std::min<int64_t>((ncols + 7) / 8, 1 << 20));
-            const unsigned bb = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ncols, (int64_t)ps.nsm * 8));
-            k_sort_warp<I, V><<<wbk, 256, 0, st>>>(ocolptr, 0, 0, ncols, (I *)orows, (V *)ovals);
-            if (cap > 32)
-                k_sort_block<I, V, 1024><<<bb, 256, (int)(1024 * (4 + sizeof(V))), st>>>(
-                    ocolptr, 0, 0, ncols, 32, cap, (I *)orows, (V *)ovals);
-            if (cap > 1024)
-                k_sort_block<I, V, 8192><<<bb, 512, (int)(8192 * (4 + sizeof(V))), st>>>(
-                    ocolptr, 0, 0, ncols, 1024, cap, (I *)orows, (V *)ovals);
+        if (ps.defer_sort && ncols > 0) {
+            // columns of up to 256 kept entries by a warp, 1024 and 8192 by a CTA
+            const unsigned wbk = (unsigned)std::max<int64_t>(1, std::min<int64_t>((ncols + 7) / 8, (int64_t)ps.nsm * 8));
+            const unsigned bb = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ncols, (int64_t)ps.nsm * 4));
+            const int slot = 4 + (int)sizeof(V);
+            k_sort_cols<I, V, 512, false><<<wbk, 256, 8 * 512 * slot, st>>>(ocolptr, ncols, 0, (I *)orows, (V *)ovals);
+            if (topk > 256)
+                k_sort_cols<I, V, 2048, true><<<bb, 512, 2048 * slot, st>>>(ocolptr, ncols, 256, (I *)orows, (V *)ovals);
+            if (topk > 1024)
+                k_sort_cols<I, V, 16384, true><<<bb, 512, 16384 * slot, st>>>(ocolptr, ncols, 1024, (I *)orows,
+                                                                             (V *)ovals);
             ps.timer.launches += 3;
             SPG_CK(cudaGetLastError());
         }

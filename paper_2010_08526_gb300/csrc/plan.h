@@ -128,10 +128,10 @@ class CallScratch {
 
 int64_t scan_partials_len(int64_t n);
 
-// Workspace of the column prune (per column: kept count, mode, selection
-// list, selected key and tie quota; scan partials).
+// Workspace of the column prune (per column: kept count, mode, selection list;
+// scan partials).
 struct PruneWs {
-    DevBuf arena, keep, mode, sel, nsel, key, quota, part, row;
+    DevBuf arena, keep, mode, sel, nsel, part;
     int64_t cols = -1;   // columns that the parts hold
     cudaError_t ensure(int64_t ncols) {
         if (ncols <= cols) return cudaSuccess;
@@ -139,14 +139,13 @@ struct PruneWs {
         cols = -1;
         const cudaError_t e = carve<SPGEMM_MEM_DEVICE>(
             arena, {{&keep, sizeof(int64_t) * c}, {&mode, c + 15}, {&sel, sizeof(int64_t) * c},
-                    {&nsel, sizeof(unsigned long long) * 2}, {&key, sizeof(uint64_t) * c},
-                    {&quota, sizeof(int64_t) * c}, {&row, sizeof(uint32_t) * c},
+                    {&nsel, sizeof(unsigned long long) * 2},
                     {&part, sizeof(int64_t) * (size_t)scan_partials_len(ncols + 1)}});
         if (e == cudaSuccess) cols = ncols;
         return e;
     }
     size_t bytes() const {
-        return keep.bytes + mode.bytes + sel.bytes + nsel.bytes + key.bytes + quota.bytes + part.bytes + row.bytes;
+        return keep.bytes + mode.bytes + sel.bytes + nsel.bytes + part.bytes;
     }
     void release(bool synced = false) {
         arena.release(synced);
