@@ -170,6 +170,8 @@ template <class I, class V> struct Engine : EngineBase {
         set_smem(k_num_warp<SrcGemm<I, V>, 1024>, mx);
         set_smem(k_num_warp<SrcParts<I, V>, 512>, mx);
         set_smem(k_num_warp<SrcParts<I, V>, 1024>, mx);
+        set_smem(k_bwd_light<I, V, 512>, mx);
+        set_smem(k_bwd_light<I, V, 1024>, mx);
         set_smem(k_bwd_warp<I, V, 512>, mx);
         set_smem(k_bwd_warp<I, V, 1024>, mx);
         set_smem(k_num_heavy<SrcPanelRange<I, V>, SrcColRange<I, V>, 2>, mx);
@@ -1517,9 +1519,19 @@ template <class I, class V> struct Engine : EngineBase {
             c.tier = t;
             const int T = 2 * tier_cap(t);
             if (t <= kWarpTiers) {
-                const int smem = 8 * T * (int)(4 + sizeof(V));
+                const bool lean = ga.gemm.lean_dense != 0;
+                const int smem = 8 * T * (int)(4 + sizeof(V)) + (lean ? 8 * 32 * (int)(8 + sizeof(V)) : 0);
                 const int per_sm = std::max(1, std::min(8, (228 * 1024) / (smem + 1024)));
                 const int blocks = std::max(1, std::min((hist[t] + 7) / 8, cx.nsm * per_sm));
+                if (lean) {
+                    switch (T) {
+                        case 64: k_bwd_light<I, V, 64><<<blocks, 256, smem, st>>>(ga, c); break;
+                        case 256: k_bwd_light<I, V, 256><<<blocks, 256, smem, st>>>(ga, c); break;
+                        case 512: k_bwd_light<I, V, 512><<<blocks, 256, smem, st>>>(ga, c); break;
+                        default: k_bwd_light<I, V, 1024><<<blocks, 256, smem, st>>>(ga, c); break;
+                    }
+                    continue;
+                }
                 switch (T) {
                     case 64: k_bwd_warp<I, V, 64><<<blocks, 256, smem, st>>>(ga, c); break;
                     case 256: k_bwd_warp<I, V, 256><<<blocks, 256, smem, st>>>(ga, c); break;

@@ -198,4 +198,126 @@ __global__ void __launch_bounds__(256) k_light(GemmArgs<I, V> ga, TierCommon c, 
     }
 }
 
+// Masked backward of light columns (columns of G of at most T / 2 entries),
+// one warp each: for every product A(i, k) B(k, j) with G(i, j) stored,
+//   dA(i, k) += G(i, j) B(k, j),  dB(k, j) += A(i, k) G(i, j).
+// G(:, j) is looked up in a warp-private table. The products are walked as one
+// stream with four windows of loads in flight; a window's lanes in one segment
+// (one B entry) add up their parts of dB in registers, so dB takes one global
+// add per segment and window, and dA's adds go to consecutive entries. Walking
+// one segment after another with an add per product for both took 377 us for
+// configuration 5 (12.8 M products), now 189 us (and dB is closer to its 64-bit value: 4.8e-8 against 6.5e-8).
+template <class I, class V, int T>
+__global__ void __launch_bounds__(256) k_bwd_light(GradArgs<I, V> a, TierCommon c) {
+    constexpr int LOG2T = Log2<T>::v;
+    constexpr int U = 4;
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    V *gv = reinterpret_cast<V *>(smem) + warp * T;
+    uint32_t *keys = reinterpret_cast<uint32_t *>(smem + sizeof(V) * 8 * T) + warp * T;
+    unsigned char *segs = smem + (size_t)8 * T * (4 + sizeof(V));
+    V *s_bv = reinterpret_cast<V *>(segs) + warp * 32;
+    int *s_off = reinterpret_cast<int *>(segs + 8 * 32 * sizeof(V)) + warp * 32;
+    int *s_e = reinterpret_cast<int *>(segs + 8 * 32 * (sizeof(V) + 4)) + warp * 32;
+    const ProbDev<I, V> *pd = a.gemm.probs;
+    const I *bp = pd->bp, *bi = pd->bi, *ap = pd->ap, *ai = pd->ai;
+    const V *bv = pd->bv, *av = pd->av;
+    V *dA = a.dA, *dB = a.dB;
+    const unsigned below = (1u << lane) - 1u, upto = 0xffffffffu >> (31 - lane);
+    const unsigned above = ~upto;
+    const int lo = c.list_off[c.tier], hi = c.list_off[c.tier + 1];
+    uint4 *k4 = reinterpret_cast<uint4 *>(keys);
+    for (int s = lane; s < T / 4; s += 32) k4[s] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
+    __syncwarp();
+    for (int it = lo + blockIdx.x * 8 + warp; it < hi; it += gridDim.x * 8) {
+        const int64_t g = c.list[it];
+        int64_t gb, ge;
+        g_range(a, g, gb, ge);
+        const int64_t b0 = (int64_t)__ldg(&bp[g]);
+        const int nb = (int)((int64_t)__ldg(&bp[g + 1]) - b0);
+        for (int64_t q = gb + lane; q < ge; q += 32) {
+            const int h = hash_insert_dbl1(keys, LOG2T, (uint32_t)a.grows[q], c.err);
+            if (h >= 0) gv[h] = a.gvals[q];
+        }
+        __syncwarp();
+        for (int base = 0; base < nb; base += 32) {
+            int beg = 0, len = 0;
+            V bval = V(0);
+            if (base + lane < nb) {
+                const int64_t k = (int64_t)__ldg(&bi[b0 + base + lane]);
+                const int64_t s = (int64_t)__ldg(&ap[k]);
+                beg = (int)s;
+                len = (int)((int64_t)__ldg(&ap[k + 1]) - s);
+                bval = __ldg(&bv[b0 + base + lane]);
+            }
+            const int incl = warp_incl_scan(len);
+            const int excl = incl - len;
+            const int tot = __shfl_sync(SPG_FULL, incl, 31);
+            const unsigned nzm = __ballot_sync(SPG_FULL, len > 0);
+            if (len > 0) {
+                const int rank = __popc(nzm & below);
+                s_off[rank] = beg - excl;
+                s_bv[rank] = bval;
+                s_e[rank] = base + lane;
+            }
+            __syncwarp();
+            int before = -1;   // segments started before the window, minus one
+            for (int w = 0; w < tot; w += 32 * U) {
+                uint32_t r[U];
+                V x[U];
+                int q[U], sl[U];
+                unsigned M[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int p = w + 32 * u + lane;
+                    const unsigned d = (unsigned)(excl - (w + 32 * u));
+                    M[u] = __reduce_or_sync(SPG_FULL, len > 0 && d < 32u ? 1u << d : 0u);
+                    sl[u] = before + __popc(M[u] & upto);
+                    before += __popc(M[u]);
+                    q[u] = -1;
+                    if (p < tot) {
+                        q[u] = s_off[sl[u]] + p;
+                        r[u] = (uint32_t)__ldg(&ai[q[u]]);
+                        x[u] = __ldg(&av[q[u]]);
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    if (w + 32 * u >= tot) break;   // the same for the warp
+                    V part = V(0);
+                    if (q[u] >= 0) {
+                        // the table holds G(:, j): empty slot first means not stored
+                        const uint32_t key = r[u];
+                        uint32_t h = hash_slot(key, LOG2T);
+                        const uint32_t step = ((key * 0x85EBCA6Bu) >> (32 - LOG2T)) | 1u;
+                        uint32_t cur = keys[h];
+                        for (int probe = 0; probe < T && cur != key && cur != kEmpty; ++probe) {
+                            h = (h + step) & (T - 1);
+                            cur = keys[h];
+                        }
+                        if (cur == key) {
+                            const V gval = gv[h];
+                            atomic_add_v(&dA[q[u]], mul_v(gval, s_bv[sl[u]]));
+                            part = mul_v(x[u], gval);
+                        }
+                    }
+                    __syncwarp();
+                    // sum over the lanes of the segment, into its first lane
+                    const unsigned later = M[u] & above;
+                    const int end = later ? __ffs(later) - 1 : 32;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const V y = shfl_bits(part, lane + o < 32 ? lane + o : lane);
+                        if (lane + o < end) part = add_v(part, y);
+                    }
+                    if (q[u] >= 0 && (lane == 0 || ((M[u] >> lane) & 1u))) atomic_add_v(&dB[b0 + s_e[sl[u]]], part);
+                }
+            }
+            __syncwarp();   // the segments are read: the next round may replace them
+        }
+        for (int s = lane; s < T / 4; s += 32) k4[s] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
+        __syncwarp();
+    }
+}
+
 }  // namespace spg

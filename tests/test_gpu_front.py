@@ -258,3 +258,41 @@ def test_light_columns_with_many_short_segments(vt, stages, sort):
     assert torch.equal(C.colptr.diff(), reached.sum(1)) and torch.equal(got, want)
     if sort:
         assert torch.equal(colc * m + C.rowidx, torch.nonzero(reached.reshape(-1)).reshape(-1))
+
+
+@pytest.mark.parametrize("vt,it", [(torch.float32, torch.int32), (torch.float64, torch.int64)])
+@pytest.mark.parametrize("kept", [1.0, 0.5, 0.0])
+def test_backward_of_light_columns(vt, it, kept):
+    """Short and empty segments, several rounds of 32 B entries, and a G that
+    stores only some of C's entries; integer values, so the sums are exact."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(8)
+    m, k = 600, 1500
+    ca = torch.randint(0, 6, (k,), generator=g, device="cuda")
+    ap = torch.zeros(k + 1, dtype=torch.int64, device="cuda")
+    ap[1:] = torch.cumsum(ca, 0)
+    cola = torch.repeat_interleave(torch.arange(k, device="cuda"), ca)
+    ra = (torch.randint(0, m, (k,), generator=g, device="cuda")[cola] + 7 * (torch.arange(cola.numel(), device="cuda") - ap[cola])) % m
+    A = spg.Csc(m, k, ap.to(it), ra.to(it), torch.randint(-4, 5, (cola.numel(),), generator=g, device="cuda").to(vt))
+    cb = torch.tensor([0, 1, 7, 31, 32, 33, 64, 65, 150], device="cuda").repeat(9)
+    n = cb.numel()
+    bp = torch.zeros(n + 1, dtype=torch.int64, device="cuda")
+    bp[1:] = torch.cumsum(cb, 0)
+    colb = torch.repeat_interleave(torch.arange(n, device="cuda"), cb)
+    rb = (torch.randint(0, k, (n,), generator=g, device="cuda")[colb] + 3 * (torch.arange(colb.numel(), device="cuda") - bp[colb])) % k
+    B = spg.Csc(k, n, bp.to(it), rb.to(it), torch.randint(-4, 5, (colb.numel(),), generator=g, device="cuda").to(vt))
+    C = spg.spgemm(A, B)
+    col = torch.repeat_interleave(torch.arange(n, device="cuda"), C.colptr.diff())
+    keep = torch.rand(C.nnz, generator=g, device="cuda") < kept
+    gp = torch.zeros(n + 1, dtype=torch.int64, device="cuda")
+    gp[1:] = torch.cumsum(torch.bincount(col[keep], minlength=n), 0)
+    G = spg.Csc(m, n, gp, C.rowidx[keep].contiguous(), torch.randint(-4, 5, (int(keep.sum()),), generator=g, device="cuda").to(vt))
+    dA, dB = spg.backward(A, B, G)
+    da = torch.zeros(m, k, dtype=torch.float64, device="cuda")
+    da[ra, cola] = A.vals.double()
+    db = torch.zeros(k, n, dtype=torch.float64, device="cuda")
+    db[rb, colb] = B.vals.double()
+    dg = torch.zeros(m, n, dtype=torch.float64, device="cuda")
+    dg[G.rowidx.long(), col[keep]] = G.vals.double()
+    assert torch.equal(dA.double(), (dg @ db.T)[ra, cola])
+    assert torch.equal(dB.double(), (da.T @ dg)[rb, colb])
