@@ -446,7 +446,7 @@ spgemm_status spgemm_backward(spgemm_plan *plan, const spgemm_csc *G, void *dA_v
 
 namespace spg {
 void MultiState::release_all() {
-    DevBuf *bufs[] = {&probs, &f, &cnt, &colptr, &tier, &list, &off, &hist, &err,
+    DevBuf *bufs[] = {&probs, &f, &cnt, &colptr, &tier, &list, &off, &hist, &err, &prob_of,
                       &scan_part, &rows, &vals, &counter, &gsize, &gtab_off, &gkeys, &gvals};
     for (auto *b : bufs) b->release();
     h_small.release();

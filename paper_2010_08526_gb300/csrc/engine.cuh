@@ -1764,6 +1764,7 @@ template <class I, class V> struct Engine : EngineBase {
         GA a{};
         a.probs = ms.probs.as<PD>();
         a.nprob = ms.nprob;
+        a.prob_of = ms.prob_of.as<int32_t>();
         a.k0 = 0; a.k1 = INT64_MAX;
         return a;
     }
@@ -1788,6 +1789,7 @@ template <class I, class V> struct Engine : EngineBase {
         SPG_CK(ms.cnt.ensure(sizeof(int64_t) * (n + 1)));
         SPG_CK(ms.colptr.ensure(sizeof(int64_t) * (n + 1)));
         SPG_CK(ms.tier.ensure(n + 16));
+        SPG_CK(ms.prob_of.ensure(sizeof(int32_t) * (n + 1)));
         SPG_CK(ms.list.ensure(sizeof(int32_t) * (n + 1)));
         SPG_CK(ms.off.ensure(sizeof(int32_t) * 64));
         SPG_CK(ms.hist.ensure(sizeof(int32_t) * kBinInts));
@@ -1799,8 +1801,8 @@ template <class I, class V> struct Engine : EngineBase {
         Ctx cx = multi_ctx(ms);
         SPG_CK(cudaMemsetAsync(cx.hist, 0, sizeof(int32_t) * 64, st));
         if (n > 0)
-            k_flops_bin<SrcGemm<I, V>><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(
-                multi_args(ms), 0, n, cx.tun.hash_cap_max, ms.f.as<int64_t>(),
+            k_multi_bin<I, V><<<(unsigned)((n * kBinLanes + 255) / 256), 256, 0, st>>>(
+                multi_args(ms), n, cx.tun.hash_cap_max, ms.prob_of.as<int32_t>(), ms.f.as<int64_t>(),
                 ms.tier.as<uint8_t>(), ms.cnt.as<int64_t>(), cx.hist);
         SPG_CK(cudaGetLastError());
         SPG_CK(exclusive_scan_i64(ms.f.as<int64_t>(), n, ms.colptr.as<int64_t>(),
@@ -1835,24 +1837,30 @@ template <class I, class V> struct Engine : EngineBase {
         }
         SPG_CK(ms.counter.ensure(sizeof(unsigned long long) * 4));
         // shared memory of the persistent passes: the largest CTA table or
-        // the warps' private tables, whichever is larger
-        const size_t sv = sizeof(V) + 4;
+        // the warps' private tables, whichever is larger; the symbolic pass needs
+        // the keys only, so more of its CTAs are resident
         const size_t nw = (size_t)ms.threads / 32;
-        ms.smem = std::max((size_t)2 * ms.tun.hash_cap_max * sv, nw * 2 * tier_cap(ms.warp_tiers) * sv);
-        int per_sm = 0;
-        cudaError_t oe = ms.threads == 512
-            ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_multi_pass<SrcGemm<I, V>, 512, 1>, 512, ms.smem)
-            : ms.threads == 256
-            ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_multi_pass<SrcGemm<I, V>, 256, 1>, 256, ms.smem)
-            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_multi_pass<SrcGemm<I, V>, 128, 1>, 128, ms.smem);
-        SPG_CK(oe);
-        if (per_sm < 1) {
-            set_error("the batched tables do not fit shared memory: lower hash_max_cap or warp_max_cap");
-            return SPGEMM_ERR_INVALID;
+        for (int mode = 0; mode < 2; ++mode) {
+            const size_t slot = 4 + (mode ? sizeof(V) : 0);
+            ms.smem[mode] = std::max((size_t)2 * ms.tun.hash_cap_max, nw * 2 * tier_cap(ms.warp_tiers)) * slot;
+            int per_sm = 0;
+            SPG_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, multi_kernel(ms.threads, mode), ms.threads,
+                                                                 ms.smem[mode]));
+            if (per_sm < 1) {
+                set_error("the batched tables do not fit shared memory: lower hash_max_cap or warp_max_cap");
+                return SPGEMM_ERR_INVALID;
+            }
+            ms.grid[mode] = ms.nsm * per_sm;
         }
-        ms.grid = ms.nsm * per_sm;
         ms.enqueue = &multi_enqueue;
         return SPGEMM_OK;
+    }
+
+    using MultiKernel = void (*)(GA, TierCommon, MultiQueue, I *, V *);
+    static MultiKernel multi_kernel(int threads, int mode) {
+        if (threads == 512) return mode ? k_multi_pass<SrcGemm<I, V>, 512, 1> : k_multi_pass<SrcGemm<I, V>, 512, 0>;
+        if (threads == 256) return mode ? k_multi_pass<SrcGemm<I, V>, 256, 1> : k_multi_pass<SrcGemm<I, V>, 256, 0>;
+        return mode ? k_multi_pass<SrcGemm<I, V>, 128, 1> : k_multi_pass<SrcGemm<I, V>, 128, 0>;
     }
 
     // flops, symbolic, scan and numeric for all problems; no host
@@ -1865,8 +1873,8 @@ template <class I, class V> struct Engine : EngineBase {
         SPG_CK(cudaMemsetAsync(ms.counter.p, 0, sizeof(unsigned long long) * 4, st));
         if (n > 0) {
             // tiers by the flop bound min(f_j, m), the same as at creation
-            k_flops_bin<SrcGemm<I, V>><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(
-                ga, 0, n, cx.tun.hash_cap_max, nullptr, ms.tier.as<uint8_t>(),
+            k_multi_bin<I, V><<<(unsigned)((n * kBinLanes + 255) / 256), 256, 0, st>>>(
+                ga, n, cx.tun.hash_cap_max, ms.prob_of.as<int32_t>(), nullptr, ms.tier.as<uint8_t>(),
                 ms.cnt.as<int64_t>(), cx.hist);
             k_bin_scatter<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(
                 ms.tier.as<uint8_t>(), 0, n, cx.hist, cx.cursor, ms.list.as<int32_t>(),
@@ -1877,14 +1885,7 @@ template <class I, class V> struct Engine : EngineBase {
         MultiQueue mq{ms.list.as<int32_t>(), ms.off.as<int32_t>(), ms.counter.as<unsigned long long>(),
                       ms.gtab_off.as<int64_t>(), ms.gkeys.as<uint32_t>(), ms.gvals.p, ms.warp_tiers};
         // one persistent launch counts every column of every problem ...
-        if (n > 0) {
-            if (ms.threads == 512)
-                k_multi_pass<SrcGemm<I, V>, 512, 0><<<ms.grid, 512, ms.smem, st>>>(ga, c, mq, nullptr, nullptr);
-            else if (ms.threads == 256)
-                k_multi_pass<SrcGemm<I, V>, 256, 0><<<ms.grid, 256, ms.smem, st>>>(ga, c, mq, nullptr, nullptr);
-            else
-                k_multi_pass<SrcGemm<I, V>, 128, 0><<<ms.grid, 128, ms.smem, st>>>(ga, c, mq, nullptr, nullptr);
-        }
+        if (n > 0) multi_kernel(ms.threads, 0)<<<ms.grid[0], ms.threads, ms.smem[0], st>>>(ga, c, mq, nullptr, nullptr);
         SPG_CK(cudaGetLastError());
         SPG_CK(exclusive_scan_i64(ms.cnt.as<int64_t>(), n, ms.colptr.as<int64_t>(),
                                   ms.scan_part.as<int64_t>(), 1, st));
@@ -1892,17 +1893,9 @@ template <class I, class V> struct Engine : EngineBase {
         c.colptr = ms.colptr.as<int64_t>();
         c.out_base = 0;
         mq.counter = ms.counter.as<unsigned long long>() + 2;
-        if (n > 0) {
-            if (ms.threads == 512)
-                k_multi_pass<SrcGemm<I, V>, 512, 1><<<ms.grid, 512, ms.smem, st>>>(ga, c, mq, ms.rows.as<I>(),
+        if (n > 0)
+            multi_kernel(ms.threads, 1)<<<ms.grid[1], ms.threads, ms.smem[1], st>>>(ga, c, mq, ms.rows.as<I>(),
                                                                                     ms.vals.as<V>());
-            else if (ms.threads == 256)
-                k_multi_pass<SrcGemm<I, V>, 256, 1><<<ms.grid, 256, ms.smem, st>>>(ga, c, mq, ms.rows.as<I>(),
-                                                                                    ms.vals.as<V>());
-            else
-                k_multi_pass<SrcGemm<I, V>, 128, 1><<<ms.grid, 128, ms.smem, st>>>(ga, c, mq, ms.rows.as<I>(),
-                                                                                    ms.vals.as<V>());
-        }
         SPG_CK(cudaGetLastError());
         return SPGEMM_OK;
     }

@@ -102,6 +102,7 @@ template <class I, class V> struct GemmArgs {
     const int32_t *apc_off;
     const uint32_t *apc_row;  // global rows
     const V *apc_val;
+    const int32_t *prob_of;   // many problems: the problem of every global column, or null
     int lean_dense;           // heavy items may use 32-bit entry offsets (nnz(A) < 2^31)
     int lean_sym;             // the heavy symbolic may use 32-bit stream positions too
 };
@@ -123,7 +124,7 @@ template <class I, class V> struct SrcGemm {
     const ProbDev<I, V> *p;
     int64_t b0, nb, k0, k1;
     __device__ __forceinline__ void open(const Args &a, int64_t g) {
-        p = a.probs + locate_prob(a.probs, a.nprob, g);
+        p = a.probs + (a.prob_of ? a.prob_of[g] : locate_prob(a.probs, a.nprob, g));
         const int64_t bc = g - p->gcol0;
         b0 = (int64_t)p->bp[bc];
         nb = (int64_t)p->bp[bc + 1] - b0;
@@ -916,32 +917,44 @@ __global__ void __launch_bounds__(256) k_col_tier(typename Src::Args sa, int64_t
 }
 
 // Both steps in one launch for the columns of many problems (the batched
-// products): one warp per column computes f_j; the CTA keeps a tier histogram.
-template <class Src>
-__global__ void __launch_bounds__(256) k_flops_bin(typename Src::Args sa, int64_t c_lo,
-                                                   int64_t c_hi, int hash_cap_max, int64_t *f_out,
-                                                   uint8_t *tier_out, int64_t *cnt_out,
+// products), which also records every column's problem. A group of kBinLanes
+// lanes takes a column (the columns are short: a warp per column with 32
+// columns in a row took 54 us for 69,000 columns, this 10 us); the CTA
+// keeps a tier histogram.
+constexpr int kBinLanes = 8;
+template <class I, class V>
+__global__ void __launch_bounds__(256) k_multi_bin(GemmArgs<I, V> sa, int64_t n, int hash_cap_max, int32_t *prob_of,
+                                                   int64_t *f_out, uint8_t *tier_out, int64_t *cnt_out,
                                                    int32_t *tier_hist) {
     __shared__ int s_hist[kTiers];
     if (threadIdx.x < kTiers) s_hist[threadIdx.x] = 0;
     __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t cbase = c_lo + (int64_t)blockIdx.x * 256;
-    for (int c = 0; c < 32; ++c) {
-        const int64_t g = cbase + warp * 32 + c;
-        if (g >= c_hi) break;
-        Src src;
-        src.open(sa, g);
-        const int64_t f = src.flops();
-        if (lane == 0) {
-            const int64_t u = f < src.m() ? f : src.m();
-            int t = hash_tier_of(u, hash_cap_max);
-            if (t < 0) t = heavy_subtier(u);
-            if (f_out) f_out[g] = f;
-            tier_out[g] = (uint8_t)t;
-            if (cnt_out) cnt_out[g] = 0;
-            if (t) atomicAdd(&s_hist[t], 1);
+    const int sub = threadIdx.x % kBinLanes;
+    const int64_t g = (int64_t)blockIdx.x * (256 / kBinLanes) + threadIdx.x / kBinLanes;
+    int64_t f = 0;
+    const ProbDev<I, V> *p = sa.probs;
+    if (g < n) {
+        const int pr = locate_prob(sa.probs, sa.nprob, g);
+        p += pr;
+        const int64_t bc = g - p->gcol0;
+        const int64_t b0 = (int64_t)__ldg(&p->bp[bc]), b1 = (int64_t)__ldg(&p->bp[bc + 1]);
+        const I *bi = p->bi, *ap = p->ap;
+        for (int64_t e = b0 + sub; e < b1; e += kBinLanes) {
+            const int64_t k = (int64_t)__ldg(&bi[e]);
+            f += (int64_t)__ldg(&ap[k + 1]) - (int64_t)__ldg(&ap[k]);
         }
+        if (sub == 0 && prob_of) prob_of[g] = pr;
+    }
+#pragma unroll
+    for (int o = kBinLanes / 2; o > 0; o >>= 1) f += __shfl_xor_sync(SPG_FULL, f, o);
+    if (sub == 0 && g < n) {
+        const int64_t u = f < p->m ? f : p->m;
+        int t = hash_tier_of(u, hash_cap_max);
+        if (t < 0) t = heavy_subtier(u);
+        if (f_out) f_out[g] = f;
+        tier_out[g] = (uint8_t)t;
+        if (cnt_out) cnt_out[g] = 0;
+        if (t) atomicAdd(&s_hist[t], 1);
     }
     __syncthreads();
     if (threadIdx.x < kTiers && s_hist[threadIdx.x])

@@ -3,6 +3,12 @@
 // formula): the symbolic count and the numeric hash accumulation of every
 // column of every problem run as work items of a single kernel.
 //
+// Measured, 64 graphs of 500 to 2000 vertices (25.5 M products), bins / symbolic /
+// numeric: 54 / 348 / 575 us before, 10 / 228 / 492 us with the problem of a
+// column looked up instead of searched, the symbolic pass's shared memory holding
+// keys only (12 CTAs per SM, not 7), the walk of k_light, and CTA items
+// written from per-warp runs of slots.
+//
 // Work comes from the tier lists of k_bin_scatter (list, off[t]) through two
 // device counters. First the CTA items: the columns above the largest
 // shared-memory table (heaviest tier first), then the CTA-sized columns
@@ -50,12 +56,17 @@ __device__ __forceinline__ int64_t ghash_insert(uint32_t *keys, int log2T, uint3
     return -1;
 }
 
-template <class V> __device__ __forceinline__ void gatomic_add_v(V *p, V v) { atomic_add_v(p, v); }
+// The same sum in global memory (64-bit integer adds are native there).
+template <class V> __device__ __forceinline__ void gatomic_add_v(V *p, V v) {
+    if constexpr (std::is_same<V, int64_t>::value)
+        atomicAdd(reinterpret_cast<unsigned long long *>(p), static_cast<unsigned long long>(v));
+    else atomic_add_v(p, v);
+}
 
 // MODE 0: symbolic (count distinct rows into c.cnt[g]); MODE 1: numeric
 // (accumulate, write column g at c.colptr[g] - c.out_base, unsorted).
 template <class Src, int NT, int MODE>
-__global__ void __launch_bounds__(NT) k_multi_pass(typename Src::Args sa, TierCommon c, MultiQueue mq,
+__global__ void __launch_bounds__(NT, MODE == 0 ? 1536 / NT : 0) k_multi_pass(typename Src::Args sa, TierCommon c, MultiQueue mq,
                                                    typename Src::Idx *out_rows, typename Src::Val *out_vals) {
     using V = typename Src::Val;
     using I = typename Src::Idx;
@@ -97,7 +108,7 @@ __global__ void __launch_bounds__(NT) k_multi_pass(typename Src::Args sa, TierCo
                 while ((1ll << log2T) < 2 * bound) ++log2T;
                 const int T = 1 << log2T;
                 V *vals = reinterpret_cast<V *>(smem);
-                uint32_t *keys = reinterpret_cast<uint32_t *>(smem + sizeof(V) * T);
+                uint32_t *keys = reinterpret_cast<uint32_t *>(smem + (MODE == 1 ? sizeof(V) * T : 0));
                 for (int s = threadIdx.x; s < T; s += NT) { keys[s] = kEmpty; if (MODE == 1) vals[s] = V(0); }
                 __syncthreads();
                 int mine = 0;
@@ -121,22 +132,28 @@ __global__ void __launch_bounds__(NT) k_multi_pass(typename Src::Args sa, TierCo
                         if (threadIdx.x == 0) c.cnt[g] = v;
                     }
                 } else {
-                    for (int s0 = 0; s0 < T; s0 += NT) {
-                        const int s = s0 + threadIdx.x;
-                        const uint32_t key = s < T ? keys[s] : kEmpty;
+                    // a warp owns a run of slots: count, one barrier, write
+                    const int per = (T + NW - 1) / NW;
+                    const int slo = min(T, warp * per), shi = min(T, slo + per);
+                    int n = 0;
+                    for (int s = slo + lane; s < shi; s += 32) n += keys[s] != kEmpty;
+                    n = warp_sum(n);
+                    int o = warp_offset(n, sh.red, warp, NW, lane);
+                    for (int s0 = slo; s0 < shi; s0 += 32) {
+                        const int s = s0 + lane;
+                        const uint32_t key = s < shi ? keys[s] : kEmpty;
                         const bool occ = key != kEmpty;
                         const unsigned bal = __ballot_sync(SPG_FULL, occ);
-                        int wbase = 0;
-                        if (lane == 0 && bal) wbase = atomicAdd(&sh.pos, __popc(bal));
-                        wbase = __shfl_sync(SPG_FULL, wbase, 0);
                         if (occ) {
-                            const int r = wbase + __popc(bal & ((1u << lane) - 1u));
+                            const int r = o + __popc(bal & ((1u << lane) - 1u));
                             if (r < want) {
                                 out_rows[out0 + r] = (I)key;
                                 out_vals[out0 + r] = vals[s];
                             }
                         }
+                        o += __popc(bal);
                     }
+                    if (warp == NW - 1 && lane == 0) sh.pos = o;
                     __syncthreads();
                     if (threadIdx.x == 0) {
                         if (sh.pos != want) atomicOr(c.err, kErrCount);
@@ -204,52 +221,108 @@ __global__ void __launch_bounds__(NT) k_multi_pass(typename Src::Args sa, TierCo
         }
     }
     // warp-sized columns: every warp takes kWarpGrab at a time (one counter
-    // update per grab), each with a warp-private table. In the numeric pass the
-    // table is cleared once and the compaction puts back the slots it reads
-    // occupied; the symbolic pass clears it per column.
+    // update per grab), each with a warp-private table, cleared once; a
+    // column's output leaves it clean. The walk is the one of k_light.
     constexpr int kWarpGrab = 8;
-    if (MODE == 1) {
-        V *vals = reinterpret_cast<V *>(smem) + warp * TW;
-        uint32_t *keys = reinterpret_cast<uint32_t *>(smem + sizeof(V) * NW * TW) + warp * TW;
-        for (int s = lane; s < TW; s += 32) { keys[s] = kEmpty; vals[s] = V(0); }
-        __syncwarp();
+    constexpr int U = 4;   // windows whose loads are in flight
+    V *vals = MODE == 1 ? reinterpret_cast<V *>(smem) + warp * TW : nullptr;
+    uint32_t *keys = reinterpret_cast<uint32_t *>(smem + (MODE == 1 ? sizeof(V) * NW * TW : 0)) + warp * TW;
+    const unsigned below = (1u << lane) - 1u, upto = 0xffffffffu >> (31 - lane);
+    // the non-empty segments of a round in stream order: offset to the entry
+    // index, and B value
+    __shared__ int64_t s_off[NW][32];
+    __shared__ V s_bv[MODE == 1 ? NW : 1][32];
+    for (int s = lane; s < TW; s += 32) {
+        keys[s] = kEmpty;
+        if (MODE == 1) vals[s] = V(0);
     }
+    __syncwarp();
     for (;;) {
         long long wb = 0;
         if (lane == 0) wb = (long long)atomicAdd(mq.counter + 1, (unsigned long long)kWarpGrab);
         wb = __shfl_sync(SPG_FULL, wb, 0);
         if (wb >= nwarp) break;
-        for (long long wi = wb; wi < wb + kWarpGrab && wi < nwarp; ++wi) {
-            const int pos = mq.off[1] + (int)wi;
-            const int64_t g = mq.list[pos];
+        // the grab's columns, one per lane: column, problem and B range are on
+        // their way before the first one is walked
+        int64_t gl = 0, b0l = 0;
+        int nbl = 0, prl = 0;
+        if (lane < kWarpGrab && wb + lane < nwarp) {
+            gl = mq.list[mq.off[1] + (int)wb + lane];
+            prl = sa.prob_of[gl];
+            const auto *p = sa.probs + prl;
+            const int64_t bc = gl - p->gcol0;
+            b0l = (int64_t)__ldg(&p->bp[bc]);
+            nbl = (int)((int64_t)__ldg(&p->bp[bc + 1]) - b0l);
+        }
+        for (int wi = 0; wi < kWarpGrab && wb + wi < nwarp; ++wi) {
+            const int pos = mq.off[1] + (int)wb + wi;
+            const int64_t g = __shfl_sync(SPG_FULL, gl, wi);
+            const int64_t b0 = __shfl_sync(SPG_FULL, b0l, wi);
+            const int nb = __shfl_sync(SPG_FULL, nbl, wi);
+            const auto *p = sa.probs + __shfl_sync(SPG_FULL, prl, wi);
+            const I *bi = p->bi, *ap = p->ap, *ai = p->ai;
+            const V *bv = p->bv, *av = p->av;
             int t = 1;
             while (t < wt && mq.off[t + 1] <= pos) ++t;
             int log2T = 1;   // 2 * cap(t) slots
             while ((1 << log2T) < 2 * tier_cap(t)) ++log2T;
             const int T = 1 << log2T;
-            V *vals = reinterpret_cast<V *>(smem) + warp * TW;
-            uint32_t *keys = reinterpret_cast<uint32_t *>(smem + sizeof(V) * NW * TW) + warp * TW;
-            Src src;
-            src.open(sa, g);
-            if (MODE == 0) {
-                for (int s = lane; s < T; s += 32) keys[s] = kEmpty;
+            int mine = 0;
+            for (int base = 0; base < nb; base += 32) {
+                int64_t beg = 0;
+                int len = 0;
+                V bval = V(0);
+                if (base + lane < nb) {
+                    const int64_t k = (int64_t)__ldg(&bi[b0 + base + lane]);
+                    beg = (int64_t)__ldg(&ap[k]);
+                    len = (int)((int64_t)__ldg(&ap[k + 1]) - beg);
+                    if (MODE == 1) bval = __ldg(&bv[b0 + base + lane]);
+                }
+                const int incl = warp_incl_scan(len);
+                const int excl = incl - len;
+                const int tot = __shfl_sync(SPG_FULL, incl, 31);
+                const unsigned nzm = __ballot_sync(SPG_FULL, len > 0);
+                if (len > 0) {
+                    const int rank = __popc(nzm & below);
+                    s_off[warp][rank] = beg - excl;
+                    if (MODE == 1) s_bv[warp][rank] = bval;
+                }
+                __syncwarp();
+                int before = -1;   // segments started before the window, minus one
+                for (int w = 0; w < tot; w += 32 * U) {
+                    uint32_t r[U];
+                    V x[U];
+                    bool ok[U];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int at = w + 32 * u + lane;
+                        const unsigned d = (unsigned)(excl - (w + 32 * u));
+                        const unsigned M = __reduce_or_sync(SPG_FULL, len > 0 && d < 32u ? 1u << d : 0u);
+                        const int sl = before + __popc(M & upto);
+                        before += __popc(M);
+                        ok[u] = at < tot;
+                        if (ok[u]) {
+                            const int64_t q = s_off[warp][sl] + at;
+                            r[u] = (uint32_t)__ldg(&ai[q]);
+                            if (MODE == 1) x[u] = mul_v(__ldg(&av[q]), s_bv[warp][sl]);
+                        }
+                    }
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        if (!ok[u]) continue;
+                        bool nw;
+                        const int h = hash_insert_dbl1(keys, log2T, r[u], c.err, nw);
+                        if (MODE == 0) mine += nw;
+                        else if (h >= 0) atomic_add_v(&vals[h], x[u]);
+                    }
+                }
                 __syncwarp();
             }
-            int mine = 0;
-            auto ld = [&](int64_t q, V bv) {
-                return RowVal<V>{src.row(q), MODE == 1 ? src.val(q, bv) : V(0)};
-            };
-            auto ap = [&](const RowVal<V> &e) {
-                bool nw;
-                const int h = hash_insert_dbl1(keys, log2T, e.r, c.err, nw);
-                if (MODE == 0) mine += nw;
-                else if (h >= 0) atomic_add_v(&vals[h], e.x);
-            };
-            warp_walk_flat<4>(src, ld, ap);
-            __syncwarp();
             if (MODE == 0) {
                 mine = warp_sum(mine);
                 if (lane == 0) c.cnt[g] = mine;
+                uint4 *k4 = reinterpret_cast<uint4 *>(keys);
+                for (int s = lane; s < T / 4; s += 32) k4[s] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
             } else {
                 const int64_t out0 = c.colptr[g] - c.out_base;
                 const int64_t want = c.colptr[g + 1] - c.colptr[g];
@@ -260,7 +333,7 @@ __global__ void __launch_bounds__(NT) k_multi_pass(typename Src::Args sa, TierCo
                     const bool occ = key != kEmpty;
                     const unsigned bal = __ballot_sync(SPG_FULL, occ);
                     if (occ) {
-                        const int r = pos2 + __popc(bal & ((1u << lane) - 1u));
+                        const int r = pos2 + __popc(bal & below);
                         if (r < want) {
                             out_rows[out0 + r] = (I)key;
                             out_vals[out0 + r] = vals[s];

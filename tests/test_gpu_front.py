@@ -296,3 +296,57 @@ def test_backward_of_light_columns(vt, it, kept):
     dg[G.rowidx.long(), col[keep]] = G.vals.double()
     assert torch.equal(dA.double(), (dg @ db.T)[ra, cola])
     assert torch.equal(dB.double(), (da.T @ dg)[rb, colb])
+
+
+@pytest.mark.parametrize("warp_cap,cap,threads", [(32, 256, 128), (128, 1024, 128), (256, 1024, 256), (512, 8192, 512)])
+def test_batched_products_of_uneven_columns(warp_cap, cap, threads):
+    """Warp and CTA items at every table size, short and empty segments, columns
+    above the shared tables, and int64 sums that wrap and change sign."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(threads + cap)
+    As, Bs, want = [], [], []
+    for i, (m, k, n) in enumerate([(40, 50, 30), (900, 700, 300), (20000, 400, 60)]):
+        A, cola = ragged(m, k, i + 3)
+        A.vals.copy_(torch.randint(-(1 << 62), 1 << 62, (A.nnz,), generator=g, device="cuda"))
+        B, colb = ragged(k, n, i + 13)
+        keep = torch.rand(B.nnz, generator=g, device="cuda") < 0.7
+        ptr = torch.zeros(n + 1, dtype=torch.int64, device="cuda")
+        ptr[1:] = torch.cumsum(torch.bincount(colb[keep], minlength=n), 0)
+        # distinct (row, column) pairs only, as ragged() gives for k > 2100 rows
+        key = torch.unique(B.rowidx[keep].long() + colb[keep] * k)
+        colb, rb = key // k, key % k
+        ptr[1:] = torch.cumsum(torch.bincount(colb, minlength=n), 0)
+        B = spg.Csc(k, n, ptr.int(), rb.int(), torch.randint(-9, 9, (key.numel(),), generator=g, device="cuda"))
+        keya = torch.unique(A.rowidx.long() + cola * m)
+        cola, ra = keya // m, keya % m
+        pa = torch.zeros(k + 1, dtype=torch.int64, device="cuda")
+        pa[1:] = torch.cumsum(torch.bincount(cola, minlength=k), 0)
+        A = spg.Csc(m, k, pa.int(), ra.int(), A.vals[:keya.numel()].contiguous())
+        As.append(A)
+        Bs.append(B)
+        # products of every B entry, summed modulo 2^64 on the host's integers
+        da = torch.zeros(k, m, dtype=torch.int64, device="cuda")
+        da[cola, ra] = A.vals
+        sa = torch.zeros(k, m, dtype=torch.bool, device="cuda")
+        sa[cola, ra] = True
+        c = torch.zeros(n, m, dtype=torch.int64, device="cuda")
+        s = torch.zeros(n, m, dtype=torch.bool, device="cuda")
+        for e in range(key.numel()):
+            c[colb[e]] += da[rb[e]] * B.vals[e]
+            s[colb[e]] |= sa[rb[e]]
+        want.append((c, s))
+    multi = spg.Multi(As, Bs, tuning=spg.Tuning(hash_max_cap=cap, warp_max_cap=warp_cap, block_tier_threads=threads))
+    for _ in range(2):
+        multi.run()
+        colptr, rows, vals = multi.output()
+        c0 = 0
+        for (c, s), B in zip(want, Bs):
+            ptr = colptr[c0:c0 + B.ncols + 1]
+            assert torch.equal(ptr.diff(), s.sum(1))
+            a, z = int(ptr[0]), int(ptr[-1])
+            col = torch.repeat_interleave(torch.arange(B.ncols, device="cuda"), ptr.diff())
+            got = torch.zeros_like(c)
+            got[col, rows[a:z].long()] = vals[a:z]
+            assert torch.equal(got, c)
+            c0 += B.ncols
+    multi.close()
