@@ -4,10 +4,11 @@
 // column of every problem run as work items of a single kernel.
 //
 // Measured, 64 graphs of 500 to 2000 vertices (25.5 M products), bins / symbolic /
-// numeric: 54 / 348 / 575 us before, 10 / 228 / 492 us with the problem of a
+// numeric: 54 / 348 / 575 us before, 10 / 186 / 453 us with the problem of a
 // column looked up instead of searched, the symbolic pass's shared memory holding
-// keys only (12 CTAs per SM, not 7), the walk of k_light, and CTA items
-// written from per-warp runs of slots.
+// keys only (12 CTAs per SM, not 7), numeric tables sized by the exact count, CTA
+// items written from per-warp runs of slots, and one barrier-free walk for warp
+// and CTA items (walk_entries; the CTA-wide walk alone cost 34 and 27 us more).
 //
 // Work comes from the tier lists of k_bin_scatter (list, off[t]) through two
 // device counters. First the CTA items: the columns above the largest
@@ -63,6 +64,67 @@ template <class V> __device__ __forceinline__ void gatomic_add_v(V *p, V v) {
     else atomic_add_v(p, v);
 }
 
+// A warp's part of the products of one column: of the rounds of 32 B entries
+// it takes r0, r0 + rs, ..., and of the 32-wide windows of a round's product
+// stream w0, w0 + ws, ...; insert(row, product) for each, with the loads of four
+// windows in flight. off / sbv: 32 places per warp in shared memory for the
+// non-empty segments of a round, in stream order (offset to the entry index, B
+// value). All lanes call it.
+template <int MODE, class I, class V, class F>
+__device__ __forceinline__ void walk_entries(const ProbDev<I, V> *p, int64_t b0, int nb, int r0, int rs, int w0,
+                                             int ws, int64_t *off, V *sbv, F &&insert) {
+    constexpr int U = 4;
+    const int lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u, upto = 0xffffffffu >> (31 - lane);
+    const I *bi = p->bi, *ap = p->ap, *ai = p->ai;
+    const V *bv = p->bv, *av = p->av;
+    for (int base = 32 * r0; base < nb; base += 32 * rs) {
+        int64_t beg = 0;
+        int len = 0;
+        V bval = V(0);
+        if (base + lane < nb) {
+            const int64_t k = (int64_t)__ldg(&bi[b0 + base + lane]);
+            beg = (int64_t)__ldg(&ap[k]);
+            len = (int)((int64_t)__ldg(&ap[k + 1]) - beg);
+            if (MODE == 1) bval = __ldg(&bv[b0 + base + lane]);
+        }
+        const int incl = warp_incl_scan(len);
+        const int excl = incl - len;
+        const int tot = __shfl_sync(SPG_FULL, incl, 31);
+        const unsigned nzm = __ballot_sync(SPG_FULL, len > 0);
+        if (len > 0) {
+            const int rank = __popc(nzm & below);
+            off[rank] = beg - excl;
+            if (MODE == 1) sbv[rank] = bval;
+        }
+        __syncwarp();
+        for (int w = 32 * w0; w < tot; w += 32 * U * ws) {
+            uint32_t r[U];
+            V x[U];
+            bool ok[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                // the segment of a lane: the last one starting at or before it
+                const int wu = w + 32 * u * ws;
+                const unsigned d = (unsigned)(excl - wu);
+                const unsigned M = __reduce_or_sync(SPG_FULL, len > 0 && d < 32u ? 1u << d : 0u);
+                const int before = __popc(__ballot_sync(SPG_FULL, len > 0 && excl < wu));
+                const int sl = before + __popc(M & upto) - 1;
+                ok[u] = wu + lane < tot;
+                if (ok[u]) {
+                    const int64_t q = off[sl] + wu + lane;
+                    r[u] = (uint32_t)__ldg(&ai[q]);
+                    if (MODE == 1) x[u] = mul_v(__ldg(&av[q]), sbv[sl]);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (ok[u]) insert(r[u], MODE == 1 ? x[u] : V(0));
+        }
+        __syncwarp();   // the segments are read: the next round may replace them
+    }
+}
+
 // MODE 0: symbolic (count distinct rows into c.cnt[g]); MODE 1: numeric
 // (accumulate, write column g at c.colptr[g] - c.out_base, unsorted).
 template <class Src, int NT, int MODE>
@@ -74,6 +136,8 @@ __global__ void __launch_bounds__(NT, MODE == 0 ? 1536 / NT : 0) k_multi_pass(ty
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ BlockShared<V, NT> sh;
     __shared__ long long s_item;
+    __shared__ int64_t s_off[NW][32];   // scratch of walk_entries
+    __shared__ V s_bv[MODE == 1 ? NW : 1][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int wt = mq.warp_tiers;
     const int nbig = mq.off[kTiers] - mq.off[wt + 1];
@@ -104,24 +168,31 @@ __global__ void __launch_bounds__(NT, MODE == 0 ? 1536 / NT : 0) k_multi_pass(ty
                 want = c.colptr[g + 1] - c.colptr[g];
             }
             if (!heavy) {
-                int log2T = 1;
-                while ((1ll << log2T) < 2 * bound) ++log2T;
+                // the numeric pass knows the exact count
+                const int64_t rows = MODE == 1 && want < bound ? want : bound;
+                int log2T = 7;
+                while ((1ll << log2T) < 2 * rows) ++log2T;
                 const int T = 1 << log2T;
                 V *vals = reinterpret_cast<V *>(smem);
                 uint32_t *keys = reinterpret_cast<uint32_t *>(smem + (MODE == 1 ? sizeof(V) * T : 0));
-                for (int s = threadIdx.x; s < T; s += NT) { keys[s] = kEmpty; if (MODE == 1) vals[s] = V(0); }
+                uint4 *k4 = reinterpret_cast<uint4 *>(keys);
+                for (int s = threadIdx.x; s < T / 4; s += NT) k4[s] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
+                if (MODE == 1)
+                    for (int s = threadIdx.x; s < T; s += NT) vals[s] = V(0);
                 __syncthreads();
+                // the warps share a column by rounds of B entries when there are
+                // enough of them, else by windows of each round's stream
                 int mine = 0;
-                auto emit = load_apply(
-                    [&](int64_t q, V bv, int64_t) { return RowVal<V>{src.row(q), MODE == 1 ? src.val(q, bv) : V(0)}; },
-                    [&](const RowVal<V> &e, bool valid) {
-                        if (!valid) return;
-                        bool nw;
-                        const int h = hash_insert_dbl1(keys, log2T, e.r, c.err, nw);
-                        if (MODE == 0) mine += nw;
-                        else if (h >= 0) atomic_add_v(&vals[h], e.x);
-                    });
-                block_walk<kWalkBatch>(src, emit, c.short_seg, c.huge_seg, sh);
+                auto insert = [&](uint32_t r, V x) {
+                    bool nw;
+                    const int h = hash_insert_dbl1(keys, log2T, r, c.err, nw);
+                    if (MODE == 0) mine += nw;
+                    else if (h >= 0) atomic_add_v(&vals[h], x);
+                };
+                const bool rounds = src.nb >= 64 * NW;
+                walk_entries<MODE>(src.p, src.b0, (int)src.nb, rounds ? warp : 0, rounds ? NW : 1, rounds ? 0 : warp,
+                                   rounds ? 1 : NW, s_off[warp], s_bv[MODE == 1 ? warp : 0], insert);
+                __syncthreads();
                 if (MODE == 0) {
                     mine = warp_sum(mine);
                     if (lane == 0) sh.red[warp] = mine;
@@ -224,14 +295,9 @@ __global__ void __launch_bounds__(NT, MODE == 0 ? 1536 / NT : 0) k_multi_pass(ty
     // update per grab), each with a warp-private table, cleared once; a
     // column's output leaves it clean. The walk is the one of k_light.
     constexpr int kWarpGrab = 8;
-    constexpr int U = 4;   // windows whose loads are in flight
     V *vals = MODE == 1 ? reinterpret_cast<V *>(smem) + warp * TW : nullptr;
     uint32_t *keys = reinterpret_cast<uint32_t *>(smem + (MODE == 1 ? sizeof(V) * NW * TW : 0)) + warp * TW;
-    const unsigned below = (1u << lane) - 1u, upto = 0xffffffffu >> (31 - lane);
-    // the non-empty segments of a round in stream order: offset to the entry
-    // index, and B value
-    __shared__ int64_t s_off[NW][32];
-    __shared__ V s_bv[MODE == 1 ? NW : 1][32];
+    const unsigned below = (1u << lane) - 1u;
     for (int s = lane; s < TW; s += 32) {
         keys[s] = kEmpty;
         if (MODE == 1) vals[s] = V(0);
@@ -260,72 +326,33 @@ __global__ void __launch_bounds__(NT, MODE == 0 ? 1536 / NT : 0) k_multi_pass(ty
             const int64_t b0 = __shfl_sync(SPG_FULL, b0l, wi);
             const int nb = __shfl_sync(SPG_FULL, nbl, wi);
             const auto *p = sa.probs + __shfl_sync(SPG_FULL, prl, wi);
-            const I *bi = p->bi, *ap = p->ap, *ai = p->ai;
-            const V *bv = p->bv, *av = p->av;
+            // 2 * cap(t) slots by the column's tier; the numeric pass knows the
+            // exact count, usually a smaller table
             int t = 1;
             while (t < wt && mq.off[t + 1] <= pos) ++t;
-            int log2T = 1;   // 2 * cap(t) slots
-            while ((1 << log2T) < 2 * tier_cap(t)) ++log2T;
+            int64_t out0 = 0;
+            int want = tier_cap(t);
+            if (MODE == 1) {
+                out0 = c.colptr[g] - c.out_base;
+                want = (int)min(c.colptr[g + 1] - c.colptr[g], (int64_t)want);
+            }
+            int log2T = 6;
+            while ((1 << log2T) < 2 * want) ++log2T;
             const int T = 1 << log2T;
             int mine = 0;
-            for (int base = 0; base < nb; base += 32) {
-                int64_t beg = 0;
-                int len = 0;
-                V bval = V(0);
-                if (base + lane < nb) {
-                    const int64_t k = (int64_t)__ldg(&bi[b0 + base + lane]);
-                    beg = (int64_t)__ldg(&ap[k]);
-                    len = (int)((int64_t)__ldg(&ap[k + 1]) - beg);
-                    if (MODE == 1) bval = __ldg(&bv[b0 + base + lane]);
-                }
-                const int incl = warp_incl_scan(len);
-                const int excl = incl - len;
-                const int tot = __shfl_sync(SPG_FULL, incl, 31);
-                const unsigned nzm = __ballot_sync(SPG_FULL, len > 0);
-                if (len > 0) {
-                    const int rank = __popc(nzm & below);
-                    s_off[warp][rank] = beg - excl;
-                    if (MODE == 1) s_bv[warp][rank] = bval;
-                }
-                __syncwarp();
-                int before = -1;   // segments started before the window, minus one
-                for (int w = 0; w < tot; w += 32 * U) {
-                    uint32_t r[U];
-                    V x[U];
-                    bool ok[U];
-#pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        const int at = w + 32 * u + lane;
-                        const unsigned d = (unsigned)(excl - (w + 32 * u));
-                        const unsigned M = __reduce_or_sync(SPG_FULL, len > 0 && d < 32u ? 1u << d : 0u);
-                        const int sl = before + __popc(M & upto);
-                        before += __popc(M);
-                        ok[u] = at < tot;
-                        if (ok[u]) {
-                            const int64_t q = s_off[warp][sl] + at;
-                            r[u] = (uint32_t)__ldg(&ai[q]);
-                            if (MODE == 1) x[u] = mul_v(__ldg(&av[q]), s_bv[warp][sl]);
-                        }
-                    }
-#pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        if (!ok[u]) continue;
-                        bool nw;
-                        const int h = hash_insert_dbl1(keys, log2T, r[u], c.err, nw);
-                        if (MODE == 0) mine += nw;
-                        else if (h >= 0) atomic_add_v(&vals[h], x[u]);
-                    }
-                }
-                __syncwarp();
-            }
+            auto insert = [&](uint32_t r, V x) {
+                bool nw;
+                const int h = hash_insert_dbl1(keys, log2T, r, c.err, nw);
+                if (MODE == 0) mine += nw;
+                else if (h >= 0) atomic_add_v(&vals[h], x);
+            };
+            walk_entries<MODE>(p, b0, nb, 0, 1, 0, 1, s_off[warp], s_bv[MODE == 1 ? warp : 0], insert);
             if (MODE == 0) {
                 mine = warp_sum(mine);
                 if (lane == 0) c.cnt[g] = mine;
                 uint4 *k4 = reinterpret_cast<uint4 *>(keys);
                 for (int s = lane; s < T / 4; s += 32) k4[s] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
             } else {
-                const int64_t out0 = c.colptr[g] - c.out_base;
-                const int64_t want = c.colptr[g + 1] - c.colptr[g];
                 int pos2 = 0;
                 for (int s0 = 0; s0 < T; s0 += 32) {
                     const int s = s0 + lane;
