@@ -407,23 +407,27 @@ template <class I, class V> struct Engine : EngineBase {
     // Products: f receives the multiplications per column, total_out their
     // sum, and nnz_b is the number of B entries. recap (optional) may lower or
     // raise the hash cap once the total is known; the columns are then binned
-    // again.
+    // again. zeroed: cx.hist and f are zero already; rows_c: rows of C (products).
     template <class Src>
     static spgemm_status sym_pass(Ctx &cx, const typename Src::Args &sa, int64_t c_lo, int64_t c_hi,
                            const int64_t *bound, int64_t *f, uint8_t *tier, int64_t *cnt_out,
                            int32_t *list, int32_t *off, int32_t *heavy_ord_w,
                            const int32_t *heavy_ord_r, DevBuf *pcnt_grow, int32_t *pcnt_ptr,
                            int *hist_out, cudaStream_t st, bool allow_heavy = true, int64_t nnz_b = 0,
-                           int64_t *total_out = nullptr, const std::function<int(int64_t)> &recap = nullptr) {
+                           int64_t *total_out = nullptr, const std::function<int(int64_t)> &recap = nullptr,
+                           bool zeroed = false, int64_t rows_c = 0) {
         const int64_t nc = c_hi - c_lo;
         int hist[16];
         int64_t total = 0;
         for (bool again = false;; again = true) {
-          SPG_CK(cudaMemsetAsync(cx.hist, 0, sizeof(int32_t) * kBinInts, st));
+          const bool small = !Src::kParts && !bound && nc > 0 && nc <= kBinSmall;
+          // k_bin_small writes the words that a second binning needs
+          if (!(zeroed && !again) && !(small && again))
+              SPG_CK(cudaMemsetAsync(cx.hist, 0, sizeof(int32_t) * kBinInts, st));
           if (nc > 0) {
             const int tb = cx.tbegin(kPhFlopsBin, st);
             if (!Src::kParts && !again) {   // all columns of one product
-                SPG_CK(cudaMemsetAsync(f, 0, sizeof(int64_t) * (size_t)nc, st));
+                if (!zeroed) SPG_CK(cudaMemsetAsync(f, 0, sizeof(int64_t) * (size_t)nc, st));
                 const int64_t per = 256 * kFlopsEntries;
                 if constexpr (!Src::kParts) {
                     if (nnz_b > 0) {
@@ -434,11 +438,22 @@ template <class I, class V> struct Engine : EngineBase {
                     }
                 }
             }
-            k_col_tier<Src><<<(unsigned)((nc + 255) / 256), 256, 0, st>>>(
-                sa, c_lo, c_hi, cx.tun.hash_cap_max, cx.cap_full, bound, f, tier, cnt_out, cx.hist, cx.hist + kOverFull);
-            k_bin_scatter<<<(unsigned)((nc + 255) / 256), 256, 0, st>>>(tier, c_lo, c_hi, cx.hist,
-                                                                       cx.cursor, list, off,
-                                                                       heavy_ord_w);
+            bool binned = false;
+            if constexpr (!Src::kParts) {
+                if (small) {
+                    k_bin_small<<<1, 1024, 0, st>>>(f, rows_c, cx.cap_full, nullptr, nullptr, c_lo, (int)nc,
+                                                    cx.tun.hash_cap_max, tier, cnt_out, list, off, heavy_ord_w, cx.hist,
+                                                    cx.hist + kOverFull, cx.cursor);
+                    binned = true;
+                }
+            }
+            if (!binned) {
+                k_col_tier<Src><<<(unsigned)((nc + 255) / 256), 256, 0, st>>>(
+                    sa, c_lo, c_hi, cx.tun.hash_cap_max, cx.cap_full, bound, f, tier, cnt_out, cx.hist, cx.hist + kOverFull);
+                k_bin_scatter<<<(unsigned)((nc + 255) / 256), 256, 0, st>>>(tier, c_lo, c_hi, cx.hist,
+                                                                           cx.cursor, list, off,
+                                                                           heavy_ord_w);
+            }
             cx.tend(tb, st);
             cx.launched(2);
             SPG_CK(cudaGetLastError());
@@ -522,11 +537,16 @@ template <class I, class V> struct Engine : EngineBase {
         c.out_base = o.out_base;
         if (any_hash && nc > 0) {
             const int th = cx.tbegin(cx.ph_hash, st);
-            SPG_CK(cudaMemsetAsync(cx.hist, 0, sizeof(int32_t) * kBinInts, st));
-            k_numeric_tier<<<(unsigned)((nc + 255) / 256), 256, 0, st>>>(
-                cnt, dense_sel, c_lo, c_hi, cx.tun.hash_cap_max, tier, cx.hist);
-            k_bin_scatter<<<(unsigned)((nc + 255) / 256), 256, 0, st>>>(
-                tier, c_lo, c_hi, cx.hist, cx.cursor, list, off, nullptr);
+            if (nc <= kBinSmall) {
+                k_bin_small<<<1, 1024, 0, st>>>(nullptr, 0, 0, cnt, dense_sel, c_lo, (int)nc, cx.tun.hash_cap_max, tier,
+                                                nullptr, list, off, nullptr, cx.hist, nullptr, cx.cursor);
+            } else {
+                SPG_CK(cudaMemsetAsync(cx.hist, 0, sizeof(int32_t) * kBinInts, st));
+                k_numeric_tier<<<(unsigned)((nc + 255) / 256), 256, 0, st>>>(
+                    cnt, dense_sel, c_lo, c_hi, cx.tun.hash_cap_max, tier, cx.hist);
+                k_bin_scatter<<<(unsigned)((nc + 255) / 256), 256, 0, st>>>(
+                    tier, c_lo, c_hi, cx.hist, cx.cursor, list, off, nullptr);
+            }
             SPG_CK(cudaGetLastError());
             c.list = list; c.list_off = off;
             for (int t = 1; t <= 8; ++t) {
@@ -678,13 +698,15 @@ template <class I, class V> struct Engine : EngineBase {
         const size_t stages = ps.s > 1 ? (size_t)ps.s * c : 0;
         SPG_CK(carve<SPGEMM_MEM_DEVICE>(
             ps.arena,
-            {{&ps.probs, sizeof(PD)}, {&ps.f, i64 * c}, {&ps.cnt, i64 * c}, {&ps.colptr, i64 * c},
-             {&ps.col_ws, std::max(i64 * c, i32 * tier_words(ps))}, {&ps.tier, c + 15}, {&ps.list_sym, i32 * c},
-             {&ps.list_num, i32 * c}, {&ps.heavy_ord, i32 * c}, {&ps.hist, i32 * kBinInts}, {&ps.off_sym, i32 * 64},
-             {&ps.off_num, i32 * 64}, {&ps.err, sizeof(int) * 4}, {&ps.scan_part, i64 * (size_t)scan_partials_len(n + 1)},
+            // err, hist and f are zeroed together; colptr and col_ws are read back
+            // together (as h_colptr and h_tier_blk below)
+            {{&ps.probs, sizeof(PD)}, {&ps.err, sizeof(int) * 4}, {&ps.hist, i32 * kBinInts}, {&ps.f, i64 * c},
+             {&ps.cnt, i64 * c}, {&ps.colptr, i64 * c}, {&ps.col_ws, std::max(i64 * c, i32 * tier_words(ps))},
+             {&ps.tier, c + 15}, {&ps.list_sym, i32 * c}, {&ps.list_num, i32 * c}, {&ps.heavy_ord, i32 * c},
+             {&ps.off_sym, i32 * 64}, {&ps.off_num, i32 * 64}, {&ps.scan_part, i64 * (size_t)scan_partials_len(n + 1)},
              {&ps.stage_cnt, i64 * stages}, {&ps.stage_colptr, i64 * stages}}));
         SPG_CK(carve<SPGEMM_MEM_PINNED_HOST>(
-            ps.h_arena, {{&ps.h_colptr, i64 * c}, {&ps.h_small, 4096}, {&ps.h_tier_blk, i32 * tier_words(ps)},
+            ps.h_arena, {{&ps.h_colptr, i64 * c}, {&ps.h_tier_blk, i32 * tier_words(ps)}, {&ps.h_small, 4096},
                          {&ps.h_stage_colptr, i64 * stages}}));
         SPG_CK(cudaMemcpyAsync(ps.probs.p, &pd, sizeof(PD), cudaMemcpyHostToDevice, st));
         SPG_CK(cudaMemsetAsync(ps.err.p, 0, sizeof(int) * 4, st));
@@ -697,7 +719,8 @@ template <class I, class V> struct Engine : EngineBase {
         ps.panels_built = false;
         ps.tun.hash_cap_max = heavy_rule(ps);
         Ctx cx = make_ctx(ps);
-        SPG_CK(cudaMemsetAsync(ps.err.p, 0, sizeof(int) * 4, st));
+        // the error word, the bins and the flops lie next to each other
+        SPG_CK(cudaMemsetAsync(ps.err.p, 0, (size_t)((char *)ps.f.p - (char *)ps.err.p) + sizeof(int64_t) * (size_t)(n + 1), st));
         // the rule's cap stays where the flops bound C to a single batch
         const auto recap = [&](int64_t flops) {
             return cx.tun.hash_cap_max == ps.cap_full || one_batch(ps, flops) ? cx.tun.hash_cap_max : ps.cap_full;
@@ -707,7 +730,7 @@ template <class I, class V> struct Engine : EngineBase {
                                        ps.tier.as<uint8_t>(), ps.cnt.as<int64_t>(),
                                        ps.list_sym.as<int32_t>(), ps.off_sym.as<int32_t>(),
                                        ps.heavy_ord.as<int32_t>(), ps.heavy_ord.as<int32_t>(),
-                                       &ps.pcnt, nullptr, ps.sym_hist, st, true, ps.B.nnz, &ps.flops, recap));
+                                       &ps.pcnt, nullptr, ps.sym_hist, st, true, ps.B.nnz, &ps.flops, recap, true, ps.m));
         ps.tun.hash_cap_max = cx.tun.hash_cap_max;
         // heavy columns by the rule alone: their workspace is not the budget's
         ps.rule_only = ps.tun.hash_cap_max < ps.cap_full && cx.over_full == 0;
@@ -732,7 +755,7 @@ template <class I, class V> struct Engine : EngineBase {
                                                ps.col_ws.as<int64_t>(), ps.tier.as<uint8_t>(), scnt,
                                                ps.list_num.as<int32_t>(), ps.off_num.as<int32_t>(),
                                                nullptr, ps.heavy_ord.as<int32_t>(), nullptr, spc,
-                                               nullptr, st, true, ps.B.nnz));
+                                               nullptr, st, true, ps.B.nnz, nullptr, nullptr, false, ps.m));
                 SPG_CK(exclusive_scan_i64(scnt, n, ps.stage_colptr.as<int64_t>() + (size_t)t * (n + 1),
                                           ps.scan_part.as<int64_t>(), 1, st));
                 cx.launched(3);
@@ -758,7 +781,7 @@ template <class I, class V> struct Engine : EngineBase {
                                                    ps.col_ws.as<int64_t>(), ps.tier.as<uint8_t>(), pc,
                                                    ps.list_num.as<int32_t>(), ps.off_num.as<int32_t>(),
                                                    nullptr, ps.heavy_ord.as<int32_t>(), nullptr, pp,
-                                                   nullptr, st, true, ps.B.nnz));
+                                                   nullptr, st, true, ps.B.nnz, nullptr, nullptr, false, ps.m));
                     SPG_CK(exclusive_scan_i64(pc, n, ps.pref_colptr.as<int64_t>() + (size_t)(u - 1) * (n + 1),
                                               ps.scan_part.as<int64_t>(), 1, st));
                     cx.launched(3);
@@ -767,8 +790,6 @@ template <class I, class V> struct Engine : EngineBase {
                                        sizeof(int64_t) * (size_t)nu * (n + 1), cudaMemcpyDeviceToHost, st));
             }
         }
-        SPG_CK(cudaMemcpyAsync(ps.h_colptr.p, ps.colptr.p, sizeof(int64_t) * (n + 1),
-                               cudaMemcpyDeviceToHost, st));
         SPG_ST(count_tiers(ps, cx, st));
         if (ps.nheavy) SPG_ST(build_panels(ps, st));
         // products alone: a hash item may span any number of panels (one run
@@ -918,7 +939,8 @@ template <class I, class V> struct Engine : EngineBase {
         return (size_t)tier_tables(ps) * (size_t)tier_block_count(ps.n) * 16 + 1;
     }
 
-    // Enqueues the counts and their copy to the host (with the error word last).
+    // Enqueues the counts and the copy of C's offsets and the counts to the host
+    // (the error word last).
     static spgemm_status count_tiers(PlanState &ps, const Ctx &cx, cudaStream_t st) {
         const int64_t n = ps.n, nblk = tier_block_count(n);
         const int nt = tier_tables(ps);
@@ -934,7 +956,9 @@ template <class I, class V> struct Engine : EngineBase {
         }
         cx.launched(nt);
         SPG_CK(cudaGetLastError());
-        SPG_CK(cudaMemcpyAsync(ps.h_tier_blk.p, blk, sizeof(int32_t) * words, cudaMemcpyDeviceToHost, st));
+        // the offsets and the counts behind them, in one copy
+        const size_t gap = (size_t)((char *)blk - ps.colptr.as<char>());
+        SPG_CK(cudaMemcpyAsync(ps.h_colptr.p, ps.colptr.p, gap + sizeof(int32_t) * words, cudaMemcpyDeviceToHost, st));
         return SPGEMM_OK;
     }
 

@@ -1450,6 +1450,16 @@ __global__ void k_heavy_items_one(const int32_t *list, const int32_t *list_off, 
                                   int64_t room, HeavyItem *items, int32_t *order, int64_t *total);
 __global__ void k_small_excl_scan(int32_t *a, int n, int64_t *total);
 
+// The binning of few columns in one launch of one CTA (defined in
+// util_kernels.cu): tier, histogram, offsets and list, for the symbolic step (f
+// given: k_col_tier's rule, cnt and heavy ordinals too) or the numeric one (cnt
+// and sel given: num_tier); hist is written, and the cursors behind it are
+// zeroed.
+constexpr int kBinSmall = 16384;
+__global__ void k_bin_small(const int64_t *f, int64_t m, int cap_full, const int64_t *num_cnt, const int64_t *num_sel,
+                            int64_t c_lo, int n, int hash_cap_max, uint8_t *tier, int64_t *cnt_out, int32_t *list,
+                            int32_t *list_off, int32_t *heavy_ord, int32_t *hist, int32_t *over, int32_t *cursor);
+
 // Tier populations per block of kTierBlock columns (blk[b * 16 + t]) from the
 // offsets cp (sel: the offsets of C when cp are a stage's), and the error word
 // (defined in util_kernels.cu).

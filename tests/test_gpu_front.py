@@ -22,7 +22,7 @@ def diagonal(n, it):
 
 
 @pytest.mark.parametrize("it", [torch.int32, torch.int64])
-@pytest.mark.parametrize("n", [1, 31, 2047, 2048, 2049, 8192, 8193, 57344, 57345, 70001, (1 << 23) + 8191])
+@pytest.mark.parametrize("n", [1, 31, 1024, 1025, 2047, 2048, 2049, 8192, 8193, 16384, 16385, 57344, 57345, 70001, (1 << 23) + 8191])
 def test_offsets_and_flops_of_ragged_columns(n, it):
     g = torch.Generator(device="cuda")
     g.manual_seed(n)
