@@ -161,6 +161,12 @@ template <class I, class V> struct Engine : EngineBase {
         set_smem(k_num_dense<SrcPanel<I, V>>, mx);
         set_smem(k_num_dense<SrcPartsPanel<I, V>>, mx);
         set_smem(k_bwd_dense<I, V>, mx);
+        set_smem(k_mid<I, V, 4096, 0>, mx);
+        set_smem(k_mid<I, V, 4096, 1>, mx);
+        set_smem(k_mid<I, V, 8192, 0>, mx);
+        set_smem(k_mid<I, V, 8192, 1>, mx);
+        set_smem(k_mid<I, V, 16384, 0>, mx);
+        set_smem(k_mid<I, V, 16384, 1>, mx);
         set_smem(k_light<I, V, 1024, 0>, mx);
         set_smem(k_light<I, V, 512, 1>, mx);
         set_smem(k_light<I, V, 1024, 1>, mx);
@@ -201,6 +207,28 @@ template <class I, class V> struct Engine : EngineBase {
     }
 
     // ---- tier launches -----------------------------------------------------
+    // A CTA tier of a product with nnz(A) < 2^31 (a run of a column of A fits 32
+    // bits anyway; larger products keep block_walk). count < 0: unknown.
+    static bool launch_mid(const Ctx &cx, const GA &sa, const TierCommon &c, int T, int thr, int mode, int count,
+                           I *rows, V *vals, cudaStream_t st) {
+        if (!sa.lean_dense) return false;
+        using Kernel = void (*)(GA, TierCommon, I *, V *);
+        Kernel k = nullptr;
+        switch (T) {
+            case 512: k = mode ? k_mid<I, V, 512, 1> : k_mid<I, V, 512, 0>; break;
+            case 1024: k = mode ? k_mid<I, V, 1024, 1> : k_mid<I, V, 1024, 0>; break;
+            case 2048: k = mode ? k_mid<I, V, 2048, 1> : k_mid<I, V, 2048, 0>; break;
+            case 4096: k = mode ? k_mid<I, V, 4096, 1> : k_mid<I, V, 4096, 0>; break;
+            case 8192: k = mode ? k_mid<I, V, 8192, 1> : k_mid<I, V, 8192, 0>; break;
+            default: k = mode ? k_mid<I, V, 16384, 1> : k_mid<I, V, 16384, 0>; break;
+        }
+        const int smem = mid_smem<V>(T, thr, mode);
+        const int per_sm = std::max(1, std::min(2048 / thr, (227 * 1024) / (smem + 1536)));
+        const int want = count < 0 ? cx.nsm * per_sm : count;
+        k<<<std::max(1, std::min(want, cx.nsm * per_sm)), thr, smem, st>>>(sa, c, rows, vals);
+        return true;
+    }
+
     // count < 0: population unknown on the host (device-driven persistent grid)
     template <class Src>
     static void launch_sym_tier(const Ctx &cx, const typename Src::Args &sa, TierCommon c, int t,
@@ -233,9 +261,12 @@ template <class I, class V> struct Engine : EngineBase {
             return;
         }
         const int thr = block_tier_threads(T, cx.tun);
+        c.next_col = cx.cursor + 32 + t;   // zeroed with the cursors at the start of the pass
+        if constexpr (!Src::kParts) {
+            if (launch_mid(cx, sa, c, T, thr, 0, count, nullptr, nullptr, st)) return;
+        }
         const int smem = T * 4;
         const int per_sm = std::max(1, std::min(2048 / thr, (228 * 1024) / (smem + 34 * 1024)));
-        c.next_col = cx.cursor + 32 + t;   // zeroed with the cursors at the start of the pass
         const int want = count < 0 ? cx.nsm * per_sm : count;
         const int blocks = std::max(1, std::min(want, cx.nsm * per_sm));
         switch (T) {
@@ -278,13 +309,16 @@ template <class I, class V> struct Engine : EngineBase {
             return;
         }
         const int thr = block_tier_threads(T, cx.tun);
+        // the tier's column counter: binning cursors 32 + t, zeroed with the
+        // cursors at the start of the pass
+        c.next_col = cx.cursor + 32 + t;
+        if constexpr (!Src::kParts) {
+            if (!c.hybrid_sort && launch_mid(cx, sa, c, T, thr, 1, count, rows, vals, st)) return;
+        }
         const int smem = T * (int)(4 + sizeof(V));
         const int per_sm = std::max(1, std::min(2048 / thr, (228 * 1024) / (smem + 34 * 1024)));
         const int want = count < 0 ? cx.nsm * per_sm : count;
         const int blocks = std::max(1, std::min(want, cx.nsm * per_sm));
-        // the tier's column counter: binning cursors 32 + t, zeroed with the
-        // cursors at the start of the pass
-        c.next_col = cx.cursor + 32 + t;
         switch (T) {
             case 512: k_num_block<Src, 512><<<blocks, thr, smem, st>>>(sa, c, rows, vals); break;
             case 1024: k_num_block<Src, 1024><<<blocks, thr, smem, st>>>(sa, c, rows, vals); break;

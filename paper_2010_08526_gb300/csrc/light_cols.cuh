@@ -198,6 +198,179 @@ __global__ void __launch_bounds__(256) k_light(GemmArgs<I, V> ga, TierCommon c, 
     }
 }
 
+// A warp's part of the products of one column with k in [k0, k1): of the rounds
+// of 32 B entries it takes r0, r0 + rs, ..., and of the 32-wide windows of a round's product
+// stream w0, w0 + ws, ...; insert(row, product) for each, with the loads of four
+// windows in flight. off / sbv: 32 places per warp in shared memory for the
+// non-empty segments of a round, in stream order (offset to the entry index, B
+// value). All lanes call it.
+template <int MODE, class I, class V, class F>
+__device__ __forceinline__ void walk_entries(const ProbDev<I, V> *p, int64_t k0, int64_t k1, int64_t b0, int nb,
+                                             int r0, int rs, int w0, int ws, int64_t *off, V *sbv, F &&insert) {
+    constexpr int U = 4;
+    const int lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u, upto = 0xffffffffu >> (31 - lane);
+    const I *bi = p->bi, *ap = p->ap, *ai = p->ai;
+    const V *bv = p->bv, *av = p->av;
+    for (int base = 32 * r0; base < nb; base += 32 * rs) {
+        int64_t beg = 0;
+        int len = 0;
+        V bval = V(0);
+        if (base + lane < nb) {
+            const int64_t k = (int64_t)__ldg(&bi[b0 + base + lane]);
+            if (k >= k0 && k < k1) {
+                beg = (int64_t)__ldg(&ap[k]);
+                len = (int)((int64_t)__ldg(&ap[k + 1]) - beg);
+            }
+            if (MODE == 1) bval = __ldg(&bv[b0 + base + lane]);
+        }
+        const int incl = warp_incl_scan(len);
+        const int excl = incl - len;
+        const int tot = __shfl_sync(SPG_FULL, incl, 31);
+        const unsigned nzm = __ballot_sync(SPG_FULL, len > 0);
+        if (len > 0) {
+            const int rank = __popc(nzm & below);
+            off[rank] = beg - excl;
+            if (MODE == 1) sbv[rank] = bval;
+        }
+        __syncwarp();
+        for (int w = 32 * w0; w < tot; w += 32 * U * ws) {
+            uint32_t r[U];
+            V x[U];
+            bool ok[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                // the segment of a lane: the last one starting at or before it
+                const int wu = w + 32 * u * ws;
+                const unsigned d = (unsigned)(excl - wu);
+                const unsigned M = __reduce_or_sync(SPG_FULL, len > 0 && d < 32u ? 1u << d : 0u);
+                const int before = __popc(__ballot_sync(SPG_FULL, len > 0 && excl < wu));
+                const int sl = before + __popc(M & upto) - 1;
+                ok[u] = wu + lane < tot;
+                if (ok[u]) {
+                    const int64_t q = off[sl] + wu + lane;
+                    r[u] = (uint32_t)__ldg(&ai[q]);
+                    if (MODE == 1) x[u] = mul_v(__ldg(&av[q]), sbv[sl]);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (ok[u]) insert(r[u], MODE == 1 ? x[u] : V(0));
+        }
+        __syncwarp();   // the segments are read: the next round may replace them
+    }
+}
+
+// Columns of the CTA tiers (tables of up to 16384 slots), one CTA each, taken
+// from a device counter: the symbolic count (MODE 0) and the numeric
+// accumulation (MODE 1: table order, or ascending with c.sort). The warps share a
+// column without a barrier (walk_entries): by rounds of B entries when there are
+// enough of them, else by windows of each round's stream, which every warp lays out
+// for itself. A CTA-wide scan per chunk of B entries (block_walk) waited on
+// four barriers for the few dozen entries of such a column and took 29 KB of
+// shared memory from the tables. Issue of the shared-memory CAS and add bounds
+// the walk now. Measured against block_walk, protein product of 100k columns
+// (int64 indices, float): numeric 1173 -> 1091 us (8192 slots), 504 -> 390 us
+// (4096), 168 -> 149 us (2048), symbolic 163 -> 125 us (4096); a stage of R-MAT
+// scale 15 split in four: numeric 155 -> 135 us (16384), 91 -> 79 us (8192),
+// symbolic 95 -> 79 us (16384).
+template <class V> constexpr int mid_smem(int T, int threads, int mode) {
+    return T * (4 + (mode == 1 ? (int)sizeof(V) : 0)) + threads * (8 + (mode == 1 ? (int)sizeof(V) : 0));
+}
+
+template <class I, class V, int T, int MODE>
+__global__ void __launch_bounds__(1024, 1) k_mid(GemmArgs<I, V> ga, TierCommon c, I *out_rows, V *out_vals) {
+    constexpr int LOG2T = Log2<T>::v;
+    extern __shared__ __align__(16) unsigned char smem[];
+    V *vals = reinterpret_cast<V *>(smem);
+    uint32_t *keys = reinterpret_cast<uint32_t *>(smem + (MODE == 1 ? sizeof(V) * T : 0));
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    int64_t *off = reinterpret_cast<int64_t *>(keys + T) + warp * 32;
+    V *sbv = reinterpret_cast<V *>(reinterpret_cast<int64_t *>(keys + T) + nw * 32) + warp * 32;
+    __shared__ SortShared ss;
+    __shared__ int s_it, s_red[33];
+    const ProbDev<I, V> *pd = ga.probs;
+    const I *bp = pd->bp;
+    const int lo = c.list_off[c.tier], hi = c.list_off[c.tier + 1];
+    uint4 *k4 = reinterpret_cast<uint4 *>(keys);
+    for (int s = threadIdx.x; s < T / 4; s += blockDim.x) k4[s] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
+    if (MODE == 1)
+        for (int s = threadIdx.x; s < T; s += blockDim.x) vals[s] = V(0);
+    // thread 0 reserves the next column when it starts one
+    int ahead = 0;
+    if (threadIdx.x == 0) ahead = atomicAdd(c.next_col, 1);
+    for (;;) {
+        if (threadIdx.x == 0) {
+            s_it = lo + ahead;
+            ahead = atomicAdd(c.next_col, 1);
+        }
+        __syncthreads();   // the table is clean, too
+        const int it = s_it;
+        if (it >= hi) break;
+        const int64_t g = c.list[it];
+        const int64_t b0 = (int64_t)__ldg(&bp[g]);
+        const int nb = (int)((int64_t)__ldg(&bp[g + 1]) - b0);
+        int64_t out0 = 0;
+        int want = 0;
+        if (MODE == 1) {
+            out0 = c.colptr[g] - c.out_base;
+            want = (int)(c.colptr[g + 1] - c.colptr[g]);
+        }
+        int mine = 0;
+        auto insert = [&](uint32_t r, V x) {
+            bool fresh;
+            const int h = hash_insert_dbl1(keys, LOG2T, r, c.err, fresh);
+            if (MODE == 0) mine += fresh;
+            else if (h >= 0) atomic_add_v(&vals[h], x);
+        };
+        const bool rounds = nb >= 64 * nw;
+        walk_entries<MODE>(pd, ga.k0, ga.k1, b0, nb, rounds ? warp : 0, rounds ? nw : 1, rounds ? 0 : warp,
+                           rounds ? 1 : nw, off, sbv, insert);
+        if (MODE == 0) {
+            mine = warp_sum(mine);
+            if (lane == 0) s_red[warp] = mine;
+            __syncthreads();
+            if (warp == 0) {
+                const int v = warp_sum(lane < nw ? s_red[lane] : 0);
+                if (lane == 0) c.cnt[g] = v;
+            }
+            for (int s = threadIdx.x; s < T / 4; s += blockDim.x) k4[s] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
+            __syncthreads();   // before thread 0 names the next column
+            continue;
+        }
+        __syncthreads();
+        if (c.sort) {
+            sorted_emit<true>(keys, vals, T, want, &ss, c.err, out_rows + out0, out_vals + out0);
+            continue;
+        }
+        // a warp owns a run of slots: count, one barrier, write and clear
+        const int per = (T + nw - 1) / nw;
+        const int slo = min(T, warp * per), shi = min(T, slo + per);
+        int n = 0;
+        for (int s = slo + lane; s < shi; s += 32) n += keys[s] != kEmpty;
+        n = warp_sum(n);
+        int o = warp_offset(n, s_red, warp, nw, lane);
+        for (int s0 = slo; s0 < shi; s0 += 32) {
+            const int s = s0 + lane;
+            const uint32_t key = s < shi ? keys[s] : kEmpty;
+            const bool occ = key != kEmpty;
+            const unsigned bal = __ballot_sync(SPG_FULL, occ);
+            if (occ) {
+                const int r = o + __popc(bal & ((1u << lane) - 1u));
+                if (r < want) {
+                    out_rows[out0 + r] = (I)key;
+                    out_vals[out0 + r] = vals[s];
+                }
+                keys[s] = kEmpty;
+                vals[s] = V(0);
+            }
+            o += __popc(bal);
+        }
+        if (warp == nw - 1 && lane == 0 && o != want) atomicOr(c.err, kErrCount);
+        __syncthreads();
+    }
+}
+
 // Masked backward of light columns (columns of G of at most T / 2 entries),
 // one warp each: for every product A(i, k) B(k, j) with G(i, j) stored,
 //   dA(i, k) += G(i, j) B(k, j),  dB(k, j) += A(i, k) G(i, j).

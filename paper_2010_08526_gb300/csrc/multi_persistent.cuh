@@ -64,67 +64,6 @@ template <class V> __device__ __forceinline__ void gatomic_add_v(V *p, V v) {
     else atomic_add_v(p, v);
 }
 
-// A warp's part of the products of one column: of the rounds of 32 B entries
-// it takes r0, r0 + rs, ..., and of the 32-wide windows of a round's product
-// stream w0, w0 + ws, ...; insert(row, product) for each, with the loads of four
-// windows in flight. off / sbv: 32 places per warp in shared memory for the
-// non-empty segments of a round, in stream order (offset to the entry index, B
-// value). All lanes call it.
-template <int MODE, class I, class V, class F>
-__device__ __forceinline__ void walk_entries(const ProbDev<I, V> *p, int64_t b0, int nb, int r0, int rs, int w0,
-                                             int ws, int64_t *off, V *sbv, F &&insert) {
-    constexpr int U = 4;
-    const int lane = threadIdx.x & 31;
-    const unsigned below = (1u << lane) - 1u, upto = 0xffffffffu >> (31 - lane);
-    const I *bi = p->bi, *ap = p->ap, *ai = p->ai;
-    const V *bv = p->bv, *av = p->av;
-    for (int base = 32 * r0; base < nb; base += 32 * rs) {
-        int64_t beg = 0;
-        int len = 0;
-        V bval = V(0);
-        if (base + lane < nb) {
-            const int64_t k = (int64_t)__ldg(&bi[b0 + base + lane]);
-            beg = (int64_t)__ldg(&ap[k]);
-            len = (int)((int64_t)__ldg(&ap[k + 1]) - beg);
-            if (MODE == 1) bval = __ldg(&bv[b0 + base + lane]);
-        }
-        const int incl = warp_incl_scan(len);
-        const int excl = incl - len;
-        const int tot = __shfl_sync(SPG_FULL, incl, 31);
-        const unsigned nzm = __ballot_sync(SPG_FULL, len > 0);
-        if (len > 0) {
-            const int rank = __popc(nzm & below);
-            off[rank] = beg - excl;
-            if (MODE == 1) sbv[rank] = bval;
-        }
-        __syncwarp();
-        for (int w = 32 * w0; w < tot; w += 32 * U * ws) {
-            uint32_t r[U];
-            V x[U];
-            bool ok[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                // the segment of a lane: the last one starting at or before it
-                const int wu = w + 32 * u * ws;
-                const unsigned d = (unsigned)(excl - wu);
-                const unsigned M = __reduce_or_sync(SPG_FULL, len > 0 && d < 32u ? 1u << d : 0u);
-                const int before = __popc(__ballot_sync(SPG_FULL, len > 0 && excl < wu));
-                const int sl = before + __popc(M & upto) - 1;
-                ok[u] = wu + lane < tot;
-                if (ok[u]) {
-                    const int64_t q = off[sl] + wu + lane;
-                    r[u] = (uint32_t)__ldg(&ai[q]);
-                    if (MODE == 1) x[u] = mul_v(__ldg(&av[q]), sbv[sl]);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < U; ++u)
-                if (ok[u]) insert(r[u], MODE == 1 ? x[u] : V(0));
-        }
-        __syncwarp();   // the segments are read: the next round may replace them
-    }
-}
-
 // MODE 0: symbolic (count distinct rows into c.cnt[g]); MODE 1: numeric
 // (accumulate, write column g at c.colptr[g] - c.out_base, unsorted).
 template <class Src, int NT, int MODE>
@@ -190,7 +129,7 @@ __global__ void __launch_bounds__(NT, MODE == 0 ? 1536 / NT : 0) k_multi_pass(ty
                     else if (h >= 0) atomic_add_v(&vals[h], x);
                 };
                 const bool rounds = src.nb >= 64 * NW;
-                walk_entries<MODE>(src.p, src.b0, (int)src.nb, rounds ? warp : 0, rounds ? NW : 1, rounds ? 0 : warp,
+                walk_entries<MODE>(src.p, 0, INT64_MAX, src.b0, (int)src.nb, rounds ? warp : 0, rounds ? NW : 1, rounds ? 0 : warp,
                                    rounds ? 1 : NW, s_off[warp], s_bv[MODE == 1 ? warp : 0], insert);
                 __syncthreads();
                 if (MODE == 0) {
@@ -346,7 +285,7 @@ __global__ void __launch_bounds__(NT, MODE == 0 ? 1536 / NT : 0) k_multi_pass(ty
                 if (MODE == 0) mine += nw;
                 else if (h >= 0) atomic_add_v(&vals[h], x);
             };
-            walk_entries<MODE>(p, b0, nb, 0, 1, 0, 1, s_off[warp], s_bv[MODE == 1 ? warp : 0], insert);
+            walk_entries<MODE>(p, 0, INT64_MAX, b0, nb, 0, 1, 0, 1, s_off[warp], s_bv[MODE == 1 ? warp : 0], insert);
             if (MODE == 0) {
                 mine = warp_sum(mine);
                 if (lane == 0) c.cnt[g] = mine;
