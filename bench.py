@@ -539,7 +539,7 @@ def bench_multi(spg, torch, args):
     torch.cuda.empty_cache()
     r = {"problems": n, "flops": flops, "multi_ms": t_multi * 1e3, "plain_ms": t_plain * 1e3,
          "speedup": t_plain / t_multi, "multi_gflops": 2 * flops / t_multi / 1e9,
-         "launches_per_run": "flop count, tier binning, 1 symbolic pass, 3-kernel scan, 1 numeric pass",
+         "launches_per_run": "flop count, tier binning, 1 symbolic pass, scan, 1 numeric pass",
          "plain_path": "512 plans made once and reused: symbolic + numeric per product per run",
          "tuning": autotune.describe([(best, 0.0)])[0], "autotune_trials": autotune.describe(trials)}
     if not args.no_cpu:

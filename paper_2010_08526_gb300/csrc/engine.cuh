@@ -489,7 +489,7 @@ template <class I, class V> struct Engine : EngineBase {
                                                                            heavy_ord_w);
             }
             cx.tend(tb, st);
-            cx.launched(2);
+            cx.launched(binned ? 1 : 2);
             SPG_CK(cudaGetLastError());
           }
           SPG_CK(cudaMemcpyAsync(cx.h_small, cx.hist, sizeof(int32_t) * (kOverFull + 1), cudaMemcpyDeviceToHost, st));
@@ -588,7 +588,7 @@ template <class I, class V> struct Engine : EngineBase {
                 const int cntt = tc ? tc[t] : -1;
                 if (cntt != 0) { launch_num_tier<Src>(cx, sa, c, t, cntt, o.rows, o.vals, st); cx.launched(); }
             }
-            cx.launched(2);
+            cx.launched(nc <= kBinSmall ? 1 : 2);
             cx.tend(th, st);
         }
         if (heavy) {
@@ -774,7 +774,7 @@ template <class I, class V> struct Engine : EngineBase {
         SPG_CK(exclusive_scan_i64(ps.cnt.as<int64_t>(), n, ps.colptr.as<int64_t>(),
                                   ps.scan_part.as<int64_t>(), 1, st));
         cx.tend(tsc, st);
-        cx.launched(3);
+        cx.launched(scan_launches(n));
         // k-split stages: per-stage counts nnz(D_t(:, j)) (LocalSymbolic per stage,
         // Algorithm 3), panel counts for the heavy columns
         if (ps.s > 1) {
@@ -792,7 +792,7 @@ template <class I, class V> struct Engine : EngineBase {
                                                nullptr, st, true, ps.B.nnz, nullptr, nullptr, false, ps.m));
                 SPG_CK(exclusive_scan_i64(scnt, n, ps.stage_colptr.as<int64_t>() + (size_t)t * (n + 1),
                                           ps.scan_part.as<int64_t>(), 1, st));
-                cx.launched(3);
+                cx.launched(scan_launches(n));
             }
             SPG_CK(cudaMemcpyAsync(ps.h_stage_colptr.p, ps.stage_colptr.p,
                                    sizeof(int64_t) * (size_t)ps.s * (n + 1), cudaMemcpyDeviceToHost, st));
@@ -818,7 +818,7 @@ template <class I, class V> struct Engine : EngineBase {
                                                    nullptr, st, true, ps.B.nnz, nullptr, nullptr, false, ps.m));
                     SPG_CK(exclusive_scan_i64(pc, n, ps.pref_colptr.as<int64_t>() + (size_t)(u - 1) * (n + 1),
                                               ps.scan_part.as<int64_t>(), 1, st));
-                    cx.launched(3);
+                    cx.launched(scan_launches(n));
                 }
                 SPG_CK(cudaMemcpyAsync(ps.h_pref_colptr.p, ps.pref_colptr.p,
                                        sizeof(int64_t) * (size_t)nu * (n + 1), cudaMemcpyDeviceToHost, st));
@@ -889,7 +889,7 @@ template <class I, class V> struct Engine : EngineBase {
         k_items_by_batch<<<ob, 256, 0, st>>>(items, ps.n_items, bounds, nb, pe, 1, cnt,
                                              ps.item_order.as<int32_t>());
         k_batch_item_starts<<<(unsigned)((nb + 1 + 255) / 256), 256, 0, st>>>(cnt, nb, pe, ps.n_items, bounds);
-        ps.timer.launches += 6;
+        ps.timer.launches += 3 + scan_launches(nbins, true);
         SPG_CK(cudaGetLastError());
         std::vector<int64_t> off((size_t)nb + 1);
         SPG_CK(cudaMemcpyAsync(off.data(), bounds, sizeof(int64_t) * (size_t)(nb + 1), cudaMemcpyDeviceToHost, st));
@@ -951,7 +951,7 @@ template <class I, class V> struct Engine : EngineBase {
                                                       ps.ap_row.as<uint16_t>(), ps.ap_val.as<V>(),
                                                       ps.apc_row.as<uint32_t>(), ps.apc_val.as<V>());
         ps.timer.end(tp, st);
-        ps.timer.launches += 6;
+        ps.timer.launches += (nnzA > 0 ? 3 : 1) + scan_launches(N, true);
         SPG_CK(cudaGetLastError());
         ps.panels_built = true;
         return SPGEMM_OK;
@@ -1512,7 +1512,7 @@ template <class I, class V> struct Engine : EngineBase {
         SPG_ST(prune_plan(colptr, (const V *)vals, ncols, thr, topk, ws, ocolptr, st));
         SPG_ST(prune_fill<I>(colptr, (const I *)rows, (const V *)vals, ncols, thr, topk, tie_by_row, ws, ocolptr,
                              (I *)orows, (V *)ovals, ps.nsm, st));
-        ps.timer.launches += 6;
+        ps.timer.launches += (ncols <= 0 ? 0 : topk > 0 ? 3 : 2) + scan_launches(ncols);
         if (ps.defer_sort && ncols > 0) {
             // columns of up to 256 kept entries by a warp, 1024 and 8192 by a CTA
             const unsigned wbk = (unsigned)std::max<int64_t>(1, std::min<int64_t>((ncols + 7) / 8, (int64_t)ps.nsm * 8));
@@ -1524,7 +1524,7 @@ template <class I, class V> struct Engine : EngineBase {
             if (topk > 1024)
                 k_sort_cols<I, V, 16384, true><<<bb, 512, 16384 * slot, st>>>(ocolptr, ncols, 1024, (I *)orows,
                                                                              (V *)ovals);
-            ps.timer.launches += 3;
+            ps.timer.launches += 1 + (topk > 256) + (topk > 1024);
             SPG_CK(cudaGetLastError());
         }
         return SPGEMM_OK;
@@ -1557,7 +1557,7 @@ template <class I, class V> struct Engine : EngineBase {
             k_fill_zero<V><<<(unsigned)((ps.A.nnz + 255) / 256), 256, 0, st>>>((V *)dA, ps.A.nnz);
         if (ps.B.nnz)
             k_fill_zero<V><<<(unsigned)((ps.B.nnz + 255) / 256), 256, 0, st>>>((V *)dB, ps.B.nnz);
-        cx.launched(2);
+        cx.launched((ps.A.nnz > 0) + (ps.B.nnz > 0));
         if (n == 0) { cx.tend(tbw, st); return SPGEMM_OK; }
         SPG_CK(cudaMemsetAsync(cx.hist, 0, sizeof(int32_t) * kBinInts, st));
         k_bwd_tier<I, V><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(ga, n, cx.tun.hash_cap_max,

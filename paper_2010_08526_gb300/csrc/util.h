@@ -10,6 +10,7 @@ int64_t scan_partials_len(int64_t n);
 // out[i] = sum_{j<i} in[j], i in [0, n) (and out[n] = total when write_total).
 cudaError_t exclusive_scan_i64(const int64_t *in, int64_t n, int64_t *out, int64_t *partials,
                                int write_total, cudaStream_t st);
+int scan_launches(int64_t n, bool in_place = false);   // launches of that scan
 cudaError_t rebase_colptr(const int64_t *src, int64_t n, void *dst, int dst_is_i64,
                           cudaStream_t st);
 cudaError_t validate_csc(const void *colptr, const void *rowidx, int idx64, int64_t ncols,

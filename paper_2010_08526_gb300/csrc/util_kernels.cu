@@ -436,6 +436,11 @@ int64_t scan_partials_len(int64_t n) { return (n + kScanTile - 1) / kScanTile + 
 // which saves the launch between (3 us). Beyond, three launches.
 constexpr int64_t kDirectScan = 56 * 1024;
 constexpr int64_t kFoldPartials = 1024;
+int scan_launches(int64_t n, bool in_place) {
+    const int64_t nb = n > 0 ? (n + kScanTile - 1) / kScanTile : 1;
+    if ((!in_place && n <= kDirectScan) || nb == 1) return 1;
+    return nb <= kFoldPartials ? 2 : 3;
+}
 cudaError_t exclusive_scan_i64(const int64_t *in, int64_t n, int64_t *out, int64_t *partials,
                                int write_total, cudaStream_t st) {
     const int64_t nb = n > 0 ? (n + kScanTile - 1) / kScanTile : 1;
