@@ -673,12 +673,17 @@ template <class I, class V> struct Engine : EngineBase {
         a.apc_off = ps.apc_off.as<int32_t>();
         a.apc_row = ps.apc_row.as<uint32_t>();
         a.apc_val = ps.P == 1 ? ps.ap_val.as<V>() : ps.apc_val.as<V>();   // one panel: the same order
-        a.lean_dense = ps.A.nnz < (int64_t(1) << 31) ? 1 : 0;
+        a.lean_dense = narrow(ps) ? 1 : 0;
         // a chunk's stream is at most kSymChunk columns of A, each of at most
         // min(m, nnz(A)) entries
         a.lean_sym = a.lean_dense && std::min<int64_t>(ps.A.nrows, ps.A.nnz) * kSymChunk < (int64_t(1) << 31);
         return a;
     }
+
+    // Whether the kernels with 32-bit entry offsets and stream positions may run: a
+    // walk looks up to kLeanSlack positions past the stream it is in.
+    static constexpr int64_t kLeanSlack = 8192;
+    static bool narrow(const PlanState &ps) { return ps.A.nnz < (int64_t(1) << 31) - kLeanSlack; }
 
     // Columns above this many rows are heavy (k_sym_heavy32, k_num_heavy32),
     // unless the caller gave hash_max_cap. The largest table that fits a CTA
@@ -696,7 +701,7 @@ template <class I, class V> struct Engine : EngineBase {
     // A k-split keeps 8192 (its stages read every heavy column again: 4-stage R-MAT 15
     // 8.07 -> 8.24 ms), and so does a product that the budget may cut into batches.
     static int heavy_rule(const PlanState &ps) {
-        if (!ps.cap_rule || ps.s > 1 || ps.opts.prune || ps.A.nnz >= (int64_t(1) << 31)) return ps.cap_full;
+        if (!ps.cap_rule || ps.s > 1 || ps.opts.prune || !narrow(ps)) return ps.cap_full;
         if (ps.P == 1) {
             int cap = 256;
             while (cap < ps.cap_full && (int64_t)cap * 16 < ps.m) cap *= 2;
@@ -830,7 +835,7 @@ template <class I, class V> struct Engine : EngineBase {
         // of the column-grouped copy of A); the items that k_sort_items orders
         // and the k-split's part-by-part merges keep the narrower form
         const int max_panels = (ps.s > 1 || !ps.A.nnz || (ps.opts.sort_output && !heavy32(cx, gemm_args(ps, 0, ps.k))) ||
-                                ps.A.nnz >= (int64_t(1) << 31))
+                                !narrow(ps))
                                    ? kRangeMaxPanels : std::max(kRangeMaxPanels, ps.P);
         SPG_ST(build_items(cx, ps.nheavy, ps.list_sym.as<int32_t>(), ps.off_sym.as<int32_t>(),
                            ps.cnt.as<int64_t>(), ps.pcnt.as<int32_t>(), ps.items, ps.item_cnt,

@@ -1,7 +1,7 @@
 // Light columns of a product, one warp each, with a warp-private hash table in
 // shared memory (C(:, j) = A * B(:, j), Sec. II-C's column formula): the
 // symbolic count and the numeric accumulation, with 32-bit entry offsets (the
-// caller guarantees nnz(A) < 2^31).
+// caller guarantees nnz(A) < 2^31 less the look-ahead of a walk).
 //
 // A column of some hundred products is a chain of dependent loads (column
 // list, colptr of B, its rows, colptr of A, A's entries) around little work, so
@@ -198,12 +198,14 @@ __global__ void __launch_bounds__(256) k_light(GemmArgs<I, V> ga, TierCommon c, 
     }
 }
 
-// A warp's part of the products of one column with k in [k0, k1): of the rounds
-// of 32 B entries it takes r0, r0 + rs, ..., and of the 32-wide windows of a round's product
-// stream w0, w0 + ws, ...; insert(row, product) for each, with the loads of four
-// windows in flight. off / sbv: 32 places per warp in shared memory for the
-// non-empty segments of a round, in stream order (offset to the entry index, B
-// value). All lanes call it.
+// A warp's part of the products of one column with k in [k0, k1): of the rounds of
+// 32 B entries it takes r0, r0 + rs, ..., and of the 32-wide windows of a round's
+// product stream w0, w0 + ws, ...; insert(row, product) for each, with the loads of
+// four windows in flight. Stream positions are 32-bit: the runs of a column of a
+// hash tier have at most as many entries as the column (rows are distinct in a
+// column of A), or nnz(A) is below 2^31 less the look-ahead. off / sbv: 32 places
+// per warp in shared memory for the non-empty segments of a round, in stream order
+// (offset to the entry index, B value). All lanes call it.
 template <int MODE, class I, class V, class F>
 __device__ __forceinline__ void walk_entries(const ProbDev<I, V> *p, int64_t k0, int64_t k1, int64_t b0, int nb,
                                              int r0, int rs, int w0, int ws, int64_t *off, V *sbv, F &&insert) {
