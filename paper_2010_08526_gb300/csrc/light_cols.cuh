@@ -276,12 +276,16 @@ __device__ __forceinline__ void walk_entries(const ProbDev<I, V> *p, int64_t k0,
 // (4096), 168 -> 149 us (2048), symbolic 163 -> 125 us (4096); a stage of R-MAT
 // scale 15 split in four: numeric 155 -> 135 us (16384), 91 -> 79 us (8192),
 // symbolic 95 -> 79 us (16384).
+// Registers: 64 let one CTA of 1024 threads run; the symbolic tables up to 8192 slots
+// leave room for half as many threads again at 40 (protein symbolic 330 -> 270 us at 8192,
+// 125 -> 102 us at 4096), which slows the numeric pass (8192 slots 1090 -> 1107 us, 16384
+// slots 139 -> 163 us per stage of the R-MAT).
 template <class V> constexpr int mid_smem(int T, int threads, int mode) {
     return T * (4 + (mode == 1 ? (int)sizeof(V) : 0)) + threads * (8 + (mode == 1 ? (int)sizeof(V) : 0));
 }
 
 template <class I, class V, int T, int MODE>
-__global__ void __launch_bounds__(1024, 1) k_mid(GemmArgs<I, V> ga, TierCommon c, I *out_rows, V *out_vals) {
+__global__ void __maxnreg__(MODE == 0 && T <= 8192 ? 40 : 64) k_mid(GemmArgs<I, V> ga, TierCommon c, I *out_rows, V *out_vals) {
     constexpr int LOG2T = Log2<T>::v;
     extern __shared__ __align__(16) unsigned char smem[];
     V *vals = reinterpret_cast<V *>(smem);
