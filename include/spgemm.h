@@ -109,10 +109,15 @@ typedef struct {
  * the Python package fills these from timed trials.
  *   hash_max_cap   largest column (distinct rows) kept in a shared-memory hash
  *                  table; larger columns use the dense row-panel accumulator.
- *                  Powers of two from 256 to 8192.
- *   panel_rows     rows per dense row panel (2^13, 2^14 or 2^15).
+ *                  Powers of two from 256 to 8192. By default the library
+ *                  chooses: 8192, or less by the number of rows of C when the
+ *                  product is unsplit, unpruned and sure to fit one batch.
+ *   panel_rows     rows per dense row panel (2^13, 2^14 or 2^15; by default 2^14
+ *                  for 4-byte values and 2^13 for others, fewer where all rows of
+ *                  C fit a smaller power of two).
  *   short_seg      A-column segments up to this length are walked by one thread;
- *                  longer ones by a whole warp (1..64).
+ *                  longer ones by a whole warp (1..64), in the kernels of merges,
+ *                  of the backward and of products with nnz(A) >= 2^31.
  *   huge_seg       segments longer than this are walked by the whole CTA.
  *   block_tier_threads  threads per CTA of the hash tiers (128..1024).
  *   hybrid_sort    1: a column of the CTA hash tiers whose products fit its

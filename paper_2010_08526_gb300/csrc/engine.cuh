@@ -207,8 +207,8 @@ template <class I, class V> struct Engine : EngineBase {
     }
 
     // ---- tier launches -----------------------------------------------------
-    // A CTA tier of a product with nnz(A) < 2^31 (a run of a column of A fits 32
-    // bits anyway; larger products keep block_walk). count < 0: unknown.
+    // A CTA tier of a product with 32-bit stream positions (narrow; larger products
+    // keep block_walk). count < 0: population unknown.
     static bool launch_mid(const Ctx &cx, const GA &sa, const TierCommon &c, int T, int thr, int mode, int count,
                            I *rows, V *vals, cudaStream_t st) {
         if (!sa.lean_dense) return false;

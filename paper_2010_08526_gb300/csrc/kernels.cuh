@@ -19,7 +19,11 @@
 //   heavy tier  : symbolic -- a shared-memory bitmap over up to ~1.5M rows;
 //                 numeric  -- dense accumulation of one row panel in shared
 //                 memory per CTA.
-// Hash tables are sort-free (Sec. IV-D): rows are emitted in table order.
+// A product with nnz(A) < 2^31 runs its warp and block tiers in light_cols.cuh and
+// its heavy tier in sym_heavy32.cuh and dense_items.cuh; the kernels here serve the
+// merge and larger products.
+// Hash tables are sort-free (Sec. IV-D): rows are emitted in table order, or in row
+// order straight from the table where the output is to be sorted (sort_smem.cuh).
 #pragma once
 
 #include <cstdint>

@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(256) k_light(GemmArgs<I, V> ga, TierCommon c, 
         if (MODE == 1) { o0 = c.colptr[g]; o1 = c.colptr[g + 1]; }
         int mine = 0;
         for (int base = 0;;) {
-            // this round's segments, one per lane, as a stream [0, tot)
+            // the segments of these 32 entries, one per lane, as a stream [0, tot)
             const int incl = warp_incl_scan(len);
             const int excl = incl - len;
             const int tot = __shfl_sync(SPG_FULL, incl, 31);

@@ -1,12 +1,11 @@
 // Sorted final output and the column-wise prune of a result batch.
 //
 // Sorting: the paper keeps the final C sorted within each column (Sec. IV-D:
-// only the intermediate products are left unsorted). The numeric pass leaves
-// a column in one of three states: a light column (at most hash_cap_max rows,
-// hash order), or a heavy column made of work items in panel order whose
-// dense items are already in row order and whose hash-range items (at most
-// kRangeCap rows each) are in hash order. So sorting the batch means sorting
-// segments of at most 8192 entries: the light columns and the hash items.
+// only the intermediate products are left unsorted). The numeric kernels write
+// row order themselves (sort_smem.cuh, dense items by nature). Two sorts of
+// written output remain: the hash-range items of heavy columns where the generic
+// heavy kernel made them (the merge, nnz(A) >= 2^31; k_sort_items), and the pruned
+// columns of a batch (k_sort_cols).
 //
 // Prune: the consumer the column batches are shaped for keeps the largest
 // entries of every column (Markov clustering, Sec. III; HipMCL prunes each
