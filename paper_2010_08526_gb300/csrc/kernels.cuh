@@ -945,7 +945,7 @@ __global__ void __launch_bounds__(256) k_multi_bin(GemmArgs<I, V> sa, int64_t n,
         const I *bi = p->bi, *ap = p->ap;
         for (int64_t e = b0 + sub; e < b1; e += kBinLanes) {
             const int64_t k = (int64_t)__ldg(&bi[e]);
-            f += (int64_t)__ldg(&ap[k + 1]) - (int64_t)__ldg(&ap[k]);
+            if (k >= 0) f += (int64_t)__ldg(&ap[k + 1]) - (int64_t)__ldg(&ap[k]);   // as the walks skip it
         }
         if (sub == 0 && prob_of) prob_of[g] = pr;
     }

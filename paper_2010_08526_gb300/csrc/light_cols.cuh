@@ -402,6 +402,7 @@ __global__ void __launch_bounds__(256) k_bwd_light(GradArgs<I, V> a, TierCommon 
     const I *bp = pd->bp, *bi = pd->bi, *ap = pd->ap, *ai = pd->ai;
     const V *bv = pd->bv, *av = pd->av;
     V *dA = a.dA, *dB = a.dB;
+    const int64_t k0 = a.gemm.k0, k1 = a.gemm.k1;
     const unsigned below = (1u << lane) - 1u, upto = 0xffffffffu >> (31 - lane);
     const unsigned above = ~upto;
     const int lo = c.list_off[c.tier], hi = c.list_off[c.tier + 1];
@@ -424,9 +425,11 @@ __global__ void __launch_bounds__(256) k_bwd_light(GradArgs<I, V> a, TierCommon 
             V bval = V(0);
             if (base + lane < nb) {
                 const int64_t k = (int64_t)__ldg(&bi[b0 + base + lane]);
-                const int64_t s = (int64_t)__ldg(&ap[k]);
-                beg = (int)s;
-                len = (int)((int64_t)__ldg(&ap[k + 1]) - s);
+                if (k >= k0 && k < k1) {   // an index outside [0, k) is skipped, as everywhere
+                    const int64_t s = (int64_t)__ldg(&ap[k]);
+                    beg = (int)s;
+                    len = (int)((int64_t)__ldg(&ap[k + 1]) - s);
+                }
                 bval = __ldg(&bv[b0 + base + lane]);
             }
             const int incl = warp_incl_scan(len);
