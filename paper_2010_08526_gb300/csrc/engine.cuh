@@ -711,7 +711,9 @@ template <class I, class V> struct Engine : EngineBase {
     }
 
     // Whether C fits one batch whatever its columns' overlap is: with as many
-    // entries as multiplications, and the heavy columns' workspace at its largest.
+    // entries as multiplications, and the heavy columns' workspace at its largest
+    // (in place of what an earlier step left of it, so that every symbolic step on
+    // a plan decides the same).
     static bool one_batch(const PlanState &ps, int64_t flops) {
         const int64_t si = ps.idx64 ? 8 : 4, sv = sizeof(V), r = si + sv;
         const int64_t inputs = (int64_t)(ps.A.nnz + ps.B.nnz) * r + (ps.A.ncols + ps.B.ncols + 2) * si;
@@ -719,7 +721,8 @@ template <class I, class V> struct Engine : EngineBase {
                               ps.n * ((int64_t)ps.P * 4 + 64) + (1 << 20);
         const int64_t items = ps.P == 1 ? 0 : std::min(ps.n * (int64_t)ps.P, flops) * 28;
         const int ring = ps.opts.ring_depth > 0 ? ps.opts.ring_depth : 2;
-        return inputs + (int64_t)ps.workspace_bytes() + heavy + items + ring * (flops * r + 8 * ps.n) <= (int64_t)ps.budget;
+        const int64_t other = (int64_t)ps.workspace_bytes() - (int64_t)ps.heavy_bytes();
+        return inputs + other + heavy + items + ring * (flops * r + 8 * ps.n) <= (int64_t)ps.budget;
     }
 
     static bool incremental(const PlanState &ps) {

@@ -1,0 +1,79 @@
+"""Which columns are heavy by default: the line, the budgets it applies to and
+what the plan reports of it."""
+from __future__ import annotations
+
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():  # pragma: no cover
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+import paper_2010_08526_gb300 as spg  # noqa: E402
+
+
+def columns(nrows, counts, g, vt=torch.float32):
+    """Columns of counts[j] distinct rows in a run from a random start."""
+    ptr = torch.zeros(counts.numel() + 1, dtype=torch.int64, device="cuda")
+    ptr[1:] = torch.cumsum(counts, 0)
+    col = torch.repeat_interleave(torch.arange(counts.numel(), device="cuda"), counts)
+    start = torch.randint(0, nrows, (counts.numel(),), generator=g, device="cuda")
+    rows = (start[col] + torch.arange(col.numel(), device="cuda") - ptr[col]) % nrows
+    vals = torch.randint(1, 5, (col.numel(),), generator=g, device="cuda").to(vt)
+    return spg.Csc(nrows, counts.numel(), ptr.int(), rows.int(), vals)
+
+
+def operands(m, most, seed, k=600, n=500, per=40):
+    """A product whose columns have up to min(m, most + a few hundred) rows and many products each."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    A = columns(m, torch.randint(1, most, (k,), generator=g, device="cuda"), g)
+    B = columns(k, torch.randint(0, per, (n,), generator=g, device="cuda"), g)
+    return A, B
+
+
+def info_at(A, B, budget, **kw):
+    plan = spg.Plan(A, B, budget=budget, **kw)
+    try:
+        return plan.symbolic()
+    except spg.SpgemmError as e:
+        return dict(status=e.status, heavy_columns=0)
+    finally:
+        plan.close()
+
+
+def line_budget(A, B):
+    """(lo, hi): the default line applies at hi bytes and not at lo, 4 KiB below."""
+    lo, hi = 1 << 20, 1 << 34
+    assert info_at(A, B, hi)["heavy_columns"] > 0 and info_at(A, B, lo)["heavy_columns"] == 0
+    while hi - lo > 4096:
+        mid = (lo + hi) // 2
+        if info_at(A, B, mid)["heavy_columns"] > 0:
+            hi = mid
+        else:
+            lo = mid
+    return lo, hi
+
+
+@pytest.mark.parametrize("m", [5000, 40000])
+def test_repeated_symbolic_steps_plan_the_same(m):
+    """The workspace that one symbolic step leaves on a plan does not change the
+    next one's heavy columns, batches or cap, at budgets around the one from
+    which the default line applies."""
+    A, B = operands(m, m // 2 if m < 8192 else 7000, m)
+    if m > 8192:   # one B entry a column: no column above the fixed line
+        g = torch.Generator(device="cuda")
+        g.manual_seed(3)
+        B = columns(B.nrows, torch.ones(B.ncols, dtype=torch.int64, device="cuda"), g)
+    lo, hi = line_budget(A, B)
+    for budget in (lo, hi, hi + (64 << 10), hi + (1 << 20), hi + (32 << 20)):
+        want = info_at(A, B, budget)
+        plan = spg.Plan(A, B, budget=budget)
+        for _ in range(3):
+            try:
+                got = plan.symbolic()
+            except spg.SpgemmError as e:
+                got = dict(status=e.status, heavy_columns=0)
+            assert got == want, budget - hi
+        plan.close()
