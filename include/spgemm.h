@@ -276,7 +276,10 @@ spgemm_status spgemm_plan_destroy(spgemm_plan *plan);
  *                                                  per column (topk <= 0: nnz(C(:,j)))
  * The cap of one batch (spgemm_plan_info.batch_cap_bytes) is (budget -
  * r (nnz(A) + nnz(B)) - index bytes (ncols(A) + ncols(B) + 2) - plan
- * workspace) / ring_depth. Starting at column 0, each range is extended while
+ * workspace) / ring_depth. Where the library chose a lower hash_max_cap than 8192
+ * (spgemm_tuning), the workspace in this formula is the one of hash_max_cap 8192, so
+ * that the plan does not depend on the choice; such a product is a single batch, and the
+ * budget holds it with the workspace that it has. Starting at column 0, each range is extended while
  * the next column still fits under the cap; b is the number of ranges.
  * Errors: SPGEMM_ERR_BUDGET (inputs alone exceed the budget, or one column's
  * output exceeds a batch), SPGEMM_ERR_CUDA, SPGEMM_ERR_OOM.

@@ -364,9 +364,9 @@ template <class I, class V> struct Engine : EngineBase {
 
     // Cut the heavy columns of the symbolic list into work items (dense
     // panels and hash ranges) from their per-panel output counts, dense items
-    // before hash items, each by first panel. The total is left on the device
-    // (ioff[0]) and copied to item_total(cx), read by the caller after its next
-    // wait: with one panel a column has at most one item, so there is room for
+    // before hash items, each by first panel. The total and the part of it that
+    // columns above cap_full make are left on the device (ioff[0], ioff[1]) and copied
+    // to item_total(cx) and full_items(cx), read by the caller after its next wait: with one panel a column has at most one item, so there is room for
     // all before the total is known. Otherwise it is read here, between the
     // count and the items. Few columns and panels take one launch (a product
     // of 3,000 rows spent 55 us on eight launches and two waits).
@@ -377,12 +377,17 @@ template <class I, class V> struct Engine : EngineBase {
         std::memcpy(&t, cx.h_small + 256, sizeof(t));
         return t;
     }
+    static int64_t full_items(const Ctx &cx) {
+        int64_t t;
+        std::memcpy(&t, cx.h_small + 258, sizeof(t));
+        return t;
+    }
     static spgemm_status build_items(const Ctx &cx, int nheavy, const int32_t *sym_list,
                                      const int32_t *sym_off, const int64_t *sel,
                                      const int32_t *pcnt, DevBuf &items, DevBuf &icnt,
                                      DevBuf &ioff, DevBuf &order, cudaStream_t st,
                                      int max_panels = kRangeMaxPanels) {
-        std::memset(cx.h_small + 256, 0, sizeof(int64_t));
+        std::memset(cx.h_small + 256, 0, 2 * sizeof(int64_t));
         if (!nheavy) return SPGEMM_OK;
         SPG_CK(icnt.ensure(sizeof(int64_t) * (size_t)(std::max(nheavy, cx.P) + 1)));
         SPG_CK(ioff.ensure(sizeof(int64_t) * (nheavy + 1)));
@@ -397,17 +402,17 @@ template <class I, class V> struct Engine : EngineBase {
         const bool one = (int64_t)nheavy * cx.P <= kItemsOne && 2 * cx.P <= kItemBins;
         const unsigned nb = (unsigned)((nheavy + 255) / 256);
         auto read_total = [&]() {
-            return cudaMemcpyAsync(cx.h_small + 256, total_d, sizeof(int64_t), cudaMemcpyDeviceToHost, st);
+            return cudaMemcpyAsync(cx.h_small + 256, total_d, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost, st);
         };
         auto run_one = [&](int64_t room) {
-            k_heavy_items_one<<<1, 1024, 0, st>>>(sym_list, sym_off, sel, cx.tun.hash_cap_max, pcnt, cx.P, dmin, rcap,
-                                                  max_panels, room, items.as<HeavyItem>(), order.as<int32_t>(),
+            k_heavy_items_one<<<1, 1024, 0, st>>>(sym_list, sym_off, sel, cx.tun.hash_cap_max, cx.cap_full, pcnt, cx.P,
+                                                  dmin, rcap, max_panels, room, items.as<HeavyItem>(), order.as<int32_t>(),
                                                   total_d);
             cx.launched();
         };
         auto run_bins = [&](int mode) {
-            k_heavy_items<<<nb, 256, 0, st>>>(sym_list, sym_off, sel, cx.tun.hash_cap_max, pcnt, cx.P, dmin, rcap,
-                                              max_panels, mode, bins, items.as<HeavyItem>(), order.as<int32_t>());
+            k_heavy_items<<<nb, 256, 0, st>>>(sym_list, sym_off, sel, cx.tun.hash_cap_max, cx.cap_full, pcnt, cx.P, dmin,
+                                              rcap, max_panels, mode, bins, items.as<HeavyItem>(), order.as<int32_t>());
             cx.launched();
         };
         auto size_items = [&](int64_t cnt) -> cudaError_t {
@@ -418,7 +423,7 @@ template <class I, class V> struct Engine : EngineBase {
         if (one) {
             run_one(cx.P == 1 ? nheavy : 0);
         } else {
-            SPG_CK(cudaMemsetAsync(bins, 0, sizeof(int32_t) * 2 * (size_t)cx.P, st));
+            SPG_CK(cudaMemsetAsync(bins, 0, sizeof(int32_t) * (2 * (size_t)cx.P + 1), st));
             run_bins(0);
             k_small_excl_scan<<<1, 1024, 0, st>>>(bins, 2 * cx.P, total_d);
             cx.launched();
@@ -725,6 +730,14 @@ template <class I, class V> struct Engine : EngineBase {
         return inputs + other + heavy + items + ring * (flops * r + 8 * ps.n) <= (int64_t)ps.budget;
     }
 
+    // The heavy columns' workspace if the line were at cap_full.
+    static size_t full_line_bytes(const PlanState &ps) {
+        if (ps.over_full == 0) return 0;
+        const size_t nh = (size_t)ps.over_full, np = (size_t)ps.P, it = np == 1 ? nh : (size_t)ps.full_items;
+        return ps.panel_bytes() + sizeof(int32_t) * nh * np + sizeof(int64_t) * (std::max(nh, np) + 1) +
+               sizeof(int64_t) * (nh + 1) + (sizeof(HeavyItem) + sizeof(int32_t)) * (it + 1);
+    }
+
     static bool incremental(const PlanState &ps) {
         return ps.s > 1 && ps.opts.merge_mode == SPGEMM_MERGE_INCREMENTAL;
     }
@@ -774,8 +787,7 @@ template <class I, class V> struct Engine : EngineBase {
                                        ps.heavy_ord.as<int32_t>(), ps.heavy_ord.as<int32_t>(),
                                        &ps.pcnt, nullptr, ps.sym_hist, st, true, ps.B.nnz, &ps.flops, recap, true, ps.m));
         ps.tun.hash_cap_max = cx.tun.hash_cap_max;
-        // heavy columns by the rule alone: their workspace is not the budget's
-        ps.rule_only = ps.tun.hash_cap_max < ps.cap_full && cx.over_full == 0;
+        ps.over_full = cx.over_full;
         ps.nheavy = 0;
         for (int t = kHeavyTier0; t < kTiers; ++t) ps.nheavy += ps.sym_hist[t];
         const int tsc = cx.tbegin(kPhScan, st);
@@ -845,6 +857,7 @@ template <class I, class V> struct Engine : EngineBase {
                            ps.item_off, ps.item_order, st, max_panels));
         SPG_CK(cudaStreamSynchronize(st));
         ps.n_items = item_total(cx);
+        ps.full_items = full_items(cx);
         const int errw = ps.h_tier_blk.as<int32_t>()[tier_words(ps) - 1];
         if (errw) {
             set_error("symbolic: device error flags " + std::to_string(errw));
@@ -1037,15 +1050,16 @@ template <class I, class V> struct Engine : EngineBase {
         const int64_t ptr_bytes = 8;
         const int64_t inputs = (int64_t)(ps.A.nnz + ps.B.nnz) * r +
                                (ps.A.ncols + 1 + ps.B.ncols + 1) * (ps.idx64 ? 8 : 4);
-        // heavy columns that only heavy_rule made heavy: the product was shown to
-        // fit one batch with their workspace, which is left out here so that
-        // the reported cap per batch does not depend on the rule
+        // columns that only heavy_rule made heavy: the product was shown to fit one
+        // batch with their workspace, and the cap per batch is the one of the fixed
+        // line, whose workspace for heavy columns is counted here
+        const int64_t heavy = (int64_t)(ps.tun.hash_cap_max < ps.cap_full ? full_line_bytes(ps) : ps.heavy_bytes());
         // the stage partial buffers are part of each batch's bytes (w_j counts
         // the unmerged entries), so they are not workspace here; this keeps the
         // plan identical across repeated symbolic calls on one plan
         const int64_t ws = (int64_t)ps.workspace_bytes() - (int64_t)ps.drows.bytes -
                            (int64_t)ps.dvals.bytes - (int64_t)ps.parts_tab.bytes -
-                           (ps.rule_only ? (int64_t)ps.heavy_bytes() : 0);
+                           (int64_t)ps.heavy_bytes() + heavy;
         const int64_t avail = (int64_t)ps.budget - inputs - ws;
         const int ring = ps.opts.ring_depth > 0 ? ps.opts.ring_depth : 2;
         if (avail <= 0) {

@@ -1447,10 +1447,10 @@ struct HeavyItem {
 constexpr int kItemBins = 2048;   // (kind, first panel) bins that a CTA counts in shared memory
 constexpr int kItemsOne = 16384;  // columns x panels that one CTA cuts by itself
 __global__ void k_heavy_items(const int32_t *list, const int32_t *list_off, const int64_t *sel, int hash_cap_max,
-                              const int32_t *pcnt, int P, int dense_min, int range_cap, int max_panels, int mode,
+                              int cap_full, const int32_t *pcnt, int P, int dense_min, int range_cap, int max_panels, int mode,
                               int32_t *bins, HeavyItem *items, int32_t *order);
 __global__ void k_heavy_items_one(const int32_t *list, const int32_t *list_off, const int64_t *sel, int hash_cap_max,
-                                  const int32_t *pcnt, int P, int dense_min, int range_cap, int max_panels,
+                                  int cap_full, const int32_t *pcnt, int P, int dense_min, int range_cap, int max_panels,
                                   int64_t room, HeavyItem *items, int32_t *order, int64_t *total);
 __global__ void k_small_excl_scan(int32_t *a, int n, int64_t *total);
 

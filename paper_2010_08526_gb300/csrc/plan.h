@@ -242,7 +242,8 @@ struct PlanState {
     AllocFns alloc;          // workspace allocator (opts->allocator, copied)
     Tuning tun;              // tun.hash_cap_max: the cap of the last symbolic step
     int cap_full = 8192;     // the largest hash table (the caller's hash_max_cap, or the default)
-    bool rule_only = false;  // heavy columns exist only by the engine's rule
+    int over_full = 0;       // columns above cap_full by their multiplications
+    int64_t full_items = 0;  // heavy items of the columns above cap_full
     bool cap_rule = true;    // no hash_max_cap given: the engine's rule by size applies
     int idx64 = 0, vtype = 0;
     int64_t m = 0, k = 0, n = 0;
@@ -290,9 +291,12 @@ struct PlanState {
     int64_t bytes_per_nnz = 0;
 
     size_t workspace_bytes() const;
-    size_t heavy_bytes() const {   // workspace of the heavy columns
+    size_t panel_bytes() const {   // the panelised copies of A
         return ap_end.bytes + ap_row.bytes + ap_val.bytes + apc_off.bytes + apc_row.bytes + apc_val.bytes +
-               merge_tmp.bytes + pcnt.bytes + items.bytes + item_cnt.bytes + item_off.bytes + item_order.bytes;
+               merge_tmp.bytes;
+    }
+    size_t heavy_bytes() const {   // workspace of the heavy columns
+        return panel_bytes() + pcnt.bytes + items.bytes + item_cnt.bytes + item_off.bytes + item_order.bytes;
     }
     void release_all();
 };

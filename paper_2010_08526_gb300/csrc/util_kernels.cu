@@ -165,9 +165,10 @@ __device__ __forceinline__ void cut_items(int64_t g, const int32_t *pc, int P, i
 // (dense items before hash items, each by first panel). One thread per heavy
 // column runs the greedy cut over its P panel counts. For up to kItemBins bins
 // a CTA counts its items in shared memory and takes each bin's run with one
-// global atomic.
+// global atomic. Mode 0 also adds the items of columns above cap_full to
+// bins[2 P].
 __global__ void __launch_bounds__(256) k_heavy_items(const int32_t *list, const int32_t *list_off, const int64_t *sel,
-                                                     int hash_cap_max, const int32_t *pcnt, int P, int dense_min,
+                                                     int hash_cap_max, int cap_full, const int32_t *pcnt, int P, int dense_min,
                                                      int range_cap, int max_panels, int mode, int32_t *bins,
                                                      HeavyItem *items, int32_t *order) {
     __shared__ int s_cnt[kItemBins], s_base[kItemBins];
@@ -178,6 +179,13 @@ __global__ void __launch_bounds__(256) k_heavy_items(const int32_t *list, const 
     const int64_t g = h < hi - lo ? list[lo + h] : 0;
     const bool mine = h < hi - lo && sel[g] > hash_cap_max;
     const int32_t *pc = pcnt + h * P;
+    if (mode == 0) {
+        int full = 0;
+        if (mine && sel[g] > cap_full)
+            cut_items(g, pc, P, dense_min, range_cap, max_panels, [&](int, const HeavyItem &) { ++full; });
+        full = warp_sum(full);
+        if ((threadIdx.x & 31) == 0 && full) atomicAdd(&bins[nbins], full);
+    }
     if (local) {
         for (int b = threadIdx.x; b < nbins; b += blockDim.x) s_cnt[b] = 0;
         __syncthreads();
@@ -202,13 +210,15 @@ __global__ void __launch_bounds__(256) k_heavy_items(const int32_t *list, const 
 
 // The same in one launch of one CTA, for few columns and panels (nheavy * P
 // <= kItemsOne): counts, bin prefix, items if there is room for them, and the
-// total.
+// totals (of all items, of those of columns above cap_full).
 __global__ void __launch_bounds__(1024) k_heavy_items_one(const int32_t *list, const int32_t *list_off,
-                                                          const int64_t *sel, int hash_cap_max, const int32_t *pcnt,
-                                                          int P, int dense_min, int range_cap, int max_panels,
+                                                          const int64_t *sel, int hash_cap_max, int cap_full,
+                                                          const int32_t *pcnt, int P, int dense_min, int range_cap, int max_panels,
                                                           int64_t room, HeavyItem *items, int32_t *order,
                                                           int64_t *total) {
     __shared__ int s_bin[kItemBins];
+    __shared__ int s_full;
+    if (threadIdx.x == 0) s_full = 0;
     const int lo = list_off[kHeavyTier0], nh = list_off[kTiers] - lo;
     const int nbins = 2 * P;
     for (int b = threadIdx.x; b < nbins; b += blockDim.x) s_bin[b] = 0;
@@ -217,7 +227,10 @@ __global__ void __launch_bounds__(1024) k_heavy_items_one(const int32_t *list, c
         const int64_t g = list[lo + h];
         if (sel[g] > hash_cap_max)
             cut_items(g, pcnt + (int64_t)h * P, P, dense_min, range_cap, max_panels,
-                      [&](int kind, const HeavyItem &it) { atomicAdd(&s_bin[kind * P + it.p0], 1); });
+                      [&](int kind, const HeavyItem &it) {
+                          atomicAdd(&s_bin[kind * P + it.p0], 1);
+                          if (sel[g] > cap_full) atomicAdd(&s_full, 1);
+                      });
     }
     __syncthreads();
     if (threadIdx.x < 32) {
@@ -229,7 +242,7 @@ __global__ void __launch_bounds__(1024) k_heavy_items_one(const int32_t *list, c
             if (b < nbins) s_bin[b] = carry + incl - v;
             carry += __shfl_sync(SPG_FULL, incl, 31);
         }
-        if (threadIdx.x == 0) *total = carry;
+        if (threadIdx.x == 0) { total[0] = carry; total[1] = s_full; }
     }
     __syncthreads();
     for (int h = threadIdx.x; h < nh; h += blockDim.x) {
@@ -287,7 +300,8 @@ __global__ void k_batch_item_starts(const unsigned long long *cnt, int64_t nb, i
     start[t] = t == 0 ? 0 : t == nb ? n : (int64_t)cnt[t * 2 * pe - 1];
 }
 
-// exclusive scan of n ints in place (one CTA); the sum goes to total
+// exclusive scan of n ints in place (one CTA); the sum goes to total[0], a[n] to
+// total[1]
 __global__ void __launch_bounds__(1024) k_small_excl_scan(int32_t *a, int n, int64_t *total) {
     __shared__ int32_t s_warp[33];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -306,7 +320,7 @@ __global__ void __launch_bounds__(1024) k_small_excl_scan(int32_t *a, int n, int
         carry += all;
         __syncthreads();
     }
-    if (threadIdx.x == 0) *total = carry;
+    if (threadIdx.x == 0) { total[0] = carry; total[1] = a[n]; }
 }
 
 // ---- exclusive scan of int64 (three phases, all on the device) ------------

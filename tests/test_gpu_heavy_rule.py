@@ -77,3 +77,19 @@ def test_repeated_symbolic_steps_plan_the_same(m):
                 got = dict(status=e.status, heavy_columns=0)
             assert got == want, budget - hi
         plan.close()
+
+
+@pytest.mark.parametrize("m,most,k", [(5000, 2500, 600), (16000, 8000, 600), (40000, 12000, 600), (300000, 12000, 3000)])
+@pytest.mark.parametrize("sort", [False, True])
+def test_cap_per_batch_is_the_fixed_lines(m, most, k, sort):
+    """No column above 8192 rows, some of them, in one panel and in several:
+    the cap of a batch is the one of the 8192-row line, after a first and a
+    second symbolic step."""
+    A, B = operands(m, most, m, k=k, n=2 * k, per=6)
+    fixed = info_at(A, B, 1 << 34, sort_output=sort, tuning=spg.Tuning(hash_max_cap=8192))
+    plan = spg.Plan(A, B, budget=1 << 34, sort_output=sort)
+    for _ in range(2):
+        info = plan.symbolic()
+        assert info["heavy_columns"] > fixed["heavy_columns"]     # the lower line is in use
+        assert info["batch_cap_bytes"] == fixed["batch_cap_bytes"]
+    plan.close()
