@@ -48,6 +48,25 @@ __host__ __device__ inline int num_tier(int64_t n, int64_t sel, int hash_cap_max
 // columns per entry of k_tier_blocks
 constexpr int kTierBlock = 256;
 
+// The last column in [c, last] that starts at or before entry q (ptr[c] <= q),
+// near c or far away: doubling steps, then a search between the last two. A walk
+// over the entries of a matrix with long runs of empty columns takes the logarithm
+// of a run's length, not the run.
+template <class P>
+__device__ __forceinline__ int64_t column_from(const P *ptr, int64_t c, int64_t last, int64_t q) {
+    int64_t step = 1;
+    while (c + step <= last && (int64_t)__ldg(&ptr[c + step]) <= q) {
+        c += step;
+        step *= 2;
+    }
+    int64_t hi = c + step - 1 < last ? c + step - 1 : last;
+    while (c < hi) {
+        const int64_t mid = (c + hi + 1) >> 1;
+        if ((int64_t)__ldg(&ptr[mid]) <= q) c = mid; else hi = mid - 1;
+    }
+    return c;
+}
+
 // Multiplicative (Fibonacci) hashing: the top log2(T) bits of key * 2^32/phi.
 __device__ __forceinline__ uint32_t hash_slot(uint32_t key, int log2T) {
     return (key * 0x9E3779B1u) >> (32 - log2T);

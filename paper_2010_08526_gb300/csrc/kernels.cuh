@@ -845,10 +845,14 @@ __global__ void __launch_bounds__(256) k_col_flops(GemmArgs<I, V> ga, int64_t n,
 #pragma unroll
         for (int i = 0; i < kFlopsEntries; ++i) {
             if (q0 + i >= e_end) break;
-            while (q0 + i >= next) {
+            if (q0 + i >= next) {
                 if (sum) atomicAdd(&f[g], (unsigned long long)sum);
                 sum = 0;
                 next = (int64_t)__ldg(&bp[++g + 1]);
+                if (q0 + i >= next) {   // empty columns between
+                    g = column_from(bp, g + 1, n - 1, q0 + i);
+                    next = (int64_t)__ldg(&bp[g + 1]);
+                }
             }
             sum += len[i];
             all += len[i];
