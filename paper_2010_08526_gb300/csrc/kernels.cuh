@@ -1803,7 +1803,17 @@ __device__ __forceinline__ void panel_runs(const I *ap, const I *ai, int64_t ka,
     for (int w = 0; w < kPanelWindow; w += 32) {
         const int64_t q = w0 + w + lane;
         const bool active = q < a1;
-        while (active && q >= end) { ++col; beg = end; end = (int64_t)__ldg(&ap[col + 1]); }
+        // a few short columns are stepped over, longer runs (empty ones) searched
+        for (int step = 0; active && q >= end && step < 4; ++step) {
+            ++col;
+            beg = end;
+            end = (int64_t)__ldg(&ap[col + 1]);
+        }
+        if (active && q >= end) {
+            col = column_from(ap, col + 1, ka - 1, q);
+            beg = (int64_t)__ldg(&ap[col]);
+            end = (int64_t)__ldg(&ap[col + 1]);
+        }
         const int64_t r = active ? (int64_t)__ldg(&ai[q]) : 0;
         const int64_t p = r >> log2R;
         const int64_t pcol = __shfl_up_sync(SPG_FULL, col, 1);

@@ -55,3 +55,34 @@ def test_flops_across_empty_columns(places, it):
     assert plan.info["flops"] == int(want.sum()) and int(got.sum()) == int(want.sum())
     assert torch.equal(got[cols], want)
     plan.close()
+
+
+@pytest.mark.parametrize("it", [torch.int32, torch.int64])
+@pytest.mark.parametrize("ordered", [True, False])
+def test_panel_copies_across_empty_columns(ordered, it):
+    """A product with a heavy column copies A by row panels: columns of one entry
+    and of thousands, neighbours and 20,000,000 columns apart."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(4)
+    ka, m = 40_000_000, 100_000
+    cols = torch.tensor([0, 1, 2, 9, 20_000_000, 20_000_001, 39_999_990, 39_999_999], device="cuda")
+    lens = torch.tensor([60_000, 1, 1, 3, 1, 30_000, 2, 60_000], device="cuda")
+    counts = torch.zeros(ka, dtype=torch.int64, device="cuda")
+    counts[cols] = lens
+    rows = [torch.randperm(m, generator=g, device="cuda")[:int(x)] for x in lens]
+    if ordered:
+        rows = [torch.sort(r).values for r in rows]
+    rows = torch.cat(rows)
+    vals = torch.randint(1, 9, (rows.numel(),), generator=g, device="cuda").float()
+    A = csc(m, ka, counts, rows, vals, it)
+    scale = torch.arange(1, 9, device="cuda").float()
+    B = csc(ka, 1, torch.tensor([8], device="cuda"), cols, scale, it)
+    plan = spg.Plan(A, B, budget=1 << 36, sort_output=True)
+    assert seconds(plan.symbolic) < 0.5
+    assert plan.info["heavy_columns"] == 1
+    C = plan.numeric(0)
+    plan.check_errors()
+    dense = torch.zeros(m, device="cuda").index_add_(0, rows, vals * torch.repeat_interleave(scale, lens))
+    where = torch.nonzero(dense).reshape(-1)
+    assert torch.equal(C.rowidx.long(), where) and torch.equal(C.vals, dense[where])
+    plan.close()
