@@ -110,8 +110,9 @@ typedef struct {
  *   hash_max_cap   largest column (distinct rows) kept in a shared-memory hash
  *                  table; larger columns use the dense row-panel accumulator.
  *                  Powers of two from 256 to 8192. By default the library
- *                  chooses: 8192, or less by the number of rows of C when the
- *                  product is unsplit, unpruned and sure to fit one batch.
+ *                  chooses: 8192, or less by the number of rows of C and the
+ *                  multiplications of its columns when the product is unsplit,
+ *                  unpruned and sure to fit one batch.
  *   panel_rows     rows per dense row panel (2^13, 2^14 or 2^15; by default 2^14
  *                  for 4-byte values and 2^13 for others, fewer where all rows of
  *                  C fit a smaller power of two).

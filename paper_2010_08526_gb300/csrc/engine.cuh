@@ -39,11 +39,13 @@ inline int block_tier_threads(int T, const Tuning &tun) {
 
 // The binning words of a pass, zeroed together: [0, 16) tier histogram,
 // [kFlopTotal, +2) total multiplications (64 bits), [kOverFull] columns above
-// the plan's largest hash table, [64, 128) list cursors and the work counters of
+// the plan's largest hash table, [kAbove, +6) sums over the columns above the line in
+// use (three of 64 bits, see k_col_tier), [64, 128) list cursors and the work counters of
 // the persistent kernels.
 constexpr int kBinInts = 128;
 constexpr int kFlopTotal = 32;
 constexpr int kOverFull = 34;
+constexpr int kAbove = kOverFull + 2;
 
 // Scratch shared by one symbolic / numeric pass.
 struct Ctx {
@@ -111,6 +113,12 @@ template <class I, class V> struct NumOut {
     int64_t out_base;
     I *rows;
     V *vals;
+};
+
+// The columns above the hash line: their number, and k_col_tier's sums of their
+// multiplications, of the logarithms (in 64ths) and of the squares of these.
+struct Above {
+    int64_t n = 0, sum = 0, lg = 0, sq = 0;
 };
 
 template <class I, class V> struct Engine : EngineBase {
@@ -445,15 +453,15 @@ template <class I, class V> struct Engine : EngineBase {
     // heavy_ord_w (optional) receives the heavy ordinals (full pass only).
     // Products: f receives the multiplications per column, total_out their
     // sum, and nnz_b is the number of B entries. recap (optional) may lower or
-    // raise the hash cap once the total is known; the columns are then binned
-    // again. zeroed: cx.hist and f are zero already; rows_c: rows of C (products).
+    // raise the hash cap once the total and the columns above the line (their number and
+    // the sums of k_col_tier) are known; the columns are then binned again. zeroed: cx.hist and f are zero already; rows_c: rows of C (products).
     template <class Src>
     static spgemm_status sym_pass(Ctx &cx, const typename Src::Args &sa, int64_t c_lo, int64_t c_hi,
                            const int64_t *bound, int64_t *f, uint8_t *tier, int64_t *cnt_out,
                            int32_t *list, int32_t *off, int32_t *heavy_ord_w,
                            const int32_t *heavy_ord_r, DevBuf *pcnt_grow, int32_t *pcnt_ptr,
                            int *hist_out, cudaStream_t st, bool allow_heavy = true, int64_t nnz_b = 0,
-                           int64_t *total_out = nullptr, const std::function<int(int64_t)> &recap = nullptr,
+                           int64_t *total_out = nullptr, const std::function<int(int64_t, const Above &)> &recap = nullptr,
                            bool zeroed = false, int64_t rows_c = 0) {
         const int64_t nc = c_hi - c_lo;
         int hist[16];
@@ -497,12 +505,15 @@ template <class I, class V> struct Engine : EngineBase {
             cx.launched(binned ? 1 : 2);
             SPG_CK(cudaGetLastError());
           }
-          SPG_CK(cudaMemcpyAsync(cx.h_small, cx.hist, sizeof(int32_t) * (kOverFull + 1), cudaMemcpyDeviceToHost, st));
+          SPG_CK(cudaMemcpyAsync(cx.h_small, cx.hist, sizeof(int32_t) * (kAbove + 6), cudaMemcpyDeviceToHost, st));
           SPG_CK(cudaStreamSynchronize(st));
           cx.over_full = cx.h_small[kOverFull];
           std::memcpy(hist, cx.h_small, sizeof(hist));
           if (!again) std::memcpy(&total, cx.h_small + kFlopTotal, sizeof(int64_t));
-          const int cap = recap && !again ? recap(total) : cx.tun.hash_cap_max;
+          Above above;
+          for (int t = kHeavyTier0; t < kTiers; ++t) above.n += hist[t];
+          std::memcpy(&above.sum, cx.h_small + kAbove, 3 * sizeof(int64_t));
+          const int cap = recap && !again ? recap(total, above) : cx.tun.hash_cap_max;
           if (cap == cx.tun.hash_cap_max) break;
           cx.tun.hash_cap_max = cap;
         }
@@ -692,17 +703,30 @@ template <class I, class V> struct Engine : EngineBase {
 
     // Columns above this many rows are heavy (k_sym_heavy32, k_num_heavy32),
     // unless the caller gave hash_max_cap. The largest table that fits a CTA
-    // (8192 rows) is not the best line: a dense item accumulates without
-    // probing, leaves its rows in order, and three run per SM against one
-    // 1024-thread CTA with the 8192-row table. Measured steps (sorted, cap 8192 ->
-    // this rule's):
-    //   m in one panel, m / 16: R-MAT 14 1.88 -> 1.34 ms, R-MAT of 3,000 rows
-    //     0.48 -> 0.35 ms, fp64 min-plus of 7,919 rows 1.08 -> 0.79 ms, uniform 16384
-    //     with 3,600 rows a column 1.64 -> 1.15 ms (m / 32 loses where columns stay
-    //     sparse: uniform 10,000 with 1,000 rows a column 0.56 -> 0.73 ms);
-    //   more panels, 4096: protein stand-in 20,011 / 100,000 columns 2.11 -> 1.83 /
-    //     12.9 -> 12.5 ms, R-MAT of 60,000 rows 6.20 -> 5.89 ms; from about 500,000 rows
-    //     on, the symbolic bitmaps leave one CTA per SM (1,000,000 columns 133 -> 135 ms).
+    // (8192 rows) is not always the best line: a dense item accumulates without
+    // probing, leaves its rows in order, three run per SM against one
+    // 1024-thread CTA with the 8192-row table, and one launch takes the place of a launch
+    // per tier; but it scans all its rows twice, and the panel copies and item lists are
+    // launches of their own (some 45 us). Measured steps, unsorted / sorted, ms, cap 8192
+    // -> the lower line:
+    //   m in one panel, m / 16, columns of many sizes: fp32 R-MAT of 1,000 rows 0.247 -> 0.208 /
+    //     0.262 -> 0.210, of 16,000 1.63 -> 1.22 / 1.81 -> 1.26, protein stand-in of 8,000 rows
+    //     0.297 -> 0.224 / 0.317 -> 0.240 (860 products a column above the line); fp64 R-MAT of
+    //     8,000 rows 1.18 -> 0.88 / 1.26 -> 0.90; int64 0.84 -> 0.89 / 0.96 -> 0.91;
+    //   columns of one size (uniform graphs), one well-filled tier: fp32 5,000 rows with 620
+    //     products a column 0.173 -> 0.274 / 0.188 -> 0.307, with 1,400 0.228 -> 0.304 /
+    //     0.254 -> 0.300, with 3,500 0.334 -> 0.342 / 0.392 -> 0.337, 10,000 with 2,900
+    //     0.587 -> 0.656 / 0.698 -> 0.663, 2,000 with 5,000 0.183 -> 0.200 / 0.192 -> 0.200; but
+    //     16,000 with 4,600 1.54 -> 1.13 / 1.83 -> 1.16, fp64 4,000 with 5,900 0.405 -> 0.362 /
+    //     0.464 -> 0.366, int64 0.368 -> 0.395 / 0.427 -> 0.398 (lower_pays);
+    //   more panels, 4096: fp32 protein stand-in 20,011 / 100,000 columns 1.66 -> 1.49 /
+    //     1.96 -> 1.71 and 10.0 -> 9.7 / 12.1 -> 11.8, R-MAT of 60,000 rows 7.24 -> 7.17 /
+    //     8.02 -> 7.75; from about 500,000 rows on, the symbolic bitmaps leave one CTA per
+    //     SM. With 8-byte values only up to two panels (uniform 16,000 with 11,000
+    //     3.10 -> 2.22 / 3.76 -> 2.24): the panels are half as wide, and a column of a few
+    //     thousand rows is cut into as many items (uniform 40,000 with 7,500 rows a column
+    //     0.98 -> 1.23 / 1.18 -> 1.23, 500,000 12.6 -> 16.5 / 15.2 -> 19.7, int64 40,000
+    //     0.90 -> 1.50 / 1.11 -> 1.51).
     // A k-split keeps 8192 (its stages read every heavy column again: 4-stage R-MAT 15
     // 8.07 -> 8.24 ms), and so does a product that the budget may cut into batches.
     static int heavy_rule(const PlanState &ps) {
@@ -712,7 +736,18 @@ template <class I, class V> struct Engine : EngineBase {
             while (cap < ps.cap_full && (int64_t)cap * 16 < ps.m) cap *= 2;
             return cap;
         }
-        return ps.m <= (int64_t(1) << 19) ? std::min(ps.cap_full, 4096) : ps.cap_full;
+        const int64_t most = int64_t(1) << (sizeof(V) == 4 ? 19 : 14);
+        return ps.m <= most ? std::min(ps.cap_full, 4096) : ps.cap_full;
+    }
+
+    // Whether the columns above the lower line gain by it: their multiplications
+    // spread (a variance of log2 of 1/3: a uniform graph's is below 0.1, R-MAT's and
+    // the protein stand-in's 0.4 to 2.9), or they are many on average and in total. Each counts
+    // up to kRuleMost and by its logarithm, so that a few hubs do not speak for the rest.
+    static bool lower_pays(const Above &a) {
+        const double n = (double)a.n, mean = a.n ? (double)a.lg / n : 0.0;
+        const bool spread = (double)a.sq - n * mean * mean >= n * (64.0 * 64.0 / 3.0);
+        return spread || (a.sum >= 4096 * a.n && a.sum >= (int64_t(1) << 24));
     }
 
     // Whether C fits one batch whatever its columns' overlap is: with as many
@@ -776,9 +811,11 @@ template <class I, class V> struct Engine : EngineBase {
         Ctx cx = make_ctx(ps);
         // the error word, the bins and the flops lie next to each other
         SPG_CK(cudaMemsetAsync(ps.err.p, 0, (size_t)((char *)ps.f.p - (char *)ps.err.p) + sizeof(int64_t) * (size_t)(n + 1), st));
-        // the rule's cap stays where the flops bound C to a single batch
-        const auto recap = [&](int64_t flops) {
-            return cx.tun.hash_cap_max == ps.cap_full || one_batch(ps, flops) ? cx.tun.hash_cap_max : ps.cap_full;
+        // the rule's cap stays where the columns above it gain by it and the flops
+        // bound C to a single batch
+        const auto recap = [&](int64_t flops, const Above &above) {
+            const bool keep = lower_pays(above) && one_batch(ps, flops);
+            return cx.tun.hash_cap_max == ps.cap_full || keep ? cx.tun.hash_cap_max : ps.cap_full;
         };
         // full product: flops, counts, heavy list
         SPG_ST(sym_pass<SrcGemm<I, V>>(cx, gemm_args(ps, 0, ps.k), 0, n, nullptr, ps.f.as<int64_t>(),

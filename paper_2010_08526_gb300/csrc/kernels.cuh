@@ -883,16 +883,42 @@ __global__ void __launch_bounds__(256) k_col_flops(GemmArgs<I, V> ga, int64_t n,
 // histogram. bound (optional) is the exact count of the unsplit product when a
 // k-stage is binned: columns with bound > hash_cap_max go to the heavy tier
 // (their stage output must be panel-grouped), others use min(f, bound) as
-// their size. over counts the columns above cap_full, the largest line.
+// their size. over[0] counts the columns above cap_full, the largest line; where the
+// line is lower, the 64-bit words at over[2], over[4] and over[6] sum, over the columns
+// above it, x = min(f, kRuleMost), log2(x) in 64ths and its square (Engine::lower_pays).
+constexpr int kRuleMost = 16384;
+struct AboveSums {
+    int64_t x = 0, lg = 0, sq = 0;
+    __device__ __forceinline__ void add(int64_t f) {
+        const int v = (int)min(f, (int64_t)kRuleMost), l = (int)(log2f((float)v) * 64.0f);
+        x += v;
+        lg += l;
+        sq += l * l;
+    }
+    // the warp's sums into three words; all lanes call it
+    __device__ __forceinline__ void warp_add(unsigned long long *to) const {
+        if (!__any_sync(SPG_FULL, x > 0)) return;
+        const int64_t a = warp_sum(x), b = warp_sum(lg), c = warp_sum(sq);
+        if ((threadIdx.x & 31) == 0) {
+            atomicAdd(&to[0], (unsigned long long)a);
+            atomicAdd(&to[1], (unsigned long long)b);
+            atomicAdd(&to[2], (unsigned long long)c);
+        }
+    }
+};
 template <class Src>
 __global__ void __launch_bounds__(256) k_col_tier(typename Src::Args sa, int64_t c_lo, int64_t c_hi,
                                                   int hash_cap_max, int cap_full, const int64_t *bound, const int64_t *f_in,
                                                   uint8_t *tier_out, int64_t *cnt_out, int32_t *tier_hist,
                                                   int32_t *over) {
     __shared__ int s_hist[kTiers + 1];
+    __shared__ unsigned long long s_above[3];
     if (threadIdx.x <= kTiers) s_hist[threadIdx.x] = 0;
+    if (threadIdx.x < 3) s_above[threadIdx.x] = 0;
     __syncthreads();
     const int64_t g = c_lo + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const bool rule = !Src::kParts && hash_cap_max < cap_full;
+    AboveSums above;
     if (g < c_hi) {
         int64_t f, m;
         if constexpr (Src::kParts) {
@@ -906,6 +932,7 @@ __global__ void __launch_bounds__(256) k_col_tier(typename Src::Args sa, int64_t
         }
         int64_t u = f < m ? f : m;
         if (u > cap_full) atomicAdd(&s_hist[kTiers], 1);
+        if (rule && u > hash_cap_max) above.add(f);
         int t;
         if (bound && bound[g] > hash_cap_max) {
             t = heavy_subtier(f);
@@ -918,10 +945,13 @@ __global__ void __launch_bounds__(256) k_col_tier(typename Src::Args sa, int64_t
         if (cnt_out) cnt_out[g] = 0;
         if (t) atomicAdd(&s_hist[t], 1);
     }
+    if (rule) above.warp_add(s_above);
     __syncthreads();
     if (threadIdx.x < kTiers && s_hist[threadIdx.x])
         atomicAdd(&tier_hist[threadIdx.x], s_hist[threadIdx.x]);
     if (threadIdx.x == kTiers && s_hist[kTiers]) atomicAdd(over, s_hist[kTiers]);
+    if (threadIdx.x < 3 && s_above[threadIdx.x])
+        atomicAdd(reinterpret_cast<unsigned long long *>(over + 2) + threadIdx.x, s_above[threadIdx.x]);
 }
 
 // Both steps in one launch for the columns of many problems (the batched
@@ -1462,7 +1492,7 @@ __global__ void k_small_excl_scan(int32_t *a, int n, int64_t *total);
 // util_kernels.cu): tier, histogram, offsets and list, for the symbolic step (f
 // given: k_col_tier's rule, cnt and heavy ordinals too) or the numeric one (cnt
 // and sel given: num_tier); hist is written, and the cursors behind it are
-// zeroed.
+// zeroed. over as in k_col_tier.
 constexpr int kBinSmall = 16384;
 __global__ void k_bin_small(const int64_t *f, int64_t m, int cap_full, const int64_t *num_cnt, const int64_t *num_sel,
                             int64_t c_lo, int n, int hash_cap_max, uint8_t *tier, int64_t *cnt_out, int32_t *list,

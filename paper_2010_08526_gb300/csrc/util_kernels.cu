@@ -78,13 +78,17 @@ __global__ void __launch_bounds__(1024) k_bin_small(const int64_t *f, int64_t m,
                                                     int32_t *heavy_ord, int32_t *hist, int32_t *over,
                                                     int32_t *cursor) {
     __shared__ int s_cnt[kTiers], s_off[kTiers + 1], s_over;
+    __shared__ unsigned long long s_above[3];
     const int lane = threadIdx.x & 31;
     if (threadIdx.x < kTiers) s_cnt[threadIdx.x] = 0;
     if (threadIdx.x == 0) s_over = 0;
+    if (threadIdx.x < 3) s_above[threadIdx.x] = 0;
     if (threadIdx.x < 64) cursor[threadIdx.x] = 0;
     __syncthreads();
     constexpr int kPer = kBinSmall / 1024;
     int mine[kPer];   // tier and rank inside the tier
+    const bool rule = f && hash_cap_max < cap_full;
+    AboveSums above;
 #pragma unroll
     for (int i = 0; i < kPer; ++i) {
         mine[i] = 0;
@@ -96,6 +100,7 @@ __global__ void __launch_bounds__(1024) k_bin_small(const int64_t *f, int64_t m,
             if (f) {
                 const int64_t u = f[g] < m ? f[g] : m;
                 if (u > cap_full) atomicAdd(&s_over, 1);
+                if (rule && u > hash_cap_max) above.add(f[g]);
                 t = hash_tier_of(u, hash_cap_max);
                 if (t < 0) t = heavy_subtier(u);
                 cnt_out[g] = 0;
@@ -111,12 +116,16 @@ __global__ void __launch_bounds__(1024) k_bin_small(const int64_t *f, int64_t m,
         base = __shfl_sync(SPG_FULL, base, lead);
         mine[i] = t | (base + __popc(peers & ((1u << lane) - 1u))) << 5;
     }
+    if (rule) above.warp_add(s_above);
     __syncthreads();
     if (threadIdx.x == 0) {
         int acc = 0;
         for (int t = 0; t < kTiers; ++t) { s_off[t] = acc; acc += t ? s_cnt[t] : 0; }
         s_off[kTiers] = acc;
-        if (over) *over = s_over;
+        if (over) {
+            *over = s_over;
+            for (int i = 0; i < 3; ++i) reinterpret_cast<unsigned long long *>(over + 2)[i] = s_above[i];
+        }
     }
     __syncthreads();
     if (threadIdx.x <= kTiers) list_off[threadIdx.x] = s_off[threadIdx.x];
