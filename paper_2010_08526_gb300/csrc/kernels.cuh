@@ -1250,7 +1250,7 @@ __device__ __forceinline__ void num_block_sorted(const Src &src, const TierCommo
         });
     block_walk<kWalkBatch>(src, emit, c.short_seg, c.huge_seg, sh);
     const int n = sh.pos < T ? sh.pos : T;
-    block_bitonic<T>(keys, vals, n);
+    bitonic<true>(keys, vals, n);
     // runs of equal rows: a run's first entry sums it and writes it at the
     // number of runs before it
     int base = 0;

@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(512, 2) k_sort_items(const HeavyItem *items, c
         const int W = (int)((((int64_t)(item.p1 - item.p0)) << log2R) >> 5);
         if (W > wcap) {
             for (int i = threadIdx.x; i < n; i += blockDim.x) { sk[i] = (uint32_t)rows[a + i]; sv[i] = vals[a + i]; }
-            block_bitonic<CAP>(sk, sv, n);
+            bitonic<true>(sk, sv, n);
             for (int i = threadIdx.x; i < n; i += blockDim.x) { rows[a + i] = (I)sk[i]; vals[a + i] = sv[i]; }
             __syncthreads();
             continue;

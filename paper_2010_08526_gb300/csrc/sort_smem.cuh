@@ -13,7 +13,8 @@
 //      same bucket, so the loads broadcast);
 //   3. the write, whose lanes go to neighbouring places: coalesced stores.
 // The work is O(n) for spread-out rows. Clusters that overfill a bucket
-// (kSortMaxBucket) fall back to the bitonic network over the front entries.
+// (kSortMaxBucket, kSortMaxBucketWarp) fall back to the bitonic network over the
+// front entries.
 //
 // It takes the place of a bitonic sort of the written output in a kernel of
 // its own (two more passes over C, 91 barrier-separated stages at 8192
@@ -25,34 +26,45 @@
 
 namespace spg {
 
-// Bitonic sort of one segment of n <= CAP entries in shared memory (keys
-// padded with 0xffffffff to the next power of two). All threads call it.
-template <int CAP, class V>
-__device__ __forceinline__ void block_bitonic(uint32_t *sk, V *sv, int n) {
+// The group working on one table: a whole CTA, or one warp (ss unused).
+template <bool BLOCK> __device__ __forceinline__ void sort_sync() {
+    if constexpr (BLOCK) __syncthreads(); else __syncwarp();
+}
+
+// Bitonic sort of n entries in shared memory by the group (keys padded with
+// 0xffffffff to the next power of two). All its threads call it.
+template <bool BLOCK, class V>
+__device__ __forceinline__ void bitonic(uint32_t *sk, V *sv, int n) {
+    const int t = BLOCK ? (int)threadIdx.x : (int)(threadIdx.x & 31), nt = BLOCK ? (int)blockDim.x : 32;
     int np2 = 1;
     while (np2 < n) np2 <<= 1;
-    for (int i = n + threadIdx.x; i < np2; i += blockDim.x) { sk[i] = 0xffffffffu; sv[i] = V(0); }
-    __syncthreads();
+    for (int i = n + t; i < np2; i += nt) { sk[i] = 0xffffffffu; sv[i] = V(0); }
+    sort_sync<BLOCK>();
     for (int k = 2; k <= np2; k <<= 1) {
         for (int jj = k >> 1; jj > 0; jj >>= 1) {
-            for (int i = threadIdx.x; i < np2; i += blockDim.x) {
-                const int l = i ^ jj;
-                if (l > i) {
-                    const bool up = (i & k) == 0;
-                    const uint32_t a = sk[i], b = sk[l];
-                    if (up ? a > b : a < b) {
-                        sk[i] = b; sk[l] = a;
-                        const V t = sv[i]; sv[i] = sv[l]; sv[l] = t;
-                    }
+            for (int p = t; p < np2 / 2; p += nt) {   // pair p: entries i and i + jj
+                const int i = ((p & ~(jj - 1)) << 1) | (p & (jj - 1)), l = i | jj;
+                const bool up = (i & k) == 0;
+                const uint32_t a = sk[i], b = sk[l];
+                if (up ? a > b : a < b) {
+                    sk[i] = b; sk[l] = a;
+                    const V x = sv[i]; sv[i] = sv[l]; sv[l] = x;
                 }
             }
-            __syncthreads();
+            sort_sync<BLOCK>();
         }
     }
 }
 
-// a bucket above this many entries sends the CTA's segment to the bitonic sort
-constexpr int kSortMaxBucket = 512;
+// A bucket above this many entries sends a CTA's (a warp's) table to the bitonic
+// sort: counting costs a bucket its square. Columns of clusters of consecutive rows far
+// apart, ranked however full a bucket is (up to 512 in a CTA) -> with these lines,
+// fp32, times an identity: 1 x 500 rows (40,000 columns, a warp each) 1.86 -> 0.80 ms, 1 x 250
+// (80,000) 0.96 -> 0.73, 2 x 500 (20,000, a CTA each) 1.65 -> 1.03, 8 x 500 (6,000) 2.02 -> 1.59;
+// 128 in a CTA loses (16 x 250 rows 1.24 against 1.65 ms), and so does 64 in a warp (1 x 90
+// rows 0.71 against 0.92).
+constexpr int kSortMaxBucket = 256;
+constexpr int kSortMaxBucketWarp = 128;
 
 // CTA-wide scratch of the sorted compaction (a warp needs none)
 struct SortShared {
@@ -61,11 +73,6 @@ struct SortShared {
     int most;            // fullest bucket
     int red[33];
 };
-
-// The group working on one table: a whole CTA, or one warp (ss unused).
-template <bool BLOCK> __device__ __forceinline__ void sort_sync() {
-    if constexpr (BLOCK) __syncthreads(); else __syncwarp();
-}
 
 // To be called (followed by a barrier) before each sort_front of a CTA that
 // did not go through compact_front.
@@ -175,13 +182,20 @@ __device__ __forceinline__ void sort_front(uint32_t *keys, V *vals, int T, int n
         const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
         most = __reduce_max_sync(SPG_FULL, most);
         if (lane == 31) ss->red[warp] = incl;
-        if (lane == 0 && shift > 9) atomicMax(&ss->most, (int)most);   // at most 2^shift per bucket
+        if (lane == 0 && shift > 8) atomicMax(&ss->most, (int)most);   // at most 2^shift per bucket
         __syncthreads();
         const int w = lane < nw ? ss->red[lane] : 0;
         const int wi = warp_incl_scan(w);
         run += __shfl_sync(SPG_FULL, wi - w, warp);
         if (ss->most > kSortMaxBucket) {   // the same for the whole CTA
-            block_bitonic<0>(keys, vals, n);
+            bitonic<true>(keys, vals, n);
+            for (int i = t; i < n && i < want; i += nt) { out_rows[i] = (I)keys[i]; out_vals[i] = vals[i]; }
+            return;
+        }
+    } else if (shift > 7) {   // likewise
+        most = __reduce_max_sync(SPG_FULL, most);
+        if (most > kSortMaxBucketWarp) {   // the same for the warp
+            bitonic<false>(keys, vals, n);
             for (int i = t; i < n && i < want; i += nt) { out_rows[i] = (I)keys[i]; out_vals[i] = vals[i]; }
             return;
         }
