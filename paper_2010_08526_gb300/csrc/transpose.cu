@@ -28,26 +28,54 @@ __global__ void k_t_count(const I *rowidx, int64_t nnz, int64_t m, unsigned long
     }
 }
 
-// One thread per entry: its column is the last one starting at or before it
-// (a search in colptr that the lanes of a warp mostly share). A warp per
-// column left 30 lanes idle on columns of two entries, the shape of a k-mer
-// matrix: 55.6 us for 800,018 entries, now 20.9 us.
+// A warp takes `window` consecutive entries, four per lane at a time: the columns of
+// the first and of the last one by a search in colptr (half of the lanes each), and every
+// entry's column between these two. A warp per column left 30 lanes idle on columns of
+// two entries, the shape of a k-mer matrix (the call on 800,018 entries 0.34 ms, now 0.10); a
+// whole search per entry cost more than it saved on long columns of neighbouring rows, whose
+// cursors stay in cache (warp per column / search per entry / now, int32, ms: 2,000,000
+// columns of 50 rows 1.90 / 2.65 / 1.61, 4,000,000 of 16 1.66 / 1.98 / 1.15, 100,000 of
+// 1000 2.27 / 2.68 / 2.27). 256 entries a warp from kTransLarge on (with 128: 1.74, 1.31,
+// 2.37); fewer entries need the warps (4096 columns of 8 rows 0.075 against 0.081).
+constexpr int64_t kTransLarge = int64_t(1) << 22;
 template <class P, class I, class W>
 __global__ void __launch_bounds__(256) k_t_scatter(const P *colptr, const I *rowidx, const W *vals, int64_t ncols,
-                                                   int64_t nnz, int64_t m, unsigned long long *cursor, I *out_rows,
-                                                   W *out_vals) {
+                                                   int64_t nnz, int64_t m, int window, unsigned long long *cursor,
+                                                   I *out_rows, W *out_vals) {
+    constexpr int U = 4;
+    const int lane = threadIdx.x & 31;
     const int64_t base = (int64_t)colptr[0];
-    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < nnz; q += (int64_t)gridDim.x * blockDim.x) {
-        int64_t lo = 0, hi = ncols - 1;
+    auto column = [&](int64_t q, int64_t lo, int64_t hi) {   // the last one starting at or before q
         while (lo < hi) {
             const int64_t mid = (lo + hi + 1) >> 1;
             if ((int64_t)__ldg(&colptr[mid]) - base <= q) lo = mid; else hi = mid - 1;
         }
-        const int64_t i = (int64_t)rowidx[q];
-        if (i < 0 || i >= m) continue;
-        const unsigned long long pos = atomicAdd(&cursor[i], 1ull);
-        out_rows[pos] = (I)lo;
-        out_vals[pos] = vals[q];
+        return lo;
+    };
+    const int64_t step = (((int64_t)gridDim.x * blockDim.x) >> 5) * window;
+    for (int64_t w = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * window; w < nnz; w += step) {
+        const int64_t ends = column(lane < 16 ? w : min(w + window, nnz) - 1, 0, ncols - 1);
+        const int64_t c0 = __shfl_sync(0xffffffffu, ends, 0), c1 = __shfl_sync(0xffffffffu, ends, 31);
+        for (int64_t w1 = w; w1 < min(w + window, nnz); w1 += 32 * U) {
+            int64_t i[U], c[U];
+            W v[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int64_t q = w1 + 32 * u + lane;
+                i[u] = q < nnz ? (int64_t)rowidx[q] : -1;
+                if (q < nnz) v[u] = vals[q];
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                c[u] = i[u] >= 0 && i[u] < m ? column(w1 + 32 * u + lane, c0, c1) : -1;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (c[u] < 0) continue;
+                const unsigned long long pos = atomicAdd(&cursor[i[u]], 1ull);
+                out_rows[pos] = (I)c[u];
+                out_vals[pos] = v[u];
+            }
+        }
     }
 }
 
@@ -76,6 +104,8 @@ static spgemm_status transpose_typed(const spgemm_csc *in, spgemm_csc *out, cuda
         (e = cudaMemsetAsync(err.p, 0, sizeof(int), st)) != cudaSuccess)
         return cuda_fail(e, "cudaMemsetAsync");
     const unsigned eb = (unsigned)std::max<int64_t>(1, std::min<int64_t>((nnz + 255) / 256, 1 << 20));
+    const int window = nnz >= kTransLarge ? 256 : 128;
+    const unsigned wb = (unsigned)std::max<int64_t>(1, std::min<int64_t>((nnz + 8 * window - 1) / (8 * window), 1 << 20));
     const unsigned mb = (unsigned)std::max<int64_t>(1, std::min<int64_t>((m + 256) / 256, 1 << 20));
     // entry q of the input is rowidx[q - colptr[0]] (the pointers address
     // the first entry), as everywhere in the library
@@ -86,8 +116,8 @@ static spgemm_status transpose_typed(const spgemm_csc *in, spgemm_csc *out, cuda
     if (out->ptr_type == SPGEMM_I64) k_t_colptr<int64_t><<<mb, 256, 0, st>>>(scan.as<int64_t>(), m + 1, (int64_t *)out->colptr);
     else k_t_colptr<int32_t><<<mb, 256, 0, st>>>(scan.as<int64_t>(), m + 1, (int32_t *)out->colptr);
     if (nnz > 0)
-        k_t_scatter<P, I, W><<<eb, 256, 0, st>>>((const P *)in->colptr, (const I *)in->rowidx, (const W *)in->vals, n,
-                                                 nnz, m, scan.as<unsigned long long>(), (I *)out->rowidx, (W *)out->vals);
+        k_t_scatter<P, I, W><<<wb, 256, 0, st>>>((const P *)in->colptr, (const I *)in->rowidx, (const W *)in->vals, n,
+                                                 nnz, m, window, scan.as<unsigned long long>(), (I *)out->rowidx, (W *)out->vals);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "transpose kernels");
     // the workspace is freed on return: wait for the kernels that use it
     int herr = 0;
