@@ -321,7 +321,14 @@ template <class I, class V> struct Engine : EngineBase {
         // cursors at the start of the pass
         c.next_col = cx.cursor + 32 + t;
         if constexpr (!Src::kParts) {
-            if (!c.hybrid_sort && launch_mid(cx, sa, c, T, thr, 1, count, rows, vals, st)) return;
+            // The largest tables, unsorted: one CTA of 32 warps per SM, which k_mid's windows of a
+            // few dozen B entries do not fill evenly, and no sort to gain on. Numeric tiers, ms, a
+            // warp's walk (k_mid) / a CTA's (k_num_block): uniform 500,000 rows, 4,500 a column fp64
+            // 7.18 / 6.63, int64 6.58 / 5.93, 150,000 with 7,500 2.57 / 2.56, 2.27 / 2.13; R-MAT of
+            // 60,000 rows fp64 1.52 / 1.64 of a step of 12.9. A stage of a k-split keeps k_mid (155 ->
+            // 135 us for one of R-MAT 15).
+            const bool cta_walk = c.hybrid_sort || (T == 16384 && !c.sort && sa.whole);
+            if (!cta_walk && launch_mid(cx, sa, c, T, thr, 1, count, rows, vals, st)) return;
         }
         const int smem = T * (int)(4 + sizeof(V));
         const int per_sm = std::max(1, std::min(2048 / thr, (228 * 1024) / (smem + 34 * 1024)));
@@ -683,6 +690,7 @@ template <class I, class V> struct Engine : EngineBase {
         a.probs = ps.probs.as<PD>();
         a.nprob = 1;
         a.k0 = k0; a.k1 = k1;
+        a.whole = k0 == 0 && k1 == ps.k;
         a.ap_end = ps.ap_end.as<int64_t>();
         a.ap_row = ps.ap_row.as<uint16_t>();
         a.ap_val = ps.ap_val.as<V>();

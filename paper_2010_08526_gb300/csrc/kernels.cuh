@@ -107,6 +107,7 @@ template <class I, class V> struct GemmArgs {
     const uint32_t *apc_row;  // global rows
     const V *apc_val;
     const int32_t *prob_of;   // many problems: the problem of every global column, or null
+    int whole;                // all of the inner dimension, not a stage of it
     int lean_dense;           // heavy items may use 32-bit entry offsets (nnz(A) < 2^31)
     int lean_sym;             // the heavy symbolic may use 32-bit stream positions too
 };
