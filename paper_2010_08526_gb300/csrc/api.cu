@@ -27,46 +27,86 @@ spgemm_status cuda_fail(cudaError_t e, const char *where) {
 
 thread_local AllocFns tl_alloc;
 
+uint64_t context_id() {
+    // driver functions, looked up through the runtime (the library links no libcuda)
+    struct Driver {
+        int (*current)(void **) = nullptr;                  // cuCtxGetCurrent
+        int (*id)(void *, unsigned long long *) = nullptr;  // cuCtxGetId
+        Driver() {
+            auto find = [](const char *name) -> void * {
+                void *p = nullptr;
+                cudaDriverEntryPointQueryResult found;
+                const cudaError_t e = cudaGetDriverEntryPointByVersion(name, &p, 12000, cudaEnableDefault, &found);
+                return e == cudaSuccess && found == cudaDriverEntryPointSuccess ? p : nullptr;
+            };
+            current = reinterpret_cast<int (*)(void **)>(find("cuCtxGetCurrent"));
+            id = reinterpret_cast<int (*)(void *, unsigned long long *)>(find("cuCtxGetId"));
+            cudaGetLastError();
+        }
+    };
+    static const Driver drv;
+    if (!drv.current || !drv.id) return 0;
+    void *ctx = nullptr;
+    if (drv.current(&ctx) != 0) return 0;
+    int dev = 0;
+    if (!ctx && (cudaGetDevice(&dev) != cudaSuccess || cudaSetDevice(dev) != cudaSuccess || drv.current(&ctx) != 0))
+        return 0;   // a thread gets the device's context with its first call
+    unsigned long long id = 0;
+    return ctx && drv.id(ctx, &id) == 0 ? (uint64_t)id : 0;
+}
+
 namespace {
-constexpr int kMaxDevices = 64;
-struct CallBlock { void *p = nullptr; bool taken = false; };
-CallBlock g_call_block[kMaxDevices];
+struct CallBlock { uint64_t ctx = 0; void *p = nullptr; bool taken = false; };
+constexpr int kCallBlocks = 64;   // contexts of a process that get one
+CallBlock g_call_block[kCallBlocks];
 std::mutex g_call_mu;
 
-// Frees the current device's idle block; whether there was one.
+// The current context's entry (a fresh one for a new context), or null. A block
+// whose context is gone went with it; its entry is never found again.
+CallBlock *call_block(bool fresh) {
+    const uint64_t id = context_id();
+    if (id == 0) return nullptr;
+    for (CallBlock &b : g_call_block) {
+        if (b.ctx == id) return &b;
+        if (b.ctx == 0) {
+            if (!fresh) return nullptr;
+            b.ctx = id;
+            return &b;
+        }
+    }
+    return nullptr;
+}
+
+// Frees the current context's idle block; whether there was one.
 bool drop_call_block() {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return false;
     std::lock_guard<std::mutex> lk(g_call_mu);
-    CallBlock &b = g_call_block[dev];
-    if (!b.p || b.taken) return false;
-    cudaFree(b.p);
-    b.p = nullptr;
+    CallBlock *b = call_block(false);
+    if (!b || !b->p || b->taken) return false;
+    cudaFree(b->p);
+    b->p = nullptr;
     return true;
 }
 }  // namespace
 
 CallScratch::CallScratch(DevBuf &arena, cudaStream_t st) : arena_(arena), st_(st) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return;
     std::lock_guard<std::mutex> lk(g_call_mu);
-    CallBlock &b = g_call_block[dev];
-    if (b.taken) return;
-    if (!b.p && cudaMalloc(&b.p, kCallScratch) != cudaSuccess) {
+    CallBlock *b = call_block(true);
+    if (!b || b->taken) return;
+    if (!b->p && cudaMalloc(&b->p, kCallScratch) != cudaSuccess) {
         cudaGetLastError();   // the call allocates what it needs itself
-        b.p = nullptr;
+        b->p = nullptr;
         return;
     }
-    b.taken = true;
-    dev_ = dev;
-    arena.borrow(b.p, kCallScratch);
+    b->taken = true;
+    block_ = b;
+    arena.borrow(b->p, kCallScratch);
 }
 
 CallScratch::~CallScratch() {
-    if (dev_ < 0) return;
+    if (!block_) return;
     cudaStreamSynchronize(st_);   // on every way out of the call
     std::lock_guard<std::mutex> lk(g_call_mu);
-    g_call_block[dev_].taken = false;
+    static_cast<CallBlock *>(block_)->taken = false;
 }
 
 void *alloc_mem(const AllocFns &a, size_t bytes, int kind, cudaError_t &e) {

@@ -105,9 +105,15 @@ template <int KIND> cudaError_t carve(Buf<KIND> &arena, std::initializer_list<Wa
     return cudaSuccess;
 }
 
+// The calling thread's CUDA context, by a number that no other context of the process has
+// or will have; 0 if there is none. Memory and function attributes belong to a
+// context: what is kept of them is kept by this number, since a device gets a new
+// context after cudaDeviceReset, and may have several.
+uint64_t context_id();
+
 // Scratch of the calls without a plan (transpose, prune, merge): a cudaMalloc
 // and its cudaFree cost them 60 to 150 us each. One block of kCallScratch bytes
-// per device is kept between calls; a call borrows it for its own length, and a
+// per context is kept between calls; a call borrows it for its own length, and a
 // call that needs more, or finds it taken by another thread, allocates as
 // before. A call waits for its stream before it gives the block back, so the
 // next one may use it on any stream. A failing cudaMalloc of the library gives
@@ -123,7 +129,7 @@ class CallScratch {
   private:
     DevBuf &arena_;
     cudaStream_t st_;
-    int dev_ = -1;                                 // >= 0: this call has the block
+    void *block_ = nullptr;                        // set: this call has the block
 };
 
 int64_t scan_partials_len(int64_t n);
