@@ -37,6 +37,9 @@
  *   - A plan is not thread-safe; use one plan per host thread.
  *   - There is no CPU fallback: without a usable sm_103a device every compute
  *     call returns SPGEMM_ERR_CUDA.
+ *   - spgemm_transpose, spgemm_prune and spgemm_merge keep one device block of 32 MiB
+ *     per CUDA context between calls. It counts toward no budget; the library frees it
+ *     when one of its allocations fails or an allocator refuses device memory.
  */
 #ifndef SPGEMM_GB300_H
 #define SPGEMM_GB300_H
@@ -151,7 +154,9 @@ typedef struct {
  * caching allocator) hands it to the library through these callbacks.
  *   alloc(ctx, bytes, kind) returns `bytes` of memory of `kind`, aligned to
  *     256 bytes, or NULL when it cannot (the call then fails with
- *     SPGEMM_ERR_OOM and frees what it had allocated for the failed step);
+ *     SPGEMM_ERR_OOM and frees what it had allocated for the failed step; where the
+ *     device is short of memory and the library holds scratch between calls, it
+ *     first frees that and asks once more);
  *   free(ctx, p, bytes, kind) returns a block that alloc gave. The library
  *     calls it only after the device has finished every use of the block
  *     (it synchronises the device first), when a buffer grows or when the

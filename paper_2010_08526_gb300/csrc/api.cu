@@ -113,6 +113,14 @@ void *alloc_mem(const AllocFns &a, size_t bytes, int kind, cudaError_t &e) {
     void *p = nullptr;
     if (a.alloc) {
         p = a.alloc(a.ctx, bytes, kind);
+        if (!p && kind == SPGEMM_MEM_DEVICE) {
+            // the scratch kept between calls goes back to the device; asked again only
+            // where that can have made the difference
+            size_t free_b = 0, total_b = 0;
+            const bool scarce = cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && free_b < bytes + kCallScratch;
+            if (drop_call_block() && scarce) p = a.alloc(a.ctx, bytes, kind);
+            cudaGetLastError();
+        }
         if (!p) { e = cudaErrorMemoryAllocation; return nullptr; }
         if (reinterpret_cast<uintptr_t>(p) % 256) {   // the callbacks promise 256-byte alignment
             a.free(a.ctx, p, bytes, kind);

@@ -117,7 +117,8 @@ uint64_t context_id();
 // call that needs more, or finds it taken by another thread, allocates as
 // before. A call waits for its stream before it gives the block back, so the
 // next one may use it on any stream. A failing cudaMalloc of the library gives
-// the block back to the device and tries again.
+// the block back to the device and tries again; so does an allocator's refusal of device
+// memory, and it is asked again if the device was short of memory.
 constexpr size_t kCallScratch = size_t(32) << 20;
 class CallScratch {
   public:
