@@ -96,7 +96,7 @@ inline TierCommon common_of(const Ctx &c) {
 
 // Allow a kernel the largest dynamic shared memory the device permits next to
 // its static shared memory (opt-in maximum minus static size).
-template <class K> static void set_smem(K kern, int) {
+template <class K> static void set_smem(K kern) {
     int dev = 0, optin = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
@@ -126,92 +126,91 @@ template <class I, class V> struct Engine : EngineBase {
     using GA = GemmArgs<I, V>;
     using PA = PartsArgs<I, V>;
 
-    // ---- one-time attributes ----------------------------------------------
+    // ---- function attributes ------------------------------------------------
+    // the shared memory limits of the kernels, which belong to a context
     static void attrs() {
-        static bool done = false;
-        if (done) return;
-        const int sv = (int)(sizeof(V) + 4);
-        const int mx = 220 * 1024;
-        set_smem(k_sym_block<SrcGemm<I, V>, 512>, mx);
-        set_smem(k_sym_block<SrcGemm<I, V>, 1024>, mx);
-        set_smem(k_sym_block<SrcGemm<I, V>, 2048>, mx);
-        set_smem(k_sym_block<SrcGemm<I, V>, 4096>, mx);
-        set_smem(k_sym_block<SrcGemm<I, V>, 8192>, mx);
-        set_smem(k_sym_block<SrcGemm<I, V>, 16384>, mx);
-        set_smem(k_sym_block<SrcParts<I, V>, 512>, mx);
-        set_smem(k_sym_block<SrcParts<I, V>, 1024>, mx);
-        set_smem(k_sym_block<SrcParts<I, V>, 2048>, mx);
-        set_smem(k_sym_block<SrcParts<I, V>, 4096>, mx);
-        set_smem(k_sym_block<SrcParts<I, V>, 8192>, mx);
-        set_smem(k_sym_block<SrcParts<I, V>, 16384>, mx);
-        set_smem(k_num_block<SrcGemm<I, V>, 512>, mx);
-        set_smem(k_num_block<SrcGemm<I, V>, 1024>, mx);
-        set_smem(k_num_block<SrcGemm<I, V>, 2048>, mx);
-        set_smem(k_num_block<SrcGemm<I, V>, 4096>, mx);
-        set_smem(k_num_block<SrcGemm<I, V>, 8192>, mx);
-        set_smem(k_num_block<SrcGemm<I, V>, 16384>, mx);
-        set_smem(k_num_block<SrcParts<I, V>, 512>, mx);
-        set_smem(k_num_block<SrcParts<I, V>, 1024>, mx);
-        set_smem(k_num_block<SrcParts<I, V>, 2048>, mx);
-        set_smem(k_num_block<SrcParts<I, V>, 4096>, mx);
-        set_smem(k_num_block<SrcParts<I, V>, 8192>, mx);
-        set_smem(k_num_block<SrcParts<I, V>, 16384>, mx);
-        set_smem(k_bwd_block<I, V, 512>, mx);
-        set_smem(k_bwd_block<I, V, 1024>, mx);
-        set_smem(k_bwd_block<I, V, 2048>, mx);
-        set_smem(k_bwd_block<I, V, 4096>, mx);
-        set_smem(k_bwd_block<I, V, 8192>, mx);
-        set_smem(k_bwd_block<I, V, 16384>, mx);
-        set_smem(k_sym_bitmap<SrcGemm<I, V>>, mx);
-        set_smem(k_sym_heavy32<I, V, 1024, 1>, mx);
-        set_smem(k_sym_heavy32<I, V, 512, 3>, mx);
-        set_smem(k_sym_bitmap<SrcParts<I, V>>, mx);
-        set_smem(k_num_dense<SrcPanel<I, V>>, mx);
-        set_smem(k_num_dense<SrcPartsPanel<I, V>>, mx);
-        set_smem(k_bwd_dense<I, V>, mx);
-        set_smem(k_mid<I, V, 4096, 0>, mx);
-        set_smem(k_mid<I, V, 4096, 1>, mx);
-        set_smem(k_mid<I, V, 8192, 0>, mx);
-        set_smem(k_mid<I, V, 8192, 1>, mx);
-        set_smem(k_mid<I, V, 16384, 0>, mx);
-        set_smem(k_mid<I, V, 16384, 1>, mx);
-        set_smem(k_light<I, V, 1024, 0>, mx);
-        set_smem(k_light<I, V, 512, 1>, mx);
-        set_smem(k_light<I, V, 1024, 1>, mx);
-        set_smem(k_sym_warp<SrcGemm<I, V>, 1024>, mx);
-        set_smem(k_sym_warp<SrcParts<I, V>, 1024>, mx);
-        set_smem(k_num_warp<SrcGemm<I, V>, 512>, mx);
-        set_smem(k_num_warp<SrcGemm<I, V>, 1024>, mx);
-        set_smem(k_num_warp<SrcParts<I, V>, 512>, mx);
-        set_smem(k_num_warp<SrcParts<I, V>, 1024>, mx);
-        set_smem(k_bwd_light<I, V, 512>, mx);
-        set_smem(k_bwd_light<I, V, 1024>, mx);
-        set_smem(k_bwd_warp<I, V, 512>, mx);
-        set_smem(k_bwd_warp<I, V, 1024>, mx);
-        set_smem(k_num_heavy<SrcPanelRange<I, V>, SrcColRange<I, V>, 2>, mx);
-        set_smem(k_num_heavy<SrcPartsRange<I, V>, SrcPartsRange<I, V>, 2>, mx);
-        set_smem(k_num_heavy<SrcPanelRange<I, V>, SrcColRange<I, V>, 3>, mx);
-        set_smem(k_num_heavy<SrcPartsRange<I, V>, SrcPartsRange<I, V>, 3>, mx);
-        set_smem(k_multi_pass<SrcGemm<I, V>, 512, 0>, mx);
-        set_smem(k_multi_pass<SrcGemm<I, V>, 512, 1>, mx);
-        set_smem(k_multi_pass<SrcGemm<I, V>, 256, 0>, mx);
-        set_smem(k_multi_pass<SrcGemm<I, V>, 256, 1>, mx);
-        set_smem(k_multi_pass<SrcGemm<I, V>, 128, 0>, mx);
-        set_smem(k_multi_pass<SrcGemm<I, V>, 128, 1>, mx);
-        set_smem(k_num_heavy32<I, V, 1, false>, mx);
-        set_smem(k_num_heavy32<I, V, 1, true>, mx);
-        set_smem(k_num_heavy32<I, V, 2, false>, mx);
-        set_smem(k_num_heavy32<I, V, 2, true>, mx);
-        set_smem(k_num_heavy32<I, V, 3, false>, mx);
-        set_smem(k_num_heavy32<I, V, 3, true>, mx);
-        set_smem(k_sort_cols<I, V, 512, false>, mx);
-        set_smem(k_sort_cols<I, V, 2048, true>, mx);
-        set_smem(k_sort_cols<I, V, 16384, true>, mx);
-        set_smem(k_prune_select<I, V, I>, mx);
-        set_smem(k_sort_items<I, V, 8192>, mx);
-        set_smem(k_sort_items<I, V, 4096>, mx);
-        (void)sv;
-        done = true;
+        static ContextOnce once;
+        once.run([] { set_limits(); });
+    }
+    static void set_limits() {
+        set_smem(k_sym_block<SrcGemm<I, V>, 512>);
+        set_smem(k_sym_block<SrcGemm<I, V>, 1024>);
+        set_smem(k_sym_block<SrcGemm<I, V>, 2048>);
+        set_smem(k_sym_block<SrcGemm<I, V>, 4096>);
+        set_smem(k_sym_block<SrcGemm<I, V>, 8192>);
+        set_smem(k_sym_block<SrcGemm<I, V>, 16384>);
+        set_smem(k_sym_block<SrcParts<I, V>, 512>);
+        set_smem(k_sym_block<SrcParts<I, V>, 1024>);
+        set_smem(k_sym_block<SrcParts<I, V>, 2048>);
+        set_smem(k_sym_block<SrcParts<I, V>, 4096>);
+        set_smem(k_sym_block<SrcParts<I, V>, 8192>);
+        set_smem(k_sym_block<SrcParts<I, V>, 16384>);
+        set_smem(k_num_block<SrcGemm<I, V>, 512>);
+        set_smem(k_num_block<SrcGemm<I, V>, 1024>);
+        set_smem(k_num_block<SrcGemm<I, V>, 2048>);
+        set_smem(k_num_block<SrcGemm<I, V>, 4096>);
+        set_smem(k_num_block<SrcGemm<I, V>, 8192>);
+        set_smem(k_num_block<SrcGemm<I, V>, 16384>);
+        set_smem(k_num_block<SrcParts<I, V>, 512>);
+        set_smem(k_num_block<SrcParts<I, V>, 1024>);
+        set_smem(k_num_block<SrcParts<I, V>, 2048>);
+        set_smem(k_num_block<SrcParts<I, V>, 4096>);
+        set_smem(k_num_block<SrcParts<I, V>, 8192>);
+        set_smem(k_num_block<SrcParts<I, V>, 16384>);
+        set_smem(k_bwd_block<I, V, 512>);
+        set_smem(k_bwd_block<I, V, 1024>);
+        set_smem(k_bwd_block<I, V, 2048>);
+        set_smem(k_bwd_block<I, V, 4096>);
+        set_smem(k_bwd_block<I, V, 8192>);
+        set_smem(k_bwd_block<I, V, 16384>);
+        set_smem(k_sym_bitmap<SrcGemm<I, V>>);
+        set_smem(k_sym_heavy32<I, V, 1024, 1>);
+        set_smem(k_sym_heavy32<I, V, 512, 3>);
+        set_smem(k_sym_bitmap<SrcParts<I, V>>);
+        set_smem(k_num_dense<SrcPanel<I, V>>);
+        set_smem(k_num_dense<SrcPartsPanel<I, V>>);
+        set_smem(k_bwd_dense<I, V>);
+        set_smem(k_mid<I, V, 4096, 0>);
+        set_smem(k_mid<I, V, 4096, 1>);
+        set_smem(k_mid<I, V, 8192, 0>);
+        set_smem(k_mid<I, V, 8192, 1>);
+        set_smem(k_mid<I, V, 16384, 0>);
+        set_smem(k_mid<I, V, 16384, 1>);
+        set_smem(k_light<I, V, 1024, 0>);
+        set_smem(k_light<I, V, 512, 1>);
+        set_smem(k_light<I, V, 1024, 1>);
+        set_smem(k_sym_warp<SrcGemm<I, V>, 1024>);
+        set_smem(k_sym_warp<SrcParts<I, V>, 1024>);
+        set_smem(k_num_warp<SrcGemm<I, V>, 512>);
+        set_smem(k_num_warp<SrcGemm<I, V>, 1024>);
+        set_smem(k_num_warp<SrcParts<I, V>, 512>);
+        set_smem(k_num_warp<SrcParts<I, V>, 1024>);
+        set_smem(k_bwd_light<I, V, 512>);
+        set_smem(k_bwd_light<I, V, 1024>);
+        set_smem(k_bwd_warp<I, V, 512>);
+        set_smem(k_bwd_warp<I, V, 1024>);
+        set_smem(k_num_heavy<SrcPanelRange<I, V>, SrcColRange<I, V>, 2>);
+        set_smem(k_num_heavy<SrcPartsRange<I, V>, SrcPartsRange<I, V>, 2>);
+        set_smem(k_num_heavy<SrcPanelRange<I, V>, SrcColRange<I, V>, 3>);
+        set_smem(k_num_heavy<SrcPartsRange<I, V>, SrcPartsRange<I, V>, 3>);
+        set_smem(k_multi_pass<SrcGemm<I, V>, 512, 0>);
+        set_smem(k_multi_pass<SrcGemm<I, V>, 512, 1>);
+        set_smem(k_multi_pass<SrcGemm<I, V>, 256, 0>);
+        set_smem(k_multi_pass<SrcGemm<I, V>, 256, 1>);
+        set_smem(k_multi_pass<SrcGemm<I, V>, 128, 0>);
+        set_smem(k_multi_pass<SrcGemm<I, V>, 128, 1>);
+        set_smem(k_num_heavy32<I, V, 1, false>);
+        set_smem(k_num_heavy32<I, V, 1, true>);
+        set_smem(k_num_heavy32<I, V, 2, false>);
+        set_smem(k_num_heavy32<I, V, 2, true>);
+        set_smem(k_num_heavy32<I, V, 3, false>);
+        set_smem(k_num_heavy32<I, V, 3, true>);
+        set_smem(k_sort_cols<I, V, 512, false>);
+        set_smem(k_sort_cols<I, V, 2048, true>);
+        set_smem(k_sort_cols<I, V, 16384, true>);
+        set_smem(k_prune_select<I, V, I>);
+        set_smem(k_sort_items<I, V, 8192>);
+        set_smem(k_sort_items<I, V, 4096>);
     }
 
     // ---- tier launches -----------------------------------------------------

@@ -1,9 +1,11 @@
 // Plan state shared by the C ABI and the typed engines.
 #pragma once
 
+#include <algorithm>
 #include <cstdint>
 #include <array>
 #include <initializer_list>
+#include <mutex>
 #include <string>
 #include <vector>
 #include <cuda_runtime.h>
@@ -110,6 +112,23 @@ template <int KIND> cudaError_t carve(Buf<KIND> &arena, std::initializer_list<Wa
 // context: what is kept of them is kept by this number, since a device gets a new
 // context after cudaDeviceReset, and may have several.
 uint64_t context_id();
+
+// Runs a function once per context (the other threads wait for it); where there is
+// no context yet, every time.
+class ContextOnce {
+  public:
+    template <class F> void run(F &&f) {
+        const uint64_t id = context_id();
+        std::lock_guard<std::mutex> lk(mu_);
+        if (id && std::find(done_.begin(), done_.end(), id) != done_.end()) return;
+        f();
+        if (id) done_.push_back(id);
+    }
+
+  private:
+    std::mutex mu_;
+    std::vector<uint64_t> done_;
+};
 
 // Scratch of the calls without a plan (transpose, prune, merge): a cudaMalloc
 // and its cudaFree cost them 60 to 150 us each. One block of kCallScratch bytes

@@ -78,3 +78,96 @@ for _ in range(3):
     transposed()
     ok(rt.cudaDeviceReset())
 """)
+
+
+PRODUCT = """
+def product():
+    # six of A's columns a column: about 4,100 rows, tables of 128 KB
+    A = csc(M, N, ptr, rows.ravel(), vals.ravel())
+    n = 40
+    pick = np.concatenate([rng.choice(N, 6, replace=False) for _ in range(n)]).astype(np.int32)
+    B = csc(N, n, (6 * np.arange(n + 1)).astype(np.int32), pick, np.ones(6 * n, np.float32))
+    o = C.SpgemmOpts()
+    o.budget_bytes = 1 << 33
+    o.kstages = 1
+    o.sort_output = 1
+    h = ctypes.c_void_p()
+    C.check(lib.spgemm_plan_create(ctypes.byref(A), ctypes.byref(B), ctypes.byref(o), 1, None, ctypes.byref(h)))
+    C.check(lib.spgemm_symbolic(h, None))
+    info = C.SpgemmPlanInfo()
+    C.check(lib.spgemm_plan_query(h, ctypes.byref(info)))
+    out = csc(M, n, np.zeros(n + 1, np.int64), np.zeros(info.nnz_c, np.int32), np.zeros(info.nnz_c, np.float32), C.I64)
+    C.check(lib.spgemm_numeric(h, 0, ctypes.byref(out), None))
+    C.check(lib.spgemm_plan_check(h, None))
+    C.check(lib.spgemm_plan_destroy(h))
+    cp = host(out.colptr, n + 1, np.int64)
+    r, v = host(out.rowidx, info.nnz_c, np.int32), host(out.vals, info.nnz_c, np.float32)
+    for j in range(n):
+        dense = np.zeros(M, np.float32)
+        for k in pick[6 * j:6 * j + 6]:
+            dense[rows[k]] += vals[k]
+        where = np.flatnonzero(dense)
+        assert np.array_equal(r[cp[j]:cp[j + 1]], where) and np.array_equal(v[cp[j]:cp[j + 1]], dense[where])
+    # and the prune, whose selection stages 100 KB
+    for fill in (False, True):
+        if not fill:
+            res = C.SpgemmCsc(M, n, 0, dev(np.zeros(n + 1, np.int64)), 0, 0, C.I64, C.I32, C.F32)
+        else:
+            res.rowidx, res.vals = dev(np.zeros(res.nnz, np.int32)), dev(np.zeros(res.nnz, np.float32))
+        C.check(lib.spgemm_prune(ctypes.byref(out), ctypes.c_double(0.0), 100, ctypes.byref(res), None))
+    pv = host(res.vals, res.nnz, np.float32)
+    for j in range(n):
+        assert np.array_equal(np.sort(pv[100 * j:100 * j + 100]), np.sort(v[cp[j]:cp[j + 1]])[-100:])
+"""
+
+
+def test_product_and_prune_after_a_reset():
+    run(PRODUCT + """
+for _ in range(3):
+    product()
+    ok(rt.cudaDeviceReset())
+""")
+
+
+def test_first_calls_of_several_threads():
+    """Every thread waits until the kernels' limits are set."""
+    run(PRODUCT + """
+import threading
+failed = []
+gate = threading.Barrier(6)
+
+def go():
+    gate.wait()
+    try:
+        product()
+    except BaseException as e:
+        failed.append(e)
+
+threads = [threading.Thread(target=go) for _ in range(6)]
+[t.start() for t in threads]
+[t.join() for t in threads]
+assert not failed, failed
+""")
+
+
+def test_a_second_context_of_the_device():
+    """A context of the caller's own beside the runtime's, and back."""
+    run(PRODUCT + """
+product()
+transposed()
+drv = ctypes.CDLL("libcuda.so.1")
+mine, first = ctypes.c_void_p(), ctypes.c_void_p()
+ok(drv.cuCtxGetCurrent(ctypes.byref(first)))
+ok(drv.cuCtxCreate_v4(ctypes.byref(mine), None, 0, 0))
+product()
+transposed()
+ok(rt.cudaDeviceSynchronize())
+ok(drv.cuCtxSetCurrent(first))
+product()
+transposed()
+ok(rt.cudaDeviceSynchronize())
+ok(drv.cuCtxDestroy_v2(mine))
+ok(drv.cuCtxSetCurrent(first))
+product()
+transposed()
+""")
