@@ -9,8 +9,8 @@
 // reads land in a static host array, one per device. Each GPU that loads this
 // library keeps the array until the process exits.
 //
-// The array's address is looked up once per device (cudaGetSymbolAddress, with
-// that device current) on that device's first call. Every call synchronises its
+// The array's address is looked up (cudaGetSymbolAddress) on a device's first call and
+// again when its context is another one than the last call's. Every call synchronises its
 // stream once, to read the merged size. All calls on one device share that device's array and
 // host staging, and the array keeps the last call's contents; the merge clears
 // what it reads before writing. Calls on one device that overlap (other
@@ -31,6 +31,7 @@ __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
 
 constexpr int kMaxDevices = 64;
 void *g_scratch_addr[kMaxDevices] = {};
+uint64_t g_scratch_ctx[kMaxDevices] = {};
 int g_nsm[kMaxDevices] = {};
 std::mutex g_setup_mu;
 int32_t g_host_stage[kMaxDevices][1024];   // host staging of small device-to-host reads
@@ -46,9 +47,11 @@ extern "C" spgemm_status spgemm_merge_noalloc(const spgemm_csc *parts, int npart
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
     if (dev < 0 || dev >= kMaxDevices) { set_error("device ordinal out of range"); return SPGEMM_ERR_INVALID; }
+    void *scratch = nullptr;
     {
         std::lock_guard<std::mutex> lk(g_setup_mu);
-        if (!g_scratch_addr[dev]) {
+        const uint64_t ctx = context_id();
+        if (!g_scratch_addr[dev] || !ctx || g_scratch_ctx[dev] != ctx) {
             // the host-side name of the array is not a device address: ask the
             // runtime for this device's copy
             void *p = nullptr;
@@ -59,9 +62,11 @@ extern "C" spgemm_status spgemm_merge_noalloc(const spgemm_csc *parts, int npart
             if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceGetAttribute");
             g_nsm[dev] = nsm;
             g_scratch_addr[dev] = p;
+            g_scratch_ctx[dev] = ctx;
         }
+        scratch = g_scratch_addr[dev];
     }
     return merge_noalloc_dispatch(parts, nparts, out, stream,
-                                  static_cast<unsigned char *>(g_scratch_addr[dev]),
+                                  static_cast<unsigned char *>(scratch),
                                   kNoAllocScratchBytes, g_host_stage[dev], g_nsm[dev]);
 }

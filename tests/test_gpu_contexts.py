@@ -171,3 +171,41 @@ ok(drv.cuCtxSetCurrent(first))
 product()
 transposed()
 """)
+
+
+MERGE = """
+def merged():
+    n = 300
+    parts = (C.SpgemmCsc * 2)(*[csc(M, n, ptr[:n + 1], rows[i * n:(i + 1) * n].ravel(), vals[i * n:(i + 1) * n].ravel())
+                                for i in range(2)])
+    out = C.SpgemmCsc(M, n, 0, dev(np.zeros(n + 1, np.int64)), 0, 0, C.I64, C.I32, C.F32)
+    C.check(lib.spgemm_merge_noalloc(parts, 2, ctypes.byref(out), None))
+    out.rowidx, out.vals = dev(np.zeros(out.nnz, np.int32)), dev(np.zeros(out.nnz, np.float32))
+    C.check(lib.spgemm_merge_noalloc(parts, 2, ctypes.byref(out), None))
+    cp = host(out.colptr, n + 1, np.int64)
+    r, v = host(out.rowidx, out.nnz, np.int32), host(out.vals, out.nnz, np.float32)
+    for j in range(n):
+        dense = np.zeros(M, np.float32)
+        for i in range(2):
+            dense[rows[i * n + j]] += vals[i * n + j]
+        got = np.zeros(M, np.float32)
+        got[r[cp[j]:cp[j + 1]]] = v[cp[j]:cp[j + 1]]
+        assert np.array_equal(got, dense) and cp[j + 1] - cp[j] == np.count_nonzero(dense)
+"""
+
+
+def test_merge_without_allocation_in_other_contexts():
+    run(MERGE + """
+merged()
+drv = ctypes.CDLL("libcuda.so.1")
+mine, first = ctypes.c_void_p(), ctypes.c_void_p()
+ok(drv.cuCtxGetCurrent(ctypes.byref(first)))
+ok(drv.cuCtxCreate_v4(ctypes.byref(mine), None, 0, 0))
+merged()
+ok(drv.cuCtxSetCurrent(first))
+merged()
+ok(drv.cuCtxDestroy_v2(mine))
+ok(drv.cuCtxSetCurrent(first))
+ok(rt.cudaDeviceReset())
+merged()
+""")
