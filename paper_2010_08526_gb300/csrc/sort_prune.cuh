@@ -205,6 +205,8 @@ constexpr int kPruneThreads = 512;
 // skipped, and the digits spread over the bins instead of crowding into a few.
 // Keys are staged in shared memory when the column fits (cap), so the
 // passes read the values from memory once.
+// Places in a column are unsigned 32-bit numbers: a column has fewer than 2^31 entries, and
+// the passes step past its end.
 // Equal keys at the cut: the earlier stored ones are kept, or (tie_by_row != 0)
 // the smaller rows, found by a second select over the ties' rows.
 // Measured (protein stand-in, 20,011 columns in 4 batches, top 100): counting,
@@ -222,7 +224,8 @@ __global__ void __launch_bounds__(kPruneThreads, 2) k_prune_select(const int64_t
     K *sk = reinterpret_cast<K *>(smem);
     __shared__ uint32_t hist[4][256];
     __shared__ K s_min[NW], s_max[NW];
-    __shared__ int s_digit, s_k, s_in;
+    __shared__ int s_digit;
+    __shared__ uint32_t s_k, s_in;
     __shared__ int s_hi[NW], s_tie[NW];
     __shared__ long long s_item;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -233,7 +236,7 @@ __global__ void __launch_bounds__(kPruneThreads, 2) k_prune_select(const int64_t
     // the digit (highest bin for keys, lowest for rows) at which the count
     // from the top (bottom) reaches k: s_digit, s_k = what remains of k in it,
     // s_in = entries in it. All threads call it.
-    auto pick = [&](int k, bool from_top) {
+    auto pick = [&](uint32_t k, bool from_top) {
         __syncthreads();
         if (warp == 0) {
             uint32_t c8[8], mine = 0;
@@ -243,15 +246,15 @@ __global__ void __launch_bounds__(kPruneThreads, 2) k_prune_select(const int64_t
                 c8[i] = hist[0][bin] + hist[1][bin] + hist[2][bin] + hist[3][bin];
                 mine += c8[i];
             }
-            int acc = (int)(warp_incl_scan(mine) - mine);
+            uint32_t acc = warp_incl_scan(mine) - mine;
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
-                if (acc < k && acc + (int)c8[i] >= k) {   // one lane and bin
+                if (acc < k && acc + c8[i] >= k) {   // one lane and bin
                     s_digit = from_top ? 255 - (lane * 8 + i) : lane * 8 + i;
                     s_k = k - acc;
-                    s_in = (int)c8[i];
+                    s_in = c8[i];
                 }
-                acc += (int)c8[i];
+                acc += c8[i];
             }
         }
         __syncthreads();
@@ -269,12 +272,12 @@ __global__ void __launch_bounds__(kPruneThreads, 2) k_prune_select(const int64_t
         if (s >= ns) break;
         const int64_t j = sel_list[s];
         const int64_t a = colptr[j] - colptr[0];
-        const int n = (int)(colptr[j + 1] - colptr[j]);
-        const bool staged = n <= cap;
-        auto key_at = [&](int i) -> K { return staged ? sk[i] : prune_key<V, K>(vals[a + i], thr); };
+        const uint32_t n = (uint32_t)(colptr[j + 1] - colptr[j]);
+        const bool staged = n <= (uint32_t)cap;
+        auto key_at = [&](uint32_t i) -> K { return staged ? sk[i] : prune_key<V, K>(vals[a + i], thr); };
         // every key of the column, four loads in flight per thread
         auto each = [&](auto &&f) {
-            for (int i0 = threadIdx.x; i0 < n; i0 += 4 * kPruneThreads) {
+            for (uint32_t i0 = threadIdx.x; i0 < n; i0 += 4 * kPruneThreads) {
                 K x[4];
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
@@ -286,14 +289,14 @@ __global__ void __launch_bounds__(kPruneThreads, 2) k_prune_select(const int64_t
         };
         // keys and their span
         K lo = ~K(0), hi = 0;
-        for (int i0 = threadIdx.x; i0 < n; i0 += 4 * kPruneThreads) {
+        for (uint32_t i0 = threadIdx.x; i0 < n; i0 += 4 * kPruneThreads) {
             V v[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u)
                 if (i0 + u * kPruneThreads < n) v[u] = vals[a + i0 + u * kPruneThreads];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                const int i = i0 + u * kPruneThreads;
+                const uint32_t i = i0 + u * kPruneThreads;
                 if (i >= n) break;
                 const K k = prune_key<V, K>(v[u], thr);
                 if (staged) sk[i] = k;
@@ -312,13 +315,13 @@ __global__ void __launch_bounds__(kPruneThreads, 2) k_prune_select(const int64_t
         // radix select on key - lo; rb: bits below the ones decided
         int rb = hi == lo ? 0 : 64 - __clzll((long long)(uint64_t)(hi - lo));
         K prefix = 0;
-        int k = (int)topk;
+        uint32_t k = (uint32_t)topk;
         bool whole = false;   // every entry of the selected bin is kept
         while (rb > 0) {
             const int w = min(8, rb), sh = rb - w;
             clear_hist();
             const bool first = rb == (int)sizeof(K) * 8;   // a shift by the whole width is undefined
-            each([&](int, K key) {
+            each([&](uint32_t, K key) {
                 const K d = key - lo;
                 if (!first && (K)(d >> rb) != prefix) return;
                 atomicAdd(&hist[warp & 3][(uint32_t)(d >> sh) & ((1u << w) - 1u)], 1u);
@@ -334,11 +337,10 @@ __global__ void __launch_bounds__(kPruneThreads, 2) k_prune_select(const int64_t
         uint32_t rmax = 0xffffffffu;
         if (!whole && tie_by_row) {
             // the k-th smallest row among the ties (rows are distinct)
-            uint32_t rpre = 0;
-            int rk = k;
+            uint32_t rpre = 0, rk = k;
             for (int sh = 24; sh >= 0; sh -= 8) {
                 clear_hist();
-                each([&](int i, K key) {
+                each([&](uint32_t i, K key) {
                     if ((K)((key - lo) >> rb) != prefix) return;
                     const uint32_t r = (uint32_t)rows[a + i];
                     if (sh < 24 && (r >> (sh + 8)) != rpre) return;
@@ -352,15 +354,15 @@ __global__ void __launch_bounds__(kPruneThreads, 2) k_prune_select(const int64_t
         }
         // stable compaction: a warp takes 128 consecutive entries of a step
         const int64_t o = out_colptr[j] - out_colptr[0];
-        int done_hi = 0, done_tie = 0;
-        for (int c0 = 0; c0 < n; c0 += 4 * kPruneThreads) {
-            const int i0 = c0 + warp * 128 + lane;
+        uint32_t done_hi = 0, done_tie = 0;
+        for (uint32_t c0 = 0; c0 < n; c0 += 4 * kPruneThreads) {
+            const uint32_t i0 = c0 + warp * 128 + lane;
             bool up[4], tie[4];
             int nh = 0, nt = 0;
             unsigned bh[4], bt[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                const int i = i0 + 32 * u;
+                const uint32_t i = i0 + 32 * u;
                 up[u] = tie[u] = false;
                 if (i < n) {
                     const K key = key_at(i);
@@ -383,8 +385,8 @@ __global__ void __launch_bounds__(kPruneThreads, 2) k_prune_select(const int64_t
             __syncthreads();
             const int vh = lane < NW ? s_hi[lane] : 0, vt = lane < NW ? s_tie[lane] : 0;
             const int ih = warp_incl_scan(vh), itl = warp_incl_scan(vt);
-            int h0 = done_hi + __shfl_sync(SPG_FULL, ih - vh, warp);
-            int t0 = done_tie + __shfl_sync(SPG_FULL, itl - vt, warp);
+            uint32_t h0 = done_hi + __shfl_sync(SPG_FULL, ih - vh, warp);
+            uint32_t t0 = done_tie + __shfl_sync(SPG_FULL, itl - vt, warp);
             done_hi += __shfl_sync(SPG_FULL, ih, 31);
             done_tie += __shfl_sync(SPG_FULL, itl, 31);
             // the entries of all four windows are read before any is written
@@ -393,7 +395,7 @@ __global__ void __launch_bounds__(kPruneThreads, 2) k_prune_select(const int64_t
             int64_t d[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                const int tb = t0 + __popc(bt[u] & below);   // ties before this entry
+                const uint32_t tb = t0 + __popc(bt[u] & below);   // ties before this entry
                 const int64_t q = a + i0 + 32 * u;
                 d[u] = -1;
                 if (up[u] || (tie[u] && tb < k)) {
