@@ -121,7 +121,8 @@ typedef struct {
  *                  C fit a smaller power of two).
  *   short_seg      A-column segments up to this length are walked by one thread;
  *                  longer ones by a whole warp (1..64), in the kernels of merges,
- *                  of the backward and of products with nnz(A) >= 2^31.
+ *                  of the backward and of products with nnz(A) or an
+ *                  inner dimension of 2^31 - 8192 or more.
  *   huge_seg       segments longer than this are walked by the whole CTA.
  *   block_tier_threads  threads per CTA of the hash tiers (128..1024).
  *   hybrid_sort    1: a column of the CTA hash tiers whose products fit its

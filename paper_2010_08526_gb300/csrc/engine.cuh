@@ -218,7 +218,7 @@ template <class I, class V> struct Engine : EngineBase {
     // keep block_walk). count < 0: population unknown.
     static bool launch_mid(const Ctx &cx, const GA &sa, const TierCommon &c, int T, int thr, int mode, int count,
                            I *rows, V *vals, cudaStream_t st) {
-        if (!sa.lean_dense) return false;
+        if (!sa.lean_walk) return false;
         using Kernel = void (*)(GA, TierCommon, I *, V *);
         Kernel k = nullptr;
         switch (T) {
@@ -249,7 +249,7 @@ template <class I, class V> struct Engine : EngineBase {
             const int want = count < 0 ? cx.nsm * per_sm : (count + 7) / 8;
             const int blocks = std::max(1, std::min(want, cx.nsm * per_sm));
             if constexpr (!Src::kParts) {
-                if (sa.lean_dense) {
+                if (sa.lean_walk) {
                     switch (T) {
                         case 64: k_light<I, V, 64, 0><<<blocks, 256, smem, st>>>(sa, c, nullptr, nullptr); break;
                         case 256: k_light<I, V, 256, 0><<<blocks, 256, smem, st>>>(sa, c, nullptr, nullptr); break;
@@ -297,7 +297,7 @@ template <class I, class V> struct Engine : EngineBase {
             const int want = count < 0 ? cx.nsm * per_sm : (count + 7) / 8;
             const int blocks = std::max(1, std::min(want, cx.nsm * per_sm));
             if constexpr (!Src::kParts) {
-                if (sa.lean_dense) {
+                if (sa.lean_walk) {
                     switch (T) {
                         case 64: k_light<I, V, 64, 1><<<blocks, 256, smem, st>>>(sa, c, rows, vals); break;
                         case 256: k_light<I, V, 256, 1><<<blocks, 256, smem, st>>>(sa, c, rows, vals); break;
@@ -365,7 +365,7 @@ template <class I, class V> struct Engine : EngineBase {
     }
 
     // Whether the products of heavy columns run in k_num_heavy32: every entry
-    // index < nnz(A) < 2^31, and the largest hash table of an item lies inside
+    // index < nnz(A) < 2^31 - 8192, and the largest hash table of an item lies inside
     // the accumulator.
     static bool heavy32(const Ctx &cx, const GA &ga) {
         return ga.lean_dense && 2 * range_cap(cx) * (int)(sizeof(V) + 4) <= (1 << cx.tun.log2R) * (int)sizeof(V);
@@ -697,6 +697,7 @@ template <class I, class V> struct Engine : EngineBase {
         a.apc_row = ps.apc_row.as<uint32_t>();
         a.apc_val = ps.P == 1 ? ps.ap_val.as<V>() : ps.apc_val.as<V>();   // one panel: the same order
         a.lean_dense = narrow(ps) ? 1 : 0;
+        a.lean_walk = narrow_walk(ps) ? 1 : 0;
         // a chunk's stream is at most kSymChunk columns of A, each of at most
         // min(m, nnz(A)) entries
         a.lean_sym = a.lean_dense && std::min<int64_t>(ps.A.nrows, ps.A.nnz) * kSymChunk < (int64_t(1) << 31);
@@ -704,9 +705,11 @@ template <class I, class V> struct Engine : EngineBase {
     }
 
     // Whether the kernels with 32-bit entry offsets and stream positions may run: a
-    // walk looks up to kLeanSlack positions past the stream it is in.
-    static constexpr int64_t kLeanSlack = 8192;
-    static bool narrow(const PlanState &ps) { return ps.A.nnz < (int64_t(1) << 31) - kLeanSlack; }
+    // walk looks up to 8192 positions past the stream it is in, and those of light
+    // columns as far past the column of B (at most k entries).
+    static constexpr int64_t kLeanMost = (int64_t(1) << 31) - 8192;
+    static bool narrow(const PlanState &ps) { return ps.A.nnz < kLeanMost; }
+    static bool narrow_walk(const PlanState &ps) { return narrow(ps) && ps.k < kLeanMost; }
 
     // Columns above this many rows are heavy (k_sym_heavy32, k_num_heavy32),
     // unless the caller gave hash_max_cap. The largest table that fits a CTA
@@ -1643,7 +1646,7 @@ template <class I, class V> struct Engine : EngineBase {
             c.tier = t;
             const int T = 2 * tier_cap(t);
             if (t <= kWarpTiers) {
-                const bool lean = ga.gemm.lean_dense != 0;
+                const bool lean = ga.gemm.lean_walk != 0;
                 const int smem = 8 * T * (int)(4 + sizeof(V)) + (lean ? 8 * 32 * (int)(8 + sizeof(V)) : 0);
                 const int per_sm = std::max(1, std::min(8, (228 * 1024) / (smem + 1024)));
                 const int blocks = std::max(1, std::min((hist[t] + 7) / 8, cx.nsm * per_sm));

@@ -19,9 +19,11 @@
 //   heavy tier  : symbolic -- a shared-memory bitmap over up to ~1.5M rows;
 //                 numeric  -- dense accumulation of one row panel in shared
 //                 memory per CTA.
-// A product with nnz(A) < 2^31 runs its warp and block tiers in light_cols.cuh and
-// its heavy tier in sym_heavy32.cuh and dense_items.cuh; the kernels here serve the
-// merge and larger products.
+// A product runs its warp and block tiers in light_cols.cuh while nnz(A) and the inner
+// dimension are below 2^31 - 8192 (lean_walk), the heavy numeric tier in dense_items.cuh
+// while nnz(A) is (lean_dense), and the heavy symbolic in sym_heavy32.cuh while also min(m,
+// nnz(A)) * 1024 < 2^31 (lean_sym: up to 2^21 rows, or fewer entries). The kernels here
+// serve the merge, larger products, and unsorted columns of the largest table.
 // Hash tables are sort-free (Sec. IV-D): rows are emitted in table order, or in row
 // order straight from the table where the output is to be sorted (sort_smem.cuh).
 #pragma once
@@ -108,8 +110,9 @@ template <class I, class V> struct GemmArgs {
     const V *apc_val;
     const int32_t *prob_of;   // many problems: the problem of every global column, or null
     int whole;                // all of the inner dimension, not a stage of it
-    int lean_dense;           // heavy items may use 32-bit entry offsets (nnz(A) < 2^31)
-    int lean_sym;             // the heavy symbolic may use 32-bit stream positions too
+    int lean_dense;           // heavy items may use 32-bit entry offsets (nnz(A) < 2^31 - 8192)
+    int lean_walk;            // so may the walks of light columns (the inner dimension, too)
+    int lean_sym;             // so may the heavy symbolic's streams (min(m, nnz(A)) * 1024 < 2^31)
 };
 
 template <class I, class V> struct PartsArgs {
