@@ -56,6 +56,10 @@ __device__ __forceinline__ void bitonic(uint32_t *sk, V *sv, int n) {
     }
 }
 
+// The warp's network as a call: inlined, it spills the walks around it (k_light with
+// 256 int64 slots 28 -> 140 bytes, 2-path counts of 50,021 vertices 463 -> 485 us).
+template <class V> __device__ __noinline__ void bitonic_warp(uint32_t *sk, V *sv, int n) { bitonic<false>(sk, sv, n); }
+
 // A bucket above this many entries sends a CTA's (a warp's) table to the bitonic
 // sort: counting costs a bucket its square. Columns of clusters of consecutive rows far
 // apart, ranked however full a bucket is (up to 512 in a CTA) -> with these lines,
@@ -192,10 +196,10 @@ __device__ __forceinline__ void sort_front(uint32_t *keys, V *vals, int T, int n
             for (int i = t; i < n && i < want; i += nt) { out_rows[i] = (I)keys[i]; out_vals[i] = vals[i]; }
             return;
         }
-    } else if (shift > 7) {   // likewise
+    } else if (cap > kSortMaxBucketWarp && shift > 7) {   // likewise; cap is the caller's constant
         most = __reduce_max_sync(SPG_FULL, most);
         if (most > kSortMaxBucketWarp) {   // the same for the warp
-            bitonic<false>(keys, vals, n);
+            bitonic_warp(keys, vals, n);
             for (int i = t; i < n && i < want; i += nt) { out_rows[i] = (I)keys[i]; out_vals[i] = vals[i]; }
             return;
         }
