@@ -732,11 +732,13 @@ template <class I, class V> struct Engine : EngineBase {
     //   more panels, 4096: fp32 protein stand-in 20,011 / 100,000 columns 1.66 -> 1.49 /
     //     1.96 -> 1.71 and 10.0 -> 9.7 / 12.1 -> 11.8, R-MAT of 60,000 rows 7.24 -> 7.17 /
     //     8.02 -> 7.75; from about 500,000 rows on, the symbolic bitmaps leave one CTA per
-    //     SM. With 8-byte values only up to two panels (uniform 16,000 with 11,000
+    //     SM. With 8-byte values up to two panels (uniform 16,000 with 11,000 products
     //     3.10 -> 2.22 / 3.76 -> 2.24): the panels are half as wide, and a column of a few
     //     thousand rows is cut into as many items (uniform 40,000 with 7,500 rows a column
     //     0.98 -> 1.23 / 1.18 -> 1.23, 500,000 12.6 -> 16.5 / 15.2 -> 19.7, int64 40,000
-    //     0.90 -> 1.50 / 1.11 -> 1.51).
+    //     0.90 -> 1.50 / 1.11 -> 1.51); fp64 columns of many sizes up to eight (R-MAT of 17,000 rows
+    //     2.29 -> 1.96 / 2.46 -> 2.06, 40,000 5.78 -> 5.58 / 6.10 -> 5.85, 120,000 22.7 -> 22.6 /
+    //     24.6 -> 24.7), int64 ones not (30,000 2.77 -> 2.90 / 3.05 -> 3.09).
     // A k-split keeps 8192 (its stages read every heavy column again: 4-stage R-MAT 15
     // 8.07 -> 8.24 ms), and so does a product that the budget may cut into batches.
     static int heavy_rule(const PlanState &ps) {
@@ -746,7 +748,7 @@ template <class I, class V> struct Engine : EngineBase {
             while (cap < ps.cap_full && (int64_t)cap * 16 < ps.m) cap *= 2;
             return cap;
         }
-        const int64_t most = int64_t(1) << (sizeof(V) == 4 ? 19 : 14);
+        const int64_t most = int64_t(1) << (sizeof(V) == 4 ? 19 : kIntValue ? 14 : 16);
         return ps.m <= most ? std::min(ps.cap_full, 4096) : ps.cap_full;
     }
 
@@ -754,9 +756,11 @@ template <class I, class V> struct Engine : EngineBase {
     // spread (a variance of log2 of 1/3: a uniform graph's is below 0.1, R-MAT's and
     // the protein stand-in's 0.4 to 2.9), or they are many on average and in total. Each counts
     // up to kRuleMost and by its logarithm, so that a few hubs do not speak for the rest.
-    static bool lower_pays(const Above &a) {
+    static constexpr bool kIntValue = std::is_integral<typename Storage<V>::type>::value;
+    static bool lower_pays(const PlanState &ps, const Above &a) {
         const double n = (double)a.n, mean = a.n ? (double)a.lg / n : 0.0;
         const bool spread = (double)a.sq - n * mean * mean >= n * (64.0 * 64.0 / 3.0);
+        if (sizeof(V) == 8 && ps.m > (int64_t(1) << 14)) return spread;
         return spread || (a.sum >= 4096 * a.n && a.sum >= (int64_t(1) << 24));
     }
 
@@ -824,7 +828,7 @@ template <class I, class V> struct Engine : EngineBase {
         // the rule's cap stays where the columns above it gain by it and the flops
         // bound C to a single batch
         const auto recap = [&](int64_t flops, const Above &above) {
-            const bool keep = lower_pays(above) && one_batch(ps, flops);
+            const bool keep = lower_pays(ps, above) && one_batch(ps, flops);
             return cx.tun.hash_cap_max == ps.cap_full || keep ? cx.tun.hash_cap_max : ps.cap_full;
         };
         // full product: flops, counts, heavy list

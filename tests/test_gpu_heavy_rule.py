@@ -102,7 +102,10 @@ def test_cap_per_batch_is_the_fixed_lines(m, most, k, sort):
     (5000, torch.int64, [6], False), (5000, torch.int64, [7], True),
     # columns of several sizes, few products: 600 to 1,800 and 1,200 to 1,800
     (5000, torch.float32, [1, 1, 3], True), (5000, torch.float32, [2, 3], False),
-    # several panels: 4-byte values up to 2^19 rows, 8-byte ones up to two panels
+    # several panels: 4-byte values up to 2^19 rows, 8-byte ones up to two panels, and
+    # doubles of several sizes up to 2^16 rows
+    (40000, torch.float64, [6, 6, 22], True), (40000, torch.int64, [6, 6, 22], False),
+    (65537, torch.float64, [6, 6, 22], False),
     (40000, torch.float32, [8], True), (40000, torch.float64, [8], False), (40000, torch.int64, [8], False),
     (16384, torch.float64, [8], True), (16385, torch.float64, [8], False),
     ((1 << 19) + 1, torch.float32, [8], False)])
@@ -120,11 +123,12 @@ def test_lower_line_where_it_pays(m, vt, sizes, lower):
         for tuning in (None, spg.Tuning(hash_max_cap=8192)):
             plan = spg.Plan(A, B, budget=1 << 36, sort_output=True, tuning=tuning)
             info = plan.symbolic()
+            assert info["nbatches"] == 1
             out.append((info["heavy_columns"], info["batch_cap_bytes"], plan.numeric(0)))
             plan.check_errors()
             plan.close()
         (heavy, cap, C), (none, cap8, W) = out
-        assert none == 0 and (heavy > 0) == lower and cap == cap8
+        assert (heavy > none) == lower and cap == cap8
         assert torch.equal(C.colptr, W.colptr) and torch.equal(C.rowidx, W.rowidx) and torch.equal(C.vals, W.vals)
 
 
