@@ -753,13 +753,13 @@ template <class I, class V> struct Engine : EngineBase {
     }
 
     // Whether the columns above the lower line gain by it: their multiplications
-    // spread (a variance of log2 of 1/3: a uniform graph's is below 0.1, R-MAT's and
-    // the protein stand-in's 0.4 to 2.9), or they are many on average and in total. Each counts
+    // spread (a variance of log2 of 1/8: a uniform graph's is below 0.08, R-MAT's 0.4 to 2.9,
+    // the protein stand-in's 0.17 to 2.3), or they are many on average and in total. Each counts
     // up to kRuleMost and by its logarithm, so that a few hubs do not speak for the rest.
     static constexpr bool kIntValue = std::is_integral<typename Storage<V>::type>::value;
     static bool lower_pays(const PlanState &ps, const Above &a) {
         const double n = (double)a.n, mean = a.n ? (double)a.lg / n : 0.0;
-        const bool spread = (double)a.sq - n * mean * mean >= n * (64.0 * 64.0 / 3.0);
+        const bool spread = (double)a.sq - n * mean * mean >= n * (64.0 * 64.0 / 8.0);
         if (sizeof(V) == 8 && ps.m > (int64_t(1) << 14)) return spread;
         return spread || (a.sum >= 4096 * a.n && a.sum >= (int64_t(1) << 24));
     }

@@ -1,7 +1,7 @@
 // Light columns of a product, one warp each, with a warp-private hash table in
 // shared memory (C(:, j) = A * B(:, j), Sec. II-C's column formula): the
 // symbolic count and the numeric accumulation, with 32-bit entry offsets (the
-// caller guarantees nnz(A) < 2^31 less the look-ahead of a walk).
+// caller guarantees nnz(A) and the inner dimension < 2^31 less the look-ahead of a walk).
 //
 // A column of some hundred products is a chain of dependent loads (column
 // list, colptr of B, its rows, colptr of A, A's entries) around little work, so
@@ -24,10 +24,20 @@ template <class V> constexpr int light_smem(int T, int mode) {
     return 8 * (T + 32) * (4 + (mode == 1 ? (int)sizeof(V) : 0));
 }
 
+// CTAs per SM that the registers are fitted to (0: the compiler's choice): what the large
+// numeric tables leave room for, so that the walk is not spilled for CTAs that cannot come
+// (1024 int64 slots: 80 registers instead of 64 and 36 bytes spilled, numeric tiers of 77,906
+// vertices' 2-path counts 634 -> 611 us). Fewer for 512 8-byte slots costs more than the spills
+// (50,021 vertices 272 us, 303 with 3).
+template <class V> constexpr int light_min_ctas(int T, int mode) {
+    return mode == 0 ? 0 : T == 1024 ? 3 : T == 512 && sizeof(V) == 4 ? 5 : 0;
+}
+
 // MODE 0: symbolic (c.cnt[g]); MODE 1: numeric, rows in table order or
 // ascending (c.sort).
 template <class I, class V, int T, int MODE>
-__global__ void __launch_bounds__(256) k_light(GemmArgs<I, V> ga, TierCommon c, I *out_rows, V *out_vals) {
+__global__ void __launch_bounds__(256, light_min_ctas<V>(T, MODE))
+    k_light(GemmArgs<I, V> ga, TierCommon c, I *out_rows, V *out_vals) {
     constexpr int LOG2T = Log2<T>::v;
     constexpr int U = 4;   // windows whose loads are in flight
     // how a lane finds its segment: a shuffle search over the lanes, or one
