@@ -17,7 +17,7 @@
 //      a window crossing segment starts finds every lane's segment with one
 //      shared load per lane and one OR-reduce of the start bits;
 //   3. keeps the gathers of kDenseBatch windows in flight before applying them.
-// Offsets inside a panel are 32-bit (the caller guarantees nnz(A) < 2^31), so
+// Offsets inside a panel are 32-bit (the caller guarantees nnz(A) < 2^31 - 8192), so
 // the walk's bookkeeping is plain int arithmetic.
 //
 // Presence without a per-product flag: a row is taken as present when its

@@ -669,7 +669,8 @@ __device__ __forceinline__ void warp_walk_flat(const Src &src, Load &load, Apply
 }
 
 // ---------------------------------------------------------------------------
-// Shared-memory hash tables (linear probing, 32-bit keys)
+// Shared-memory hash tables (32-bit keys): hash_insert and hash_find probe linearly,
+// hash_insert_dbl and hash_insert_dbl1 by double hashing
 // ---------------------------------------------------------------------------
 
 // Insert key; returns its slot and sets is_new when this call claimed it.

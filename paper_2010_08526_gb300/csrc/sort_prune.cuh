@@ -4,7 +4,7 @@
 // only the intermediate products are left unsorted). The numeric kernels write
 // row order themselves (sort_smem.cuh, dense items by nature). Two sorts of
 // written output remain: the hash-range items of heavy columns where the generic
-// heavy kernel made them (the merge, nnz(A) >= 2^31; k_sort_items), and the pruned
+// heavy kernel made them (the merge, nnz(A) >= 2^31 - 8192; k_sort_items), and the pruned
 // columns of a batch (k_sort_cols).
 //
 // Prune: the consumer the column batches are shaped for keeps the largest
